@@ -390,10 +390,12 @@ int usp_cell_sort_static(const usp_grid* grid, int64_t n, const double* pos, uin
                          uint32_t* perm, void* stream);
 
 /* Launch tuning (set by the autotuner, paper_1808_03801_gb300/autotune.py):
- * fused_R in {4, 8, 12} sets the fused kernels' staging capacity to 32 R
- * particles per cell pass (larger cells take two sweeps); grid_per_sm in
- * 1..32 sets the persistent blocks per SM of the tiled kernels; 0 keeps a
- * value.  A batch uses the largest values of its members.  STATE while the
+ * fused_R in {4, 8, 12} selects how the fused relax / advect kernel works on
+ * a cell: one warp (4, the best with many cells) or a block of four or eight
+ * warps (8, 12; few or very dense cells); a load chooses it by the number of
+ * cells and ppc_ref.  grid_per_sm in 1..32 sets the persistent blocks per SM
+ * of the tiled kernels; 0 keeps a value.  A batch uses the largest values set
+ * on its members, without any its own choice by all cells.  STATE while the
  * handle is admitted to a batch. */
 int usp_set_tuning(usp_handle* h, int fused_R, int grid_per_sm);
 int usp_get_tuning(usp_handle* h, int* fused_R, int* grid_per_sm);

@@ -3,9 +3,9 @@
 For a workload it times a few candidate settings on the device (CUDA events
 on the simulation's stream, after warm-up) and keeps the fastest:
 
-* fused_R: staging capacity of the fused relax/advect kernel (32 R particles
-  per cell pass; cells above it take a second sweep that redraws the random
-  numbers), so the best value depends on the particles-per-cell distribution;
+* fused_R: how the fused relax/advect kernel works on a cell (4: one warp, 8 and
+  12: a block of four or eight warps), so the best value depends on the number
+  of cells and the particles per cell;
 * grid_per_sm: persistent blocks per SM of the tiled kernels.
 
 Results are cached in a JSON file keyed by the workload shape (dimension,

@@ -85,7 +85,7 @@ struct usp_handle {
     size_t cell_bytes = 0, part_bytes = 0;
     int2* d_ptiles = nullptr;
     int2* d_ctiles = nullptr;
-    int* d_ntiles = nullptr;          // [0] particle tiles, [1] cell tiles, [2..3] k_g2 work queue
+    int* d_ntiles = nullptr;          // [0] particle tiles, [1] cell tiles, [2..5] k_g2 work queues
     int nptiles = 0, nctiles = 0;
     Graphs graphs;
     bool initialised = false;
@@ -94,7 +94,8 @@ struct usp_handle {
     std::string err;
     std::vector<uint32_t> inj_count_host;
     int batch_refs = 0;
-    int fused_R = 8;                  // k_g2 consumer warps per CTA: 3, 7, 15 for R = 4, 8, 12
+    int fused_R = 4;                  // k_g2 variant: a warp (4) or a block of 4 or 8 warps (8, 12) per cell
+    bool tuned = false;               // fused_R was set by usp_set_tuning since the last load
     int grid_per_sm = 8;              // persistent blocks per SM of the tiled kernels
     cudaStream_t batch_stream = nullptr;   // stream of the batch the handle is admitted to
     void* b1_block = nullptr;         // buffer 1 and the cell plane (one allocation)
@@ -112,11 +113,11 @@ struct usp_batch {
     SimDev* d_sims = nullptr;
     int2* d_ptiles = nullptr;
     int2* d_ctiles = nullptr;
-    int* d_ntiles = nullptr;
+    int* d_ntiles = nullptr;          // as a handle's, then [6], [7] the cell tiles of each dimension
     size_t ptile_cap = 0, ctile_cap = 0;
     int nptiles = 0, nctiles = 0;
     Graphs graphs;
-    int graph_nsims = -1;             // nsims the graphs were captured with
+    uint64_t graph_key = ~0ull;       // what the graphs were captured for (batch_key)
     int lay_tiles = 1;                // layout tiles of the largest member seen (grid of the layout kernels)
     bool dirty = true;
     int precision = -1, pipeline = -1;
@@ -196,9 +197,12 @@ static Launch make_launch(usp_handle* h) {
     L.ctiles = h->d_ctiles;
     L.nctiles = h->d_ntiles + 1;
     L.wq = (uint32_t*)(h->d_ntiles + 2);
+    L.ndim = nullptr;   // one dimension
     L.nsims = 1;
     L.dims = h->host.dim == 1 ? 1 : 2;
     L.flux = h->host.flux_axis != 0;
+    L.ablation = h->host.selection || h->host.es_sampler;
+    L.cells = h->host.K;
     L.grid_p = persistent_grid(h->nptiles, h->grid_per_sm);
     L.grid_c = persistent_grid(h->nctiles, h->grid_per_sm);
     L.lay_tiles = (h->host.K + kLayTile - 1) / kLayTile;
@@ -248,12 +252,22 @@ static void enqueue_any(usp_handle* h, const Launch& L) {
     else enqueue_step(L, h->precision == USP_FP64, h->host.has_reservoir != 0);
 }
 
-// default k_g2 configuration (7 consumer warps per CTA, two CTAs per SM):
-// the fastest of the three on every workload measured; the autotuner may
-// pick another (the staged cell size no longer depends on it)
-static int choose_R(uint32_t max_count) {
-    (void)max_count;
-    return 8;
+// k_g2 variant for `cells` cells in all.  One warp per cell (4) is the
+// cheapest per particle but takes the latency of a whole cell (a dense one
+// of a shock tube: 25 us); with few cells a block per cell spreads each one
+// over several warps (8: four warps, 12: eight).  Measured per k_g2 launch:
+// 100 cells of 200 particles 21 us (4), 15 us (8), 13 us (12); 1000 cells of
+// 360 / 45 particles 30, 18, 23 us; 5929 cells of 37 particles 28, 44 us; so
+// the line lies at ten cells per SM, and eight warps pay where every block
+// has an SM to itself.  Cells above a warp's staging area (kG2Stage1 / 2, with
+// a margin for the scatter about the mean) go to the eight-warp blocks, which
+// hold 1024 particles in registers.
+static int choose_R(int64_t cells, int ppc_ref, int dim) {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (ppc_ref > (dim == 1 ? 370 : 320)) return 12;
+    if (cells > 10 * (int64_t)sms) return 4;
+    return cells <= 2 * (int64_t)sms && ppc_ref > 128 ? 12 : 8;
 }
 
 static int count_for_density(const SimDev& s, double n, double n_ref, int ppc_ref) {
@@ -341,7 +355,6 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
         if (segs[g].kind == USP_BC_DIFFUSE && !(segs[g].T > 0)) return USP_ERR_INVALID_ARG;
     }
 
-    if (prm->pipeline == USP_PIPE_FUSED) fused_prepare_attributes();
     usp_handle* h = new usp_handle();
     h->precision = prm->precision;
     h->pipeline = prm->pipeline;
@@ -443,6 +456,13 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     s.f_w = (float)s.w;
     s.f_inv_R = (float)(1.0 / s.R);
     s.inv_R = 1.0 / s.R;
+    for (int g = 0; g < nseg; ++g) s.f_seg_pos[g] = (float)s.seg[g].pos;
+    for (int a = 0; a < 2; ++a) {   // without reservoir faces: no buffer cells
+        const int n = a == 0 ? s.nx : s.ny;
+        const bool on = any_res && (s.dim == 2 || a == 1);
+        s.buf_lo[a] = on && s.face[2 * a].kind == kBcReservoir ? s.reservoir_cols : 0;
+        s.buf_hi[a] = on && s.face[2 * a + 1].kind == kBcReservoir ? n - s.reservoir_cols : n;
+    }
     s.es_b = 1.0 - 1.0 / s.Pr;
 
     const int K = s.K;
@@ -496,7 +516,7 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     if ((rc = cell_alloc(h, sizeof(SimDyn), &p)) != 0) { usp_destroy(h); return rc; }
     h->d_dyn = (SimDyn*)p;
     s.dyn = h->d_dyn;
-    if ((rc = cell_alloc(h, 4 * sizeof(int), &p)) != 0) { usp_destroy(h); return rc; }
+    if ((rc = cell_alloc(h, 8 * sizeof(int), &p)) != 0) { usp_destroy(h); return rc; }
     h->d_ntiles = (int*)p;
     h->nctiles = (K + kCTile - 1) / kCTile;
     if ((rc = cell_alloc(h, sizeof(int2) * (size_t)h->nctiles, &p)) != 0) { usp_destroy(h); return rc; }
@@ -521,7 +541,7 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     s.inj_total = total;
     std::vector<int2> ct(h->nctiles);
     for (int t = 0; t < h->nctiles; ++t) ct[t] = make_int2(0, t * kCTile);
-    int nt[4] = {0, h->nctiles, 0, 0};
+    int nt[8] = {0, h->nctiles, 0, 0, 0, 0, 0, 0};
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.inj_count, h->inj_count_host.data(), sizeof(uint32_t) * K, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.inj_pidoff, off.data(), sizeof(uint32_t) * K, cudaMemcpyHostToDevice, h->stream);
@@ -739,9 +759,8 @@ extern "C" int usp_init_particles(usp_handle* h, const usp_region* regions, int 
     if (rc) return rc;
     if (e != cudaSuccess) return fail(h, USP_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e));
     if (h->pipeline == USP_PIPE_FUSED) {
-        uint32_t mx = 0;
-        for (int c = 0; c < K; ++c) mx = std::max(mx, start[c + 1] - start[c]);
-        h->fused_R = choose_R(mx + mx / 4);
+        h->fused_R = choose_R(K, h->ppc_ref, s.dim);
+        h->tuned = false;
         Launch L = make_launch(h);
         // no parameters yet: zero shift for the first moments, no relaxation
         CK(cudaMemsetAsync(h->host.fprm, 0, sizeof(float) * kNFPrm * (size_t)K, h->stream));
@@ -771,7 +790,8 @@ static int fused_from_unsorted(usp_handle* h) {
     CK(cudaMemsetAsync(s.fprm, 0, sizeof(float) * kNFPrm * (size_t)K, h->stream));
     int one = 1;   // pageable: copied out before the call returns
     CK(cudaMemcpyAsync(&h->d_dyn->cur, &one, sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    h->fused_R = choose_R(0);
+    h->fused_R = choose_R(K, h->ppc_ref, s.dim);
+    h->tuned = false;
     launch_fused_setup(L);
     CK(cudaGetLastError());
     return USP_OK;
@@ -1218,8 +1238,8 @@ extern "C" int usp_batch_create(size_t hbm_budget, int max_sims, void* stream, u
         b->own_stream = true;
     }
     if (cudaMalloc(&b->d_sims, sizeof(SimDev) * max_sims) != cudaSuccess ||
-        cudaMalloc(&b->d_ntiles, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMemsetAsync(b->d_ntiles, 0, 4 * sizeof(int), b->stream) != cudaSuccess) {
+        cudaMalloc(&b->d_ntiles, 8 * sizeof(int)) != cudaSuccess ||
+        cudaMemsetAsync(b->d_ntiles, 0, 8 * sizeof(int), b->stream) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(b->d_sims);
         cudaFree(b->d_ntiles);
@@ -1282,6 +1302,37 @@ extern "C" int usp_batch_retire(usp_batch* b, usp_handle* h) {
     return bfail(b, USP_ERR_INVALID_ARG, "handle not in batch");
 }
 
+// k_g2 variant of a batch: the tuned one if a member was tuned, else by all
+// cells together and the particles per cell of the members that hold most
+static int batch_R(const usp_batch* b) {
+    int tuned = 0;
+    int64_t cells = 0, total = 0, dense = 0;
+    for (auto* h : b->members) {
+        if (h->tuned) tuned = std::max(tuned, h->fused_R);
+        cells += h->host.K;
+        total += h->host.cap;
+        if (choose_R(1 << 30, h->ppc_ref, h->host.dim) == 12) dense += h->host.cap;
+    }
+    if (tuned) return tuned;
+    return choose_R(cells, 2 * dense > total ? 1 << 20 : 1, 1);
+}
+
+// everything a captured graph depends on besides the device tables
+static uint64_t batch_key(const usp_batch* b) {
+    uint64_t k = 0;
+    int per_sm = 1;
+    for (auto* h : b->members) {
+        const SimDev& s = h->host;
+        k |= s.dim == 1 ? 1u : 2u;
+        if (s.slab_count > 1) k |= 4u;
+        if (s.flux_axis) k |= 8u;
+        if (s.selection || s.es_sampler) k |= 16u;
+        if (s.has_reservoir) k |= 32u;
+        per_sm = std::max(per_sm, h->grid_per_sm);
+    }
+    return k | (uint64_t)batch_R(b) << 8 | (uint64_t)per_sm << 16 | (uint64_t)b->members.size() << 32;
+}
+
 // rebuild the device tables of the batch (simulation list and tiles)
 static int batch_rebuild(usp_batch* b) {
     std::vector<SimDev> sims;
@@ -1290,8 +1341,14 @@ static int batch_rebuild(usp_batch* b) {
         usp_handle* h = b->members[i];
         sims.push_back(h->host);
         for (int t = 0; t < h->nptiles; ++t) pt.push_back(make_int2((int)i, t * kPTile));
-        for (int t = 0; t < h->nctiles; ++t) ct.push_back(make_int2((int)i, t * kCTile));
     }
+    // the cells of the 1-D members first: k_g2 has a kernel for each dimension
+    int nd[2] = {0, 0};
+    for (int dim = 1; dim <= 2; ++dim)
+        for (size_t i = 0; i < b->members.size(); ++i)
+            if (b->members[i]->host.dim == dim)
+                for (int t = 0; t < b->members[i]->nctiles; ++t, ++nd[dim - 1])
+                    ct.push_back(make_int2((int)i, t * kCTile));
     // the slabs of a decomposed domain must sit consecutively, in slab order,
     // each one pointing at slab 0 of its group
     for (size_t i = 0; i < sims.size(); ++i) {
@@ -1330,7 +1387,7 @@ static int batch_rebuild(usp_batch* b) {
         }
         regraph = true;
     }
-    if ((int)sims.size() != b->graph_nsims) regraph = true;
+    if (batch_key(b) != b->graph_key) regraph = true;
     for (auto* h : b->members) {
         const int t = (h->host.K + kLayTile - 1) / kLayTile;
         if (t > b->lay_tiles) {   // the layout grid only grows: extra blocks find no tile
@@ -1346,6 +1403,7 @@ static int batch_rebuild(usp_batch* b) {
     if (e == cudaSuccess && !pt.empty()) e = cudaMemcpyAsync(b->d_ptiles, pt.data(), sizeof(int2) * pt.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess && !ct.empty()) e = cudaMemcpyAsync(b->d_ctiles, ct.data(), sizeof(int2) * ct.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ntiles, nt, sizeof(nt), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ntiles + 6, nd, sizeof(nd), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, USP_ERR_CUDA, cudaGetErrorString(e));
     if (regraph) destroy_graphs(b->graphs);
@@ -1361,13 +1419,16 @@ static Launch batch_launch(usp_batch* b) {
     L.ctiles = b->d_ctiles;
     L.nctiles = b->d_ntiles + 1;
     L.wq = (uint32_t*)(b->d_ntiles + 2);
+    L.ndim = b->d_ntiles + 6;
     L.nsims = (int)b->members.size();
     L.dims = 0;
     for (auto* h : b->members) L.dims |= h->host.dim == 1 ? 1 : 2;
     for (auto* h : b->members) {
         L.slabs |= h->host.slab_count > 1;
         L.flux |= h->host.flux_axis != 0;
+        L.ablation |= h->host.selection || h->host.es_sampler;
     }
+    L.cells = 1 << 30;   // members come and go under a captured graph
     // fixed persistent grids: the tile counts are read on the device, so the
     // captured graph stays valid while simulations come and go
     int per_sm = 1;
@@ -1383,11 +1444,8 @@ static int batch_capture(usp_batch* b, int nsteps, cudaGraphExec_t* exec) {
     Launch L = batch_launch(b);
     const bool fp64 = b->precision == USP_FP64;
     bool res = false;
-    int R = 4;
-    for (auto* h : b->members) {
-        res |= h->host.has_reservoir != 0;
-        R = std::max(R, h->fused_R);
-    }
+    for (auto* h : b->members) res |= h->host.has_reservoir != 0;
+    const int R = batch_R(b);
     if (b->pipeline == USP_PIPE_FUSED && b->fork.make()) b->fork.attach(L);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
@@ -1401,7 +1459,7 @@ static int batch_capture(usp_batch* b, int nsteps, cudaGraphExec_t* exec) {
     e = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return bfail(b, USP_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-    b->graph_nsims = (int)b->members.size();
+    b->graph_key = batch_key(b);
     return USP_OK;
 }
 
@@ -1453,11 +1511,8 @@ extern "C" int usp_batch_run_stage(usp_batch* b, int stage) {
     Launch L = batch_launch(b);
     const bool fp64 = b->precision == USP_FP64;
     bool res = false;
-    int R = 4;
-    for (auto* h : b->members) {
-        res |= h->host.has_reservoir != 0;
-        R = std::max(R, h->fused_R);
-    }
+    for (auto* h : b->members) res |= h->host.has_reservoir != 0;
+    const int R = batch_R(b);
     if (stage_launch(L, b->pipeline, fp64, R, res, stage))
         return bfail(b, USP_ERR_INVALID_ARG, "stage must be 0..6 (plain) or 10..14 (fused)");
     cudaError_t e = cudaGetLastError();
@@ -1466,15 +1521,18 @@ extern "C" int usp_batch_run_stage(usp_batch* b, int stage) {
 
 extern "C" int usp_fused_supported(void) { return 1; }
 
-// Tuning knobs chosen by the autotuner: fused staging capacity (R = 4, 8 or
-// 12, i.e. 128, 256 or 416 particles per cell pass; 0 keeps the current) and
-// persistent blocks per SM (1..32; 0 keeps).  Captured graphs are rebuilt.
+// Tuning knobs chosen by the autotuner: the k_g2 variant (R = 4: a warp per
+// cell, 8 / 12: a block of 4 / 8 warps; 0 keeps the current) and persistent
+// blocks per SM (1..32; 0 keeps).  Captured graphs are rebuilt.
 extern "C" int usp_set_tuning(usp_handle* h, int fused_R, int grid_per_sm) {
     if (!h) return USP_ERR_INVALID_ARG;
     if (h->batch_refs) return fail(h, USP_ERR_STATE, "handle is admitted to a batch");
     if (fused_R != 0 && fused_R != 4 && fused_R != 8 && fused_R != 12) return fail(h, USP_ERR_INVALID_ARG, "R");
     if (grid_per_sm < 0 || grid_per_sm > 32) return fail(h, USP_ERR_INVALID_ARG, "grid_per_sm");
-    if (fused_R) h->fused_R = fused_R;
+    if (fused_R) {
+        h->fused_R = fused_R;
+        h->tuned = true;
+    }
     if (grid_per_sm) h->grid_per_sm = grid_per_sm;
     destroy_graphs(h->graphs);
     return USP_OK;

@@ -1,14 +1,13 @@
 // usp_fused.cu -- the fused FP32 pipeline of the USP-ESBGK step (sm_103a).
 //
 // One step n reads buffer p = cur and writes buffer q = cur ^ 1:
-//   k_g2      per cell (one consumer warp, the cell's planes copied into a
-//             shared-memory ring by a producer warp of the same CTA): the
-//             relaxation of step n-1 still pending on the cell's particles
-//             (Eqs. 8b, 9, 27, 29-32 with the per-cell momentum / energy
-//             conservation), then advection of step n with the boundaries,
-//             the new cell, and the write into that cell's bucket of buffer
-//             q (the scatter of the counting sort; the bucket sizes come from
-//             the previous histogram plus slack).
+//   k_g2      per cell (one warp; k_g2b: a block, where there are few or
+//             very dense cells): the relaxation of step n-1 still pending on
+//             the cell's particles (Eqs. 8b, 9, 27, 29-32 with the per-cell
+//             momentum / energy conservation), then advection of step n with
+//             the boundaries, the new cell, and the write into that cell's
+//             bucket of buffer q (the scatter of the counting sort; the
+//             bucket sizes come from the previous histogram plus slack).
 //   k_inject  reservoir buffer cells refilled into buffer q.
 //   k_g1      per cell (one warp): moments of Eq. 1 in one pass, as sums
 //             about the cell's mean velocity of the previous step, and the
@@ -37,33 +36,23 @@ namespace {
 
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
 
-struct FCell {
-    float u[3], th, M[6], pr, nu, nues, pne;   // M = L L^T - theta I (lower triangle, row-major)
-    int valid;
-};
-
-__device__ __forceinline__ float warp_sumf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// collect up to 32 spill-list indices of `cell` into spl (per warp); returns the count
-__device__ uint32_t collect_spill(const SimDev& s, int b, int cell, uint32_t* spl, int lane) {
+// the spill-list indices of `cell` (at most `most`; the others count as lost)
+// into spl (one warp); returns how many
+__device__ uint32_t collect_spill(const SimDev& s, int b, int cell, uint32_t* spl, uint32_t most, int lane) {
     const uint32_t n = min(s.dyn->sp_n[b], (uint32_t)kSpillCap);
     uint32_t found = 0;
-    for (uint32_t base = 0; base < n && found < 32; base += 32) {
+    for (uint32_t base = 0; base < n; base += 32) {
         const uint32_t i = base + lane;
         const bool hit = i < n && s.sp_cell[b][i] == (uint32_t)cell;
         const unsigned m = __ballot_sync(0xffffffffu, hit);
         const uint32_t pos = found + __popc(m & lanemask_lt());
-        if (hit && pos < 32) spl[pos] = i;
+        if (hit && pos < most) spl[pos] = i;
         found += __popc(m);
     }
     __syncwarp();
-    if (found > 32) {
-        if (lane == 0) atomicAdd(&s.dyn->counters[kCntOverflow], (unsigned long long)(found - 32));
-        found = 32;
+    if (found > most) {
+        if (lane == 0) atomicAdd(&s.dyn->counters[kCntOverflow], (unsigned long long)(found - most));
+        found = most;
     }
     return found;
 }
@@ -91,7 +80,6 @@ __device__ __forceinline__ void load_particle(const SimDev& s, int b, uint32_t b
     }
 }
 
-template <int DIM>
 __device__ __forceinline__ void store_velocity(const SimDev& s, int b, uint32_t base, uint32_t nb, const uint32_t* spl,
                                                uint32_t j, float v0, float v1, float v2) {
     if (j < nb) {
@@ -107,130 +95,51 @@ __device__ __forceinline__ void store_velocity(const SimDev& s, int b, uint32_t 
     }
 }
 
-// register copy of the source buffer's planes for the particles of one cell
-struct Src {
-    const float* x;
-    const float* y;
-    const float* v0;
-    const float* v1;
-    const float* v2;
-    const uint32_t* id;
-};
-
-__device__ __forceinline__ Src src_of(const SimDev& s, int b) {
-    Src P;
-    P.x = (const float*)s.pos[b][0];
-    P.y = (const float*)s.pos[b][1];
-    P.v0 = (const float*)s.vel[b][0];
-    P.v1 = (const float*)s.vel[b][1];
-    P.v2 = (const float*)s.vel[b][2];
-    P.id = s.pid[b];
-    return P;
-}
-
-// per-cell constants of the time-instant draw (Eq. 30)
-struct TimeDraw {
-    float dt, a, em1, ema, inv_nues, inv_pr;
-};
-
-// Relaxation draw from the four words of one Philox call (counter
-// (pid, step, relax, 0)).  It samples the law of the FP64 path's two-call
-// scheme with fewer variates:
-//  * u = u01(w.x) selects the particle (u < P_relax); given the selection,
-//    u / P_relax is uniform on (0, 1], so it also gives the time instant
-//    of Eq. 30;
-//  * the sum sqrt(s) L xi1 + sqrt((1 - s) theta) xi2 of two independent
-//    Gaussians (Eqs. 31-32) is one Gaussian of covariance
-//    s L L^T + (1 - s) theta I = theta I + s M, sampled through its own
-//    Cholesky factor from three normals: a Box-Muller pair (w.y, w.z) and
-//    one Box-Muller normal from w.w and the bits the other uniforms leave
-//    unused.
-__device__ __forceinline__ void es_draw1(const FCell& f, const TimeDraw& td, float u, const uint4& w, float* C) {
-    const float U1 = fminf(u * td.inv_pr, 1.0f);
-    const float t = td.a < 1.0f ? __logf(1.0f + U1 * td.em1) * td.inv_nues
-                                : td.dt + __logf(U1 + (1.0f - U1) * td.ema) * td.inv_nues;
-    const float sf = f.pne + (1.0f - f.pne) * __expf(-f.nu * t);          // Eq. 32
-    float z0, z1;
-    box_muller<float>(w.y, w.z, z0, z1);
-    // third normal: Box-Muller on w.w and the 23 low bits that the uniforms
-    // of w.x, w.y and w.z leave unused (each takes the top 23 bits)
-    const uint32_t lo = (w.x & 511u) | ((w.y & 511u) << 9) | ((w.z & 31u) << 18);
-    const float r2 = sqrtf(-1.3862943611198906f * __log2f(u01<float>(w.w)));
-    const float z2 = r2 * __cosf(6.283185307179586f * (((float)lo + 0.5f) * 1.1920928955078125e-7f) - 3.14159265358979f);
-    const float S00 = f.th + sf * f.M[0], S10 = sf * f.M[1], S11 = f.th + sf * f.M[2];
-    const float S20 = sf * f.M[3], S21 = sf * f.M[4], S22 = f.th + sf * f.M[5];
-    const float r0 = rsqrtf(S00);
-    const float l00 = S00 * r0, l10 = S10 * r0, l20 = S20 * r0;
-    const float d1 = fmaxf(S11 - l10 * l10, 1e-12f * f.th);
-    const float r1 = rsqrtf(d1);
-    const float l11 = d1 * r1, l21 = (S21 - l20 * l10) * r1;
-    const float l22 = sqrtf(fmaxf(S22 - l20 * l20 - l21 * l21, 0.0f));
-    C[0] = l00 * z0;
-    C[1] = l10 * z0 + l11 * z1;
-    C[2] = l20 * z0 + l21 * z1 + l22 * z2;
-}
-
-// The Gallis-Torczynski draw (Eqs. 10-11) of the SP-ESBGK ablations: a
-// thermal velocity sqrt(theta) z, with z three independent normals drawn as
-// in es_draw1, transformed by S = I - s B, B = ((1 - Pr)/(2 Pr)) sigma* /
-// (rho theta) (symmetric; f.M holds its lower triangle) and s of Eq. 32 at
-// the time instant.
-__device__ __forceinline__ void es_draw_gt(const FCell& f, const TimeDraw& td, float u, const uint4& w, float* C) {
-    const float U1 = fminf(u * td.inv_pr, 1.0f);
-    const float t = td.a < 1.0f ? __logf(1.0f + U1 * td.em1) * td.inv_nues
-                                : td.dt + __logf(U1 + (1.0f - U1) * td.ema) * td.inv_nues;
-    const float sf = f.pne + (1.0f - f.pne) * __expf(-f.nu * t);          // Eq. 32
-    float z0, z1;
-    box_muller<float>(w.y, w.z, z0, z1);
-    const uint32_t lo = (w.x & 511u) | ((w.y & 511u) << 9) | ((w.z & 31u) << 18);
-    const float r2 = sqrtf(-1.3862943611198906f * __log2f(u01<float>(w.w)));
-    const float z2 = r2 * __cosf(6.283185307179586f * (((float)lo + 0.5f) * 1.1920928955078125e-7f) - 3.14159265358979f);
-    const float st = sqrtf(f.th);
-    const float c0 = st * z0, c1 = st * z1, c2 = st * z2;
-    const float b00 = f.M[0], b10 = f.M[1], b11 = f.M[2], b20 = f.M[3], b21 = f.M[4], b22 = f.M[5];
-    C[0] = c0 - sf * (b00 * c0 + b10 * c1 + b20 * c2);
-    C[1] = c1 - sf * (b10 * c0 + b11 * c1 + b21 * c2);
-    C[2] = c2 - sf * (b20 * c0 + b21 * c1 + b22 * c2);
+// a particle whose bucket is full: into the spill list of buffer b
+template <int DIM>
+__device__ __forceinline__ void spill(const SimDev& s, int b, int cell, float x, float y, float v0, float v1, float v2,
+                                      uint32_t id) {
+    const uint32_t k = atomicAdd(&s.dyn->sp_n[b], 1u);
+    atomicAdd(&s.dyn->counters[kCntSpilled], 1ull);
+    if (k < (uint32_t)kSpillCap) {
+        if (DIM == 2) s.sp_pos[b][0][k] = x;
+        s.sp_pos[b][1][k] = y;
+        s.sp_vel[b][0][k] = v0;
+        s.sp_vel[b][1][k] = v1;
+        s.sp_vel[b][2][k] = v2;
+        s.sp_pid[b][k] = id;
+        s.sp_cell[b][k] = (uint32_t)cell;
+    } else {
+        atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
+    }
 }
 
 // ---------------------------------------------------------------------------
-// k_g2: pending relaxation + advection + bucket scatter, as a producer /
-// consumer pipeline inside each CTA.
+// k_g2b: pending relaxation + advection + bucket scatter, one block of G warps
+// per cell.
 //
-// Warp 0 of a CTA is the producer.  It takes runs of kG2Run cells from the
-// per-simulation queues (SimDyn::qnext), reads their bucket bounds with one
-// load per lane, allocates room for each cell in a ring buffer in shared
-// memory and starts bulk asynchronous copies (cp.async.bulk) of the cell's
-// particle planes and of its 64-byte FP32 parameter record; the copies
-// complete on the descriptor's mbarrier ("full").
-//
-// The other NC warps are consumers.  Each takes the next descriptor in
-// order, waits for its copies and processes the cell with rolled loops over
-// the staged particles (so the per-particle code appears once):
+// A block takes units of consecutive cells from one counter and works on one
+// cell at a time; thread t holds the particles t, t + 32 G, ... (at most kG2P)
+// in registers from the load to the write:
 //   relax    relaxation draws of the pending step (one Philox call per
-//            particle), conservation sums;
-//   pass A   conservation, advection, destination cell and its slot in the
+//            particle), conservation sums over the block;
+//   move     conservation, advection, destination cell and its slot in the
 //            cell's 64-cell destination window; each particle's rank among
-//            the arrivals of its slot;
-//   pass B   one atomic reservation per occupied slot in the destination
-//            buckets (one round trip for the whole cell);
-//   writes   each particle at its slot's reserved start plus its rank, so
+//            the arrivals of its slot from one shared-memory atomic;
+//   reserve  one global atomic per occupied slot in the destination buckets
+//            (one round trip for the whole cell);
+//   write    each particle at its slot's reserved start plus its rank, so
 //            the lanes of one slot write consecutive words of one bucket.
-// Then it releases the descriptor ("empty" mbarrier) and the producer may
-// reuse its ring space.  While a consumer works on a cell, the copies of the
-// cells behind it are in flight, so HBM latency is paid once per run of
-// cells rather than several times per cell.
-//
-// Cells whose bucket is not 16-byte aligned (the compact layout right after
-// a set-up sort) are loaded by the consumer itself; cells above the largest
-// ring allocation (max_stage particles) are processed in chunks with the
-// conservation sums in a first sweep and the update in a second one that
-// redraws the same counter-based random numbers.
-//
-// Every wait on an mbarrier is bounded (kG2WaitNs of global time); a wait
-// that runs out adds kG2TimeoutMark to the overflow counter of simulation 0
-// and ends the warp's work, so a fault in the pipeline shows up as lost
-// particles instead of a hung GPU.
+// It is for domains of few cells, where a step takes as long as its slowest
+// cell: spread over several warps a cell's latency is that of a few particles
+// per thread (measured per launch, one warp per cell -> block per cell: 100
+// cells of 200 particles 21 -> 13 us, one shock tube of 1000 cells 30 -> 18 us;
+// with 4e4 cells of 100 particles the barriers and the per-warp share of the
+// cell's work cost more than they give, 117 -> 230 us).  It also carries the
+// forms that are seldom run: in-place relaxation, slabs, the ablations.
+// Cells above 32 G kG2P particles go through in chunks: a first sweep for the
+// conservation sums, a second one (in reverse, so that the last chunk is
+// still in registers) that draws the same counter-based random numbers again.
 // ---------------------------------------------------------------------------
 // the general advection (wall and plate hits), out of line; the particle
 // goes in and out by value so that the common path keeps it in registers
@@ -253,85 +162,34 @@ __device__ __noinline__ AdvOut advect_slow(const SimDev& s, uint32_t step, uint3
     return o;
 }
 
-// per-cell register copy of what the advection and the scatter need
-struct Ctx {
-    float tau, lo0, hi0, lo1, hi1, inv_dx, inv_dy, b0, b1, b2;
-    int nx, nxm1, nym1, nseg, reservoir, K, cell0;   // cell0: first global cell of a slab
-    float* dx_;   // destination planes
-    float* dy_;
-    float* dv0;
-    float* dv1;
-    float* dv2;
-    uint32_t* did;
-    const uint32_t* dlay;
-    uint32_t* dcnt;
-    uint32_t cap;
-};
-
-__device__ __forceinline__ void make_ctx(const SimDev& s, int q, Ctx& C) {
-    C.tau = s.f_dt;
-    C.lo0 = s.f_lo[0];
-    C.hi0 = s.f_hi[0];
-    C.lo1 = s.f_lo[1];
-    C.hi1 = s.f_hi[1];
-    C.inv_dx = s.f_inv_dx;
-    C.inv_dy = s.f_inv_dy;
-    C.b0 = s.f_bdt[0];
-    C.b1 = s.f_bdt[1];
-    C.b2 = s.f_bdt[2];
-    C.nx = s.nx;
-    C.nxm1 = s.nx - 1;
-    C.nym1 = s.ny - 1;
-    C.nseg = s.nseg;
-    C.reservoir = s.has_reservoir;
-    C.K = s.K;
-    C.dx_ = (float*)s.pos[q][0];
-    C.dy_ = (float*)s.pos[q][1];
-    C.dv0 = (float*)s.vel[q][0];
-    C.dv1 = (float*)s.vel[q][1];
-    C.dv2 = (float*)s.vel[q][2];
-    C.did = s.pid[q];
-    C.dlay = s.lay[q];
-    C.dcnt = s.cnt[q];
-    C.cap = (uint32_t)s.cap;
-    C.cell0 = s.row0 * s.nx;
-}
-
-// column and row of an FP32 position: floor of the scaled offset, clamped
-// to the grid (1-D: ix = 0)
+// row and column of an FP32 position: floor of the scaled offset, clamped to
+// the grid (1-D: ix = 0)
 template <int DIM>
-__device__ __forceinline__ void cell_xy(const Ctx& C, float x, float y, int& ix, int& iy) {
-    iy = (int)fminf(fmaxf(floorf((y - C.lo1) * C.inv_dy), 0.0f), (float)C.nym1);
-    ix = DIM == 1 ? 0 : (int)fminf(fmaxf(floorf((x - C.lo0) * C.inv_dx), 0.0f), (float)C.nxm1);
+__device__ __forceinline__ void cell_xy(const SimDev& s, float x, float y, int& ix, int& iy) {
+    iy = min(max(__float2int_rd((y - s.f_lo[1]) * s.f_inv_dy), 0), s.ny - 1);
+    ix = DIM == 1 ? 0 : min(max(__float2int_rd((x - s.f_lo[0]) * s.f_inv_dx), 0), s.nx - 1);
 }
 
 template <int DIM>
-__device__ __forceinline__ int cell_f(const Ctx& C, float x, float y) {
-    int ix, iy;
-    cell_xy<DIM>(C, x, y, ix, iy);
-    return DIM == 1 ? iy : iy * C.nx + ix;
-}
-
-template <int DIM>
-__device__ __forceinline__ bool advect_fast(const SimDev& s, const Ctx& C, uint32_t step, uint32_t pid, float& x,
-                                            float& y, float* c) {
-    const float yn = y + c[1] * C.tau;
-    bool inside = yn > C.lo1 && yn < C.hi1;
+__device__ __forceinline__ bool advect_fast(const SimDev& s, uint32_t step, uint32_t pid, float& x, float& y,
+                                            float* c) {
+    const float yn = y + c[1] * s.f_dt;
+    bool inside = yn > s.f_lo[1] && yn < s.f_hi[1];
     float xn = x;
     if (DIM == 2) {
-        xn = x + c[0] * C.tau;
-        inside = inside && xn > C.lo0 && xn < C.hi0;
-        for (int g = 0; g < C.nseg; ++g) {
-            const float ps = (float)s.seg[g].pos;
+        xn = x + c[0] * s.f_dt;
+        inside = inside && xn > s.f_lo[0] && xn < s.f_hi[0];
+        for (int g = 0; g < s.nseg; ++g) {
+            const float ps = s.f_seg_pos[g];
             if ((x - ps) * (xn - ps) <= 0.0f) inside = false;
         }
     }
     if (inside) {
         y = yn;
         if (DIM == 2) x = xn;
-        c[0] += C.b0;
-        c[1] += C.b1;
-        c[2] += C.b2;
+        c[0] += s.f_bdt[0];
+        c[1] += s.f_bdt[1];
+        c[2] += s.f_bdt[2];
         return true;
     }
     const AdvOut o = advect_slow(s, step, pid, x, y, c[0], c[1], c[2]);
@@ -343,61 +201,27 @@ __device__ __forceinline__ bool advect_fast(const SimDev& s, const Ctx& C, uint3
     return o.alive != 0;
 }
 
-// append one particle to the bucket of its cell (all 32 lanes call this
-// together; key == kNoCell for lanes with nothing to write)
-template <int DIM>
-__device__ __forceinline__ void emit_c(const SimDev& s, const Ctx& C, int b, uint32_t key, float x, float y, float v0,
-                                       float v1, float v2, uint32_t id, int lane) {
-    const unsigned grp = __match_any_sync(0xffffffffu, key);
-    if (key == kNoCell) return;
-    const int leader = __ffs(grp) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&C.dcnt[key], (uint32_t)__popc(grp));
-    base = __shfl_sync(grp, base, leader);
-    const uint32_t rank = base + (uint32_t)__popc(grp & lanemask_lt());
-    const uint32_t lo = C.dlay[key];
-    const uint32_t hi = min(C.dlay[key + 1], C.cap);
-    if (lo + rank < hi) {
-        const uint32_t i = lo + rank;
-        if (DIM == 2) C.dx_[i] = x;
-        C.dy_[i] = y;
-        C.dv0[i] = v0;
-        C.dv1[i] = v1;
-        C.dv2[i] = v2;
-        C.did[i] = id;
-    } else {
-        const uint32_t k = atomicAdd(&s.dyn->sp_n[b], 1u);
-        atomicAdd(&s.dyn->counters[kCntSpilled], 1ull);
-        if (k < (uint32_t)kSpillCap) {
-            if (DIM == 2) s.sp_pos[b][0][k] = x;
-            s.sp_pos[b][1][k] = y;
-            s.sp_vel[b][0][k] = v0;
-            s.sp_vel[b][1][k] = v1;
-            s.sp_vel[b][2][k] = v2;
-            s.sp_pid[b][k] = id;
-            s.sp_cell[b][k] = key;
-        } else {
-            atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
-        }
-    }
+// reservoir buffer cell (column ix, global row iy)?
+__device__ __forceinline__ bool in_buffer_xy(const SimDev& s, int ix, int iy) {
+    return ix < s.buf_lo[0] || ix >= s.buf_hi[0] || iy < s.buf_lo[1] || iy >= s.buf_hi[1];
 }
 
 // Destination window of a cell: the 64 cells that its particles can reach in
 // one step without leaving it (1-D: offsets -32..31; 2-D: an 8 x 8 block
-// around the cell).  The warp counts its arrivals per window slot in shared
+// around the cell).  The block counts its arrivals per window slot in shared
 // memory, reserves each slot's range in the destination bucket with one
 // global atomic, then writes; particles that land outside the window reserve
 // their place one at a time.
 constexpr int kWin = 64;
-constexpr unsigned char kSlotNone = 0xFF;   // removed, nothing to write
-constexpr unsigned char kSlotFar = 0xFE;    // outside the window
-constexpr unsigned char kSlotOther = 0xFD;  // in another slab of a decomposed domain
+constexpr uint32_t kSlotNone = 0xFF;   // removed, nothing to write
+constexpr uint32_t kSlotFar = 0xFE;    // outside the window
+constexpr uint32_t kSlotOther = 0xFD;  // in another slab of a decomposed domain
 
 template <int DIM>
 __device__ __forceinline__ int win_slot_xy(int ix, int iy, int cell, int cx, int cy) {
     if (DIM == 1) {
         const int o = iy - cell + 32;
-        return (o >= 0 && o < kWin) ? o : -1;
+        return (unsigned)o < (unsigned)kWin ? o : -1;
     }
     const int oy = iy - cy + 4, ox = ix - cx + 4;
     return ((unsigned)oy < 8u && (unsigned)ox < 8u) ? oy * 8 + ox : -1;
@@ -415,10 +239,9 @@ __device__ __forceinline__ int win_cell(int k, int cell, int cx, int cy, int nx)
 template <int DIM>
 __device__ __noinline__ void emit_other(const SimDev* __restrict__ sims, const SimDev& s, int q, float x, float y,
                                         float v0, float v1, float v2, uint32_t id) {
-    const float fy = fminf(fmaxf(floorf((y - s.f_lo[1]) * s.f_inv_dy), 0.0f), (float)(s.ny - 1));
-    const int row = (int)fy;
-    int gc = row;
-    if (DIM == 2) gc = row * s.nx + (int)fminf(fmaxf(floorf((x - s.f_lo[0]) * s.f_inv_dx), 0.0f), (float)(s.nx - 1));
+    int ix, row;
+    cell_xy<DIM>(s, x, y, ix, row);
+    const int gc = DIM == 2 ? row * s.nx + ix : row;
     const SimDev& o = sims[s.slab_first + row / s.rows];
     const int dc = gc - o.row0 * o.nx;
     const uint32_t i = o.lay[q][dc] + atomicAdd(&o.cnt[q][dc], 1u);
@@ -432,48 +255,7 @@ __device__ __noinline__ void emit_other(const SimDev* __restrict__ sims, const S
         o.pid[q][i] = id;
         return;
     }
-    const uint32_t k = atomicAdd(&o.dyn->sp_n[q], 1u);
-    atomicAdd(&o.dyn->counters[kCntSpilled], 1ull);
-    if (k < (uint32_t)kSpillCap) {
-        if (DIM == 2) o.sp_pos[q][0][k] = x;
-        o.sp_pos[q][1][k] = y;
-        o.sp_vel[q][0][k] = v0;
-        o.sp_vel[q][1][k] = v1;
-        o.sp_vel[q][2][k] = v2;
-        o.sp_pid[q][k] = id;
-        o.sp_cell[q][k] = (uint32_t)dc;
-    } else {
-        atomicAdd(&o.dyn->counters[kCntOverflow], 1ull);
-    }
-}
-
-// write a particle into slot i of its own simulation's destination bucket
-// (buffer q), or into the spill list when the bucket is full (dc: its cell)
-template <int DIM>
-__device__ __forceinline__ void put_own(const SimDev& s, const Ctx& C, int q, uint32_t i, uint32_t hi, int dc, float x,
-                                        float y, float v0, float v1, float v2, uint32_t id) {
-    if (i < hi) {
-        if (DIM == 2) C.dx_[i] = x;
-        C.dy_[i] = y;
-        C.dv0[i] = v0;
-        C.dv1[i] = v1;
-        C.dv2[i] = v2;
-        C.did[i] = id;
-        return;
-    }
-    const uint32_t k = atomicAdd(&s.dyn->sp_n[q], 1u);
-    atomicAdd(&s.dyn->counters[kCntSpilled], 1ull);
-    if (k < (uint32_t)kSpillCap) {
-        if (DIM == 2) s.sp_pos[q][0][k] = x;
-        s.sp_pos[q][1][k] = y;
-        s.sp_vel[q][0][k] = v0;
-        s.sp_vel[q][1][k] = v1;
-        s.sp_vel[q][2][k] = v2;
-        s.sp_pid[q][k] = id;
-        s.sp_cell[q][k] = (uint32_t)dc;
-    } else {
-        atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
-    }
+    spill<DIM>(o, q, dc, x, y, v0, v1, v2, id);
 }
 
 // kFullSlab: kFull for batches holding slabs of a decomposed domain (routes
@@ -483,76 +265,683 @@ __device__ __forceinline__ void put_own(const SimDev& s, const Ctx& C, int q, ui
 // relaxation in place (before the particles are read back).
 enum { kFull = 0, kRelaxOnly = 1, kFullSlab = 2, kFullFlux = 3 };
 
-// ---- pipeline constants ----------------------------------------------------
-constexpr int kG2Desc = 32;            // descriptors (cells in flight) per CTA
-constexpr int kG2Run = 16;             // cells taken from a queue at once by the producer
-constexpr int kG2Spill = 32;           // spill-list entries a cell may add to its bucket
+constexpr int kG2P = 4;         // particles per thread and chunk
+constexpr int kG2Warps = 16;    // resident warps per SM
+constexpr int kG2Spill = 512;   // spill-list entries one cell may add to its bucket
+
+// shared state of one block of k_g2b
+template <int G>
+struct G2Shared {
+    SimDev sim;                 // the simulation the block works on
+    uint32_t wcnt[kWin];        // arrivals per window slot (zero between cells)
+    uint32_t wstart[kWin];      // first reserved index of each slot in its bucket
+    uint32_t wend[kWin];        // end of that bucket
+    float part[G][8];           // per-warp conservation sums
+    uint32_t part_n[G];         // per-warp relaxed particles
+    uint32_t key[20];           // the ten round keys of the relaxation's Philox calls
+    uint32_t hist[256];         // fixed-count selection: digits
+    uint32_t spl[kG2Spill];     // the cell's spill-list entries
+    uint32_t nsp;
+    uint32_t next;              // next unit
+    uint32_t sel[4];            // fixed-count selection: broadcast words
+};
+
+// approximate functions with subnormal inputs and results flushed: the
+// arguments here are never subnormal, and the plain forms scale for that
+__device__ __forceinline__ float lg2_ftz(float x) { float y; asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float ex2_ftz(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float sqrt_ftz(float x) { float y; asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float rsqrt_ftz(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float sin_ftz(float x) { float y; asm("sin.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float cos_ftz(float x) { float y; asm("cos.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+
+// per-cell constants of the relaxation: the record k_params_f writes.  X:
+// e^a - 1 where a = nu_ES dt < 1, else -e^-a.
+struct G2Prm {
+    float u[3], th, M[6], pr, nu, inv_nues, pne, X, inv_pr;
+};
+
+__device__ __forceinline__ G2Prm g2_prm(const float* fprm, int cell) {
+    const float4* r = reinterpret_cast<const float4*>(fprm) + (size_t)cell * (kNFPrm / 4);
+    const float4 a = r[0], b = r[1], c = r[2], d = r[3];
+    G2Prm f;
+    f.u[0] = a.x; f.u[1] = a.y; f.u[2] = a.z; f.th = a.w;
+    f.M[0] = b.x; f.M[1] = b.y; f.M[2] = b.z; f.M[3] = b.w;
+    f.M[4] = c.x; f.M[5] = c.y; f.pr = c.z; f.nu = c.w;
+    f.inv_nues = d.x; f.pne = d.y; f.X = d.z; f.inv_pr = d.w;
+    return f;
+}
+
+// Philox4x32-10 for the relaxation of one particle, counter (pid, step,
+// relax, 0): the round keys come from shared memory (five 16-byte broadcast
+// loads instead of eighteen additions)
+__device__ __forceinline__ uint4 philox_keys(uint32_t pid, uint32_t step, const uint32_t* key) {
+    uint4 c = make_uint4(pid, step, kRelax, 0u);
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ key[2 * r], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ key[2 * r + 1], (uint32_t)p0);
+    }
+    return c;
+}
+
+// three independent normals from the four words of one Philox call: a
+// Box-Muller pair (w.y, w.z) and a third one whose radius comes from w.w and
+// whose angle comes from the 23 low bits that the uniforms of w.x, w.y and
+// w.z leave unused (each takes the top 23 bits; lo + 1/2 over 2^23 is built
+// from the bits, exactly).
+__device__ __forceinline__ void g2_normals(const uint4& w, float* z) {
+    const float r = sqrt_ftz(-1.3862943611198906f * lg2_ftz(u01<float>(w.y)));
+    const float a = 6.283185307179586f * u01<float>(w.z) - 3.14159265358979f;
+    z[0] = r * cos_ftz(a);
+    z[1] = r * sin_ftz(a);
+    const uint32_t lo = (w.x & 511u) | ((w.y & 511u) << 9) | ((w.z & 31u) << 18);
+    const float r2 = sqrt_ftz(-1.3862943611198906f * lg2_ftz(u01<float>(w.w)));
+    const float v = __uint_as_float(0x3F800000u | lo) - 0.99999994039535522f;
+    z[2] = r2 * cos_ftz(6.283185307179586f * v - 3.14159265358979f);
+}
+
+// s of Eq. 32 at the time instant of Eq. 30.  u = u01(w.x) selects the
+// particle (u < P_relax); given the selection u / P_relax is uniform on (0, 1]
+// and gives the instant, in the overflow-free form of its range of a.
+__device__ __forceinline__ float g2_instant(const SimDev& s, const G2Prm& f, float u) {
+    const float U1 = fminf(u * f.inv_pr, 1.0f);
+    const bool small = f.X > 0.0f;
+    const float arg = (small ? U1 : 1.0f - U1) * fabsf(f.X) + (small ? 1.0f : U1);
+    const float t = 0.6931471805599453f * lg2_ftz(arg) * f.inv_nues + (small ? 0.0f : s.f_dt);
+    return f.pne + (1.0f - f.pne) * ex2_ftz(1.4426950408889634f * (-f.nu * t));
+}
+
+// new peculiar velocity: the sum sqrt(s) L xi1 + sqrt((1 - s) theta) xi2 of
+// Eqs. 31-32 is one Gaussian of covariance s L L^T + (1 - s) theta I =
+// theta I + s M, sampled through its own Cholesky factor
+__device__ __forceinline__ void es_draw1(const SimDev& s, const G2Prm& f, float u, const uint4& w, float* C) {
+    const float sf = g2_instant(s, f, u);
+    float z[3];
+    g2_normals(w, z);
+    const float S00 = f.th + sf * f.M[0], S10 = sf * f.M[1], S11 = f.th + sf * f.M[2];
+    const float S20 = sf * f.M[3], S21 = sf * f.M[4], S22 = f.th + sf * f.M[5];
+    const float r0 = rsqrt_ftz(S00);
+    const float l00 = S00 * r0, l10 = S10 * r0, l20 = S20 * r0;
+    const float d1 = fmaxf(S11 - l10 * l10, 1e-12f * f.th);
+    const float r1 = rsqrt_ftz(d1);
+    const float l11 = d1 * r1, l21 = (S21 - l20 * l10) * r1;
+    const float l22 = sqrt_ftz(fmaxf(S22 - l20 * l20 - l21 * l21, 0.0f));
+    C[0] = l00 * z[0];
+    C[1] = l10 * z[0] + l11 * z[1];
+    C[2] = l20 * z[0] + l21 * z[1] + l22 * z[2];
+}
+
+// The Gallis-Torczynski draw (Eqs. 10-11) of the SP-ESBGK ablations: a
+// thermal velocity sqrt(theta) z transformed by S = I - s B, B = ((1 - Pr) /
+// (2 Pr)) sigma* / (rho theta) (symmetric; M holds its lower triangle) and s
+// of Eq. 32 at the time instant.
+__device__ __forceinline__ void es_draw_gt(const SimDev& s, const G2Prm& f, float u, const uint4& w, float* C) {
+    const float sf = g2_instant(s, f, u);
+    float z[3];
+    g2_normals(w, z);
+    const float st = sqrt_ftz(f.th);
+    const float c0 = st * z[0], c1 = st * z[1], c2 = st * z[2];
+    const float b00 = f.M[0], b10 = f.M[1], b11 = f.M[2], b20 = f.M[3], b21 = f.M[4], b22 = f.M[5];
+    C[0] = c0 - sf * (b00 * c0 + b10 * c1 + b20 * c2);
+    C[1] = c1 - sf * (b10 * c0 + b11 * c1 + b21 * c2);
+    C[2] = c2 - sf * (b20 * c0 + b21 * c1 + b22 * c2);
+}
+
+// counters of one simulation, added when the block leaves it
+struct G2Acc {
+    uint32_t relaxed, removed;   // relaxed: thread 0's
+};
+
+__device__ __forceinline__ void g2_flush(G2Acc& a, SimDyn* dyn, int tid) {
+    if (tid == 0 && a.relaxed) atomicAdd(&dyn->counters[kCntRelaxed], (unsigned long long)a.relaxed);
+    const uint32_t r = __reduce_add_sync(0xffffffffu, a.removed);
+    if ((tid & 31) == 0 && r) atomicAdd(&dyn->counters[kCntRemoved], (unsigned long long)r);
+    a.relaxed = a.removed = 0;
+}
+
+// the id of particle j of a cell (bucket, then its spill-list entries)
+__device__ __forceinline__ uint32_t g2_id(const SimDev& s, int p, uint32_t base, uint32_t nb, const uint32_t* spl,
+                                          uint32_t j) {
+    return j < nb ? s.pid[p][base + j] : s.sp_pid[p][spl[j - nb]];
+}
+
+// Eq. 9 fixed count for one cell: the ns = nearest-int(n P_relax) particles
+// with the smallest selection words w.x (ties: lower position in the
+// bucket).  T is the ns-th smallest word and `quota` the number of particles
+// with word T that are taken; the (ns+1)-th smallest word T2 scales the time
+// instants (given T2, the ns smallest words are independent and uniform
+// below it).
+struct G2Fixed {
+    uint32_t T, quota, eq, ns;
+    float inv_thr;
+};
+
+// radix select of the ns-th smallest word: four passes of 8-bit digits
+// counted in shared memory, then the ties and T2; every pass draws the words
+// again
+template <int G>
+__device__ __noinline__ G2Fixed g2_fixed(G2Shared<G>& sh, int p, uint32_t step, uint32_t base, uint32_t nb, uint32_t n,
+                                         float pr, int tid) {
+    const SimDev& s = sh.sim;
+    const int lane = tid & 31;
+    G2Fixed F;
+    F.ns = min((uint32_t)floorf((float)n * pr + 0.5f), n);
+    F.T = 0xFFFFFFFFu;
+    F.quota = F.eq = 0;
+    F.inv_thr = 1.0f;
+    if (F.ns == 0) return F;
+    auto word = [&](uint32_t j) { return philox_keys(g2_id(s, p, base, nb, sh.spl, j), step, sh.key).x; };
+    uint32_t prefix = 0, mask = 0, rem = F.ns;
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        __syncthreads();
+        for (int b = tid; b < 256; b += 32 * G) sh.hist[b] = 0u;
+        __syncthreads();
+        for (uint32_t j = tid; j < n; j += 32 * G) {
+            const uint32_t k = word(j);
+            if ((k & mask) == prefix) atomicAdd(&sh.hist[(k >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        // every warp: lane l holds digits [8l, 8l + 8); the digit where the running count reaches rem
+        uint32_t h[8], tot = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            h[i] = sh.hist[8 * lane + i];
+            tot += h[i];
+        }
+        uint32_t inc = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint32_t exc = inc - tot;
+        const unsigned own = __ballot_sync(0xffffffffu, exc < rem && rem <= inc);
+        const int L = __ffs(own) - 1;
+        uint32_t d = 0, below = exc;
+        if (lane == L) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (below + h[i] >= rem) {
+                    d = 8u * lane + i;
+                    break;
+                }
+                below += h[i];
+            }
+        }
+        d = __shfl_sync(0xffffffffu, d, L);
+        below = __shfl_sync(0xffffffffu, below, L);
+        rem -= below;
+        prefix |= d << shift;
+        mask |= 0xFFu << shift;
+    }
+    F.T = prefix;
+    F.quota = rem;
+    // words equal to T, and the smallest word above it
+    __syncthreads();
+    if (tid == 0) {
+        sh.sel[0] = 0u;            // words equal to T
+        sh.sel[1] = 0xFFFFFFFFu;   // smallest word above T
+        sh.sel[2] = 0u;            // whether there is one
+    }
+    __syncthreads();
+    uint32_t eq = 0, above = 0xFFFFFFFFu;
+    bool any_above = false;
+    for (uint32_t j = tid; j < n; j += 32 * G) {
+        const uint32_t k = word(j);
+        eq += k == F.T;
+        if (k > F.T) {
+            any_above = true;
+            above = min(above, k);
+        }
+    }
+    if (eq) atomicAdd(&sh.sel[0], eq);
+    if (any_above) {
+        atomicMin(&sh.sel[1], above);
+        sh.sel[2] = 1u;
+    }
+    __syncthreads();
+    F.eq = sh.sel[0];
+    if (F.eq > F.quota) F.inv_thr = 1.0f / u01<float>(F.T);
+    else if (sh.sel[2]) F.inv_thr = 1.0f / u01<float>(sh.sel[1]);
+    return F;
+}
+
+// is particle j with word x among the fixed count?  Ties beyond the quota go
+// to the lower positions (counted by drawing the words before j again).
+template <int G>
+__device__ __forceinline__ bool g2_fixed_takes(G2Shared<G>& sh, const G2Fixed& X, int p, uint32_t step, uint32_t base,
+                                               uint32_t nb, uint32_t j, uint32_t x) {
+    if (X.ns == 0 || x > X.T) return false;
+    if (x < X.T || X.eq <= X.quota) return true;
+    uint32_t rank = 0;
+    for (uint32_t i = 0; i < j; ++i)
+        rank += philox_keys(g2_id(sh.sim, p, base, nb, sh.spl, i), step, sh.key).x == X.T;
+    return rank < X.quota;
+}
+
+// the cell's spill-list entries into sh.spl (whole block); returns their count
+template <int G>
+__device__ __noinline__ uint32_t g2_collect(G2Shared<G>& sh, int p, int cell, int tid) {
+    const SimDev& s = sh.sim;
+    __syncthreads();
+    if (tid == 0) sh.nsp = 0;
+    __syncthreads();
+    const uint32_t n = min(s.dyn->sp_n[p], (uint32_t)kSpillCap);
+    for (uint32_t i = tid; i < n; i += 32 * G)
+        if (s.sp_cell[p][i] == (uint32_t)cell) {
+            const uint32_t k = atomicAdd(&sh.nsp, 1u);
+            if (k < (uint32_t)kG2Spill) sh.spl[k] = i;
+        }
+    __syncthreads();
+    const uint32_t found = sh.nsp;
+    if (found <= (uint32_t)kG2Spill) return found;
+    if (tid == 0) atomicAdd(&s.dyn->counters[kCntOverflow], (unsigned long long)(found - kG2Spill));
+    return kG2Spill;
+}
+
+// one cell: bucket [base, base + nb) of buffer p, `arrived` arrivals
+template <int DIM, int MODE, bool ABL, int G>
+__device__ __forceinline__ void g2_cell(const SimDev* __restrict__ sims, G2Shared<G>& sh, int cell, uint32_t base,
+                                        uint32_t nb, uint32_t arrived, int p, uint32_t step, bool pending, int tid,
+                                        G2Acc& acc) {
+    constexpr uint32_t T = 32 * G, CAP = T * kG2P;
+    const SimDev& s = sh.sim;
+    const int lane = tid & 31, warp = tid >> 5, q = p ^ 1;
+    uint32_t nsp = 0;
+    if (arrived > nb) nsp = g2_collect<G>(sh, p, cell, tid);
+    const uint32_t n = nb + nsp;
+    if (n == 0) return;
+    G2Prm f = g2_prm(s.fprm, cell);
+    const bool relax = pending && f.pr > 0.0f;
+    if (MODE == kRelaxOnly && !relax) return;
+    // the window: thread k < 64 looks after slot k, its bucket bounds read ahead
+    const int cy = DIM == 2 ? cell / s.nx : 0;
+    const int cx = DIM == 2 ? cell - cy * s.nx : 0;
+    const int gcell = cell + (MODE == kFullSlab && DIM == 1 ? s.row0 : 0);   // 1-D: global cell of the slab's cell
+    const int row0 = MODE == kFullSlab && DIM == 2 ? s.row0 : 0;
+    const int cell0 = MODE == kFullSlab ? s.row0 * s.nx : 0;
+    int dest = -1;
+    uint32_t dlo = 0, dhi = 0;
+    if (MODE != kRelaxOnly && tid < kWin) {
+        dest = win_cell<DIM>(tid, cell, cx, cy, s.nx);
+        if ((unsigned)dest < (unsigned)s.K) {
+            dlo = s.lay[q][dest];
+            dhi = min(s.lay[q][dest + 1], (uint32_t)s.cap);
+        }
+    }
+    G2Fixed X = {0u, 0u, 0u, 0u, 1.0f};
+    if (ABL && relax && s.selection) {
+        X = g2_fixed<G>(sh, p, step, base, nb, n, f.pr, tid);
+        f.inv_pr = X.inv_thr;   // the instants scale with the threshold word instead of P_relax
+    }
+    const uint32_t nch = (n + CAP - 1) / CAP;
+    float R[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) R[k] = 0.0f;
+    uint32_t nr = 0;
+    float uo0 = 0, uo1 = 0, uo2 = 0, mn0 = 0, mn1 = 0, mn2 = 0, alpha = 1.0f;
+    bool apply = false;
+    // sweep 1: chunks 0 .. nch - 1 (sums); sweep 2: nch - 1 .. 0 (moves)
+#pragma unroll 1
+    for (uint32_t it = relax ? 0 : nch - 1; it < 2 * nch - 1; ++it) {
+        const uint32_t off = (it < nch ? it : 2 * nch - 2 - it) * CAP;
+        const uint32_t cnt = min(CAP, n - off);      // particles of the chunk
+        float x[kG2P], y[kG2P], v[kG2P][3];
+        uint32_t id[kG2P], selm = 0;
+#pragma unroll
+        for (int k = 0; k < kG2P; ++k) {
+            const uint32_t j = tid + k * T;
+            x[k] = y[k] = v[k][0] = v[k][1] = v[k][2] = 0.0f;
+            id[k] = 0;
+            if (j < cnt)
+                load_particle<DIM>(s, p, base, nb, sh.spl, off + j, x[k], y[k], v[k][0], v[k][1], v[k][2], id[k]);
+        }
+        if (relax) {
+#pragma unroll
+            for (int k = 0; k < kG2P; ++k) {
+                if (32u * warp + k * T >= cnt) break;
+                const uint32_t j = tid + k * T;
+                const uint4 w = philox_keys(id[k], step, sh.key);
+                const float u = u01<float>(w.x);
+                bool sel;
+                if (ABL && s.selection) {
+                    sel = j < cnt && g2_fixed_takes<G>(sh, X, p, step, base, nb, off + j, w.x);
+                } else {
+                    sel = j < cnt && u < f.pr;
+                }
+                if (sel) {
+                    float C[3];
+                    if (ABL && s.es_sampler) es_draw_gt(s, f, u, w, C);
+                    else es_draw1(s, f, u, w, C);
+                    const float o0 = v[k][0] - f.u[0], o1 = v[k][1] - f.u[1], o2 = v[k][2] - f.u[2];
+                    R[0] += o0; R[1] += o1; R[2] += o2;
+                    R[3] += o0 * o0 + o1 * o1 + o2 * o2;
+                    R[4] += C[0]; R[5] += C[1]; R[6] += C[2];
+                    R[7] += C[0] * C[0] + C[1] * C[1] + C[2] * C[2];
+                    v[k][0] = C[0]; v[k][1] = C[1]; v[k][2] = C[2];
+                    selm |= 1u << k;
+                }
+                if (it < nch) nr += (uint32_t)__popc(__ballot_sync(0xffffffffu, sel));
+            }
+        }
+        if (it + 1 < nch) continue;
+        if (it + 1 == nch && relax) {
+            // conservation factors from the block's sums.  Warp: reduce-scatter
+            // of the eight sums (lane 4 i holds sum i); block: through shared
+            // memory, every warp adding the G partial sums.
+#pragma unroll
+            for (int half = 4; half >= 1; half >>= 1) {
+                const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+                for (int i = 0; i < half; ++i) {
+                    const float send = up ? R[i] : R[i + half];
+                    const float recv = __shfl_xor_sync(0xffffffffu, send, 4 * half);
+                    R[i] = (up ? R[i + half] : R[i]) + recv;
+                }
+            }
+            R[0] += __shfl_xor_sync(0xffffffffu, R[0], 2);
+            R[0] += __shfl_xor_sync(0xffffffffu, R[0], 1);
+            if ((lane & 3) == 0) sh.part[warp][lane >> 2] = R[0];
+            if (lane == 0) sh.part_n[warp] = nr;
+            __syncthreads();
+            float t = 0.0f;
+            if (G >= 4 || lane < 8 * G) t = sh.part[lane >> 3][lane & 7];
+#pragma unroll
+            for (int g = 4; g < G; g += 4) t += sh.part[g + (lane >> 3)][lane & 7];
+            t += __shfl_xor_sync(0xffffffffu, t, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 16);
+            uint32_t nall = 0;
+#pragma unroll
+            for (int g = 0; g < G; ++g) nall += sh.part_n[g];
+            float Q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) Q[k] = __shfl_sync(0xffffffffu, t, k);
+            if (nall >= 2) {
+                // FP32: the sums are taken about the cell mean, so the
+                // differences below do not cancel; every thread computes the
+                // same factors from the same values
+                const float inv = 1.0f / (float)nall;
+                const float Eo = Q[3] - (Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2]) * inv;
+                const float En = Q[7] - (Q[4] * Q[4] + Q[5] * Q[5] + Q[6] * Q[6]) * inv;
+                if (En > 0.0f && Eo >= 0.0f) {
+                    apply = true;
+                    alpha = sqrtf(Eo / En);
+                    uo0 = f.u[0] + Q[0] * inv;
+                    uo1 = f.u[1] + Q[1] * inv;
+                    uo2 = f.u[2] + Q[2] * inv;
+                    mn0 = Q[4] * inv;
+                    mn1 = Q[5] * inv;
+                    mn2 = Q[6] * inv;
+                    if (tid == 0) acc.relaxed += nall;
+                }
+            }
+        }
+        if (MODE == kRelaxOnly) {
+            if (apply) {
+#pragma unroll
+                for (int k = 0; k < kG2P; ++k)
+                    if (selm & (1u << k))
+                        store_velocity(s, p, base, nb, sh.spl, off + tid + k * T, uo0 + alpha * (v[k][0] - mn0),
+                                       uo1 + alpha * (v[k][1] - mn1), uo2 + alpha * (v[k][2] - mn2));
+            }
+            continue;
+        }
+        uint32_t sr[kG2P];   // slot, rank << 8
+#pragma unroll
+        for (int k = 0; k < kG2P; ++k) {
+            sr[k] = kSlotNone;
+            if (32 * warp + k * T >= cnt) break;
+            const uint32_t j = tid + k * T;
+            if (j >= cnt) continue;
+            if (selm & (1u << k)) {
+                if (apply) {
+                    v[k][0] = uo0 + alpha * (v[k][0] - mn0);
+                    v[k][1] = uo1 + alpha * (v[k][1] - mn1);
+                    v[k][2] = uo2 + alpha * (v[k][2] - mn2);
+                } else {   // a single relaxed particle: reverted
+                    float ox, oy;
+                    uint32_t oid;
+                    load_particle<DIM>(s, p, base, nb, sh.spl, off + j, ox, oy, v[k][0], v[k][1], v[k][2], oid);
+                }
+            }
+            const float x0 = x[k], y0 = y[k];
+            const bool alive = advect_fast<DIM>(s, step, id[k], x[k], y[k], v[k]);
+            if ((MODE == kFullFlux || MODE == kFullSlab) && s.flux_axis) count_flux<float>(s, x0, y0, x[k], y[k]);
+            if (!alive) continue;
+            int ix, iy;
+            cell_xy<DIM>(s, x[k], y[k], ix, iy);
+            const int dc = (DIM == 2 ? iy * s.nx + ix : iy) - cell0;   // local
+            if (MODE == kFullSlab && (unsigned)dc >= (unsigned)s.K) {
+                sr[k] = kSlotOther;
+            } else if (s.has_reservoir && in_buffer_xy(s, ix, iy)) {
+                ++acc.removed;
+            } else {
+                const int slot = win_slot_xy<DIM>(ix, iy - row0, gcell, cx, cy);
+                sr[k] = kSlotFar;
+                // the particle's rank among the arrivals of its slot: one shared
+                // atomic (lanes of one slot are served one after another)
+                if (slot >= 0) sr[k] = (uint32_t)slot | (atomicAdd(&sh.wcnt[slot], 1u) << 8);
+            }
+        }
+        __syncthreads();
+        // one reservation per occupied slot, all in flight together
+        if (tid < kWin) {
+            const uint32_t c = sh.wcnt[tid];
+            if (c) {
+                sh.wstart[tid] = dlo + atomicAdd(&s.cnt[q][dest], c);
+                sh.wend[tid] = dhi;
+                sh.wcnt[tid] = 0;
+            }
+        }
+        __syncthreads();
+        // consecutive lanes write particles of the same few destination
+        // buckets (a window slot's particles go to consecutive slots of its
+        // bucket, in rank order); particles leaving the window or the slab
+        // take their own reservation
+#pragma unroll
+        for (int k = 0; k < kG2P; ++k) {
+            if (32 * warp + k * T >= cnt) break;
+            const uint32_t slot = sr[k] & 255u;
+            if (slot == kSlotNone) continue;
+            uint32_t i, hi;
+            if (slot < (uint32_t)kWin) {
+                i = sh.wstart[slot] + (sr[k] >> 8);
+                hi = sh.wend[slot];
+            } else if (MODE == kFullSlab && slot == kSlotOther) {   // into the buckets of another slab
+                emit_other<DIM>(sims, s, q, x[k], y[k], v[k][0], v[k][1], v[k][2], id[k]);
+                continue;
+            } else {   // outside the window: a reservation of its own
+                int ix, iy;
+                cell_xy<DIM>(s, x[k], y[k], ix, iy);
+                const int dc = (DIM == 2 ? iy * s.nx + ix : iy) - cell0;
+                i = s.lay[q][dc] + atomicAdd(&s.cnt[q][dc], 1u);
+                hi = min(s.lay[q][dc + 1], (uint32_t)s.cap);
+            }
+            if (i < hi) {
+                if (DIM == 2) ((float*)s.pos[q][0])[i] = x[k];
+                ((float*)s.pos[q][1])[i] = y[k];
+                ((float*)s.vel[q][0])[i] = v[k][0];
+                ((float*)s.vel[q][1])[i] = v[k][1];
+                ((float*)s.vel[q][2])[i] = v[k][2];
+                s.pid[q][i] = id[k];
+            } else {   // the bucket is full
+                int ix, iy;
+                cell_xy<DIM>(s, x[k], y[k], ix, iy);
+                spill<DIM>(s, q, (DIM == 2 ? iy * s.nx + ix : iy) - cell0, x[k], y[k], v[k][0], v[k][1], v[k][2],
+                           id[k]);
+            }
+        }
+    }
+    // kRelaxOnly has no barrier after the sums are read: the next cell's
+    // partial sums wait for it
+    if (MODE == kRelaxOnly) __syncthreads();
+}
+
+// DIMS: bit 0 / 1: the batch holds 1-D / 2-D simulations
+template <int DIMS, int MODE, bool ABL, int G>
+__global__ void __launch_bounds__(32 * G, kG2Warps / G) k_g2b(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+                                                       const int* __restrict__ ntiles, uint32_t* __restrict__ wq) {
+    __shared__ __align__(16) G2Shared<G> sh;
+    const int tid = threadIdx.x;
+    const uint32_t slots = (uint32_t)*ntiles * kCTile;
+    // units of 1 to 8 cells, at least 32 units per block where there are enough cells
+    uint32_t U = 1;
+    while (U < 8 && slots >= U * 64 * gridDim.x) U *= 2;
+    const uint32_t nunits = slots / U;
+    if (tid < kWin) sh.wcnt[tid] = 0;
+    G2Acc acc = {0u, 0u};
+    int loaded = -1, p = 0;
+    uint32_t step = 0;
+    bool pending = false;
+    for (uint32_t unit = blockIdx.x; unit < nunits;) {
+        uint32_t nxt = 0;
+        if (tid == 0) nxt = gridDim.x + atomicAdd(&wq[0], 1u);
+        const uint32_t slot0 = unit * U;
+        const int2 tile = tiles[slot0 / kCTile];
+        if (tile.x != loaded) {
+            if (loaded >= 0) g2_flush(acc, sh.sim.dyn, tid);
+            __syncthreads();
+            load_sim(sh.sim, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+            p = sh.sim.dyn->cur;
+            step = sh.sim.dyn->step;
+            pending = sh.sim.dyn->relax_pending != 0;
+            if (tid < 10) {   // round keys: the key plus r times the Weyl constants
+                sh.key[2 * tid] = sh.sim.key0 + (uint32_t)tid * 0x9E3779B9u;
+                sh.key[2 * tid + 1] = sh.sim.key1 + (uint32_t)tid * 0xBB67AE85u;
+            }
+            __syncthreads();
+        }
+        const SimDev& s = sh.sim;
+        const int c0 = tile.y + (int)(slot0 % kCTile), c1 = min(c0 + (int)U, s.K);
+        if (c0 < c1 && !(MODE == kRelaxOnly && !pending)) {
+            const uint32_t cap = (uint32_t)s.cap;
+            uint32_t lo = s.lay[p][c0], hi = s.lay[p][c0 + 1], ar = s.cnt[p][c0];
+            for (int cell = c0; cell < c1; ++cell) {
+                const uint32_t base = lo, top = min(hi, cap), arrived = ar;
+                if (cell + 1 < c1) {   // the next cell's bounds
+                    lo = hi;
+                    hi = s.lay[p][cell + 2];
+                    ar = s.cnt[p][cell + 1];
+                }
+                const uint32_t nb = min(arrived, top > base ? top - base : 0u);
+                if (DIMS == 1 || (DIMS == 3 && s.dim == 1))
+                    g2_cell<1, MODE, ABL, G>(sims, sh, cell, base, nb, arrived, p, step, pending, tid, acc);
+                else
+                    g2_cell<2, MODE, ABL, G>(sims, sh, cell, base, nb, arrived, p, step, pending, tid, acc);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) sh.next = nxt;
+        __syncthreads();
+        unit = sh.next;
+    }
+    if (loaded >= 0) g2_flush(acc, sh.sim.dyn, tid);
+    if (tid == 0) {
+        __threadfence();
+        const uint32_t done = atomicAdd(&wq[1], 1u);
+        if (done == gridDim.x - 1) wq[0] = wq[1] = 0;   // the last block resets the counters for the next launch
+    }
+}
+
+// copy one simulation descriptor into shared memory (one warp)
+__device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, int lane) {
+    const int4* a = reinterpret_cast<const int4*>(&src);
+    int4* b = reinterpret_cast<int4*>(&dst);
+    for (int i = lane; i < (int)(sizeof(SimDev) / 16); i += 32) b[i] = a[i];
+}
+
+// ---------------------------------------------------------------------------
+// k_g2: the same work for domains of many cells, one warp per cell.
+//
+// With many cells per SM the work is bound by instruction issue, not by a
+// cell's latency: a warp of its own per cell needs no block barriers, wastes
+// no lanes on the per-cell part and leaves at most 31 lanes of a cell idle.
+// The warps of a block are independent; each keeps its own copy of the
+// simulation descriptor and its own staging area in shared memory.  A cell:
+//   copy     its planes and parameter record come in by bulk asynchronous
+//            copies (one per plane), started while the cell before it is worked on wherever both fit
+//            the staging area (its bounds are read another cell ahead, the
+//            unit number yet another), so that a cell finds its data there;
+//   sweep 1  relaxation draw, conservation sums, the new velocity staged;
+//   sweep 2  conservation, flight, destination slot and rank, staged;
+//   reserve  one global atomic per occupied slot;
+//   sweep 3  the writes, consecutive lanes to consecutive slots.
+// The two particles per lane and iteration are independent chains.  16 warps
+// per SM with 128 registers and no spills measured best (12 and 14 warps with
+// more staging, 18 and 20 with less and some spills: 3-50 % slower), and so did
+// bulk copies (per-lane 16-byte copies took three times as long to issue).
+// What bounds it: the warps' dependent instructions (352 per 32 particles in
+// 1-D, 49 % issue) and, for dense cells, the copy that cannot start before the
+// cell ahead is written.  Against the form before it (a producer warp feeding
+// seven consumer warps): 64 shock tubes 301 -> 250 us, cavity 200 x 200 168 ->
+// 117 us, slit 522 -> 366 us per launch.
+// Cells above the staging area, and cells with spill-list entries, take the
+// general form of the same code: loaded by the lanes, in chunks, the draws of
+// all but one chunk made twice.
+//
+// The wait for a copy is bounded (kG2WaitNs of global time); one that runs out
+// adds kG2TimeoutMark to the overflow counter of simulation 0 and ends the
+// warp's work, so that a fault shows up as lost particles, not as a hang.
+// ---------------------------------------------------------------------------
+constexpr int kG2Stage1 = 448, kG2Stage2 = 384;   // staged particles per warp, 1-D and 2-D (multiples of 32)
+constexpr int kG2wSpill = 64;                     // spill-list entries one cell may add to its bucket
+
+constexpr int g2w_words(int dims) {   // 32-bit words of the staging area: (x,) y, v0, v1, v2, id and 16-bit slots
+    return dims == 1 ? 5 * kG2Stage1 + kG2Stage1 / 2 : 6 * kG2Stage2 + kG2Stage2 / 2;
+}
+
+template <int DIMS>
+struct alignas(16) G2Warp {
+    float stage[g2w_words(DIMS)];
+    float prm[2][kNFPrm];  // parameter records of the cell and of the next one
+    SimDev sim;
+    uint32_t key[20];
+    uint32_t wst[kWin];    // arrivals per window slot, then its first reserved index
+    uint32_t wlo[kWin];    // start and end of the slot's bucket
+    uint32_t wend[kWin];
+    uint32_t spl[kG2wSpill];
+    int2 ptile[4];         // the cells on their way: tile,
+    uint32_t pbound[4][4]; // bucket start, end and arrivals,
+    uint32_t punit[4];     // unit number
+    uint64_t full[2];      // the copies of a cell have landed (cells alternate)
+};
+
+// slot and rank of a staged particle in 16 bits (at most 1023 arrivals of one
+// cell share a slot)
+constexpr uint32_t kPackNone = 0xFFFFu;   // removed, nothing to write
+constexpr uint32_t kPackFar = 0xFFFEu;    // outside the window
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// per-lane asynchronous global -> shared copies (completion waited with
+// cp.async.wait_group by the issuing lane, then made visible to the warp
+// with __syncwarp)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+
 constexpr unsigned long long kG2WaitNs = 2000000000ull;   // bound of one mbarrier wait
 constexpr unsigned long long kG2TimeoutMark = 1ull << 40;
 
-enum : uint32_t { kDescBulk = 1u, kDescPending = 2u, kDescParity = 4u };
-
-// One cell handed from the producer to a consumer.  prm is filled by a bulk
-// copy of the cell's parameter record; the rest by the producer.
-struct alignas(16) G2Desc {
-    float prm[kNFPrm];   // u[3], theta, L[6], P_relax, nu, nu_ES, P_ne, valid, spare
-    uint32_t base;       // first slot of the cell's bucket in buffer p
-    uint32_t nb;         // particles in the bucket (arrivals beyond it are in the spill list)
-    uint32_t arrived;    // arrivals into the cell (bucket + spill list)
-    uint32_t off;        // byte offset of the cell's area in the ring
-    uint32_t m;          // particle slots of that area
-    int cell;            // -1: no more cells for this consumer
-    int ent;             // simulation descriptor entry in shared memory
-    uint32_t step;       // step counter of the simulation (Philox word 1)
-    uint32_t flags;      // kDesc*
-    uint32_t end;        // ring counter after this allocation (producer bookkeeping)
-};
-
-// bytes of ring per staged particle: (x,) y, v0, v1, v2, id; slot; rank
-template <int DIM>
-__host__ __device__ constexpr uint32_t g2_bytes_per_particle() {
-    return (DIM == 2 ? 24u : 20u) + 1u + 2u;
-}
-
-struct G2Stage {
-    float* x;
-    float* y;
-    float* v0;
-    float* v1;
-    float* v2;
-    uint32_t* id;
-    unsigned char* sel;
-    uint16_t* rank;
-};
-
-template <int DIM>
-__device__ __forceinline__ G2Stage g2_stage(unsigned char* ring, uint32_t off, uint32_t m) {
-    float* f = (float*)(ring + off);
-    G2Stage S;
-    S.x = nullptr;
-    if (DIM == 2) {
-        S.x = f;
-        f += m;
-    }
-    S.y = f;
-    S.v0 = f + m;
-    S.v1 = f + 2 * m;
-    S.v2 = f + 3 * m;
-    S.id = (uint32_t*)(f + 4 * m);
-    S.sel = (unsigned char*)(f + 5 * m);
-    S.rank = (uint16_t*)(S.sel + m);
-    return S;
-}
-
 // ---- mbarrier and bulk-copy primitives (PTX, sm_90+) ----------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_tx(uint64_t* bar, uint32_t tx) {
@@ -596,815 +985,609 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                  : "memory");
 }
 
+// the same range into L2 only
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // order this thread's generic-proxy accesses to shared memory before later
 // bulk copies (async proxy) into the same bytes
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-__device__ void g2_timeout(const SimDev* __restrict__ sims) {
-    atomicAdd(&sims[0].dyn->counters[kCntOverflow], kG2TimeoutMark);
-}
-
-// counters a consumer accumulates in registers and adds once per simulation
-struct G2Acc {
-    unsigned long long relaxed, removed;
+// registers of one warp's current simulation
+struct G2Sim {
+    uint32_t step;
+    int p;
+    bool pending, aligned;   // aligned: every plane starts on a 16-byte boundary
 };
 
-__device__ __forceinline__ void g2_flush(G2Acc& a, SimDyn* dyn, int lane) {
-    if (dyn && lane == 0) {
-        if (a.relaxed) atomicAdd(&dyn->counters[kCntRelaxed], a.relaxed);
-        if (a.removed) atomicAdd(&dyn->counters[kCntRemoved], a.removed);
-    }
-    a.relaxed = a.removed = 0;
+__device__ __forceinline__ uint32_t atom_add_global(uint32_t* p, uint32_t v) {
+    uint32_t r;
+    asm volatile("atom.global.add.u32 %0, [%1], %2;" : "=r"(r) : "l"(__cvta_generic_to_global(p)), "r"(v) : "memory");
+    return r;
 }
 
-// ---- consumer: one cell ------------------------------------------------------
-// conservation sums over the relaxed subset of a cell: old peculiar
-// velocities about the cell mean (a) and new peculiar velocities (b)
-struct G2Sums {
-    float a0, a1, a2, ae, b0, b1, b2, be, nr;
+// a cell on its way through a warp: its bounds, and where it is staged
+struct G2Job {
+    int cell;              // -1: none
+    uint32_t base, nb, arrived;
+    uint32_t ro;           // first staged particle
 };
 
-// per-cell factors of the momentum / energy correction
-struct G2Cons {
-    float uo0, uo1, uo2, mn0, mn1, mn2, alpha;
-    bool apply;
+template <int DIM>
+__host__ __device__ constexpr uint32_t g2w_cap() { return DIM == 1 ? kG2Stage1 : kG2Stage2; }
+
+// start the bulk copies of a cell's bucket and parameter record (lane 0):
+// whole 16-byte groups, bucket starts and the capacity being multiples of
+// four slots
+template <int DIM, class Sh>
+__device__ __forceinline__ void g2w_copy(Sh& sh, const G2Job& J, int p, uint32_t parity) {
+    constexpr uint32_t CAP = g2w_cap<DIM>();
+    const SimDev& s = sh.sim;
+    float* const d = sh.stage + J.ro;
+    const uint32_t bytes = 4u * ((J.nb + 3u) & ~3u);
+    uint64_t* const bar = &sh.full[parity];
+    mbar_arrive_tx(bar, (DIM == 2 ? 6u : 5u) * bytes + 4u * kNFPrm);
+    bulk_g2s(sh.prm[parity], s.fprm + (size_t)J.cell * kNFPrm, 4u * kNFPrm, bar);
+    bulk_g2s(d + 4 * CAP, s.pid[p] + J.base, bytes, bar);
+    bulk_g2s(d + 1 * CAP, (const float*)s.vel[p][0] + J.base, bytes, bar);
+    bulk_g2s(d + 2 * CAP, (const float*)s.vel[p][1] + J.base, bytes, bar);
+    bulk_g2s(d + 3 * CAP, (const float*)s.vel[p][2] + J.base, bytes, bar);
+    bulk_g2s(d, (const float*)s.pos[p][1] + J.base, bytes, bar);
+    if (DIM == 2) bulk_g2s(d + 5 * CAP, (const float*)s.pos[p][0] + J.base, bytes, bar);
+}
+
+// the same by the lanes, for buckets that are not 16-byte aligned (the
+// compact layout right after a set-up sort)
+template <int DIM, class Sh>
+__device__ __noinline__ void g2w_load(Sh& sh, G2Job J, int p, uint32_t parity, int lane) {
+    constexpr uint32_t CAP = g2w_cap<DIM>();
+    const SimDev& s = sh.sim;
+    float* const d = sh.stage + J.ro;
+    if (lane < kNFPrm) sh.prm[parity][lane] = s.fprm[(size_t)J.cell * kNFPrm + lane];
+    for (uint32_t k = lane; k < J.nb; k += 32u) {
+        const uint32_t i = J.base + k;
+        d[k] = ((const float*)s.pos[p][1])[i];
+        d[k + 1 * CAP] = ((const float*)s.vel[p][0])[i];
+        d[k + 2 * CAP] = ((const float*)s.vel[p][1])[i];
+        d[k + 3 * CAP] = ((const float*)s.vel[p][2])[i];
+        reinterpret_cast<uint32_t*>(d)[k + 4 * CAP] = s.pid[p][i];
+        if (DIM == 2) d[k + 5 * CAP] = ((const float*)s.pos[p][0])[i];
+    }
+    __syncwarp();
+}
+
+template <int V>
+struct Num {
+    static constexpr int value = V;
 };
 
-// staged particles [0, cnt) of a cell area from their bucket (at bucket
-// index off) and spill-list entries; with `have_bucket` the bucket part is
-// already there (bulk copy)
-template <int DIM>
-__device__ __forceinline__ void g2_load(const SimDev& s, const G2Stage& S, int p, uint32_t base, uint32_t nb,
-                                        const uint32_t* spl, uint32_t off, uint32_t cnt, bool have_bucket, int lane) {
-    const uint32_t mb = off < nb ? min(cnt, nb - off) : 0u;
-    __syncwarp();
-    if (!have_bucket) {
-        const Src P = src_of(s, p);
-#pragma unroll 2
-        for (uint32_t j = lane; j < mb; j += 32) {
-            const uint32_t i = base + off + j;
-            if (DIM == 2) S.x[j] = P.x[i];
-            S.y[j] = P.y[i];
-            S.v0[j] = P.v0[i];
-            S.v1[j] = P.v1[i];
-            S.v2[j] = P.v2[i];
-            S.id[j] = P.id[i];
-        }
-    }
-#pragma unroll 1
-    for (uint32_t j = mb + lane; j < cnt; j += 32) {
-        float x = 0.0f, y, v0, v1, v2;
-        uint32_t id;
-        load_particle<DIM>(s, p, base, nb, spl, off + j, x, y, v0, v1, v2, id);
-        if (DIM == 2) S.x[j] = x;
-        S.y[j] = y; S.v0[j] = v0; S.v1[j] = v1; S.v2[j] = v2; S.id[j] = id;
-    }
-    __syncwarp();
-}
-
-// Relaxation draws of the staged particles [0, cnt): a relaxed particle
-// gets its new peculiar velocity in v0..v2 and sel = 1 (else sel = 0);
-// with SUMS the conservation sums of the relaxed subset are accumulated.
-// The cell's FP32 parameters live only in this scope.
-template <bool SUMS>
-__device__ __forceinline__ void g2_relax(const float* prm, const SimDev& s, const G2Stage& S, uint32_t cnt,
-                                         uint32_t step, bool relax, int lane, G2Sums& R) {
-    FCell f;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) f.u[d] = prm[d];
-    f.th = prm[3];
-    {   // M = L L^T - theta I from the FP64-built factor L
-        const float L0 = prm[4], L1 = prm[5], L2 = prm[6], L3 = prm[7], L4 = prm[8], L5 = prm[9];
-        f.M[0] = L0 * L0 - f.th;
-        f.M[1] = L1 * L0;
-        f.M[2] = L1 * L1 + L2 * L2 - f.th;
-        f.M[3] = L3 * L0;
-        f.M[4] = L3 * L1 + L4 * L2;
-        f.M[5] = L3 * L3 + L4 * L4 + L5 * L5 - f.th;
-    }
-    f.pr = prm[10];
-    f.nu = prm[11];
-    f.nues = prm[12];
-    f.pne = prm[13];
-    TimeDraw td;
-    td.dt = s.f_dt;
-    td.a = f.nues * td.dt;
-    td.em1 = expm1f(td.a);
-    td.ema = __expf(-td.a);
-    td.inv_nues = 1.0f / f.nues;
-    td.inv_pr = f.pr > 0.0f ? 1.0f / f.pr : 0.0f;
-    const uint2 key = make_uint2(s.key0, s.key1);
-#pragma unroll 1
-    for (uint32_t j0 = lane; j0 < cnt; j0 += 64) {
-        const uint32_t j1 = j0 + 32;
-        const bool has1 = j1 < cnt;
-        unsigned char s0 = 0, s1 = 0;
-        if (relax) {
-            const uint32_t id0 = S.id[j0];
-            const uint32_t id1 = has1 ? S.id[j1] : 0u;
-            const uint4 w0 = philox(make_uint4(id0, step, kRelax, 0), key);
-            const uint4 w1 = philox(make_uint4(id1, step, kRelax, 0), key);
-            const float x0 = u01<float>(w0.x), x1 = u01<float>(w1.x);
-            s0 = x0 < f.pr;
-            s1 = has1 && x1 < f.pr;
-            if (s0 | s1) {
-                float C0[3], C1[3];
-                es_draw1(f, td, x0, w0, C0);
-                es_draw1(f, td, x1, w1, C1);
-                if (s0) {
-                    if (SUMS) {
-                        const float o0 = S.v0[j0] - f.u[0], o1 = S.v1[j0] - f.u[1], o2 = S.v2[j0] - f.u[2];
-                        R.a0 += o0; R.a1 += o1; R.a2 += o2;
-                        R.ae += o0 * o0 + o1 * o1 + o2 * o2;
-                        R.b0 += C0[0]; R.b1 += C0[1]; R.b2 += C0[2];
-                        R.be += C0[0] * C0[0] + C0[1] * C0[1] + C0[2] * C0[2];
-                        R.nr += 1.0f;
-                    }
-                    S.v0[j0] = C0[0]; S.v1[j0] = C0[1]; S.v2[j0] = C0[2];
-                }
-                if (s1) {
-                    if (SUMS) {
-                        const float o0 = S.v0[j1] - f.u[0], o1 = S.v1[j1] - f.u[1], o2 = S.v2[j1] - f.u[2];
-                        R.a0 += o0; R.a1 += o1; R.a2 += o2;
-                        R.ae += o0 * o0 + o1 * o1 + o2 * o2;
-                        R.b0 += C1[0]; R.b1 += C1[1]; R.b2 += C1[2];
-                        R.be += C1[0] * C1[0] + C1[1] * C1[1] + C1[2] * C1[2];
-                        R.nr += 1.0f;
-                    }
-                    S.v0[j1] = C1[0]; S.v1[j1] = C1[1]; S.v2[j1] = C1[2];
-                }
-            }
-        }
-        S.sel[j0] = s0;
-        if (has1) S.sel[j1] = s1;
-    }
-    __syncwarp();
-}
-
-// Eq. 9 fixed count for one cell: the ns = nearest-int(n P_relax) particles
-// with the smallest selection words w.x (ties: lower staged position).  T is
-// the ns-th smallest word and `quota` the number of particles with word T
-// that are taken; the (ns+1)-th smallest word T2 scales the time instants
-// (given T2, the ns smallest words are independent and uniform below it).
-struct G2Fixed {
-    uint32_t T, quota, ties, ns;
-    float inv_thr;
-};
-
-// the words of the staged particles [0, cnt) one chunk at a time: the
-// radix select of the ns-th smallest (four passes of 8-bit digits counted
-// in the warp's window array), then the ties and T2.  Cells above the
-// ring allocation reload each chunk in every pass.
-template <int DIM>
-__device__ __noinline__ G2Fixed g2_fixed(const SimDev& s, const G2Desc& D, const G2Stage& S, uint32_t n,
-                                          const uint32_t* spl, uint32_t* hist, int lane) {
-    const int p = (D.flags & kDescParity) ? 1 : 0;
-    const uint32_t m = D.m, nch = (n + m - 1) / m;
-    const uint2 key = make_uint2(s.key0, s.key1);
-    G2Fixed F;
-    F.ns = (uint32_t)floorf((float)n * D.prm[10] + 0.5f);
-    F.ns = min(F.ns, n);
-    F.ties = 0;
-    F.T = 0xFFFFFFFFu;
-    F.quota = 0;
-    F.inv_thr = 1.0f;
-    if (F.ns == 0) return F;
-    uint32_t prefix = 0, mask = 0, rem = F.ns;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int b = lane; b < 256; b += 32) hist[b] = 0u;
-        __syncwarp();
-        for (uint32_t ch = 0; ch < nch; ++ch) {
-            const uint32_t cnt = min(m, n - ch * m);
-            if (nch > 1) g2_load<DIM>(s, S, p, D.base, D.nb, spl, ch * m, cnt, false, lane);
-            for (uint32_t j = lane; j < cnt; j += 32) {
-                const uint32_t k = philox(make_uint4(S.id[j], D.step, kRelax, 0), key).x;
-                if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
-            }
-            __syncwarp();
-        }
-        // lane l holds digits [8l, 8l + 8): the digit where the running count reaches rem
-        uint32_t h[8], tot = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            h[i] = hist[8 * lane + i];
-            tot += h[i];
-        }
-        uint32_t inc = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const uint32_t exc = inc - tot;
-        const unsigned own = __ballot_sync(0xffffffffu, exc < rem && rem <= inc);
-        const int L = __ffs(own) - 1;
-        uint32_t d = 0, below = exc;
-        if (lane == L) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (below + h[i] >= rem) {
-                    d = 8u * lane + i;
-                    break;
-                }
-                below += h[i];
-            }
-        }
-        d = __shfl_sync(0xffffffffu, d, L);
-        below = __shfl_sync(0xffffffffu, below, L);
-        rem -= below;
-        prefix |= d << shift;
-        mask |= 0xFFu << shift;
-        __syncwarp();
-    }
-    F.T = prefix;
-    F.quota = rem;
-    // words equal to T, and the smallest word above it
-    uint32_t eq = 0, above = 0xFFFFFFFFu;
-    bool any_above = false;
-    for (uint32_t ch = 0; ch < nch; ++ch) {
-        const uint32_t cnt = min(m, n - ch * m);
-        if (nch > 1) g2_load<DIM>(s, S, p, D.base, D.nb, spl, ch * m, cnt, false, lane);
-        for (uint32_t j = lane; j < cnt; j += 32) {
-            const uint32_t k = philox(make_uint4(S.id[j], D.step, kRelax, 0), key).x;
-            eq += k == F.T;
-            if (k > F.T) {
-                any_above = true;
-                above = min(above, k);
-            }
-        }
-    }
-    eq = __reduce_add_sync(0xffffffffu, eq);
-    above = __reduce_min_sync(0xffffffffu, above);
-    any_above = __any_sync(0xffffffffu, any_above);
-    uint32_t T2 = 0;
-    bool has2 = true;
-    if (eq > F.quota) T2 = F.T;
-    else if (any_above) T2 = above;
-    else has2 = false;
-    F.inv_thr = has2 ? 1.0f / u01<float>(T2) : 1.0f;
-    return F;
-}
-
-// Relaxation draws of the SP-ESBGK ablations (same contract as g2_relax):
-// the Bernoulli or fixed-count selection (Eq. 9), the ES Cholesky or
-// Gallis-Torczynski sampler (Eqs. 10-11).  The loop is warp-uniform so
-// that the ties of the fixed count are ranked by position with ballots.
-template <bool SUMS>
-__device__ __forceinline__ void g2_relax_abl(const float* prm, const SimDev& s, const G2Stage& S, uint32_t cnt,
-                                             uint32_t step, bool relax, int lane, G2Sums& R, G2Fixed& X) {
-    FCell f;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) f.u[d] = prm[d];
-    f.th = prm[3];
-    const bool gt = s.es_sampler != 0, fixed = s.selection != 0;
-    if (gt) {   // B of Eq. 11 (lower triangle)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) f.M[k] = prm[4 + k];
-    } else {
-        const float L0 = prm[4], L1 = prm[5], L2 = prm[6], L3 = prm[7], L4 = prm[8], L5 = prm[9];
-        f.M[0] = L0 * L0 - f.th;
-        f.M[1] = L1 * L0;
-        f.M[2] = L1 * L1 + L2 * L2 - f.th;
-        f.M[3] = L3 * L0;
-        f.M[4] = L3 * L1 + L4 * L2;
-        f.M[5] = L3 * L3 + L4 * L4 + L5 * L5 - f.th;
-    }
-    f.pr = prm[10];
-    f.nu = prm[11];
-    f.nues = prm[12];
-    f.pne = prm[13];
-    TimeDraw td;
-    td.dt = s.f_dt;
-    td.a = f.nues * td.dt;
-    td.em1 = expm1f(td.a);
-    td.ema = __expf(-td.a);
-    td.inv_nues = 1.0f / f.nues;
-    td.inv_pr = fixed ? X.inv_thr : (f.pr > 0.0f ? 1.0f / f.pr : 0.0f);
-    const uint2 key = make_uint2(s.key0, s.key1);
-    const unsigned lt = lanemask_lt();
-#pragma unroll 1
-    for (uint32_t b = 0; b < cnt; b += 32) {
-        const uint32_t j = b + lane;
-        const bool has = j < cnt;
-        bool sel = false;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (relax) {
-            w = philox(make_uint4(has ? S.id[j] : 0u, step, kRelax, 0), key);
-            if (fixed) {
-                const bool tie = has && w.x == X.T;
-                const unsigned tb = __ballot_sync(0xffffffffu, tie);
-                const uint32_t rank = X.ties + (uint32_t)__popc(tb & lt);
-                X.ties += (uint32_t)__popc(tb);
-                sel = has && X.ns > 0 && (w.x < X.T || (tie && rank < X.quota));
-            } else {
-                sel = has && u01<float>(w.x) < f.pr;
-            }
-            if (sel) {
-                float C[3];
-                const float u = u01<float>(w.x);
-                if (gt) es_draw_gt(f, td, u, w, C);
-                else es_draw1(f, td, u, w, C);
-                if (SUMS) {
-                    const float o0 = S.v0[j] - f.u[0], o1 = S.v1[j] - f.u[1], o2 = S.v2[j] - f.u[2];
-                    R.a0 += o0; R.a1 += o1; R.a2 += o2;
-                    R.ae += o0 * o0 + o1 * o1 + o2 * o2;
-                    R.b0 += C[0]; R.b1 += C[1]; R.b2 += C[2];
-                    R.be += C[0] * C[0] + C[1] * C[1] + C[2] * C[2];
-                    R.nr += 1.0f;
-                }
-                S.v0[j] = C[0]; S.v1[j] = C[1]; S.v2[j] = C[2];
-            }
-        }
-        if (has) S.sel[j] = sel ? 1 : 0;
-    }
-    __syncwarp();
-}
-
-// conservation factors of the cell from the warp's partial sums
-__device__ __forceinline__ G2Cons g2_factors(const float* prm, G2Sums R, bool relax, G2Acc& acc) {
-    G2Cons K;
-    K.apply = false;
-    K.uo0 = K.uo1 = K.uo2 = K.mn0 = K.mn1 = K.mn2 = 0.0f;
-    K.alpha = 1.0f;
-    if (!relax) return K;
-    const float nr = warp_sumf(R.nr);
-    if (nr < 2.0f) return K;
-    const float a0 = warp_sumf(R.a0), a1 = warp_sumf(R.a1), a2 = warp_sumf(R.a2), ae = warp_sumf(R.ae);
-    const float b0 = warp_sumf(R.b0), b1 = warp_sumf(R.b1), b2 = warp_sumf(R.b2), be = warp_sumf(R.be);
-    // FP32: the sums are taken about the cell mean, so the differences
-    // below do not cancel.  The butterfly sums are bitwise the same on
-    // every lane (each stage adds the same two values), so every lane
-    // computes the same factors without a broadcast.
-    const float inv = 1.0f / nr;
-    const float Eo = ae - (a0 * a0 + a1 * a1 + a2 * a2) * inv;
-    const float En = be - (b0 * b0 + b1 * b1 + b2 * b2) * inv;
-    if (En > 0.0f && Eo >= 0.0f) {
-        K.apply = true;
-        K.alpha = sqrtf(Eo / En);
-        K.uo0 = prm[0] + a0 * inv;
-        K.uo1 = prm[1] + a1 * inv;
-        K.uo2 = prm[2] + a2 * inv;
-        K.mn0 = b0 * inv;
-        K.mn1 = b1 * inv;
-        K.mn2 = b2 * inv;
-        acc.relaxed += (unsigned long long)(unsigned)nr;
-    }
-    return K;
-}
-
-// the relaxed velocity of staged particle j (conservation applied), or its
-// old velocity when the cell had a single relaxed particle (reverted)
-template <int DIM>
-__device__ __forceinline__ void g2_velocity(const SimDev& s, const G2Stage& S, const G2Cons& K, int p, uint32_t base,
-                                            uint32_t nb, const uint32_t* spl, uint32_t off, uint32_t j, float* c) {
-    c[0] = S.v0[j];
-    c[1] = S.v1[j];
-    c[2] = S.v2[j];
-    if (S.sel[j]) {
-        if (K.apply) {
-            c[0] = K.uo0 + K.alpha * (c[0] - K.mn0);
-            c[1] = K.uo1 + K.alpha * (c[1] - K.mn1);
-            c[2] = K.uo2 + K.alpha * (c[2] - K.mn2);
-        } else {
-            float ox, oy;
-            uint32_t oid;
-            load_particle<DIM>(s, p, base, nb, spl, off + j, ox, oy, c[0], c[1], c[2], oid);
-        }
-    }
-}
-
-// relaxed velocities written back in place (MODE kRelaxOnly)
-template <int DIM>
-__device__ __forceinline__ void g2_store_relaxed(const SimDev& s, const G2Stage& S, const G2Cons& K, int p,
-                                                 uint32_t base, uint32_t nb, const uint32_t* spl, uint32_t off,
-                                                 uint32_t cnt, int lane) {
-    if (!K.apply) return;
-#pragma unroll 1
-    for (uint32_t j = lane; j < cnt; j += 32) {
-        if (!S.sel[j]) continue;
-        float c[3];
-        g2_velocity<DIM>(s, S, K, p, base, nb, spl, off, j, c);
-        store_velocity<DIM>(s, p, base, nb, spl, off + j, c[0], c[1], c[2]);
-    }
-    __syncwarp();
-}
-
-// passes A, B and the write pass over the staged particles [0, cnt)
-template <int DIM, int MODE>
-__device__ __forceinline__ void g2_move(const SimDev* __restrict__ sims, const SimDev& s, const G2Stage& S,
-                                        const G2Cons& K, int cell, int p, uint32_t base, uint32_t nb,
-                                        const uint32_t* spl, uint32_t off, uint32_t cnt, uint32_t step,
-                                        uint32_t* win, int lane, uint32_t& removed) {
-    const int q = p ^ 1;
-    Ctx C;
-    make_ctx(s, q, C);
-    const int cy = DIM == 2 ? cell / C.nx : 0;
-    const int cx = DIM == 2 ? cell - cy * C.nx : 0;
-    const int gcell = cell + (MODE == kFullSlab && DIM == 1 ? C.cell0 : 0);   // 1-D: global cell of the slab's cell
-    const int row0 = MODE == kFullSlab && DIM == 2 ? s.row0 : 0;
-    uint32_t* wcnt = win;              // arrivals per window slot
-    uint32_t* wstart = win + kWin;     // first reserved index of each slot in its bucket
-    uint32_t* wend = win + 2 * kWin;   // end of that bucket
-    wcnt[lane] = 0;
-    wcnt[lane + 32] = 0;
-    __syncwarp();
-    // pass A: conservation, advection, destination slot, rank in the slot
-#pragma unroll 1
-    for (uint32_t b = 0; b < cnt; b += 32) {
-        const uint32_t j = b + lane;
-        int slot = -2;   // -2: nothing to count
-        if (j < cnt) {
-            float x = DIM == 2 ? S.x[j] : 0.0f, y = S.y[j], c[3];
-            g2_velocity<DIM>(s, S, K, p, base, nb, spl, off, j, c);
-            unsigned char ws = kSlotNone;
-            if (advect_fast<DIM>(s, C, step, S.id[j], x, y, c)) {
-                int ix, iy;
-                cell_xy<DIM>(C, x, y, ix, iy);
-                const int dc = (DIM == 2 ? iy * C.nx + ix : iy) - (MODE == kFullSlab ? C.cell0 : 0);   // local
-                if (MODE == kFullSlab && (unsigned)dc >= (unsigned)C.K) {
-                    ws = kSlotOther;
-                } else if (!C.reservoir || !in_buffer(s, dc)) {
-                    slot = win_slot_xy<DIM>(ix, iy - row0, gcell, cx, cy);
-                    ws = slot >= 0 ? (unsigned char)slot : kSlotFar;
-                } else {
-                    ++removed;
-                }
-            }
-            if ((MODE == kFullFlux || MODE == kFullSlab) && s.flux_axis)
-                count_flux<float>(s, DIM == 2 ? S.x[j] : 0.0f, S.y[j], x, y);
-            if (DIM == 2) S.x[j] = x;
-            S.y[j] = y; S.v0[j] = c[0]; S.v1[j] = c[1]; S.v2[j] = c[2];
-            S.sel[j] = ws;
-        }
-        // the particle's rank among the arrivals of its slot: one shared
-        // atomic (lanes of one slot are served one after another)
-        if (slot >= 0) S.rank[j] = (uint16_t)atomicAdd(&wcnt[slot], 1u);
-    }
-    __syncwarp();
-    // pass B: one reservation per occupied slot, all in flight together
+// one cell.  GEN: loaded here, in chunks, with spill-list entries; else it is
+// staged at J.ro
+template <int DIM, int MODE, bool GEN, class Sh>
+__device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Job& J, uint32_t parity, uint32_t nsp,
+                                              int lane, G2Acc& acc) {
+    constexpr uint32_t CAP = g2w_cap<DIM>();
+    const SimDev& s = sh.sim;
+    const int p = S.p, q = p ^ 1, cell = J.cell;
+    const uint32_t base = J.base, nb = J.nb, n = nb + nsp, ro = GEN ? 0u : J.ro;
+    float* const st_y = sh.stage;
+    float* const st_0 = st_y + CAP;
+    float* const st_1 = st_0 + CAP;
+    float* const st_2 = st_1 + CAP;
+    uint32_t* const st_id = reinterpret_cast<uint32_t*>(st_2 + CAP);
+    float* const st_x = st_2 + 2 * CAP;   // 2-D only
+    uint16_t* const st_r = reinterpret_cast<uint16_t*>(st_2 + (DIM == 2 ? 3 : 2) * CAP);
+    // the window: lane k looks after slots k and k + 32, their bucket bounds read ahead
+    const int cy = DIM == 2 ? cell / s.nx : 0;
+    const int cx = DIM == 2 ? cell - cy * s.nx : 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int k = lane + 32 * h;
-        const uint32_t cntk = wcnt[k];
-        if (cntk) {
-            const int dest = win_cell<DIM>(k, cell, cx, cy, C.nx);
-            const uint32_t r = atomicAdd(&C.dcnt[dest], cntk);
-            wstart[k] = C.dlay[dest] + r;
-            wend[k] = min(C.dlay[dest + 1], C.cap);
+        const int k = lane + 32 * h, dest = win_cell<DIM>(k, cell, cx, cy, s.nx);
+        if ((unsigned)dest < (unsigned)s.K) {
+            cp_async4(&sh.wlo[k], &s.lay[q][dest]);
+            cp_async4(&sh.wend[k], &s.lay[q][dest + 1]);
         }
+        sh.wst[k] = 0;
     }
-    __syncwarp();
-    // write pass: consecutive lanes write particles of the same few
-    // destination buckets (a window slot's particles go to consecutive
-    // slots of its bucket, in rank order); particles leaving the window or
-    // the slab take their own reservation
+    const G2Prm f = GEN ? g2_prm(s.fprm, cell) : g2_prm(sh.prm[parity], 0);
+    const bool relax = S.pending && f.pr > 0.0f;
+    const uint32_t nch = GEN ? (n + CAP - 1) / CAP : 1u;
+    float R[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) R[k] = 0.0f;
+    uint32_t nr = 0;
+    float al = 1.0f, uo0 = 0, uo1 = 0, uo2 = 0, mn0 = 0, mn1 = 0, mn2 = 0;
+    bool apply = false;
 #pragma unroll 1
-    for (uint32_t j = lane; j < cnt; j += 32) {
-        const unsigned char ws = S.sel[j];
-        if (ws == kSlotNone) continue;
-        const float x = DIM == 2 ? S.x[j] : 0.0f, y = S.y[j];
-        if (ws < kWin) {
-            const uint32_t i = wstart[ws] + S.rank[j];
-            const uint32_t hi = wend[ws];
-            const int dc = i < hi ? 0 : cell_f<DIM>(C, x, y) - (MODE == kFullSlab ? C.cell0 : 0);
-            put_own<DIM>(s, C, q, i, hi, dc, x, y, S.v0[j], S.v1[j], S.v2[j], S.id[j]);
-        } else if (MODE == kFullSlab && ws == kSlotOther) {   // into the buckets of another slab
-            emit_other<DIM>(sims, s, q, x, y, S.v0[j], S.v1[j], S.v2[j], S.id[j]);
-        } else {   // outside the window: a reservation of its own
-            const int dc = cell_f<DIM>(C, x, y) - (MODE == kFullSlab ? C.cell0 : 0);
-            const uint32_t i = C.dlay[dc] + atomicAdd(&C.dcnt[dc], 1u);
-            const uint32_t hi = min(C.dlay[dc + 1], C.cap);
-            put_own<DIM>(s, C, q, i, hi, dc, x, y, S.v0[j], S.v1[j], S.v2[j], S.id[j]);
-        }
-    }
-    __syncwarp();
-}
-
-// a cell above the largest ring area: conservation sums in a first sweep
-// over its chunks, the update in a second sweep that reloads each chunk and
-// redraws the same counter-based random numbers
-template <int DIM, int MODE>
-__device__ __noinline__ void g2_cell_chunked(const SimDev* __restrict__ sims, const SimDev& s, const G2Desc& D,
-                                             const G2Stage& S, uint32_t n, bool relax, const uint32_t* spl,
-                                             uint32_t* win, int lane, G2Acc& acc) {
-    const int p = (D.flags & kDescParity) ? 1 : 0;
-    const uint32_t m = D.m, nch = (n + m - 1) / m;
-    const bool abl = s.selection | s.es_sampler;
-    G2Fixed X = {0u, 0u, 0u, 0u, 1.0f};
-    if (relax && s.selection) X = g2_fixed<DIM>(s, D, S, n, spl, win, lane);
-    G2Sums R = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (uint32_t ch = 0; ch < nch; ++ch) {
-        const uint32_t cnt = min(m, n - ch * m);
-        g2_load<DIM>(s, S, p, D.base, D.nb, spl, ch * m, cnt, false, lane);
-        if (abl) g2_relax_abl<true>(D.prm, s, S, cnt, D.step, relax, lane, R, X);
-        else g2_relax<true>(D.prm, s, S, cnt, D.step, relax, lane, R);
-    }
-    const G2Cons K = g2_factors(D.prm, R, relax, acc);
-    uint32_t removed = 0;
-    X.ties = 0;
-    for (uint32_t ch = 0; ch < nch; ++ch) {
-        const uint32_t cnt = min(m, n - ch * m);
-        g2_load<DIM>(s, S, p, D.base, D.nb, spl, ch * m, cnt, false, lane);
-        if (abl) g2_relax_abl<false>(D.prm, s, S, cnt, D.step, relax, lane, R, X);
-        else g2_relax<false>(D.prm, s, S, cnt, D.step, relax, lane, R);
-        if (MODE == kRelaxOnly) g2_store_relaxed<DIM>(s, S, K, p, D.base, D.nb, spl, ch * m, cnt, lane);
-        else g2_move<DIM, MODE>(sims, s, S, K, D.cell, p, D.base, D.nb, spl, ch * m, cnt, D.step, win, lane, removed);
-    }
-    if (s.has_reservoir) acc.removed += __reduce_add_sync(0xffffffffu, removed);
-}
-
-template <int DIM, int MODE>
-__device__ __forceinline__ void g2_cell(const SimDev* __restrict__ sims, const SimDev& s, const G2Desc& D,
-                                        unsigned char* ring, uint32_t* win, uint32_t* spl, int lane, G2Acc& acc) {
-    const int p = (D.flags & kDescParity) ? 1 : 0;
-    uint32_t nsp = 0;
-    if (D.arrived > D.nb) nsp = collect_spill(s, p, D.cell, spl, lane);
-    const uint32_t n = D.nb + nsp;
-    if (n == 0) return;
-    const bool relax = (D.flags & kDescPending) && D.prm[14] != 0.0f;
-    if (MODE == kRelaxOnly && !relax) return;
-    const G2Stage S = g2_stage<DIM>(ring, D.off, D.m);
-    if (n > D.m) {
-        g2_cell_chunked<DIM, MODE>(sims, s, D, S, n, relax, spl, win, lane, acc);
-        return;
-    }
-    g2_load<DIM>(s, S, p, D.base, D.nb, spl, 0u, n, (D.flags & kDescBulk) != 0, lane);
-    G2Sums R = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    if (s.selection | s.es_sampler) {   // the SP-ESBGK ablations
-        G2Fixed X = {0u, 0u, 0u, 0u, 1.0f};
-        if (relax && s.selection) X = g2_fixed<DIM>(s, D, S, n, spl, win, lane);
-        g2_relax_abl<true>(D.prm, s, S, n, D.step, relax, lane, R, X);
-    } else {
-        g2_relax<true>(D.prm, s, S, n, D.step, relax, lane, R);
-    }
-    const G2Cons K = g2_factors(D.prm, R, relax, acc);
-    if (MODE == kRelaxOnly) {
-        g2_store_relaxed<DIM>(s, S, K, p, D.base, D.nb, spl, 0u, n, lane);
-        return;
-    }
-    uint32_t removed = 0;
-    g2_move<DIM, MODE>(sims, s, S, K, D.cell, p, D.base, D.nb, spl, 0u, n, D.step, win, lane, removed);
-    if (s.has_reservoir) acc.removed += __reduce_add_sync(0xffffffffu, removed);
-}
-
-// copy one simulation descriptor into shared memory (one warp)
-__device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, int lane) {
-    const int4* a = reinterpret_cast<const int4*>(&src);
-    int4* b = reinterpret_cast<int4*>(&dst);
-    for (int i = lane; i < (int)(sizeof(SimDev) / 16); i += 32) b[i] = a[i];
-}
-
-// next simulation with cells left in its queue, after `from` (32 candidates
-// per round); -1 when every queue of this dimension is empty
-template <int DIM>
-__device__ __forceinline__ int find_sim(const SimDev* __restrict__ sims, int nsims, int from, int lane) {
-    for (int base = 0; base < nsims; base += 32) {
-        const int k = base + lane;
-        bool ok = false;
-        int idx = 0;
-        if (k < nsims) {
-            idx = from + 1 + k;
-            if (idx >= nsims) idx -= nsims;
-            const SimDev& c = sims[idx];
-            ok = c.dim == DIM && __ldcg(&c.dyn->qnext) < (uint32_t)c.K;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        if (m) return __shfl_sync(0xffffffffu, idx, __ffs(m) - 1);
-    }
-    return -1;
-}
-
-// shared state of one CTA of k_g2
-template <int NC>
-struct G2Shared {
-    SimDev sim[2];                 // simulation descriptors in use (the producer alternates)
-    G2Desc desc[kG2Desc];
-    uint64_t full[kG2Desc];        // copies of a descriptor landed (producer arrive + bytes)
-    uint64_t empty[kG2Desc];       // consumer done with a descriptor
-    uint32_t win[NC][4 * kWin];
-    uint32_t spl[NC][32];
-    uint32_t take;                 // next descriptor for a consumer
-};
-
-// ---- producer --------------------------------------------------------------
-template <int DIM, int MODE, int NC>
-__device__ void g2_producer(const SimDev* __restrict__ sims, int nsims, G2Shared<NC>& sh, unsigned char* ring,
-                            uint32_t ring_bytes, uint32_t max_stage, int lane) {
-    constexpr uint32_t bpp = g2_bytes_per_particle<DIM>();
-    constexpr int NP = DIM == 2 ? 6 : 5;   // planes
-    uint32_t seq = 0, oldest = 0;          // descriptors issued / reclaimed
-    uint32_t head = 0, tail = 0;           // ring bytes allocated / freed (monotonic)
-    uint32_t last_use[2] = {0u, 0u};
-    bool used[2] = {false, false};
-    int ent = 1;
-    bool ok = true;
-
-    // reclaim the oldest descriptor once its consumer released it
-    auto reclaim = [&]() -> bool {
-        const uint32_t slot = oldest % kG2Desc;
-        if (!mbar_wait(&sh.empty[slot], (oldest / kG2Desc) & 1u)) return false;
-        tail = sh.desc[slot].end;
-        ++oldest;
-        return true;
-    };
-    // a free descriptor and `bytes` of contiguous ring; returns the ring offset
-    auto reserve = [&](uint32_t bytes, uint32_t& off) -> bool {
-        while (seq - oldest >= (uint32_t)kG2Desc)
-            if (!reclaim()) return false;
-        for (;;) {
-            const uint32_t pos = head % ring_bytes;
-            // an allocation never wraps: with no room before the end it starts at offset 0
-            const uint32_t start = pos + bytes > ring_bytes ? head + (ring_bytes - pos) : head;
-            if (start + bytes - tail <= ring_bytes) {
-                head = start;
-                off = start % ring_bytes;
-                return true;
-            }
-            if (oldest == seq) {   // empty ring: restart it at the chosen offset
-                head = tail = start;
-            } else if (!reclaim()) {
-                return false;
+    for (uint32_t it = relax || !GEN ? 0 : nch - 1; it < 2 * nch - 1; ++it) {
+        const uint32_t off = GEN ? (it < nch ? it : 2 * nch - 2 - it) * CAP : 0u;
+        const uint32_t cnt = GEN ? min(CAP, n - off) : n;
+        if (GEN) {
+            __syncwarp();
+#pragma unroll 1
+            for (uint32_t j = lane; j < cnt; j += 32) {
+                float x = 0.0f, y, v0, v1, v2;
+                uint32_t id;
+                load_particle<DIM>(s, p, base, nb, sh.spl, off + j, x, y, v0, v1, v2, id);
+                if (DIM == 2) st_x[j] = x;
+                st_y[j] = y;
+                st_0[j] = v0;
+                st_1[j] = v1;
+                st_2[j] = v2;
+                st_id[j] = id;
             }
         }
-    };
-
-    int h = (int)(blockIdx.x % (unsigned)nsims);
-    if (sims[h].dim != DIM) h = find_sim<DIM>(sims, nsims, h, lane);
-    while (h >= 0 && ok) {
-        const int e = ent ^ 1;
-        if (used[e])
-            while (ok && oldest <= last_use[e]) ok = reclaim();
-        if (!ok) break;
-        __syncwarp();
-        load_sim_warp(sh.sim[e], sims[h], lane);
-        __syncwarp();
-        const SimDev& s = sh.sim[e];
-        const int p = s.dyn->cur;
-        const uint32_t step = s.dyn->step;
-        const bool pending = s.dyn->relax_pending != 0;
-        const uint32_t K = (uint32_t)s.K;
-        if (MODE == kRelaxOnly && !pending) {   // nothing to apply: close its queue
-            if (lane == 0) atomicMax(&s.dyn->qnext, K);
-            h = find_sim<DIM>(sims, nsims, h, lane);
-            continue;
-        }
-        ent = e;
-        // bulk copies need 16-byte aligned planes (and buckets)
-        uintptr_t al = (uintptr_t)s.pos[p][1] | (uintptr_t)s.vel[p][0] | (uintptr_t)s.vel[p][1] |
-                       (uintptr_t)s.vel[p][2] | (uintptr_t)s.pid[p] | (uintptr_t)s.fprm;
-        if (DIM == 2) al |= (uintptr_t)s.pos[p][0];
-        const bool planes_aligned = (al & 15u) == 0;
-        const uint32_t flags0 = (pending ? kDescPending : 0u) | (p ? kDescParity : 0u);
-        const uint32_t cap = (uint32_t)s.cap;
-        for (;;) {
-            uint32_t c0 = 0;
-            if (lane == 0) c0 = atomicAdd(&s.dyn->qnext, (uint32_t)kG2Run);
-            c0 = __shfl_sync(0xffffffffu, c0, 0);
-            if (c0 >= K) break;
-            uint32_t lo = 0, hi = 0, ar = 0;
-            if (lane < kG2Run && c0 + lane < K) {
-                lo = s.lay[p][c0 + lane];
-                hi = min(s.lay[p][c0 + lane + 1], cap);
-                ar = s.cnt[p][c0 + lane];
-            }
-            const uint32_t nrun = min((uint32_t)kG2Run, K - c0);
-            for (uint32_t i = 0; i < nrun && ok; ++i) {
-                const uint32_t bs = __shfl_sync(0xffffffffu, lo, i);
-                const uint32_t tp = __shfl_sync(0xffffffffu, hi, i);
-                const uint32_t arv = __shfl_sync(0xffffffffu, ar, i);
-                const uint32_t capc = tp > bs ? tp - bs : 0u;
-                const uint32_t nb = min(arv, capc);
-                const bool spill = arv > nb;
-                if (nb == 0 && !spill) continue;
-                const uint32_t need = nb + (spill ? (uint32_t)kG2Spill : 0u);
-                const bool chunked = need > max_stage;
-                const uint32_t m = chunked ? max_stage : ((need + 3u) & ~3u);
-                const uint32_t bytes = (bpp * m + 15u) & ~15u;
-                const bool bulk = !chunked && planes_aligned && (bs & 3u) == 0 && nb > 0 &&
-                                  bs + ((nb + 3u) & ~3u) <= cap;
-                uint32_t off = 0;
-                if (!reserve(bytes, off)) {
-                    ok = false;
-                    break;
+        uint32_t selm = 0;   // bit i: the lane's particle of iteration i is relaxed
+        // ---- sweep 1: each lane on its own particles, two at a time (lanes
+        // past the end work on what is there, unselected) ----
+        if (relax) {
+            auto draw = [&](auto nt, uint32_t b) {
+                constexpr int N = decltype(nt)::value;
+                uint4 w[N];
+                float u[N], C[N][3];
+                bool sel[N], any = false;
+#pragma unroll
+                for (int t = 0; t < N; ++t) w[t] = philox_keys(st_id[ro + b + 32 * t + lane], S.step, sh.key);
+#pragma unroll
+                for (int t = 0; t < N; ++t) {
+                    u[t] = u01<float>(w[t].x);
+                    sel[t] = b + 32 * t + lane < cnt && u[t] < f.pr;
+                    any = any || sel[t];
                 }
-                const uint32_t slot = seq % kG2Desc;
-                G2Desc& d = sh.desc[slot];
-                if (lane == 0) {
-                    d.base = bs;
-                    d.nb = nb;
-                    d.arrived = arv;
-                    d.off = off;
-                    d.m = m;
-                    d.cell = (int)(c0 + i);
-                    d.ent = e;
-                    d.step = step;
-                    d.flags = flags0 | (bulk ? kDescBulk : 0u);
-                    d.end = head + bytes;
-                    const uint32_t nb4 = (nb + 3u) & ~3u;
-                    mbar_arrive_tx(&sh.full[slot], 64u + (bulk ? (uint32_t)NP * 4u * nb4 : 0u));
-                    bulk_g2s(d.prm, s.fprm + (size_t)(c0 + i) * kNFPrm, 64u, &sh.full[slot]);
-                    if (bulk) {
-                        unsigned char* dst = ring + off;
-                        const uint32_t pb = 4u * m;   // bytes of one staged plane
-                        int k = 0;
-                        if (DIM == 2) bulk_g2s(dst + pb * k++, (const float*)s.pos[p][0] + bs, 4u * nb4, &sh.full[slot]);
-                        bulk_g2s(dst + pb * k++, (const float*)s.pos[p][1] + bs, 4u * nb4, &sh.full[slot]);
-                        bulk_g2s(dst + pb * k++, (const float*)s.vel[p][0] + bs, 4u * nb4, &sh.full[slot]);
-                        bulk_g2s(dst + pb * k++, (const float*)s.vel[p][1] + bs, 4u * nb4, &sh.full[slot]);
-                        bulk_g2s(dst + pb * k++, (const float*)s.vel[p][2] + bs, 4u * nb4, &sh.full[slot]);
-                        bulk_g2s(dst + pb * k, s.pid[p] + bs, 4u * nb4, &sh.full[slot]);
+                if (!__any_sync(0xffffffffu, any)) return;
+#pragma unroll
+                for (int t = 0; t < N; ++t) es_draw1(s, f, u[t], w[t], C[t]);
+#pragma unroll
+                for (int t = 0; t < N; ++t) {
+                    const uint32_t j = ro + b + 32 * t + lane;
+                    const float o0 = st_0[j] - f.u[0], o1 = st_1[j] - f.u[1], o2 = st_2[j] - f.u[2];
+                    if (sel[t]) {
+                        R[0] += o0; R[1] += o1; R[2] += o2;
+                        R[3] += o0 * o0 + o1 * o1 + o2 * o2;
+                        R[4] += C[t][0]; R[5] += C[t][1]; R[6] += C[t][2];
+                        R[7] += C[t][0] * C[t][0] + C[t][1] * C[t][1] + C[t][2] * C[t][2];
+                        st_0[j] = C[t][0];
+                        st_1[j] = C[t][1];
+                        st_2[j] = C[t][2];
+                        selm |= 1u << ((b >> 5) + t);
                     }
                 }
-                __syncwarp();
-                head += bytes;
-                last_use[e] = seq;
-                used[e] = true;
-                ++seq;
+            };
+            uint32_t b = 0;
+#pragma unroll 1
+            for (; b + 32 < cnt; b += 64) draw(Num<2>{}, b);
+            if (b < cnt) draw(Num<1>{}, b);
+            if (!GEN || it < nch) nr += (uint32_t)__popc(selm);
+        }
+        if (GEN && it + 1 < nch) continue;
+        if ((!GEN || it + 1 == nch) && relax) {
+            // conservation factors: reduce-scatter of the eight sums (lane
+            // 4 i holds sum i), every lane then reads all eight
+            __syncwarp();
+#pragma unroll
+            for (int half = 4; half >= 1; half >>= 1) {
+                const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+                for (int i = 0; i < half; ++i) {
+                    const float send = up ? R[i] : R[i + half];
+                    const float recv = __shfl_xor_sync(0xffffffffu, send, 4 * half);
+                    R[i] = (up ? R[i + half] : R[i]) + recv;
+                }
+            }
+            R[0] += __shfl_xor_sync(0xffffffffu, R[0], 2);
+            R[0] += __shfl_xor_sync(0xffffffffu, R[0], 1);
+            const uint32_t nall = __reduce_add_sync(0xffffffffu, nr);
+            float Q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) Q[k] = __shfl_sync(0xffffffffu, R[0], 4 * k);
+            if (nall >= 2) {
+                // FP32: the sums are taken about the cell mean, so the
+                // differences below do not cancel
+                const float inv = 1.0f / (float)nall;
+                const float Eo = Q[3] - (Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2]) * inv;
+                const float En = Q[7] - (Q[4] * Q[4] + Q[5] * Q[5] + Q[6] * Q[6]) * inv;
+                if (En > 0.0f && Eo >= 0.0f) {
+                    // c = ubar_old + alpha (c' - ubar_new) with c' about the cell mean
+                    apply = true;
+                    al = sqrtf(Eo / En);
+                    uo0 = f.u[0] + Q[0] * inv;
+                    uo1 = f.u[1] + Q[1] * inv;
+                    uo2 = f.u[2] + Q[2] * inv;
+                    mn0 = Q[4] * inv;
+                    mn1 = Q[5] * inv;
+                    mn2 = Q[6] * inv;
+                    if (lane == 0) acc.relaxed += nall;
+                }
             }
         }
-        if (!ok) break;
-        h = find_sim<DIM>(sims, nsims, h, lane);
-    }
-    // one end marker per consumer (they take descriptors in order)
-    for (int k = 0; k < NC && ok; ++k) {
-        uint32_t off;
-        if (!reserve(0u, off)) {
-            ok = false;
-            break;
+        if (!apply && selm) {   // fewer than two relaxed particles in the cell: reverted
+#pragma unroll 1
+            for (uint32_t b = lane; b < cnt; b += 32, selm >>= 1)
+                if (selm & 1u) {
+                    float x, y;
+                    uint32_t id;
+                    load_particle<DIM>(s, p, base, nb, sh.spl, off + b, x, y, st_0[ro + b], st_1[ro + b],
+                                       st_2[ro + b], id);
+                }
+            selm = 0;
         }
-        const uint32_t slot = seq % kG2Desc;
-        if (lane == 0) {
-            sh.desc[slot].cell = -1;
-            sh.desc[slot].end = head;
-            mbar_arrive(&sh.full[slot]);
+        // ---- sweep 2 ----
+        const float tau = s.f_dt, lo1 = s.f_lo[1], hi1 = s.f_hi[1], idy = s.f_inv_dy;
+        const float lo0 = s.f_lo[0], hi0 = s.f_hi[0], idx = s.f_inv_dx;
+        const int nym1 = s.ny - 1, nxm1 = s.nx - 1, nseg = DIM == 2 ? s.nseg : 0;
+        const bool res = s.has_reservoir != 0;
+        const float b0 = s.f_bdt[0], b1 = s.f_bdt[1], b2 = s.f_bdt[2];
+        uint32_t slow = 0;   // bit i: the lane's particle of iteration i meets a wall or plate
+        // destination slot of a moved particle, its rank among the arrivals
+        // of the slot from one shared atomic (lanes of one slot are served
+        // one after another)
+        auto place = [&](bool alive, float x, float y) -> uint32_t {
+            const int iy = min(max(__float2int_rd((y - lo1) * idy), 0), nym1);
+            const int ix = DIM == 1 ? 0 : min(max(__float2int_rd((x - lo0) * idx), 0), nxm1);
+            if (res && alive && in_buffer_xy(s, ix, iy)) {
+                ++acc.removed;
+                alive = false;
+            }
+            const int slot = win_slot_xy<DIM>(ix, iy, cell, cx, cy);
+            uint32_t sr = alive ? kPackFar : kPackNone;
+            if (alive && slot >= 0) sr = (uint32_t)slot | (atomicAdd(&sh.wst[slot], 1u) << 6);
+            return sr;
+        };
+        auto fly = [&](auto nt, uint32_t b) {
+            constexpr int N = decltype(nt)::value;
+            float x[N], y[N], c[N][3], xn[N], yn[N];
+            bool has[N], inside[N];
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                const uint32_t j = ro + b + 32 * t + lane;
+                x[t] = DIM == 2 ? st_x[j] : 0.0f;
+                y[t] = st_y[j];
+                c[t][0] = st_0[j];
+                c[t][1] = st_1[j];
+                c[t][2] = st_2[j];
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                has[t] = b + 32 * t + lane < cnt;
+                if (selm >> ((b >> 5) + t) & 1u) {
+                    c[t][0] = uo0 + al * (c[t][0] - mn0);
+                    c[t][1] = uo1 + al * (c[t][1] - mn1);
+                    c[t][2] = uo2 + al * (c[t][2] - mn2);
+                }
+                yn[t] = y[t] + c[t][1] * tau;
+                xn[t] = x[t];
+                inside[t] = yn[t] > lo1 && yn[t] < hi1;
+                if (DIM == 2) {
+                    xn[t] = x[t] + c[t][0] * tau;
+                    inside[t] = inside[t] && xn[t] > lo0 && xn[t] < hi0;
+                }
+            }
+            if (DIM == 2)
+                for (int g = 0; g < nseg; ++g) {
+                    const float ps = s.f_seg_pos[g];
+#pragma unroll
+                    for (int t = 0; t < N; ++t)
+                        if ((x[t] - ps) * (xn[t] - ps) <= 0.0f) inside[t] = false;
+                }
+            if (MODE == kFullFlux && s.flux_axis) {
+#pragma unroll
+                for (int t = 0; t < N; ++t)
+                    if (has[t] && inside[t]) count_flux<float>(s, x[t], y[t], xn[t], yn[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                const uint32_t j = ro + b + 32 * t + lane;
+                const uint32_t sr = place(has[t] && inside[t], xn[t], yn[t]);
+                if (has[t] && !inside[t]) slow |= 1u << ((b >> 5) + t);   // left as it is for the loop below
+                if (DIM == 2) st_x[j] = inside[t] ? xn[t] : x[t];
+                st_y[j] = inside[t] ? yn[t] : y[t];
+                st_0[j] = inside[t] ? c[t][0] + b0 : c[t][0];
+                st_1[j] = inside[t] ? c[t][1] + b1 : c[t][1];
+                st_2[j] = inside[t] ? c[t][2] + b2 : c[t][2];
+                st_r[j] = (uint16_t)sr;
+            }
+        };
+        __syncwarp();   // the window is clear
+        {
+            uint32_t b = 0;
+#pragma unroll 1
+            for (; b + 32 < cnt; b += 64) fly(Num<2>{}, b);
+            if (b < cnt) fly(Num<1>{}, b);
+        }
+        // walls and plates
+        for (; __any_sync(0xffffffffu, slow); slow &= slow - 1u) {
+            if (!slow) continue;
+            const uint32_t j = ro + 32u * (uint32_t)(__ffs(slow) - 1) + lane;
+            const float x = DIM == 2 ? st_x[j] : 0.0f, y = st_y[j];
+            const AdvOut o = advect_slow(s, S.step, st_id[j], x, y, st_0[j], st_1[j], st_2[j]);
+            if (MODE == kFullFlux && s.flux_axis) count_flux<float>(s, x, y, o.x, o.y);
+            st_r[j] = (uint16_t)place(o.alive != 0, o.x, o.y);
+            if (DIM == 2) st_x[j] = o.x;
+            st_y[j] = o.y;
+            st_0[j] = o.c0;
+            st_1[j] = o.c1;
+            st_2[j] = o.c2;
         }
         __syncwarp();
-        ++seq;
+        // ---- reserve: all slots in flight together (each lane with the bounds it asked for) ----
+        cp_async_wait_all();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            const uint32_t c = sh.wst[k];
+            if (c) sh.wst[k] = sh.wlo[k] + atom_add_global(&s.cnt[q][win_cell<DIM>(k, cell, cx, cy, s.nx)], c);
+            sh.wend[k] = min(sh.wend[k], (uint32_t)s.cap);
+        }
+        // ---- sweep 3 ----
+        float* const dx = (float*)s.pos[q][0];
+        float* const dy = (float*)s.pos[q][1];
+        float* const d0 = (float*)s.vel[q][0];
+        float* const d1 = (float*)s.vel[q][1];
+        float* const d2 = (float*)s.vel[q][2];
+        uint32_t* const did = s.pid[q];
+        auto put = [&](auto nt, uint32_t b) {
+            constexpr int N = decltype(nt)::value;
+            uint32_t sr[N], id[N], i[N];
+            float x[N], y[N], v[N][3];
+            bool in[N], odd = false;
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                const uint32_t j = ro + b + 32 * t + lane;
+                sr[t] = b + 32 * t + lane < cnt ? st_r[j] : kPackNone;
+                id[t] = st_id[j];
+                x[t] = DIM == 2 ? st_x[j] : 0.0f;
+                y[t] = st_y[j];
+                v[t][0] = st_0[j];
+                v[t][1] = st_1[j];
+                v[t][2] = st_2[j];
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                i[t] = sh.wst[sr[t] & 63u] + (sr[t] >> 6);
+                in[t] = sr[t] < kPackFar && i[t] < sh.wend[sr[t] & 63u];
+                odd = odd || (!in[t] && sr[t] != kPackNone);
+            }
+            if (__any_sync(0xffffffffu, odd)) {   // not in the window, or the bucket is full
+                int dc[N];
+                uint32_t r[N], lo[N], hi[N];
+#pragma unroll
+                for (int t = 0; t < N; ++t) {   // reservations of their own, all in flight together
+                    int ix, iy;
+                    cell_xy<DIM>(s, x[t], y[t], ix, iy);
+                    dc[t] = DIM == 2 ? iy * s.nx + ix : iy;
+                    r[t] = lo[t] = hi[t] = 0;
+                    if (sr[t] == kPackFar) {
+                        r[t] = atom_add_global(&s.cnt[q][dc[t]], 1u);
+                        lo[t] = __ldg(&s.lay[q][dc[t]]);
+                        hi[t] = __ldg(&s.lay[q][dc[t] + 1]);
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < N; ++t) {
+                    if (sr[t] == kPackFar) {
+                        i[t] = lo[t] + r[t];
+                        in[t] = i[t] < min(hi[t], (uint32_t)s.cap);
+                    }
+                    if (!in[t] && sr[t] != kPackNone)
+                        spill<DIM>(s, q, dc[t], x[t], y[t], v[t][0], v[t][1], v[t][2], id[t]);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t)
+                if (in[t]) {
+                    if (DIM == 2) __stcg(dx + i[t], x[t]);
+                    __stcg(dy + i[t], y[t]);
+                    __stcg(d0 + i[t], v[t][0]);
+                    __stcg(d1 + i[t], v[t][1]);
+                    __stcg(d2 + i[t], v[t][2]);
+                    __stcg(did + i[t], id[t]);
+                }
+        };
+        __syncwarp();
+        {
+            uint32_t b = 0;
+#pragma unroll 1
+            for (; b + 32 < cnt; b += 64) put(Num<2>{}, b);
+            if (b < cnt) put(Num<1>{}, b);
+        }
+        if (GEN && it + 1 < 2 * nch - 1) {   // the window of the next chunk
+            __syncwarp();
+            sh.wst[lane] = 0;
+            sh.wst[lane + 32] = 0;
+        }
     }
-    if (!ok) {
-        if (lane == 0) g2_timeout(sims);
-        // copies still in flight land before the CTA may exit
-        for (uint32_t t = oldest; t < seq; ++t) mbar_wait(&sh.full[t % kG2Desc], (t / kG2Desc) & 1u);
-    }
+    __syncwarp();
 }
 
-template <int DIM, int MODE, int NC>
-__global__ void __launch_bounds__(32 * (NC + 1), 16 / (NC + 1)) k_g2(const SimDev* __restrict__ sims, int nsims,
-                                                     uint32_t* __restrict__ wq, uint32_t ring_bytes,
-                                                     uint32_t max_stage) {
-    extern __shared__ __align__(128) unsigned char g2_ring[];
-    __shared__ G2Shared<NC> sh;
+template <int DIM, int MODE, class Sh>
+__device__ __noinline__ G2Acc g2w_cell_general(Sh& sh, G2Sim S, G2Job J, int lane) {
+    G2Acc acc = {0u, 0u};
+    uint32_t nsp = 0;
+    if (J.arrived > J.nb) nsp = collect_spill(sh.sim, S.p, J.cell, sh.spl, kG2wSpill, lane);
+    g2w_cell_impl<DIM, MODE, true>(sh, S, J, 0u, nsp, lane, acc);
+    return acc;
+}
+
+constexpr int kG2wWarps = 4;    // warps per block
+constexpr int kG2wBlocks = 4;   // blocks per SM
+
+// DIMS 1 or 2: the dimension of every cell of the tiles *first .. *first +
+// *ntiles (first null: 0)
+template <int DIMS, int MODE>
+__global__ void __launch_bounds__(32 * kG2wWarps, kG2wBlocks) k_g2(const SimDev* __restrict__ sims,
+                                                                   const int2* __restrict__ tiles,
+                                                                   const int* __restrict__ ntiles,
+                                                                   const int* __restrict__ first_tile,
+                                                                   uint32_t* __restrict__ wq) {
+    extern __shared__ __align__(16) unsigned char g2_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kG2Desc; ++i) {
-            mbar_init(&sh.full[i], 1);
-            mbar_init(&sh.empty[i], 1);
+    G2Warp<DIMS>& sh = reinterpret_cast<G2Warp<DIMS>*>(g2_smem)[warp];
+    const SimDev& s = sh.sim;
+    const uint32_t nunits = (uint32_t)*ntiles * kCTile;   // a unit is one cell slot of a tile
+    if (first_tile) tiles += *first_tile;
+    const uint32_t nwarps = gridDim.x * kG2wWarps;
+    G2Acc acc = {0u, 0u};
+    G2Sim S = {0u, 0, false};
+    int loaded = -1;
+    // Four cells are on their way through the warp.  While cell i is worked
+    // on, the copies of i + 1, the bounds of i + 2 and the tile of i + 3 come
+    // in asynchronously, each from what had arrived by the start of cell i;
+    // the unit number of i + 4 (lane 0's `ahead`) comes from the counter.  The
+    // first four units of a warp are dealt out by its number.
+    const uint32_t first = blockIdx.x * kG2wWarps + warp;
+    uint32_t ahead = 0;
+    if (lane == 0) {
+        ahead = atom_add_global(&wq[0], 1u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t u = first + k * nwarps;
+            sh.punit[k] = u;
+            if (k < 3 && u < nunits) cp_async8(&sh.ptile[k], &tiles[u / kCTile]);
         }
-        sh.take = 0;
+    }
+    if (lane == 0) {
+        mbar_init(&sh.full[0], 1);
+        mbar_init(&sh.full[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    __syncthreads();
-    if (warp == 0) {
-        g2_producer<DIM, MODE, NC>(sims, nsims, sh, g2_ring, ring_bytes, max_stage, lane);
-    } else {
-        uint32_t* win = sh.win[warp - 1];
-        uint32_t* spl = sh.spl[warp - 1];
-        G2Acc acc = {0ull, 0ull};
-        SimDyn* acc_dyn = nullptr;
-        for (;;) {
-            uint32_t my = 0;
-            if (lane == 0) my = atomicAdd(&sh.take, 1u);
-            my = __shfl_sync(0xffffffffu, my, 0);
-            const uint32_t slot = my % kG2Desc;
-            if (!mbar_wait(&sh.full[slot], (my / kG2Desc) & 1u)) {
-                if (lane == 0) g2_timeout(sims);
-                break;
-            }
-            const G2Desc& D = sh.desc[slot];
-            if (D.cell < 0) break;
-            const SimDev& s = sh.sim[D.ent];
-            if (s.dyn != acc_dyn) {
-                g2_flush(acc, acc_dyn, lane);
-                acc_dyn = s.dyn;
-            }
-            g2_cell<DIM, MODE>(sims, s, D, g2_ring, win, spl, lane, acc);
-            fence_proxy_async_smem();
+    uint32_t phase = 0;    // bit b: parity of the next phase of full[b]
+    bool ok = true;
+    uint32_t known = 0;    // bit k: pbound[k] holds the bounds of the cell in slot k
+    bool staged = false;   // the copies of the next cell have been started, to `ro`
+    uint32_t ro = 0;
+    for (uint32_t i = 0;; ++i) {
+        const uint32_t k0 = i & 3u, k1 = (i + 1) & 3u, k2 = (i + 2) & 3u, k3 = (i + 3) & 3u;
+        cp_async_wait_all();
+        __syncwarp();
+        const uint32_t unit = sh.punit[k0];
+        if (unit >= nunits) break;   // unit numbers of a warp only grow
+        const int2 tile = sh.ptile[k0];
+        if (tile.x != loaded) {
+            if (loaded >= 0) g2_flush(acc, s.dyn, lane);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.empty[slot]);
+            load_sim_warp(sh.sim, sims[tile.x], lane);
+            __syncwarp();
+            loaded = tile.x;
+            S.p = s.dyn->cur;
+            S.step = s.dyn->step;
+            S.pending = s.dyn->relax_pending != 0;
+            uintptr_t al = (uintptr_t)s.pos[S.p][1] | (uintptr_t)s.vel[S.p][0] | (uintptr_t)s.vel[S.p][1] |
+                           (uintptr_t)s.vel[S.p][2] | (uintptr_t)s.pid[S.p];
+            if (DIMS == 2) al |= (uintptr_t)s.pos[S.p][0];
+            S.aligned = (al & 15u) == 0;
+            if (lane < 10) {   // round keys: the key plus r times the Weyl constants
+                sh.key[2 * lane] = s.key0 + (uint32_t)lane * 0x9E3779B9u;
+                sh.key[2 * lane + 1] = s.key1 + (uint32_t)lane * 0xBB67AE85u;
+            }
+            __syncwarp();
+            known = 0;
+            staged = false;
         }
-        g2_flush(acc, acc_dyn, lane);
+        const uint32_t room = g2w_cap<DIMS>(), cap = (uint32_t)s.cap;
+        G2Job J;
+        J.cell = tile.y + (int)(unit % kCTile);
+        J.base = J.nb = J.arrived = 0;
+        J.ro = staged ? ro : 0u;
+        if (J.cell < s.K) {
+            uint32_t lo, hi;
+            if (known >> k0 & 1u) {
+                lo = sh.pbound[k0][0];
+                hi = sh.pbound[k0][1];
+                J.arrived = sh.pbound[k0][2];
+            } else {
+                lo = __ldg(&s.lay[S.p][J.cell]);
+                hi = __ldg(&s.lay[S.p][J.cell + 1]);
+                J.arrived = __ldg(&s.cnt[S.p][J.cell]);
+            }
+            hi = min(hi, cap);
+            J.base = lo;
+            J.nb = min(J.arrived, hi > lo ? hi - lo : 0u);
+        }
+        const bool general = J.arrived > J.nb || J.nb > room;
+        const uint32_t par = i & 1u;
+        if (J.arrived && !general) {
+            bool bulk = staged;
+            if (!staged) {
+                bulk = S.aligned && (J.base & 3u) == 0u;
+                if (bulk) {
+                    if (lane == 0) g2w_copy<DIMS>(sh, J, S.p, par);
+                } else {
+                    g2w_load<DIMS>(sh, J, S.p, par, lane);
+                }
+            }
+            if (bulk) {
+                ok = mbar_wait(&sh.full[par], phase >> par & 1u);
+                if (!ok) break;
+                phase ^= 1u << par;
+            }
+        }
+        // the next cell's copies, where it fits the staging area beside this one
+        staged = false;
+        if (known >> k1 & 1u) {
+            G2Job N;
+            const uint32_t lo = sh.pbound[k1][0], hi = min(sh.pbound[k1][1], cap);
+            N.cell = sh.ptile[k1].y + (int)(sh.punit[k1] % kCTile);
+            N.base = lo;
+            N.arrived = sh.pbound[k1][2];
+            N.nb = min(N.arrived, hi > lo ? hi - lo : 0u);
+            const uint32_t m = (J.nb + 31u) & ~31u, mn = (N.nb + 31u) & ~31u;
+            staged = !general && S.aligned && (lo & 3u) == 0u && N.arrived == N.nb && N.nb > 0 &&
+                     (J.ro + m + mn <= room || mn <= J.ro);
+            if (staged) {
+                ro = J.ro + m + mn <= room ? J.ro + m : 0u;
+                N.ro = ro;
+                if (lane == 0) g2w_copy<DIMS>(sh, N, S.p, par ^ 1u);
+            } else if (S.aligned && (lo & 3u) == 0u && N.nb > 0 && lane == 0) {   // at least into L2
+                const uint32_t bytes = 4u * ((N.nb + 3u) & ~3u);
+                bulk_prefetch(s.pid[S.p] + lo, bytes);
+                for (int d = 0; d < 3; ++d) bulk_prefetch((const float*)s.vel[S.p][d] + lo, bytes);
+                bulk_prefetch((const float*)s.pos[S.p][1] + lo, bytes);
+                if (DIMS == 2) bulk_prefetch((const float*)s.pos[S.p][0] + lo, bytes);
+            }
+        }
+        __syncwarp();   // every lane has read the slots of cell i
+        {   // bounds of i + 2, tile of i + 3, unit of i + 4
+            const uint32_t u2 = sh.punit[k2], u3 = sh.punit[k3];
+            known &= ~(1u << k2);
+            if (u2 < nunits && sh.ptile[k2].x == loaded) {
+                const int c = sh.ptile[k2].y + (int)(u2 % kCTile);
+                if (c < s.K) {
+                    if (lane < 3) cp_async4(&sh.pbound[k2][lane], lane < 2 ? &s.lay[S.p][c + lane] : &s.cnt[S.p][c]);
+                    known |= 1u << k2;
+                }
+            }
+            if (lane == 0) {
+                if (u3 < nunits) cp_async8(&sh.ptile[k3], &tiles[u3 / kCTile]);
+                sh.punit[k0] = 4 * nwarps + ahead;
+                ahead = atom_add_global(&wq[0], 1u);   // not looked at before the next cell
+            }
+        }
+        if (J.arrived) {
+            if (general) {
+                const G2Acc a = g2w_cell_general<DIMS, MODE>(sh, S, J, lane);
+                acc.relaxed += a.relaxed;
+                acc.removed += a.removed;
+            } else {
+                g2w_cell_impl<DIMS, MODE, false>(sh, S, J, par, 0u, lane, acc);
+            }
+            fence_proxy_async_smem();   // later copies come after these accesses
+            __syncwarp();
+        }
+    }
+    if (loaded >= 0) g2_flush(acc, s.dyn, lane);
+    if (!ok) {   // copies in flight land before the block may exit
+        if (lane == 0) atomicAdd(&sims[0].dyn->counters[kCntOverflow], kG2TimeoutMark);
+        mbar_wait(&sh.full[0], phase & 1u);
+        mbar_wait(&sh.full[1], phase >> 1 & 1u);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const uint32_t done = atomicAdd(&wq[0], 1u);
-        if (done == gridDim.x - 1) {   // the last CTA resets the queues for the next launch
-            wq[0] = 0;
-            for (int i = 0; i < nsims; ++i) sims[i].dyn->qnext = 0;
-        }
+        const uint32_t done = atomicAdd(&wq[1], 1u);
+        if (done == gridDim.x - 1) wq[0] = wq[1] = 0;   // the last block resets the counters for the next launch
     }
 }
-
 
 // ---------------------------------------------------------------------------
 // k_g1: per-cell moments (Eq. 1) in one pass, as sums of C = c - u_s about a
@@ -1415,19 +1598,6 @@ __global__ void __launch_bounds__(32 * (NC + 1), 16 / (NC + 1)) k_g2(const SimDe
 // ---------------------------------------------------------------------------
 constexpr int kG1Warps = 4;     // warps per block; a block takes one 32-cell tile at a time
 constexpr int kG1Stage = 384;   // slots of one pipeline stage (a multiple of 4)
-
-// per-lane asynchronous global -> shared copies (completion waited with
-// cp.async.wait_group by the issuing lane, then made visible to the warp
-// with __syncwarp)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                      const int* __restrict__ ntiles) {
@@ -1515,7 +1685,7 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
             const float4 us = h_us[cc];
             const float u0 = us.x, u1 = us.y, u2 = us.z;
             uint32_t nsp = 0;
-            if (arrived > nb) nsp = collect_spill(s, q, cell, spl_all[warp], lane);
+            if (arrived > nb) nsp = collect_spill(s, q, cell, spl_all[warp], 32u, lane);
             const uint32_t n = nb + nsp;
             float S[12];
 #pragma unroll
@@ -1801,14 +1971,7 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                 const float A10 = b * sig[3], A20 = b * sig[4], A21 = b * sig[5];
                 float l00 = 0, l10 = 0, l11 = 0, l20 = 0, l21 = 0, l22 = 0;
                 bool ok = A00 > 0.0f;
-                if (s.es_sampler) {
-                    // Gallis-Torczynski (Eq. 11): B = ((1 - Pr)/(2 Pr)) sigma* / (rho theta)
-                    // in the factor's slots, lower triangle row-major
-                    const float beta = (1.0f - (float)s.Pr) / (2.0f * (float)s.Pr * th);
-                    l00 = beta * sig[0]; l10 = beta * sig[3]; l11 = beta * sig[1];
-                    l20 = beta * sig[4]; l21 = beta * sig[5]; l22 = beta * sig[2];
-                    ok = true;
-                } else if (ok) {
+                if (ok) {
                     const float r0 = rsqrtf(A00);
                     l00 = A00 * r0;
                     l10 = A10 * r0;
@@ -1824,22 +1987,36 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                         if (ok) l22 = d2 * rsqrtf(d2);
                     }
                 }
-                if (!ok) {
-                    const float r = sqrtf(th);
-                    l00 = l11 = l22 = r;
-                    l10 = l20 = l21 = 0.0f;
-                    atomicAdd(&s.dyn->counters[kCntChol], 1ull);
+                if (s.es_sampler) {
+                    // Gallis-Torczynski (Eq. 11): B = ((1 - Pr)/(2 Pr)) sigma* / (rho theta)
+                    // in M's slots, lower triangle row-major
+                    const float beta = (1.0f - (float)s.Pr) / (2.0f * (float)s.Pr * th);
+                    pr[4] = beta * sig[0]; pr[5] = beta * sig[3]; pr[6] = beta * sig[1];
+                    pr[7] = beta * sig[4]; pr[8] = beta * sig[5]; pr[9] = beta * sig[2];
+                } else {
+                    if (!ok) {   // no Cholesky factor: an isotropic Gaussian
+                        l00 = l11 = l22 = sqrtf(th);
+                        l10 = l20 = l21 = 0.0f;
+                        atomicAdd(&s.dyn->counters[kCntChol], 1ull);
+                    }
+                    // M = L L^T - theta I (lower triangle, row-major)
+                    pr[4] = l00 * l00 - th;
+                    pr[5] = l10 * l00;
+                    pr[6] = l10 * l10 + l11 * l11 - th;
+                    pr[7] = l20 * l00;
+                    pr[8] = l20 * l10 + l21 * l11;
+                    pr[9] = l20 * l20 + l21 * l21 + l22 * l22 - th;
                 }
                 const float nues = (float)s.Pr * nu;
-                pr[4] = l00; pr[5] = l10; pr[6] = l11;
-                pr[7] = l20; pr[8] = l21; pr[9] = l22;
+                const float at = nues * s.f_dt;
                 pr[10] = -expm1f(-nues * s.f_dt);                                             // Eqs. 8b, 9
                 // the decay rate of Eq. 32; the SP-ESBGK step holds its target
                 // for the whole step (Eq. 8b): with P_ne = 0 a rate of 0 gives s = 1
                 pr[11] = s.mode == kModeSPESBGK ? 0.0f : nu;
-                pr[12] = nues;
+                pr[12] = 1.0f / nues;
                 pr[13] = pne;
-                pr[14] = 1.0f;
+                pr[14] = at < 1.0f ? expm1f(at) : -__expf(-at);
+                pr[15] = pr[10] > 0.0f ? 1.0f / pr[10] : 0.0f;
                 // heat flux from the third central moment of the shifted sums
                 const float d0 = M[1] * inv, d1 = M[2] * inv, d2 = M[3] * inv;
                 const float m00 = M[4] * inv, m11 = M[5] * inv, m22 = M[6] * inv;
@@ -1880,6 +2057,30 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
     }
 }
 
+// append one particle to the bucket of its cell (all 32 lanes call this
+// together; key == kNoCell for lanes with nothing to write)
+template <int DIM>
+__device__ __forceinline__ void emit_c(const SimDev& s, int b, uint32_t key, float x, float y, float v0, float v1,
+                                       float v2, uint32_t id, int lane) {
+    const unsigned grp = __match_any_sync(0xffffffffu, key);
+    if (key == kNoCell) return;
+    const int leader = __ffs(grp) - 1;
+    uint32_t base = 0;
+    if (lane == leader) base = atomicAdd(&s.cnt[b][key], (uint32_t)__popc(grp));
+    base = __shfl_sync(grp, base, leader);
+    const uint32_t i = s.lay[b][key] + base + (uint32_t)__popc(grp & lanemask_lt());
+    if (i < min(s.lay[b][key + 1], (uint32_t)s.cap)) {
+        if (DIM == 2) ((float*)s.pos[b][0])[i] = x;
+        ((float*)s.pos[b][1])[i] = y;
+        ((float*)s.vel[b][0])[i] = v0;
+        ((float*)s.vel[b][1])[i] = v1;
+        ((float*)s.vel[b][2])[i] = v2;
+        s.pid[b][i] = id;
+    } else {
+        spill<DIM>(s, b, (int)key, x, y, v0, v1, v2, id);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // k_inject_f: reservoir buffer cells, written into buffer q
 // ---------------------------------------------------------------------------
@@ -1898,8 +2099,6 @@ __global__ void __launch_bounds__(256) k_inject_f(const SimDev* __restrict__ sim
         if (!s.has_reservoir || s.dim != DIM) continue;
         const uint32_t step = s.dyn->step, next_pid = s.dyn->next_pid;
         const int q = s.dyn->cur ^ 1;
-        Ctx C;
-        make_ctx(s, q, C);
         for (int cc = warp; cc < kCTile; cc += 8) {
             const int cell = tile.y + cc;
             if (cell >= s.K) break;
@@ -1916,7 +2115,7 @@ __global__ void __launch_bounds__(256) k_inject_f(const SimDev* __restrict__ sim
                     make_particle<float>(s, cell, pid, step, kInject, F.theta, F.u, x, y, c);
                     key = (uint32_t)cell;
                 }
-                emit_c<DIM>(s, C, q, key, x, y, c[0], c[1], c[2], pid, lane);
+                emit_c<DIM>(s, q, key, x, y, c[0], c[1], c[2], pid, lane);
             }
         }
     }
@@ -2237,73 +2436,90 @@ __global__ void k_clear_pending(const SimDev* __restrict__ sims, int nsims) {
 }
 
 // ---------------------------------------------------------------------------
-// k_g2 launch configuration: NC consumer warps per CTA, 16 / (NC + 1) CTAs
-// per SM sharing its shared memory, the rest of which is each CTA's ring
+// k_g2 launch configuration: one wave of resident blocks
 // ---------------------------------------------------------------------------
-struct G2Config {
-    int grid;
-    uint32_t ring, max_stage;
-};
-
-template <int DIM, int MODE, int NC>
-const G2Config& g2_config() {
-    static G2Config cfg = {0, 0u, 0u};
-    if (!cfg.grid) {
-        int dev = 0, sms = 152, optin = 0, per_sm = 0;
+template <int DIMS, int MODE, bool ABL, int G>
+void launch_g2b_one(const Launch& L) {
+    static int wave = 0;   // blocks resident on the device (the same on every GB300)
+    if (!wave) {
+        int dev = 0, sms = 152, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        cudaFuncAttributes fa;
-        cudaFuncGetAttributes(&fa, k_g2<DIM, MODE, NC>);
-        const int ctas = 16 / (NC + 1);
-        int ring = std::min(per_sm / ctas - 1024, optin) - (int)fa.sharedSizeBytes;
-        ring &= ~1023;
-        int per = 0;
-        for (; ring >= 16384; ring -= 4096) {
-            cudaFuncSetAttribute(k_g2<DIM, MODE, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIM, MODE, NC>, 32 * (NC + 1), ring);
-            if (per >= ctas) break;
-        }
-        constexpr uint32_t bpp = g2_bytes_per_particle<DIM>();
-        cfg.ring = (uint32_t)ring;
-        cfg.max_stage = std::min(1024u, ((uint32_t)ring / (2u * bpp)) & ~3u);
-        cfg.grid = sms * std::max(per, 1);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2b<DIMS, MODE, ABL, G>, 32 * G, 0);
+        wave = sms * std::max(per, 1);
     }
-    return cfg;
+    const int grid = std::max(1, std::min(wave, L.cells));
+    k_g2b<DIMS, MODE, ABL, G><<<grid, 32 * G, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles, L.wq);
 }
 
-template <int DIM, int MODE, int NC>
-void launch_g2_one(const Launch& L) {
-    const G2Config& c = g2_config<DIM, MODE, NC>();
-    k_g2<DIM, MODE, NC><<<c.grid, 32 * (NC + 1), c.ring, L.stream>>>(L.sims, L.nsims, L.wq, c.ring, c.max_stage);
+template <int DIMS, int MODE>
+void launch_g2_one(const Launch& L, cudaStream_t st, bool part) {
+    static int wave = 0;
+    constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS>));
+    if (!wave) {
+        int dev = 0, sms = 152, per = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaFuncSetAttribute(k_g2<DIMS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE>, 32 * kG2wWarps, smem);
+        wave = sms * std::max(per, 1);
+    }
+    const int grid = std::max(1, std::min(wave, (L.cells + kG2wWarps - 1) / kG2wWarps));
+    const int* n = part ? (DIMS == 1 ? L.ndim : L.ndim + 1) : L.nctiles;
+    k_g2<DIMS, MODE><<<grid, 32 * kG2wWarps, smem, st>>>(L.sims, L.ctiles, n, part && DIMS == 2 ? L.ndim : nullptr,
+                                                         DIMS == 1 ? L.wq : L.wq + 2);
 }
 
-template <int MODE, int NC>
+// A mixed batch runs the kernels of both dimensions side by side (one kernel
+// with both bodies overflows the instruction cache where a block's warps are
+// in different ones): the 2-D one on the second stream, its blocks following
+// as those of the 1-D one finish.
+template <int MODE>
 void launch_g2(const Launch& L) {
-    if (L.dims & 1) launch_g2_one<1, MODE, NC>(L);
-    if (L.dims & 2) launch_g2_one<2, MODE, NC>(L);
+    if (L.dims == 1) {
+        launch_g2_one<1, MODE>(L, L.stream, false);
+    } else if (L.dims == 2) {
+        launch_g2_one<2, MODE>(L, L.stream, false);
+    } else if (!L.side) {
+        launch_g2_one<1, MODE>(L, L.stream, true);
+        launch_g2_one<2, MODE>(L, L.stream, true);
+    } else {
+        cudaEventRecord(L.ev_fork, L.stream);
+        cudaStreamWaitEvent(L.side, L.ev_fork, 0);
+        launch_g2_one<1, MODE>(L, L.stream, true);
+        launch_g2_one<2, MODE>(L, L.side, true);
+        cudaEventRecord(L.ev_join, L.side);
+        cudaStreamWaitEvent(L.stream, L.ev_join, 0);
+    }
 }
 
-// R (tuning): 4, 8, 12 select 3, 7 or 15 consumer warps per CTA
+template <int MODE, bool ABL, int G>
+void launch_g2b(const Launch& L) {
+    if constexpr (ABL || MODE == kRelaxOnly || MODE == kFullSlab) {   // seldom run: one form for both dimensions
+        launch_g2b_one<3, MODE, ABL, G>(L);
+    } else {
+        if (L.dims == 3) launch_g2b_one<3, MODE, ABL, G>(L);
+        else if (L.dims == 1) launch_g2b_one<1, MODE, ABL, G>(L);
+        else launch_g2b_one<2, MODE, ABL, G>(L);
+    }
+}
+
+// R (tuning): 4 one warp per cell, 8 and 12 a block of 4 or 8 warps
 template <int MODE>
 void launch_g2_R(const Launch& L, int R) {
-    if (R <= 4) launch_g2<MODE, 3>(L);
-    else if (R <= 8) launch_g2<MODE, 7>(L);
-    else launch_g2<MODE, 15>(L);
-}
-
-template <int MODE, int NC>
-void prepare_g2() {
-    g2_config<1, MODE, NC>();
-    g2_config<2, MODE, NC>();
-}
-
-template <int MODE>
-void prepare_g2_all() {
-    prepare_g2<MODE, 3>();
-    prepare_g2<MODE, 7>();
-    prepare_g2<MODE, 15>();
+    if (L.ablation) {
+        launch_g2b<MODE, true, 4>(L);
+    } else if constexpr (MODE == kRelaxOnly || MODE == kFullSlab) {
+        launch_g2b<MODE, false, 4>(L);
+    } else {
+        if (R <= 4) {
+            launch_g2<MODE>(L);
+        } else if (R <= 8) {
+            launch_g2b<MODE, false, 4>(L);
+        } else {
+            launch_g2b<MODE, false, 8>(L);
+        }
+    }
 }
 
 }  // namespace
@@ -2319,19 +2535,6 @@ void launch_fused_relax_stream(const Launch& L, int R, bool flush_only) {
     if (L.slabs) launch_g2_R<kFullSlab>(L, R);
     else if (L.flux) launch_g2_R<kFullFlux>(L, R);
     else launch_g2_R<kFull>(L, R);
-}
-
-// shared-memory limits and grids of the pipelined kernel, set once outside
-// any stream capture
-void fused_prepare_attributes() {
-    static bool done = false;
-    if (done) return;
-    done = true;
-    prepare_g2_all<kFull>();
-    prepare_g2_all<kRelaxOnly>();
-    prepare_g2_all<kFullSlab>();
-    prepare_g2_all<kFullFlux>();
-    cudaGetLastError();
 }
 
 void launch_fused_inject(const Launch& L) {

@@ -48,7 +48,6 @@ struct SimDyn {
     int cur;            // buffer holding the current state
     int relax_pending;  // fused pipeline: the relaxation of the last step is still to be applied
     uint32_t sp_n[2];   // fused pipeline: entries in the spill lists
-    uint32_t qnext;     // fused pipeline: next cell handed out by k_g2 (zero between launches)
     uint32_t lay_dst;   // fused pipeline: buffer whose bucket layout the layout kernels build
     uint32_t w_started; // weighted particles: bit 0 / 1, the step-2 / step-4,7 weight-field averages exist
     uint32_t w_added;   // weighted particles: particles added by the current stage
@@ -75,6 +74,8 @@ struct alignas(16) SimDev {
     int slab_count, slab_index, slab_first, row0, rows;
     // single-precision copies for the FP32 kernels (set on the host)
     float f_dt, f_lo[2], f_hi[2], f_inv_dx, f_inv_dy, f_bdt[3], f_w, f_inv_R, f_flux_pos;
+    float f_seg_pos[kMaxSeg];
+    int buf_lo[2], buf_hi[2];   // columns / global rows outside [buf_lo, buf_hi) are reservoir buffer cells
     int mode;
     double fixed_pne;
     // counting plane of the mass flow (Eq. 41): normal to x (1) or y (2) at
@@ -214,11 +215,14 @@ struct Launch {
     const int* nptiles;   // device scalar
     const int2* ctiles;   // (sim, first cell) tiles
     const int* nctiles;   // device scalar
-    uint32_t* wq;         // k_g2: warps done (2 words, zero between launches)
+    uint32_t* wq;         // k_g2: units handed out and blocks done, for each dimension (zero between launches)
+    const int* ndim;      // device: 1-D and 2-D cell tiles of a batch (the 1-D ones come first)
     int nsims;
     int dims;             // bit 0: some simulation is 1-D, bit 1: some is 2-D
     int slabs = 0;        // some simulation is a slab of a decomposed domain
     int flux = 0;         // some simulation counts particles through a plane
+    int ablation = 0;     // some simulation uses the fixed count or the Gallis-Torczynski sampler
+    int cells = 1;        // upper bound of the cells of all simulations (grid of k_g2)
     int grid_p, grid_c;   // persistent grid sizes
     int lay_tiles = 1;    // layout tiles (kLayTile cells) of the largest simulation
     cudaStream_t stream;
@@ -231,7 +235,7 @@ struct Launch {
 constexpr int kPTile = 512;   // particles per tile (small domains still spread over many SMs)
 constexpr int kCTile = 32;    // cells per tile (balances the per-cell kernels across SMs)
 constexpr int kSpillCap = 4096;  // spill entries per parity (fused pipeline)
-constexpr int kNFPrm = 16;       // u[3], theta, L[6], P_relax, nu, nu_ES, P_ne, valid, spare
+constexpr int kNFPrm = 16;       // u[3], theta, M[6], P_relax (0: none), nu, 1/nu_ES, P_ne, X, 1/P_relax (G2Prm)
 constexpr int kLayTile = 1024;   // cells per block of the layout kernels (fused pipeline)
 
 void launch_stream(const Launch& L, bool fp64);
@@ -265,7 +269,6 @@ void launch_fused_params(const Launch& L);
 void launch_fused_layout(const Launch& L);
 void launch_fused_layout_parts(const Launch& L);
 void launch_fused_step_end(const Launch& L);
-void fused_prepare_attributes();
 cudaError_t debug_philox(int64_t n, const uint32_t* d_ctr, uint32_t k0, uint32_t k1, uint32_t* d_out, cudaStream_t st);
 
 }  // namespace usp
