@@ -205,6 +205,7 @@ static Launch make_launch(usp_handle* h) {
     L.cells = h->host.K;
     L.grid_p = persistent_grid(h->nptiles, h->grid_per_sm);
     L.grid_c = persistent_grid(h->nctiles, h->grid_per_sm);
+    L.grid_f = persistent_grid(8 * h->nctiles, h->grid_per_sm);
     L.lay_tiles = (h->host.K + kLayTile - 1) / kLayTile;
     L.stream = h->stream;
     return L;
@@ -456,14 +457,24 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     s.f_w = (float)s.w;
     s.f_inv_R = (float)(1.0 / s.R);
     s.inv_R = 1.0 / s.R;
+    s.es_b = 1.0 - 1.0 / s.Pr;
     for (int g = 0; g < nseg; ++g) s.f_seg_pos[g] = (float)s.seg[g].pos;
+    s.f_mass = (float)s.mass;
+    s.f_mu_ref = (float)s.mu_ref;
+    s.f_T_ref = (float)s.T_ref;
+    s.f_omega = (float)s.omega;
+    s.f_Pr = (float)s.Pr;
+    s.f_R = (float)s.R;
+    s.f_es_b = (float)s.es_b;
+    s.f_fixed_pne = (float)s.fixed_pne;
+    s.f_h[0] = (float)s.dx;
+    s.f_h[1] = (float)s.dy;
     for (int a = 0; a < 2; ++a) {   // without reservoir faces: no buffer cells
         const int n = a == 0 ? s.nx : s.ny;
         const bool on = any_res && (s.dim == 2 || a == 1);
         s.buf_lo[a] = on && s.face[2 * a].kind == kBcReservoir ? s.reservoir_cols : 0;
         s.buf_hi[a] = on && s.face[2 * a + 1].kind == kBcReservoir ? n - s.reservoir_cols : n;
     }
-    s.es_b = 1.0 - 1.0 / s.Pr;
 
     const int K = s.K;
     int rc = USP_OK;
@@ -1435,6 +1446,7 @@ static Launch batch_launch(usp_batch* b) {
     for (auto* h : b->members) per_sm = std::max(per_sm, h->grid_per_sm);
     L.grid_p = persistent_grid(1 << 30, per_sm);
     L.grid_c = persistent_grid(1 << 30, per_sm);
+    L.grid_f = L.grid_c;
     L.lay_tiles = b->lay_tiles;
     L.stream = b->stream;
     return L;

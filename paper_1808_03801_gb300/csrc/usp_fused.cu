@@ -1598,11 +1598,12 @@ __global__ void __launch_bounds__(32 * kG2wWarps, kG2wBlocks) k_g2(const SimDev*
 // ---------------------------------------------------------------------------
 constexpr int kG1Warps = 4;     // warps per block; a block takes one 32-cell tile at a time
 constexpr int kG1Stage = 384;   // slots of one pipeline stage (a multiple of 4)
+constexpr int kG1Units = 1;     // units per block wanted
 
 __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                      const int* __restrict__ ntiles) {
     __shared__ uint32_t spl_all[kG1Warps][32];
-    // the tile's per-cell headers, fetched in one round for all 32 cells:
+    // the unit's per-cell headers, fetched in one round for all its cells:
     // bucket start, particles in the bucket, arrivals, and the shift u_s
     __shared__ uint32_t h_base[kCTile], h_nb[kCTile], h_arr[kCTile];
     __shared__ float4 h_us[kCTile];
@@ -1610,16 +1611,29 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
     __shared__ __align__(16) float stage[kG1Warps][2][3][kG1Stage];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ SimDev sim_sh;
+    // A unit is a whole tile or, until every block has kG1Units of them, a
+    // half, quarter or eighth of one (down to one cell per warp), so that few
+    // cells spread over all SMs: one shock tube of 1000 cells 16.6 -> 8.9 us.
+    // More units than blocks cost what the next cell's copy ahead gains
+    // (cavity 200 x 200: 34 us with 1, 37 / 42 / 54 us with 2 / 4 / 8).
     const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
+    int parts = 1;
+    while (parts < kCTile / kG1Warps && nt * parts < kG1Units * (int)gridDim.x) parts *= 2;
+    const int ncell = kCTile / parts;   // cells of a unit
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nt * parts; t += gridDim.x) {
+        int2 tile = tiles[t / parts];
+        tile.y += (t % parts) * ncell;
         __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+        if (tile.x != loaded) {
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const int K = s.K;
         const int q = s.dyn->cur ^ 1;
-        if (threadIdx.x < kCTile && tile.y + (int)threadIdx.x < K) {
+        if ((int)threadIdx.x < ncell && tile.y + (int)threadIdx.x < K) {
             const int cell = tile.y + (int)threadIdx.x;
             const uint32_t base = s.lay[q][cell];
             const uint32_t top = min(s.lay[q][cell + 1], (uint32_t)s.cap);
@@ -1639,7 +1653,7 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
         // of two stages while the chunk before it is summed: a cell's whole
         // bucket is in flight at once, and its round trip overlaps the
         // previous chunk's work.  (c, o) is the next chunk to copy.
-        auto live = [&](int c) { return c < kCTile && tile.y + c < K; };
+        auto live = [&](int c) { return c < ncell && tile.y + c < K; };
         auto copy_chunk = [&](int c, uint32_t o, int b) {
             const uint32_t g = h_base[c] + o;
             const uint32_t len = min(h_nb[c] - o, (uint32_t)kG1Stage);
@@ -1831,26 +1845,25 @@ __device__ __forceinline__ void local_nb(const SimDev& s, int cell, LocalF& L) {
     L.N = 0;
 }
 
-// state of the neighbour of `cell` along `axis` (dir = -1 / +1) for the
+// state of the neighbour of cell (ix, iy) along `axis` (dir = -1 / +1) for the
 // Kn_GLL stencil; across a slab boundary it is the adjacent slab's row.
 // Returns whether the neighbour exists and is valid.
-__device__ __forceinline__ bool nb_state(const SimDev* __restrict__ sims, const SimDev& s, int cell, int axis, int dir,
-                                         LocalF& L) {
-    const int ix = cell % s.nx, iy = cell / s.nx;
+__device__ __forceinline__ bool nb_state(const SimDev* __restrict__ sims, const SimDev& s, int ix, int iy, int axis,
+                                         int dir, LocalF& L) {
     const SimDev* t = &s;
     int c;
     if (axis == 0) {
         int j = ix + dir;
         if (j < 0 || j >= s.nx) {
             if (!s.periodic_x) return false;
-            j = (j + s.nx) % s.nx;
+            j = j < 0 ? j + s.nx : j - s.nx;
         }
         c = iy * s.nx + j;
     } else {
         int gj = s.row0 + iy + dir;   // global row
         if (gj < 0 || gj >= s.ny) {
             if (!s.periodic_y) return false;
-            gj = (gj + s.ny) % s.ny;
+            gj = gj < 0 ? gj + s.ny : gj - s.ny;
         }
         const int r = gj - s.row0;
         if (r >= 0 && r < s.rows) {
@@ -1888,9 +1901,12 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
             LocalF Nm[2] = {}, Np[2] = {};
             bool hm[2] = {false, false}, hp[2] = {false, false};
             if (s.mode == kModeUSP) {
-                for (int axis = s.dim == 1 ? 1 : 0; axis < 2; ++axis) {
-                    hm[axis] = nb_state(sims, s, cell, axis, -1, Nm[axis]);
-                    hp[axis] = nb_state(sims, s, cell, axis, +1, Np[axis]);
+                const int iy = s.dim == 1 ? cell : cell / s.nx, ix = s.dim == 1 ? 0 : cell - iy * s.nx;
+#pragma unroll
+                for (int axis = 0; axis < 2; ++axis) {
+                    if (axis == 0 && s.dim == 1) continue;
+                    hm[axis] = nb_state(sims, s, ix, iy, axis, -1, Nm[axis]);
+                    hp[axis] = nb_state(sims, s, ix, iy, axis, +1, Np[axis]);
                 }
             }
             LocalF L;
@@ -1910,14 +1926,14 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
             pr[3] = th;
             if (L.valid) {
                 const float thf = th;
-                const float rho = L.n * (float)s.mass;
+                const float rho = L.n * s.f_mass;
                 const float pf = rho * thf;
-                const float mu = (float)s.mu_ref * __powf(L.T / (float)s.T_ref, (float)s.omega);   // Eq. 35
+                const float mu = s.f_mu_ref * __powf(L.T / s.f_T_ref, s.f_omega);   // Eq. 35
                 const float nu = pf / mu;
                 const float lam = 1.2766152f * mu / sqrtf(rho * pf);     // Eq. 36: 16 / (5 sqrt(2 pi))
                 float pne;
                 if (s.mode == kModeSP || s.mode == kModeSPESBGK) pne = 0.0f;
-                else if (s.mode == kModeFixed) pne = (float)s.fixed_pne;
+                else if (s.mode == kModeFixed) pne = s.f_fixed_pne;
                 else {
                     // the cell's own stencil state: instantaneous, or the
                     // Eq. 34 average (loaded above, before this step's update)
@@ -1929,9 +1945,9 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                         gu = (float)sqrt(av[1] * av[1] + av[2] * av[2] + av[3] * av[3]);
                         gvalid = gn > 0.0f && gT > 0.0f;
                         if (gvalid) {
-                            const float gth = gT * (float)s.R;
-                            const float grho = gn * (float)s.mass;
-                            const float gmu = (float)s.mu_ref * __powf(gT / (float)s.T_ref, (float)s.omega);
+                            const float gth = gT * s.f_R;
+                            const float grho = gn * s.f_mass;
+                            const float gmu = s.f_mu_ref * __powf(gT / s.f_T_ref, s.f_omega);
                             glam = 1.2766152f * gmu / sqrtf(grho * grho * gth);   // Eq. 36 at the averaged state
                             ga = sqrtf((float)kGammaMono * gth);
                         }
@@ -1943,8 +1959,10 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                     const float Qc[3] = {gn, gT, gu};
                     const float rq[3] = {1.0f / gn, 1.0f / gT, 1.0f / fmaxf(gu, a_s)};
                     float g2[3] = {0, 0, 0};
-                    for (int axis = s.dim == 1 ? 1 : 0; axis < 2; ++axis) {
-                        const float h = (float)(axis == 0 ? s.dx : s.dy);
+#pragma unroll
+                    for (int axis = 0; axis < 2; ++axis) {
+                        if (axis == 0 && s.dim == 1) continue;
+                        const float h = s.f_h[axis];
                         const LocalF& Lm = Nm[axis];
                         const LocalF& Lp = Np[axis];
                         const int m = hm[axis] ? 1 : -1;
@@ -1963,10 +1981,10 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                 }
                 // Eq. 33
                 const float ifs = 1.0f / (1.0f + 0.5f * s.f_dt * nu * pne);
-                const float ifq = 1.0f / (1.0f + 0.5f * s.f_dt * nu * (float)s.Pr * pne);
+                const float ifq = 1.0f / (1.0f + 0.5f * s.f_dt * nu * s.f_Pr * pne);
                 const float sig[6] = {(P[0] - th) * ifs, (P[1] - th) * ifs, (P[2] - th) * ifs, P[3] * ifs, P[4] * ifs,
                                       P[5] * ifs};
-                const float b = (float)s.es_b;                                                  // Eq. 6c
+                const float b = s.f_es_b;                                                  // Eq. 6c
                 const float A00 = th + b * sig[0], A11 = th + b * sig[1], A22 = th + b * sig[2];
                 const float A10 = b * sig[3], A20 = b * sig[4], A21 = b * sig[5];
                 float l00 = 0, l10 = 0, l11 = 0, l20 = 0, l21 = 0, l22 = 0;
@@ -1990,7 +2008,7 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                 if (s.es_sampler) {
                     // Gallis-Torczynski (Eq. 11): B = ((1 - Pr)/(2 Pr)) sigma* / (rho theta)
                     // in M's slots, lower triangle row-major
-                    const float beta = (1.0f - (float)s.Pr) / (2.0f * (float)s.Pr * th);
+                    const float beta = (1.0f - s.f_Pr) / (2.0f * s.f_Pr * th);
                     pr[4] = beta * sig[0]; pr[5] = beta * sig[3]; pr[6] = beta * sig[1];
                     pr[7] = beta * sig[4]; pr[8] = beta * sig[5]; pr[9] = beta * sig[2];
                 } else {
@@ -2007,7 +2025,7 @@ __global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sim
                     pr[8] = l20 * l10 + l21 * l11;
                     pr[9] = l20 * l20 + l21 * l21 + l22 * l22 - th;
                 }
-                const float nues = (float)s.Pr * nu;
+                const float nues = s.f_Pr * nu;
                 const float at = nues * s.f_dt;
                 pr[10] = -expm1f(-nues * s.f_dt);                                             // Eqs. 8b, 9
                 // the decay rate of Eq. 32; the SP-ESBGK step holds its target
@@ -2387,6 +2405,61 @@ __global__ void __launch_bounds__(kLayTile) k_lay_scan(const SimDev* __restrict_
     }
 }
 
+// the three in one, a block per simulation, where every simulation has at
+// most kLaySmall cells (each thread a run of consecutive cells): the layout
+// then takes one latency instead of three (measured on one simulation of 1000
+// cells: 20 -> 8 us), so that it stays behind k_g1 and k_params_f
+constexpr int kLaySmall = 8 * 1024;
+
+__global__ void __launch_bounds__(1024) k_lay_small(const SimDev* __restrict__ sims) {
+    __shared__ unsigned long long sh[33];
+    const SimDev& s = sims[blockIdx.x];
+    SimDyn* dyn = s.dyn;
+    const int K = s.K, cur = dyn->cur;
+    const uint32_t* C = s.cnt[cur ^ 1];
+    uint32_t* const lay = s.lay[cur];
+    uint32_t* const cnt = s.cnt[cur];
+    const int per = (K + 1023) / 1024;   // at most 8
+    const int c0 = min((int)threadIdx.x * per, K), c1 = min(c0 + per, K);
+    uint32_t slack[8], tight[8];
+    unsigned long long f = 0, g = 0, e = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        slack[k] = tight[k] = 0;
+        if (c0 + k < c1) {
+            slack[k] = bucket_size(s, C, c0 + k);
+            tight[k] = tight_size(s, C, c0 + k);
+            f += slack[k];
+            g += tight[k];
+            e += C[c0 + k];
+        }
+    }
+    unsigned long long tot_full, tot_tight;
+    const unsigned long long xf = block_scan_1024(f, sh, &tot_full);
+    const unsigned long long xg = block_scan_1024(g, sh, &tot_tight);
+    const unsigned long long tot_exact = block_sum_1024(e, sh);
+    const unsigned long long cap = (unsigned long long)s.cap;
+    const bool full = tot_full <= cap;
+    const unsigned long long extra =
+        (!full && tot_tight < cap) ? ((cap - tot_tight) / (unsigned long long)K) & ~3ull : 0ull;
+    unsigned long long x = full ? xf : xg + extra * (unsigned long long)c0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (c0 + k < c1) {
+            lay[c0 + k] = (uint32_t)min(x, 0xFFFFFFFFull);
+            cnt[c0 + k] = 0;
+            x += full ? slack[k] : tight[k] + extra;
+        }
+    if (threadIdx.x == 0) {
+        const unsigned long long demand = tot_exact + (s.has_reservoir ? s.inj_total : 0u);
+        if (!full && demand > cap) atomicAdd(&dyn->counters[kCntOverflow], 1ull);
+        lay[K] = (uint32_t)min(full ? tot_full : tot_tight + extra * (unsigned long long)K, 0xFFFFFFFFull);
+        dyn->n = (uint32_t)min(tot_exact, 0xFFFFFFFFull);
+        dyn->sp_n[cur] = 0;
+        dyn->lay_dst = (uint32_t)cur;
+    }
+}
+
 // end of the step (after the layout and the parameters): buffers swap, the
 // step counter and the sample count advance, the relaxation becomes pending
 __global__ void k_step_end(const SimDev* __restrict__ sims, int nsims) {
@@ -2544,7 +2617,7 @@ void launch_fused_inject(const Launch& L) {
 
 void launch_fused_moments(const Launch& L, int R) {
     (void)R;
-    k_g1<<<L.grid_c, 32 * kG1Warps, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+    k_g1<<<L.grid_f, 32 * kG1Warps, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 
 void launch_fused_params(const Launch& L) { k_params_f<<<L.grid_c, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles); }
@@ -2552,6 +2625,10 @@ void launch_fused_params(const Launch& L) { k_params_f<<<L.grid_c, 32, 0, L.stre
 // the bucket layout of the next step's destination buffer (reads only the
 // arrivals of this step, so it may run beside k_g1 and k_params_f)
 void launch_fused_layout_parts(const Launch& L) {
+    if (L.lay_tiles * kLayTile <= kLaySmall) {
+        k_lay_small<<<L.nsims, 1024, 0, L.stream>>>(L.sims);
+        return;
+    }
     const dim3 grid((unsigned)std::min(L.lay_tiles, 1024), (unsigned)L.nsims);
     k_lay_sum<<<grid, kLayTile, 0, L.stream>>>(L.sims);
     k_lay_scan<<<L.nsims, kLayTile, 0, L.stream>>>(L.sims, L.nsims);

@@ -74,6 +74,7 @@ struct alignas(16) SimDev {
     int slab_count, slab_index, slab_first, row0, rows;
     // single-precision copies for the FP32 kernels (set on the host)
     float f_dt, f_lo[2], f_hi[2], f_inv_dx, f_inv_dy, f_bdt[3], f_w, f_inv_R, f_flux_pos;
+    float f_mass, f_mu_ref, f_T_ref, f_omega, f_Pr, f_R, f_es_b, f_fixed_pne, f_h[2];
     float f_seg_pos[kMaxSeg];
     int buf_lo[2], buf_hi[2];   // columns / global rows outside [buf_lo, buf_hi) are reservoir buffer cells
     int mode;
@@ -224,6 +225,7 @@ struct Launch {
     int ablation = 0;     // some simulation uses the fixed count or the Gallis-Torczynski sampler
     int cells = 1;        // upper bound of the cells of all simulations (grid of k_g2)
     int grid_p, grid_c;   // persistent grid sizes
+    int grid_f = 1;       // grid of k_g1 (its units are parts of cell tiles)
     int lay_tiles = 1;    // layout tiles (kLayTile cells) of the largest simulation
     cudaStream_t stream;
     // fused step: a second stream and two events let the layout kernels run
