@@ -204,6 +204,7 @@ static Launch make_launch(usp_handle* h) {
     L.ablation = h->host.selection || h->host.es_sampler;
     L.cells = h->host.K;
     L.grid_p = persistent_grid(h->nptiles, h->grid_per_sm);
+    L.grid_u = persistent_grid(h->nptiles * (kPTile / kPUnit), 2 * h->grid_per_sm);
     L.grid_c = persistent_grid(h->nctiles, h->grid_per_sm);
     L.grid_f = persistent_grid(8 * h->nctiles, h->grid_per_sm);
     L.lay_tiles = (h->host.K + kLayTile - 1) / kLayTile;
@@ -269,6 +270,12 @@ static int choose_R(int64_t cells, int ppc_ref, int dim) {
     if (ppc_ref > (dim == 1 ? 370 : 320)) return 12;
     if (cells > 10 * (int64_t)sms) return 4;
     return cells <= 2 * (int64_t)sms && ppc_ref > 128 ? 12 : 8;
+}
+
+// a load goes back to the default variant
+static void set_default_R(usp_handle* h) {
+    h->fused_R = choose_R(h->host.K, h->ppc_ref, h->host.dim);
+    h->tuned = false;
 }
 
 static int count_for_density(const SimDev& s, double n, double n_ref, int ppc_ref) {
@@ -458,7 +465,11 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     s.f_inv_R = (float)(1.0 / s.R);
     s.inv_R = 1.0 / s.R;
     s.es_b = 1.0 - 1.0 / s.Pr;
+    s.inv_d[0] = 1.0 / s.dx;
+    s.inv_d[1] = 1.0 / s.dy;
+    s.inv_T_ref = 1.0 / s.T_ref;
     for (int g = 0; g < nseg; ++g) s.f_seg_pos[g] = (float)s.seg[g].pos;
+    for (int d = 0; d < 3; ++d) s.f_body[d] = (float)s.body[d];
     s.f_mass = (float)s.mass;
     s.f_mu_ref = (float)s.mu_ref;
     s.f_T_ref = (float)s.T_ref;
@@ -770,8 +781,7 @@ extern "C" int usp_init_particles(usp_handle* h, const usp_region* regions, int 
     if (rc) return rc;
     if (e != cudaSuccess) return fail(h, USP_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e));
     if (h->pipeline == USP_PIPE_FUSED) {
-        h->fused_R = choose_R(K, h->ppc_ref, s.dim);
-        h->tuned = false;
+        set_default_R(h);
         Launch L = make_launch(h);
         // no parameters yet: zero shift for the first moments, no relaxation
         CK(cudaMemsetAsync(h->host.fprm, 0, sizeof(float) * kNFPrm * (size_t)K, h->stream));
@@ -801,8 +811,7 @@ static int fused_from_unsorted(usp_handle* h) {
     CK(cudaMemsetAsync(s.fprm, 0, sizeof(float) * kNFPrm * (size_t)K, h->stream));
     int one = 1;   // pageable: copied out before the call returns
     CK(cudaMemcpyAsync(&h->d_dyn->cur, &one, sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    h->fused_R = choose_R(K, h->ppc_ref, s.dim);
-    h->tuned = false;
+    set_default_R(h);
     launch_fused_setup(L);
     CK(cudaGetLastError());
     return USP_OK;
@@ -1445,6 +1454,7 @@ static Launch batch_launch(usp_batch* b) {
     int per_sm = 1;
     for (auto* h : b->members) per_sm = std::max(per_sm, h->grid_per_sm);
     L.grid_p = persistent_grid(1 << 30, per_sm);
+    L.grid_u = persistent_grid(1 << 30, 2 * per_sm);
     L.grid_c = persistent_grid(1 << 30, per_sm);
     L.grid_f = L.grid_c;
     L.lay_tiles = b->lay_tiles;

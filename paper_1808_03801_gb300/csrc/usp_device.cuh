@@ -37,16 +37,36 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+// unit t of the particle tiles: its simulation and first particle slot
+__device__ __forceinline__ int2 unit_of(const int2* tiles, int t) {
+    int2 u = tiles[t / (kPTile / kPUnit)];
+    u.y += (t % (kPTile / kPUnit)) * kPUnit;
+    return u;
+}
+
 // ---------------------------------------------------------------------------
 // cells
 // ---------------------------------------------------------------------------
+// floor((v - lo) / d), as the division gives it.  FP64: from the product with
+// 1 / d, whose error is below 1e-6 for any grid (2^28 cells); within that of a
+// whole number the division decides.  (An FP64 division costs about twenty FP64
+// instructions.)
+__device__ __forceinline__ float cell_floor(const SimDev& s, int axis, float v) {
+    return floorf((v - s.f_lo[axis]) / s.f_h[axis]);
+}
+__device__ __forceinline__ double cell_floor(const SimDev& s, int axis, double v) {
+    const double o = v - s.lo[axis], q = o * s.inv_d[axis], f = floor(q), r = q - f;
+    if (r > 1e-6 && r < 1.0 - 1e-6) return f;
+    return floor(o / (axis == 0 ? s.dx : s.dy));
+}
+
 template <class T>
 __device__ __forceinline__ int cell_index(const SimDev& s, T x, T y) {
-    T fy = dev_floor<T>((y - (T)s.lo[1]) / (T)s.dy);
+    T fy = cell_floor(s, 1, y);
     fy = fy < (T)0 ? (T)0 : (fy > (T)(s.ny - 1) ? (T)(s.ny - 1) : fy);
     int iy = (int)fy;
     if (s.dim == 1) return iy;
-    T fx = dev_floor<T>((x - (T)s.lo[0]) / (T)s.dx);
+    T fx = cell_floor(s, 0, x);
     fx = fx < (T)0 ? (T)0 : (fx > (T)(s.nx - 1) ? (T)(s.nx - 1) : fx);
     return iy * s.nx + (int)fx;
 }
@@ -149,7 +169,9 @@ __device__ __forceinline__ void diffuse(const SimDev& s, uint32_t pid, uint32_t 
 template <class T>
 __device__ __forceinline__ T wrap(T v, double lo, double hi) {
     T L = (T)(hi - lo);
-    T r = fmod(v - (T)lo, L);
+    T r = v - (T)lo;
+    if (r >= (T)0 && r < L) return (T)lo + r;   // fmod(r, L) is r
+    r = fmod(r, L);
     if (r < (T)0) r += L;
     return (T)lo + r;
 }
@@ -199,6 +221,39 @@ __device__ bool advect(const SimDev& s, uint32_t step, uint32_t pid, T& x, T& y,
             else diffuse<T>(s, pid, step, (uint32_t)k, 0, dir, G.theta, G.sqrt_theta, G.u, c);
         }
     }
+    if (s.dim == 2 && s.periodic_x) x = wrap<T>(x, s.lo[0], s.hi[0]);
+    if (s.periodic_y) y = wrap<T>(y, s.lo[1], s.hi[1]);
+    return true;
+}
+
+// the flight of a particle that stays clear of every face and plate by a
+// margin far above rounding (a ten-millionth of the domain in FP64, 1e-5 in
+// FP32), where `advect` would find no hit; false if it does not, the particle
+// left as it was.  Spares the FP64 divisions of the hit times; FP32 reads the
+// single-precision constants (a conversion is FP64 work too).
+template <class T>
+__device__ __forceinline__ bool advect_clear(const SimDev& s, T& x, T& y, T* c) {
+    constexpr bool F = sizeof(T) == 4;
+    const T eps = F ? (T)1e-5 : (T)1e-7;
+    const T tau = F ? (T)s.f_dt : (T)s.dt;
+    const T xn = x + c[0] * tau, yn = y + c[1] * tau;
+    if (!s.periodic_y) {
+        const T lo = F ? (T)s.f_lo[1] : (T)s.lo[1], hi = F ? (T)s.f_hi[1] : (T)s.hi[1], m = eps * (hi - lo);
+        if (!(yn > lo + m && yn < hi - m)) return false;
+    }
+    if (s.dim == 2) {
+        const T lo = F ? (T)s.f_lo[0] : (T)s.lo[0], hi = F ? (T)s.f_hi[0] : (T)s.hi[0], m = eps * (hi - lo);
+        if (!s.periodic_x && !(xn > lo + m && xn < hi - m)) return false;
+        for (int g = 0; g < s.nseg; ++g) {
+            const T ps = F ? (T)s.f_seg_pos[g] : (T)s.seg[g].pos;
+            const T a = x - ps, b = xn - ps;
+            if (!((a > m && b > m) || (a < -m && b < -m))) return false;
+        }
+        x = xn;
+    }
+    y = yn;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) c[d] += (F ? (T)s.f_body[d] : (T)s.body[d]) * tau;
     if (s.dim == 2 && s.periodic_x) x = wrap<T>(x, s.lo[0], s.hi[0]);
     if (s.periodic_y) y = wrap<T>(y, s.lo[1], s.hi[1]);
     return true;
@@ -298,7 +353,7 @@ __device__ __forceinline__ void local_state(const SimDev& s, int cell, Local& L,
     const double m00 = M[4 * K + cell] * inv, m11 = M[5 * K + cell] * inv, m22 = M[6 * K + cell] * inv;
     const double m01 = M[7 * K + cell] * inv, m02 = M[8 * K + cell] * inv, m12 = M[9 * K + cell] * inv;
     double P[6] = {m00 - d0 * d0, m11 - d1 * d1, m22 - d2 * d2, m01 - d0 * d1, m02 - d0 * d2, m12 - d1 * d2};
-    L.theta = (P[0] + P[1] + P[2]) / 3.0;
+    L.theta = (P[0] + P[1] + P[2]) * (1.0 / 3.0);
     if (P6)
         for (int k = 0; k < 6; ++k) P6[k] = P[k];
     if (Q3) {
@@ -315,14 +370,26 @@ __device__ __forceinline__ void local_state(const SimDev& s, int cell, Local& L,
     }
     L.valid = N >= 2 && (!s.weighted || we > 1.0) && L.theta > 0.0;
     if (!L.valid) return;
-    L.T = L.theta / s.R;
+    L.T = L.theta * s.inv_R;
     L.umag = sqrt(L.u[0] * L.u[0] + L.u[1] * L.u[1] + L.u[2] * L.u[2]);
-    L.a_sound = sqrt(kGammaMono * L.theta);
+}
+
+// (T / T_ref)^omega of Eq. 35 (a hard-sphere gas has omega = 1/2)
+__device__ __forceinline__ double visc_power(const SimDev& s, double T) {
+    const double r = T * s.inv_T_ref;
+    return s.omega == 0.5 ? sqrt(r) : pow(r, s.omega);
+}
+
+// sound speed, viscosity, collision frequency and mean free path of a valid
+// state (Eqs. 35-36)
+__device__ __forceinline__ void local_transport(const SimDev& s, Local& L) {
+    const double st = sqrt(L.theta);
+    L.a_sound = 1.2909944487358056 * st;                                        // sqrt(5/3 theta)
     L.rho = L.n * s.mass;
     L.p = L.rho * L.theta;
-    L.mu = s.mu_ref * pow(L.T / s.T_ref, s.omega);                              // Eq. 35
+    L.mu = s.mu_ref * visc_power(s, L.T);                                       // Eq. 35
     L.nu = L.p / L.mu;                                                          // nu = p / mu
-    L.lambda = 16.0 / (5.0 * sqrt(2.0 * kPi)) * L.mu / sqrt(L.rho * L.p);       // Eq. 36
+    L.lambda = 16.0 / (5.0 * sqrt(2.0 * kPi)) * L.mu / (L.rho * st);            // Eq. 36
 }
 
 // state a cell contributes to the Kn_GLL stencil (Eqs. 17-18): its
@@ -350,19 +417,22 @@ __device__ __forceinline__ void snap_avg(const SimDev& s, int cell) {
     s.gavg[(size_t)2 * K + cell] = sqrt(u0 * u0 + u1 * u1 + u2 * u2);
 }
 
-__device__ __forceinline__ void grad_from_avg(const SimDev& s, int cell, GradState& G) {
+// (lambda and the sound speed only for the cell itself)
+__device__ __forceinline__ void grad_from_avg(const SimDev& s, int cell, GradState& G, bool own) {
     const int K = s.K;
     G.n = s.gavg[cell];
     G.T = s.gavg[(size_t)K + cell];
     G.umag = s.gavg[(size_t)2 * K + cell];
     G.valid = G.n > 0.0 && G.T > 0.0;
     G.a_sound = G.lambda = 0.0;
-    if (!G.valid) return;
-    const double theta = s.R * G.T;
-    G.a_sound = sqrt(kGammaMono * theta);
-    const double rho = G.n * s.mass, p = rho * theta;
-    const double mu = s.mu_ref * pow(G.T / s.T_ref, s.omega);                 // Eq. 35
-    G.lambda = 16.0 / (5.0 * sqrt(2.0 * kPi)) * mu / sqrt(rho * p);           // Eq. 36
+    if (!G.valid || !own) return;
+    Local L;
+    L.n = G.n;
+    L.T = G.T;
+    L.theta = s.R * G.T;
+    local_transport(s, L);
+    G.a_sound = L.a_sound;
+    G.lambda = L.lambda;
 }
 
 __device__ __forceinline__ void grad_from_local(const Local& L, GradState& G) {
@@ -374,16 +444,15 @@ __device__ __forceinline__ void grad_from_local(const Local& L, GradState& G) {
     G.lambda = L.lambda;
 }
 
-// the stencil state of a cell as k_moments stored it (plain pipeline), or
-// computed from its sums when no store exists
-__device__ __forceinline__ void store_grad_state(const SimDev& s, int cell, const GradState& G) {
+// the stencil state of a cell as k_moments stores it for its neighbours
+// (plain pipeline)
+__device__ __forceinline__ void store_grad_state(const SimDev& s, int cell, bool valid, double n, double T,
+                                                 double umag) {
     const size_t K = (size_t)s.K;
-    s.gloc[cell] = G.valid ? 1.0 : 0.0;
-    s.gloc[K + cell] = G.n;
-    s.gloc[2 * K + cell] = G.T;
-    s.gloc[3 * K + cell] = G.umag;
-    s.gloc[4 * K + cell] = G.a_sound;
-    s.gloc[5 * K + cell] = G.lambda;
+    s.gloc[cell] = valid ? 1.0 : 0.0;
+    s.gloc[K + cell] = n;
+    s.gloc[2 * K + cell] = T;
+    s.gloc[3 * K + cell] = umag;
 }
 
 __device__ __forceinline__ void load_grad_state(const SimDev& s, int cell, GradState& G) {
@@ -392,8 +461,7 @@ __device__ __forceinline__ void load_grad_state(const SimDev& s, int cell, GradS
     G.n = s.gloc[K + cell];
     G.T = s.gloc[2 * K + cell];
     G.umag = s.gloc[3 * K + cell];
-    G.a_sound = s.gloc[4 * K + cell];
-    G.lambda = s.gloc[5 * K + cell];
+    G.a_sound = G.lambda = 0.0;
 }
 
 __device__ __forceinline__ int neighbor(const SimDev& s, int cell, int axis, int dir) {

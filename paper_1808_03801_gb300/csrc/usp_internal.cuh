@@ -68,13 +68,14 @@ struct alignas(16) SimDev {
     double R, mass, mu_ref, T_ref, omega, Pr, dt, w;   // w: number density carried by one particle
     double avg_keep, avg_new;                          // (n_a - 1)/n_a, 1/n_a
     double inv_R, es_b;                                // 1/R and 1 - 1/Pr (Eq. 6c), set on the host
+    double inv_d[2], inv_T_ref;                        // 1/dx, 1/dy, 1/T_ref
     // spatial decomposition: this handle owns rows [row0, row0 + rows) of the
     // grid above (K = nx * rows cells, local index = global - row0 * nx);
     // slab_first is the batch index of slab 0 (-1 outside a batch)
     int slab_count, slab_index, slab_first, row0, rows;
     // single-precision copies for the FP32 kernels (set on the host)
     float f_dt, f_lo[2], f_hi[2], f_inv_dx, f_inv_dy, f_bdt[3], f_w, f_inv_R, f_flux_pos;
-    float f_mass, f_mu_ref, f_T_ref, f_omega, f_Pr, f_R, f_es_b, f_fixed_pne, f_h[2];
+    float f_body[3], f_mass, f_mu_ref, f_T_ref, f_omega, f_Pr, f_R, f_es_b, f_fixed_pne, f_h[2];
     float f_seg_pos[kMaxSeg];
     int buf_lo[2], buf_hi[2];   // columns / global rows outside [buf_lo, buf_hi) are reservoir buffer cells
     int mode;
@@ -225,6 +226,7 @@ struct Launch {
     int ablation = 0;     // some simulation uses the fixed count or the Gallis-Torczynski sampler
     int cells = 1;        // upper bound of the cells of all simulations (grid of k_g2)
     int grid_p, grid_c;   // persistent grid sizes
+    int grid_u = 1;       // grid of the particle kernels (units of kPUnit)
     int grid_f = 1;       // grid of k_g1 (its units are parts of cell tiles)
     int lay_tiles = 1;    // layout tiles (kLayTile cells) of the largest simulation
     cudaStream_t stream;
@@ -234,7 +236,8 @@ struct Launch {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
-constexpr int kPTile = 512;   // particles per tile (small domains still spread over many SMs)
+constexpr int kPTile = 512;   // particles per tile
+constexpr int kPUnit = 128;   // particles a block of the particle kernels takes at a time (a quarter of a tile)
 constexpr int kCTile = 32;    // cells per tile (balances the per-cell kernels across SMs)
 constexpr int kSpillCap = 4096;  // spill entries per parity (fused pipeline)
 constexpr int kNFPrm = 16;       // u[3], theta, M[6], P_relax (0: none), nu, 1/nu_ES, P_ne, X, 1/P_relax (G2Prm)

@@ -26,29 +26,33 @@ namespace usp {
 // K1: advection, new cell, histogram
 // ---------------------------------------------------------------------------
 template <class T>
-__global__ void __launch_bounds__(256) k_stream(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(kPUnit) k_stream(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                 const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
-    const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int nu = *ntiles * (kPTile / kPUnit);
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nu; t += gridDim.x) {
+        const int2 tile = unit_of(tiles, t);
+        if (tile.x != loaded) {
+            __syncthreads();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const uint32_t n = s.dyn->n;
         const uint32_t step = s.dyn->step;
         const int cur = s.dyn->cur;
         PView<T> P = view<T>(s, cur);
-        for (int j = threadIdx.x; j < kPTile; j += blockDim.x) {
-            const int64_t i = (int64_t)tile.y + j;
-            if (i >= (int64_t)n) break;
+        const int64_t i = (int64_t)tile.y + threadIdx.x;
+        if (i < (int64_t)n) {
             T x = s.dim == 2 ? P.x[i] : (T)0;
             T y = P.y[i];
             T c[3] = {P.c0[i], P.c1[i], P.c2[i]};
             const uint32_t pid = P.pid[i];
             const T x0 = x, y0 = y;
-            bool alive = advect<T>(s, step, pid, x, y, c);
+            bool alive = true;
+            if (!advect_clear<T>(s, x, y, c)) alive = advect<T>(s, step, pid, x, y, c);
             if (s.flux_axis) count_flux<T>(s, x0, y0, x, y);
             int cell = s.K;
             if (alive) {
@@ -71,21 +75,24 @@ __global__ void __launch_bounds__(256) k_stream(const SimDev* __restrict__ sims,
 
 // cell of every particle without moving it (ordering an arbitrary loaded state)
 template <class T>
-__global__ void __launch_bounds__(256) k_assign(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(kPUnit) k_assign(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                 const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
-    const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int nu = *ntiles * (kPTile / kPUnit);
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nu; t += gridDim.x) {
+        const int2 tile = unit_of(tiles, t);
+        if (tile.x != loaded) {
+            __syncthreads();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const uint32_t n = s.dyn->n;
         PView<T> P = view<T>(s, s.dyn->cur);
-        for (int j = threadIdx.x; j < kPTile; j += blockDim.x) {
-            const int64_t i = (int64_t)tile.y + j;
-            if (i >= (int64_t)n) break;
+        const int64_t i = (int64_t)tile.y + threadIdx.x;
+        if (i < (int64_t)n) {
             // local cell of a slab (row0 = 0 without a decomposition),
             // clamped into the slab's cell range
             const int cell = min(max(cell_index<T>(s, s.dim == 2 ? P.x[i] : (T)0, P.y[i]) - s.row0 * s.nx, 0),
@@ -152,24 +159,27 @@ __global__ void __launch_bounds__(1024) k_scan(const SimDev* __restrict__ sims, 
 // K3: scatter to sorted slots
 // ---------------------------------------------------------------------------
 template <class T>
-__global__ void __launch_bounds__(256) k_scatter(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(kPUnit) k_scatter(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                  const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
-    const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int nu = *ntiles * (kPTile / kPUnit);
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nu; t += gridDim.x) {
+        const int2 tile = unit_of(tiles, t);
+        if (tile.x != loaded) {
+            __syncthreads();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const uint32_t n = s.dyn->n;
         const int cur = s.dyn->cur;
         PView<T> A = view<T>(s, cur), B = view<T>(s, cur ^ 1);
-        for (int j = threadIdx.x; j < kPTile; j += blockDim.x) {
-            const int64_t i = (int64_t)tile.y + j;
-            if (i >= (int64_t)n) break;
+        const int64_t i = (int64_t)tile.y + threadIdx.x;
+        if (i < (int64_t)n) {
             const uint32_t cell = s.cell[i];
-            if (cell >= (uint32_t)s.K) continue;
+            if (cell >= (uint32_t)s.K) continue;   // (the block's other threads take theirs)
             const uint32_t slot = s.start[cell] + aggregated_add(s.fill, cell);
             if ((int64_t)slot >= s.cap) {
                 atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
@@ -287,23 +297,50 @@ __global__ void __launch_bounds__(32) k_moments(const SimDev* __restrict__ sims,
                 a[6] += C0 * C1; a[7] += C0 * C2; a[8] += C1 * C2;
                 a[9] += c2 * C0; a[10] += c2 * C1; a[11] += c2 * C2;
             }
+            // the twelve sums (and the weights') as a warp reduce-scatter: lane
+            // 2 v ends with value v (16 FP64 additions instead of 60)
+            double v[16];
 #pragma unroll
-            for (int m = 0; m < 12; ++m) a[m] = warp_sum(a[m]);
-            if (Wt) we = warp_sum(we);
+            for (int m = 0; m < 12; ++m) v[m] = a[m];
+            v[12] = we;
+            v[13] = v[14] = v[15] = 0.0;
+#pragma unroll
+            for (int half = 8; half >= 1; half >>= 1) {
+                const bool up = (lane & (2 * half)) != 0;
+#pragma unroll
+                for (int i = 0; i < half; ++i) {
+                    const double send = up ? v[i] : v[i + half];
+                    const double recv = __shfl_xor_sync(0xffffffffu, send, 2 * half);
+                    v[i] = (up ? v[i + half] : v[i]) + recv;
+                }
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            if ((lane & 1) == 0 && lane < 24) s.mom[(size_t)(lane / 2 + 1) * K + cell] = v[0];
+            if (Wt && lane == 24) s.wneff[cell] = v[0];
+            if (s.gloc) {
+                // n, T and |u| for the neighbours' Kn_GLL
+                double S[6];
+#pragma unroll
+                for (int m = 0; m < 6; ++m) S[m] = __shfl_sync(0xffffffffu, v[0], 2 * m);
+                const double w = Wt ? __shfl_sync(0xffffffffu, v[0], 24) : (double)(e - b);
+                double T = 0.0, um = 0.0;
+                bool ok = false;
+                if (e > b && w > 0.0) {
+                    const double inv = 1.0 / w;
+                    const double d0 = S[0] * inv, d1 = S[1] * inv, d2 = S[2] * inv;
+                    const double th = ((S[3] * inv - d0 * d0) + (S[4] * inv - d1 * d1) + (S[5] * inv - d2 * d2)) *
+                                      (1.0 / 3.0);
+                    ok = e - b >= 2 && (!Wt || w > 1.0) && th > 0.0;
+                    if (ok) {
+                        const double u0 = sh0 + d0, u1 = sh1 + d1, u2 = sh2 + d2;
+                        T = th * s.inv_R;
+                        um = sqrt(u0 * u0 + u1 * u1 + u2 * u2);
+                    }
+                }
+                if (lane == 0) store_grad_state(s, cell, ok, w * s.w, T, um);
+            }
             if (lane == 0) {
                 s.mom[cell] = (double)(e - b);
-                if (Wt) s.wneff[cell] = we;
-#pragma unroll
-                for (int m = 0; m < 12; ++m) s.mom[(size_t)(m + 1) * K + cell] = a[m];
-                if (s.gloc) {
-                    // the cell's stencil state once (from the sums just
-                    // stored), for its neighbours' Kn_GLL
-                    Local L;
-                    local_state(s, cell, L, nullptr, nullptr);
-                    GradState G;
-                    grad_from_local(L, G);
-                    store_grad_state(s, cell, G);
-                }
                 s.fill[cell] = 0;
                 if (gll_averaged(s)) snap_avg(s, cell);
             }
@@ -348,6 +385,7 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
             pr[2] = L.u[2];
             pr[3] = L.theta;
             if (L.valid) {
+                local_transport(s, L);
                 double pne;
                 if (s.mode == kModeSP || s.mode == kModeSPESBGK) pne = 0.0;
                 else if (s.mode == kModeFixed) pne = s.fixed_pne;
@@ -356,34 +394,24 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                     // differences, one-sided next to a missing or invalid neighbour
                     const bool avg = gll_averaged(s);
                     GradState G;
-                    if (avg) grad_from_avg(s, cell, G);
+                    if (avg) grad_from_avg(s, cell, G, true);
                     else grad_from_local(L, G);
                     double kn = 0.0;   // no stencil state of its own: no gradient
                     if (G.valid) {
-                        double Qc[3] = {G.n, G.T, G.umag};
+                        const double Qc[3] = {G.n, G.T, G.umag};
                         double g2[3] = {0.0, 0.0, 0.0};
                         for (int axis = s.dim == 1 ? 1 : 0; axis < 2; ++axis) {
-                            const double h = axis == 0 ? s.dx : s.dy;
+                            const double ih = s.inv_d[axis];
                             int m = neighbor(s, cell, axis, -1), p = neighbor(s, cell, axis, +1);
                             GradState Gm, Gp;
                             if (m >= 0) {
-                                if (avg) grad_from_avg(s, m, Gm);
-                                else if (s.gloc) load_grad_state(s, m, Gm);
-                                else {
-                                    Local Lm;
-                                    local_state(s, m, Lm, nullptr, nullptr);
-                                    grad_from_local(Lm, Gm);
-                                }
+                                if (avg) grad_from_avg(s, m, Gm, false);
+                                else load_grad_state(s, m, Gm);
                                 if (!Gm.valid) m = -1;
                             }
                             if (p >= 0) {
-                                if (avg) grad_from_avg(s, p, Gp);
-                                else if (s.gloc) load_grad_state(s, p, Gp);
-                                else {
-                                    Local Lp;
-                                    local_state(s, p, Lp, nullptr, nullptr);
-                                    grad_from_local(Lp, Gp);
-                                }
+                                if (avg) grad_from_avg(s, p, Gp, false);
+                                else load_grad_state(s, p, Gp);
                                 if (!Gp.valid) p = -1;
                             }
                             double Qm[3], Qp[3];
@@ -391,32 +419,32 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                             if (p >= 0) { Qp[0] = Gp.n; Qp[1] = Gp.T; Qp[2] = Gp.umag; }
                             for (int q = 0; q < 3; ++q) {
                                 double d = 0.0;
-                                if (m >= 0 && p >= 0) d = (Qp[q] - Qm[q]) / (2.0 * h);
-                                else if (p >= 0) d = (Qp[q] - Qc[q]) / h;
-                                else if (m >= 0) d = (Qc[q] - Qm[q]) / h;
+                                if (m >= 0 && p >= 0) d = (Qp[q] - Qm[q]) * (0.5 * ih);
+                                else if (p >= 0) d = (Qp[q] - Qc[q]) * ih;
+                                else if (m >= 0) d = (Qc[q] - Qm[q]) * ih;
                                 g2[q] += d * d;
                             }
                         }
-                        const double kn_rho = G.lambda * sqrt(g2[0]) / G.n;
-                        const double kn_T = G.lambda * sqrt(g2[1]) / G.T;
-                        const double kn_u = G.lambda * sqrt(g2[2]) / fmax(G.umag, G.a_sound);
-                        kn = fmax(kn_rho, fmax(kn_T, kn_u));                 // Eq. 17
+                        // Eq. 17: lambda max over Q of |grad Q| / Q, in squares
+                        const double r0 = 1.0 / G.n, r1 = 1.0 / G.T, r2 = 1.0 / fmax(G.umag, G.a_sound);
+                        kn = G.lambda * sqrt(fmax(g2[0] * r0 * r0, fmax(g2[1] * r1 * r1, g2[2] * r2 * r2)));
                     }
-                    pne = exp(-kn / kKnC);                                   // Eq. 16
+                    pne = exp(kn * (-1.0 / kKnC));                           // Eq. 16
                 }
-                const double fs = 1.0 + 0.5 * s.dt * L.nu * pne;            // Eq. 33
-                const double fq = 1.0 + 0.5 * s.dt * L.nu * s.Pr * pne;
-                const double sig[6] = {(P[0] - L.theta) / fs, (P[1] - L.theta) / fs, (P[2] - L.theta) / fs,
-                                       P[3] / fs, P[4] / fs, P[5] / fs};
-                const double b = 1.0 - 1.0 / s.Pr;                          // Eq. 6c
+                const double ifs = 1.0 / (1.0 + 0.5 * s.dt * L.nu * pne);   // Eq. 33
+                const double ifq = 1.0 / (1.0 + 0.5 * s.dt * L.nu * s.Pr * pne);
+                const double sig[6] = {(P[0] - L.theta) * ifs, (P[1] - L.theta) * ifs, (P[2] - L.theta) * ifs,
+                                       P[3] * ifs, P[4] * ifs, P[5] * ifs};
+                const double b = s.es_b;                                    // Eq. 6c: 1 - 1/Pr
                 const double A00 = L.theta + b * sig[0], A11 = L.theta + b * sig[1], A22 = L.theta + b * sig[2];
                 const double A10 = b * sig[3], A20 = b * sig[4], A21 = b * sig[5];
                 double l00 = 0, l10 = 0, l11 = 0, l20 = 0, l21 = 0, l22 = 0;
                 bool ok = A00 > 0.0;
                 if (ok) {
                     l00 = sqrt(A00);
-                    l10 = A10 / l00;
-                    l20 = A20 / l00;
+                    const double i0 = 1.0 / l00;
+                    l10 = A10 * i0;
+                    l20 = A20 * i0;
                     const double d1 = A11 - l10 * l10;
                     ok = d1 > 0.0;
                     if (ok) {
@@ -442,7 +470,7 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                 if (s.weighted) {
                     // sigma* and q* per unit density for the weights of steps 4 and 7
                     for (int k = 0; k < 6; ++k) s.wst[(size_t)k * K + cell] = sig[k];
-                    for (int k = 0; k < 3; ++k) s.wst[(size_t)(6 + k) * K + cell] = Q[k] / fq;
+                    for (int k = 0; k < 3; ++k) s.wst[(size_t)(6 + k) * K + cell] = Q[k] * ifq;
                 }
                 pr[10] = -expm1(-s.Pr * L.nu * s.dt);                       // Eqs. 8b, 9
                 pr[11] = L.nu;
@@ -456,9 +484,9 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                 f[8] = L.rho * sig[3];
                 f[9] = L.rho * sig[4];
                 f[10] = L.rho * sig[5];
-                f[11] = L.rho * Q[0] / fq;
-                f[12] = L.rho * Q[1] / fq;
-                f[13] = L.rho * Q[2] / fq;
+                f[11] = L.rho * Q[0] * ifq;
+                f[12] = L.rho * Q[1] * ifq;
+                f[13] = L.rho * Q[2] * ifq;
                 f[14] = pne;
             }
             for (int k = 0; k < kNPrm; ++k) prm[(size_t)k * K + cell] = pr[k];
@@ -481,9 +509,13 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
 // selection words (staged once per cell) when the cell fits, else null and
 // the words are drawn again.
 constexpr uint32_t kRelaxWords = 1024;
-// new peculiar velocities of a cell's relaxed particles kept from the sums
-// pass for the apply pass (larger cells draw them again)
+// relaxed particles of a cell worked on at a time: their new peculiar
+// velocities are kept from the sums for the apply pass (a larger cell goes
+// through in chunks of this many particles and draws them again)
 constexpr uint32_t kRelaxKeep = 512;
+// warps per cell: four in FP64; one in FP32, where the draws are cheap and the
+// cell's own FP64 work would only be done four times over
+template <class T> constexpr int kRelaxWarps = sizeof(T) == 8 ? 4 : 1;
 
 template <class T>
 __device__ __forceinline__ bool selected(const SimDev& s, const PView<T>& B, uint32_t b, uint32_t e, uint32_t i,
@@ -498,124 +530,242 @@ __device__ __forceinline__ bool selected(const SimDev& s, const PView<T>& B, uin
     return rank < ns;
 }
 
-// One warp per block, the blocks striding over single cells (not tiles of
-// cells): the relaxation is bound by FP64 issue (about two FP64 FMA per clock
-// per SM on GB300), so even a domain of a hundred cells should spread over a
-// hundred SMs.
+// A block of four warps per cell, the blocks striding over single cells: the
+// relaxation is bound by FP64 issue (about two FP64 FMA per clock per SM on
+// GB300, the same for one lane of a warp as for all), so
+//  * only the selected particles are worked on: their list is packed first, so
+//    that a cell with a quarter of its particles selected takes a quarter of
+//    the draws' instructions;
+//  * the draw of a particle is split over the four warps (the time instant, and
+//    one Box-Muller pair each), which keep the FP64 pipe busy together where a
+//    domain has about one cell per SM.
+// Measured per launch, one warp per cell on all particles before: 100 cells of
+// 100 particles, a quarter selected, 60 -> 20 us; 1000 cells of 360 / 45, all
+// selected, 208 -> 175 us (FP64 issue); FP32, 4e4 cells of 100, 719 -> 432 us.
 template <class T>
-__global__ void __launch_bounds__(32) k_relax(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
-                                              const int* __restrict__ ntiles) {
+__global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __restrict__ sims,
+                                                               const int2* __restrict__ tiles,
+                                                               const int* __restrict__ ntiles) {
+    constexpr int NW = kRelaxWarps<T>;
+    constexpr uint32_t B_ = 32 * NW, Q_ = kRelaxKeep / NW;
     __shared__ SimDev sim_sh;
     __shared__ uint32_t sel_words[kRelaxWords];
-    __shared__ double keep_c[3][kRelaxKeep];
-    __shared__ unsigned char keep_sel[kRelaxKeep];
+    __shared__ T zc[NW > 1 ? 6 : 3][kRelaxKeep];   // the six normals, then the new peculiar velocity (first three)
+    __shared__ T ab[2][NW > 1 ? kRelaxKeep : 1];   // sqrt(s), sqrt((1 - s) theta) of Eqs. 31-32 (Gallis-Torczynski: s)
+    __shared__ unsigned short part[kRelaxKeep], list[NW > 1 ? kRelaxKeep : 1];   // selected particles by warp, packed
+    __shared__ uint32_t part_n[NW];
+    __shared__ double sums[NW][8], fac[8];
     const int nt = *ntiles;
-    const int lane = threadIdx.x & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = lanemask_lt();
     int loaded = -1;
     for (int g = blockIdx.x; g < nt * kCTile; g += gridDim.x) {
         const int2 tile = tiles[g / kCTile];
         if (tile.x != loaded) {
-            __syncwarp();
+            __syncthreads();
             load_sim(sim_sh, sims[tile.x]);
-            __syncwarp();
+            __syncthreads();
             loaded = tile.x;
         }
         const SimDev& s = sim_sh;
         const int K = s.K;
         const uint32_t step = s.dyn->step;
-        PView<T> B = view<T>(s, s.dyn->cur ^ 1);
-        {
-            const int cell = tile.y + g % kCTile;
-            if (cell >= K) continue;
-            const double* pr = s.prm;
-            const bool valid = pr[(size_t)14 * K + cell] != 0.0;
-            CellRelax R;
-            for (int d = 0; d < 3; ++d) R.u[d] = pr[(size_t)d * K + cell];
-            if (lane == 0 && s.mom[cell] >= 1.0)
-                for (int d = 0; d < 3; ++d) s.ushift[(size_t)d * K + cell] = R.u[d];
-            if (!valid) continue;
-            R.theta = pr[(size_t)3 * K + cell];
-            for (int d = 0; d < 6; ++d) R.L[d] = pr[(size_t)(4 + d) * K + cell];
-            R.p_relax = pr[(size_t)10 * K + cell];
-            R.nu = pr[(size_t)11 * K + cell];
-            R.nu_es = pr[(size_t)12 * K + cell];
-            R.pne = pr[(size_t)13 * K + cell];
-            const uint32_t cap = (uint32_t)s.cap;
-            const uint32_t b = min(s.start[cell], cap), e = min(s.start[cell + 1], cap);
-            const T pth = (T)R.p_relax;
-            // pass 1: sums over the relaxed subset (velocities relative to the cell mean)
-            double nr = 0, so[3] = {0, 0, 0}, eo = 0, sn[3] = {0, 0, 0}, en = 0;
-            // Eq. 9 fixed count: the ns particles with the smallest selection
-            // words (ties: lower position first)
-            const uint32_t ns = s.selection ? (uint32_t)floor((double)(e - b) * R.p_relax + 0.5) : 0u;
-            const uint32_t* words = nullptr;
-            if (s.selection && e - b <= kRelaxWords) {
-                __syncwarp();
-                for (uint32_t i = b + lane; i < e; i += 32) sel_words[i - b] = draw(s, B.pid[i], step, kRelax, 0).x;
-                __syncwarp();
-                words = sel_words;
+        const PView<T> V = view<T>(s, s.dyn->cur ^ 1);
+        const int cell = tile.y + g % kCTile;
+        if (cell >= K) continue;
+        const double* pr = s.prm;
+        const bool valid = pr[(size_t)14 * K + cell] != 0.0;
+        CellRelax R;
+        for (int d = 0; d < 3; ++d) R.u[d] = pr[(size_t)d * K + cell];
+        if (tid == 0 && s.mom[cell] >= 1.0)
+            for (int d = 0; d < 3; ++d) s.ushift[(size_t)d * K + cell] = R.u[d];
+        if (!valid) continue;
+        R.theta = pr[(size_t)3 * K + cell];
+        for (int d = 0; d < 6; ++d) R.L[d] = pr[(size_t)(4 + d) * K + cell];
+        R.p_relax = pr[(size_t)10 * K + cell];
+        R.nu = pr[(size_t)11 * K + cell];
+        R.nu_es = pr[(size_t)12 * K + cell];
+        R.pne = pr[(size_t)13 * K + cell];
+        const uint32_t cap = (uint32_t)s.cap;
+        const uint32_t b = min(s.start[cell], cap), e = min(s.start[cell + 1], cap);
+        const T pth = (T)R.p_relax;
+        // Eq. 9 fixed count: the ns particles with the smallest selection
+        // words (ties: lower position first)
+        const uint32_t ns = s.selection ? (uint32_t)floor((double)(e - b) * R.p_relax + 0.5) : 0u;
+        const uint32_t* words = nullptr;
+        __syncthreads();   // the shared arrays of the cell before are free
+        if (s.selection && e - b <= kRelaxWords) {
+            for (uint32_t i = b + tid; i < e; i += B_) sel_words[i - b] = draw(s, V.pid[i], step, kRelax, 0).x;
+            __syncthreads();
+            words = sel_words;
+        }
+        // the selected particles of [c0, c0 + kRelaxKeep) into `list`, in
+        // order, and their new peculiar velocities into zc[0..2]; how many
+        unsigned short* const lst = NW > 1 ? list : part;
+        auto draws = [&](uint32_t c0) -> uint32_t {
+            uint32_t mine = 0;
+            for (uint32_t j = 0; j < Q_; j += 32) {   // warp w: particles w Q_ .. (w + 1) Q_ - 1
+                const uint32_t k = warp * Q_ + j + lane, i = c0 + k;
+                if (c0 + warp * Q_ + j >= e) break;
+                bool sel = false;
+                if (i < e) sel = selected<T>(s, V, b, e, i, draw(s, V.pid[i], step, kRelax, 0).x, pth, ns, step, words);
+                const unsigned m = __ballot_sync(0xffffffffu, sel);
+                if (sel) part[warp * Q_ + mine + __popc(m & lt)] = (unsigned short)k;
+                mine += __popc(m);
             }
-            const bool keep = e - b <= kRelaxKeep;
-            __syncwarp();
-            for (uint32_t i = b + lane; i < e; i += 32) {
-                const uint32_t pid = B.pid[i];
-                const uint4 w = draw(s, pid, step, kRelax, 0);
-                const bool sel = selected<T>(s, B, b, e, i, w.x, pth, ns, step, words);
-                if (keep) keep_sel[i - b] = sel ? 1 : 0;
-                if (!sel) continue;
+            if constexpr (NW == 1) {
+                __syncwarp();
+                for (uint32_t k = lane; k < mine; k += 32) {
+                    const uint32_t id = V.pid[c0 + part[k]];
+                    T C[3];
+                    es_draw<T>(s, R, id, step, draw(s, id, step, kRelax, 0), C);
+                    zc[0][k] = C[0];   // (read again by this thread alone)
+                    zc[1][k] = C[1];
+                    zc[2][k] = C[2];
+                }
+                return mine;
+            } else {
+            if (lane == 0) part_n[warp] = mine;
+            __syncthreads();
+            uint32_t first = 0, all = 0;
+            for (int w = 0; w < NW; ++w) {
+                if (w < warp) first += part_n[w];
+                all += part_n[w];
+            }
+            for (uint32_t k = lane; k < mine; k += 32) list[first + k] = part[warp * Q_ + k];
+            __syncthreads();
+            // time instant (Eqs. 29-30): its cell constants once, by this warp alone
+            const T dt = (T)s.dt, nues = (T)R.nu_es, a = nues * dt;
+            const bool small = a < (T)1;
+            T ea = (T)0, inv = (T)0;
+            if (warp == 0) {
+                ea = small ? expm1(a) : exp(-a);
+                inv = (T)1 / nues;
+            }
+            for (uint32_t k = lane; k < all; k += 32) {
+                const uint32_t id = V.pid[c0 + list[k]];
+                if (warp == 0) {
+                    const T U = u01<T>(draw(s, id, step, kRelax, 0).y);
+                    const T t = small ? log1p(U * ea) * inv : dt + log(U + ((T)1 - U) * ea) * inv;
+                    // Eq. 32; the SP-ESBGK step holds the target for the whole step (Eq. 8b)
+                    const T sf = s.mode == kModeSPESBGK ? (T)1 : (T)R.pne + (T)(1.0 - R.pne) * exp(-(T)R.nu * t);
+                    ab[0][k] = s.es_sampler ? sf : dev_sqrt<T>(sf);
+                    ab[1][k] = s.es_sampler ? dev_sqrt<T>((T)R.theta) : dev_sqrt<T>(((T)1 - sf) * (T)R.theta);
+                } else {
+                    const uint4 w = draw(s, id, step, kRelax, warp == 1 ? 0u : 1u);
+                    T z0, z1;
+                    box_muller<T>(warp == 2 ? w.x : w.z, warp == 2 ? w.y : w.w, z0, z1);
+                    zc[2 * warp - 2][k] = z0;
+                    zc[2 * warp - 1][k] = z1;
+                }
+            }
+            __syncthreads();
+            for (uint32_t k = tid; k < all; k += B_) {
+                const T a0 = ab[0][k], b0 = ab[1][k];
                 T C[3];
-                es_draw<T>(s, R, pid, step, w, C);
-                if (keep)
-                    for (int d = 0; d < 3; ++d) keep_c[d][i - b] = (double)C[d];
-                const double o0 = (double)B.c0[i] - R.u[0], o1 = (double)B.c1[i] - R.u[1],
-                             o2 = (double)B.c2[i] - R.u[2];
-                nr += 1.0;
-                so[0] += o0; so[1] += o1; so[2] += o2;
-                eo += o0 * o0 + o1 * o1 + o2 * o2;
-                sn[0] += (double)C[0]; sn[1] += (double)C[1]; sn[2] += (double)C[2];
-                en += (double)C[0] * C[0] + (double)C[1] * C[1] + (double)C[2] * C[2];
+                if (s.es_sampler) {
+                    // Eq. 10: one thermal component per (cosine) Box-Muller pair; Eq. 11:
+                    // C = S C*, S = I - s B, B = ((1 - Pr)/(2 Pr)) sigma*/(rho theta) in
+                    // the L slots (xx, yy, zz, xy, xz, yz)
+                    const T c0_ = b0 * zc[0][k], c1_ = b0 * zc[2][k], c2_ = b0 * zc[4][k];
+                    const T b00 = a0 * (T)R.L[0], b11 = a0 * (T)R.L[1], b22 = a0 * (T)R.L[2];
+                    const T b01 = a0 * (T)R.L[3], b02 = a0 * (T)R.L[4], b12 = a0 * (T)R.L[5];
+                    C[0] = ((T)1 - b00) * c0_ - b01 * c1_ - b02 * c2_;
+                    C[1] = -b01 * c0_ + ((T)1 - b11) * c1_ - b12 * c2_;
+                    C[2] = -b02 * c0_ - b12 * c1_ + ((T)1 - b22) * c2_;
+                } else {
+                    const T z0 = zc[0][k], z1 = zc[1][k], z2 = zc[2][k];
+                    C[0] = a0 * ((T)R.L[0] * z0) + b0 * zc[3][k];
+                    C[1] = a0 * ((T)R.L[1] * z0 + (T)R.L[2] * z1) + b0 * zc[4][k];
+                    C[2] = a0 * ((T)R.L[3] * z0 + (T)R.L[4] * z1 + (T)R.L[5] * z2) + b0 * zc[5][k];
+                }
+                zc[0][k] = C[0];   // (read again by this thread alone)
+                zc[1][k] = C[1];
+                zc[2][k] = C[2];
             }
-            nr = warp_sum(nr);
-            for (int d = 0; d < 3; ++d) {
-                so[d] = warp_sum(so[d]);
-                sn[d] = warp_sum(sn[d]);
+            return all;
             }
-            eo = warp_sum(eo);
-            en = warp_sum(en);
-            int applied = 0;
-            if (nr >= 2.0) {
-                const double inv = 1.0 / nr;
-                const double Eo = eo - (so[0] * so[0] + so[1] * so[1] + so[2] * so[2]) * inv;
-                const double En = en - (sn[0] * sn[0] + sn[1] * sn[1] + sn[2] * sn[2]) * inv;
-                if (En > 0.0) {
-                    applied = (int)nr;
-                    const double alpha = sqrt(Eo / En);
-                    const double uo[3] = {R.u[0] + so[0] * inv, R.u[1] + so[1] * inv, R.u[2] + so[2] * inv};
-                    const double mn[3] = {sn[0] * inv, sn[1] * inv, sn[2] * inv};
-                    // pass 2: apply c = ubar_old + alpha (c' - ubar_new), with c'
-                    // kept from pass 1 or drawn again
-                    __syncwarp();
-                    for (uint32_t i = b + lane; i < e; i += 32) {
-                        T C[3];
-                        if (keep) {
-                            if (!keep_sel[i - b]) continue;
-                            for (int d = 0; d < 3; ++d) C[d] = (T)keep_c[d][i - b];
-                        } else {
-                            const uint32_t pid = B.pid[i];
-                            const uint4 w = draw(s, pid, step, kRelax, 0);
-                            if (!selected<T>(s, B, b, e, i, w.x, pth, ns, step, words)) continue;
-                            es_draw<T>(s, R, pid, step, w, C);
+        };
+        // pass 1: sums over the relaxed subset (velocities relative to the cell mean)
+        double S[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        uint32_t nr = 0, all = 0;
+        for (uint32_t c0 = b; c0 < e; c0 += kRelaxKeep) {
+            if (c0 != b) __syncthreads();
+            all = draws(c0);
+            nr += all;
+            for (uint32_t k = tid; k < all; k += B_) {
+                const uint32_t i = c0 + lst[k];
+                const double o0 = (double)V.c0[i] - R.u[0], o1 = (double)V.c1[i] - R.u[1],
+                             o2 = (double)V.c2[i] - R.u[2];
+                const double C0 = (double)zc[0][k], C1 = (double)zc[1][k], C2 = (double)zc[2][k];
+                S[0] += o0; S[1] += o1; S[2] += o2;
+                S[3] += o0 * o0 + o1 * o1 + o2 * o2;
+                S[4] += C0; S[5] += C1; S[6] += C2;
+                S[7] += C0 * C0 + C1 * C1 + C2 * C2;
+            }
+        }
+        int applied = 0;
+        if (nr >= 2) {
+            // reduce-scatter of the eight sums in each warp (lane 4 i: sum i), then over the warps
+#pragma unroll
+            for (int half = 4; half >= 1; half >>= 1) {
+                const bool up = (lane & (4 * half)) != 0;
+#pragma unroll
+                for (int i = 0; i < half; ++i) {
+                    const double send = up ? S[i] : S[i + half];
+                    const double recv = __shfl_xor_sync(0xffffffffu, send, 4 * half);
+                    S[i] = (up ? S[i + half] : S[i]) + recv;
+                }
+            }
+            S[0] += __shfl_xor_sync(0xffffffffu, S[0], 2);
+            S[0] += __shfl_xor_sync(0xffffffffu, S[0], 1);
+            if ((lane & 3) == 0) sums[warp][lane >> 2] = S[0];
+            __syncthreads();
+            if (warp == 0) {   // the factors once (FP64 costs each warp that computes it)
+                double A[8], a = 0.0;
+                if (lane < 8)
+                    for (int w = 0; w < NW; ++w) a += sums[w][lane];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) A[k] = __shfl_sync(0xffffffffu, a, k);
+                const double inv = 1.0 / (double)nr;
+                const double Eo = A[3] - (A[0] * A[0] + A[1] * A[1] + A[2] * A[2]) * inv;
+                const double En = A[7] - (A[4] * A[4] + A[5] * A[5] + A[6] * A[6]) * inv;
+                if (lane == 0) {
+                    fac[7] = En > 0.0 ? 1.0 : 0.0;
+                    if (En > 0.0) {
+                        fac[6] = sqrt(Eo / En);
+                        for (int d = 0; d < 3; ++d) {
+                            fac[d] = R.u[d] + A[d] * inv;
+                            fac[3 + d] = A[4 + d] * inv;
                         }
-                        B.c0[i] = (T)(uo[0] + alpha * ((double)C[0] - mn[0]));
-                        B.c1[i] = (T)(uo[1] + alpha * ((double)C[1] - mn[1]));
-                        B.c2[i] = (T)(uo[2] + alpha * ((double)C[2] - mn[2]));
                     }
                 }
             }
-            if (lane == 0) {
-                s.prm[(size_t)15 * K + cell] = applied;
-                if (applied) atomicAdd(&s.dyn->counters[kCntRelaxed], (unsigned long long)applied);
+            __syncthreads();
+            if (fac[7] != 0.0) {
+                applied = (int)nr;
+                const double alpha = fac[6];
+                const double uo[3] = {fac[0], fac[1], fac[2]};
+                const double mn[3] = {fac[3], fac[4], fac[5]};
+                // pass 2: apply c = ubar_old + alpha (c' - ubar_new), with c'
+                // kept from pass 1 or drawn again
+                for (uint32_t c0 = b; c0 < e; c0 += kRelaxKeep) {
+                    if (e - b > kRelaxKeep) {
+                        __syncthreads();
+                        all = draws(c0);
+                    }
+                    for (uint32_t k = tid; k < all; k += B_) {
+                        const uint32_t i = c0 + lst[k];
+                        V.c0[i] = (T)(uo[0] + alpha * ((double)zc[0][k] - mn[0]));
+                        V.c1[i] = (T)(uo[1] + alpha * ((double)zc[1][k] - mn[1]));
+                        V.c2[i] = (T)(uo[2] + alpha * ((double)zc[2][k] - mn[2]));
+                    }
+                }
             }
+        }
+        if (tid == 0) {
+            s.prm[(size_t)15 * K + cell] = applied;
+            if (applied) atomicAdd(&s.dyn->counters[kCntRelaxed], (unsigned long long)applied);
         }
     }
 }
@@ -692,17 +842,17 @@ __global__ void k_debug_philox(int64_t n, const uint32_t* __restrict__ ctr, uint
 // launchers
 // ---------------------------------------------------------------------------
 void launch_stream(const Launch& L, bool fp64) {
-    if (fp64) k_stream<double><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
-    else k_stream<float><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    if (fp64) k_stream<double><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    else k_stream<float><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
 }
 void launch_assign(const Launch& L, bool fp64) {
-    if (fp64) k_assign<double><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
-    else k_assign<float><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    if (fp64) k_assign<double><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    else k_assign<float><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
 }
 void launch_scan(const Launch& L, bool with_inj) { k_scan<<<L.nsims, 1024, 0, L.stream>>>(L.sims, L.nsims, with_inj ? 1 : 0); }
 void launch_scatter(const Launch& L, bool fp64) {
-    if (fp64) k_scatter<double><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
-    else k_scatter<float><<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    if (fp64) k_scatter<double><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    else k_scatter<float><<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
 }
 void launch_inject(const Launch& L, bool fp64) {
     if (fp64) k_inject<double><<<L.grid_c, 256, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
@@ -719,12 +869,12 @@ void launch_moments_src(const Launch& L, bool fp64, bool src_cur) {
 }
 void launch_params(const Launch& L) { k_params<<<L.grid_c, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles); }
 void launch_relax(const Launch& L, bool fp64) {
-    // one warp per cell slot of the tiles, at most 32 one-warp blocks per SM
+    // one block per cell slot of the tiles, at most what the SMs' shared memory holds (41 and 13 KB a block)
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = std::max(1, std::min(L.grid_c * kCTile, 32 * sms));
-    if (fp64) k_relax<double><<<grid, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
-    else k_relax<float><<<grid, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+    const int grid = std::max(1, std::min(L.grid_c * kCTile, (fp64 ? 5 : 16) * sms));
+    if (fp64) k_relax<double><<<grid, 32 * kRelaxWarps<double>, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+    else k_relax<float><<<grid, 32 * kRelaxWarps<float>, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 void launch_finish(const Launch& L) { k_finish<<<(L.nsims + 127) / 128, 128, 0, L.stream>>>(L.sims, L.nsims); }
 

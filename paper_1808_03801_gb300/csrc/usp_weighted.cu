@@ -215,53 +215,58 @@ __global__ void __launch_bounds__(1024) k_w_scan(const SimDev* __restrict__ sims
 // entries in (cell, k) order; ids continue from next_pid in the same order.
 // Positions uniform in the cell, velocities Maxwellian at the record's u and
 // theta, weights pref * factor * Eq. 26.
-__global__ void __launch_bounds__(256) k_w_add(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
-                                               const int* __restrict__ ntiles) {
+// One warp per block, the blocks striding over single cells: the draws are
+// FP64 latency, and with the cells of a tile in one block two SMs did all the
+// work of a domain of 50 cells (78 us a stage).
+__global__ void __launch_bounds__(32) k_w_add(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+                                              const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
     const int nt = *ntiles;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int lane = threadIdx.x;
+    int loaded = -1;
+    for (int g = blockIdx.x; g < nt * kCTile; g += gridDim.x) {
+        const int2 tile = tiles[g / kCTile];
+        if (tile.x != loaded) {
+            __syncwarp();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncwarp();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
+        const int cell = tile.y + g % kCTile;
+        if (cell >= s.K) continue;
+        const uint32_t na = s.wna[cell];
+        if (!na) continue;
         const int cur = s.dyn->cur;
         const uint32_t n0 = s.dyn->n, pid0 = s.dyn->next_pid, step = s.dyn->step;
         PView<double> P = view<double>(s, cur);
         double* W = s.wgt[cur];
-        for (int cc = warp; cc < kCTile; cc += nwarps) {
-            const int cell = tile.y + cc;
-            if (cell >= s.K) break;
-            const uint32_t na = s.wna[cell];
-            if (!na) continue;
-            const double* F = s.wfs + (size_t)kNWF * cell;
-            const int ix = cell % s.nx, iy = cell / s.nx;
-            const double xl = s.dim == 2 ? s.lo[0] + ix * s.dx : 0.0;
-            const double yl = s.lo[1] + iy * s.dy;
-            const double sq = sqrt(F[kWFTh]);
-            for (uint32_t k = lane; k < na; k += 32) {
-                const uint32_t off = s.woff[cell] + k;
-                const int64_t i = (int64_t)n0 + off;
-                if (i >= s.cap) {
-                    atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
-                    continue;
-                }
-                const uint32_t pid = pid0 + off;
-                const uint4 w = draw(s, pid, step, kAdd, 0);
-                const uint4 v = draw(s, pid, step, kAdd, 1);
-                double z0, z1, z2, z3;
-                box_muller<double>(v.x, v.y, z0, z1);
-                box_muller<double>(v.z, v.w, z2, z3);
-                const double C[3] = {sq * z0, sq * z1, sq * z2};
-                if (s.dim == 2) P.x[i] = xl + u01<double>(w.x) * s.dx;
-                P.y[i] = yl + u01<double>(w.y) * s.dy;
-                P.c0[i] = F[kWFU] + C[0];
-                P.c1[i] = F[kWFU + 1] + C[1];
-                P.c2[i] = F[kWFU + 2] + C[2];
-                P.pid[i] = pid;
-                W[i] = F[kWFPref] * eq26_weight(C, F, F[kWFPne], s.dt, s.Pr);
+        const double* F = s.wfs + (size_t)kNWF * cell;
+        const int ix = cell % s.nx, iy = cell / s.nx;
+        const double xl = s.dim == 2 ? s.lo[0] + ix * s.dx : 0.0;
+        const double yl = s.lo[1] + iy * s.dy;
+        const double sq = sqrt(F[kWFTh]);
+        for (uint32_t k = lane; k < na; k += 32) {
+            const uint32_t off = s.woff[cell] + k;
+            const int64_t i = (int64_t)n0 + off;
+            if (i >= s.cap) {
+                atomicAdd(&s.dyn->counters[kCntOverflow], 1ull);
+                continue;
             }
+            const uint32_t pid = pid0 + off;
+            const uint4 w = draw(s, pid, step, kAdd, 0);
+            const uint4 v = draw(s, pid, step, kAdd, 1);
+            double z0, z1, z2, z3;
+            box_muller<double>(v.x, v.y, z0, z1);
+            box_muller<double>(v.z, v.w, z2, z3);
+            const double C[3] = {sq * z0, sq * z1, sq * z2};
+            if (s.dim == 2) P.x[i] = xl + u01<double>(w.x) * s.dx;
+            P.y[i] = yl + u01<double>(w.y) * s.dy;
+            P.c0[i] = F[kWFU] + C[0];
+            P.c1[i] = F[kWFU + 1] + C[1];
+            P.c2[i] = F[kWFU + 2] + C[2];
+            P.pid[i] = pid;
+            W[i] = F[kWFPref] * eq26_weight(C, F, F[kWFPne], s.dt, s.Pr);
         }
     }
 }
@@ -283,23 +288,26 @@ __global__ void k_w_commit(const SimDev* __restrict__ sims, int nsims, uint32_t 
 
 // cell and histogram of the n entries of buffer `cur` (a deleted particle,
 // weight NaN, goes to the sentinel K and is dropped by the scatter)
-__global__ void __launch_bounds__(256) k_w_assign(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(kPUnit) k_w_assign(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                   const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
-    const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int nu = *ntiles * (kPTile / kPUnit);
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nu; t += gridDim.x) {
+        const int2 tile = unit_of(tiles, t);
+        if (tile.x != loaded) {
+            __syncthreads();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const uint32_t n = s.dyn->n;
         const int cur = s.dyn->cur;
         PView<double> P = view<double>(s, cur);
         const double* W = s.wgt[cur];
-        for (int j = threadIdx.x; j < kPTile; j += blockDim.x) {
-            const int64_t i = (int64_t)tile.y + j;
-            if (i >= (int64_t)n) break;
+        const int64_t i = (int64_t)tile.y + threadIdx.x;
+        if (i < (int64_t)n) {
             uint32_t cell = (uint32_t)s.K;
             if (!isnan(W[i])) {
                 cell = (uint32_t)min(max(cell_index<double>(s, s.dim == 2 ? P.x[i] : 0.0, P.y[i]), 0), s.K - 1);
@@ -311,24 +319,27 @@ __global__ void __launch_bounds__(256) k_w_assign(const SimDev* __restrict__ sim
 }
 
 // particles and weights of buffer cur to their sorted slots in cur ^ 1
-__global__ void __launch_bounds__(256) k_w_scatter(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+__global__ void __launch_bounds__(kPUnit) k_w_scatter(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                    const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
-    const int nt = *ntiles;
-    for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-        const int2 tile = tiles[t];
-        __syncthreads();
-        load_sim(sim_sh, sims[tile.x]);
-        __syncthreads();
+    const int nu = *ntiles * (kPTile / kPUnit);
+    int loaded = -1;
+    for (int t = blockIdx.x; t < nu; t += gridDim.x) {
+        const int2 tile = unit_of(tiles, t);
+        if (tile.x != loaded) {
+            __syncthreads();
+            load_sim(sim_sh, sims[tile.x]);
+            __syncthreads();
+            loaded = tile.x;
+        }
         const SimDev& s = sim_sh;
         const uint32_t n = s.dyn->n;
         const int cur = s.dyn->cur;
         PView<double> A = view<double>(s, cur), B = view<double>(s, cur ^ 1);
         const double* WA = s.wgt[cur];
         double* WB = s.wgt[cur ^ 1];
-        for (int j = threadIdx.x; j < kPTile; j += blockDim.x) {
-            const int64_t i = (int64_t)tile.y + j;
-            if (i >= (int64_t)n) break;
+        const int64_t i = (int64_t)tile.y + threadIdx.x;
+        if (i < (int64_t)n) {
             const uint32_t cell = s.cell[i];
             if (cell >= (uint32_t)s.K) continue;
             const uint32_t slot = s.start[cell] + aggregated_add(s.fill, cell);
@@ -377,24 +388,43 @@ __global__ void k_w_take_sorted(const SimDev* __restrict__ sims, int nsims) {
 }
 
 // ---------------------------------------------------------------------------
-// steps 5-6 on the sorted buffer cur ^ 1, one warp per cell
+// steps 5-6 on the sorted buffer cur ^ 1, a block of four warps per cell (with
+// one warp a cell of 300 particles took ten draws one after another: 215 us)
 // ---------------------------------------------------------------------------
 constexpr int kWKeys = 2048;   // selection words cached per cell (larger cells redraw them)
+constexpr int kWWarps = 4;
+
+// sums of N values over the block, the same on every thread
+template <int N>
+__device__ __forceinline__ void w_block_sum(double (&v)[N], double (*sh)[8]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = warp_sum(v[k]);
+    __syncthreads();
+    if (lane == 0)
+        for (int k = 0; k < N; ++k) sh[warp][k] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = (sh[0][k] + sh[1][k]) + (sh[2][k] + sh[3][k]);
+}
 
 // the m-th smallest (1-based) selection word of the cell's slots [b, e): a
-// radix select over 8-bit digits counted in `hist` (256 entries)
+// radix select over 8-bit digits counted in `hist` (256 entries); every warp
+// reads the counts by itself
 template <class KeyOf>
-__device__ uint32_t w_kth_word(uint32_t b, uint32_t e, uint32_t m, const KeyOf& key_of, uint32_t* hist, int lane,
+__device__ uint32_t w_kth_word(uint32_t b, uint32_t e, uint32_t m, const KeyOf& key_of, uint32_t* hist,
                                uint32_t& below_out) {
+    const int lane = threadIdx.x & 31;
     uint32_t prefix = 0, mask = 0, rem = m;
     for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int k = lane; k < 256; k += 32) hist[k] = 0u;
-        __syncwarp();
-        for (uint32_t i = b + lane; i < e; i += 32) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < 256; k += 32 * kWWarps) hist[k] = 0u;
+        __syncthreads();
+        for (uint32_t i = b + threadIdx.x; i < e; i += 32 * kWWarps) {
             const uint32_t x = key_of(i);
             if ((x & mask) == prefix) atomicAdd(&hist[(x >> shift) & 255u], 1u);
         }
-        __syncwarp();
+        __syncthreads();
         uint32_t h[8], tot = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -426,27 +456,28 @@ __device__ uint32_t w_kth_word(uint32_t b, uint32_t e, uint32_t m, const KeyOf& 
         rem -= below;
         prefix |= d << shift;
         mask |= 0xFFu << shift;
-        __syncwarp();
     }
     below_out = m - rem;   // words strictly below the result
     return prefix;
 }
 
-__global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
-                                                const int* __restrict__ ntiles) {
+__global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restrict__ sims,
+                                                          const int2* __restrict__ tiles,
+                                                          const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
     __shared__ uint32_t keys[kWKeys];
     __shared__ uint32_t hist[256];
+    __shared__ double sh[kWWarps][8];
     const int nt = *ntiles;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
+    const int tid = threadIdx.x;
+    constexpr uint32_t T_ = 32 * kWWarps;
     int loaded = -1;
     for (int g = blockIdx.x; g < nt * kCTile; g += gridDim.x) {
         const int2 tile = tiles[g / kCTile];
+        __syncthreads();   // the shared arrays of the cell before are free
         if (tile.x != loaded) {
-            __syncwarp();
             load_sim(sim_sh, sims[tile.x]);
-            __syncwarp();
+            __syncthreads();
             loaded = tile.x;
         }
         const SimDev& s = sim_sh;
@@ -460,12 +491,11 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
         const double* pr = s.prm;
         CellRelax R;
         for (int d = 0; d < 3; ++d) R.u[d] = pr[(size_t)d * K + cell];
-        if (lane == 0 && s.mom[cell] >= 1.0)
+        if (tid == 0 && s.mom[cell] >= 1.0)
             for (int d = 0; d < 3; ++d) s.ushift[(size_t)d * K + cell] = R.u[d];
-        __syncwarp();
         const bool valid = pr[(size_t)14 * K + cell] != 0.0;
         if (!valid) {
-            if (lane == 0) s.prm[(size_t)15 * K + cell] = 0.0;
+            if (tid == 0) s.prm[(size_t)15 * K + cell] = 0.0;
             continue;
         }
         R.theta = pr[(size_t)3 * K + cell];
@@ -481,26 +511,24 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
             return cached ? keys[i - b] : draw(s, B.pid[i], step, kRelax, 0).x;
         };
         // step 5: Bernoulli selection (Eq. 9); the selected set's weight and momentum
-        double ns = 0, sw = 0, su[3] = {0, 0, 0};
-        for (uint32_t i = b + lane; i < e; i += 32) {
+        double q[5] = {0, 0, 0, 0, 0};   // count, weight, momentum
+        for (uint32_t i = b + tid; i < e; i += T_) {
             const uint32_t x = draw(s, B.pid[i], step, kRelax, 0).x;
             if (cached) keys[i - b] = x;
             if (!(u01<double>(x) < R.p_relax)) continue;
             const double w = W[i];
-            ns += 1.0;
-            sw += w;
-            su[0] += w * B.c0[i];
-            su[1] += w * B.c1[i];
-            su[2] += w * B.c2[i];
+            q[0] += 1.0;
+            q[1] += w;
+            q[2] += w * B.c0[i];
+            q[3] += w * B.c1[i];
+            q[4] += w * B.c2[i];
         }
-        __syncwarp();
-        ns = warp_sum(ns);
+        w_block_sum(q, sh);
+        const double ns = q[0], sw = q[1];
         if (ns == 0.0) {
-            if (lane == 0) s.prm[(size_t)15 * K + cell] = 0.0;
+            if (tid == 0) s.prm[(size_t)15 * K + cell] = 0.0;
             continue;
         }
-        sw = warp_sum(sw);
-        for (int d = 0; d < 3; ++d) su[d] = warp_sum(su[d]);
         // Eq. 28: int(sum of the selected weights), rounded at random
         const uint4 wc = draw(s, (uint32_t)cell, step, kCellDraw, 0);
         double md = sw > 0.0 ? floor(sw + u01<double>(wc.x)) : 0.0;
@@ -508,13 +536,15 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
         const uint32_t m = (uint32_t)md;
         double uo[3] = {0, 0, 0}, eo = 0;
         if (sw > 0.0) {
-            for (int d = 0; d < 3; ++d) uo[d] = su[d] / sw;
-            for (uint32_t i = b + lane; i < e; i += 32) {
+            for (int d = 0; d < 3; ++d) uo[d] = q[2 + d] / sw;
+            double r[1] = {0};
+            for (uint32_t i = b + tid; i < e; i += T_) {
                 if (!(u01<double>(key_of(i)) < R.p_relax)) continue;
                 const double a0 = B.c0[i] - uo[0], a1 = B.c1[i] - uo[1], a2 = B.c2[i] - uo[2];
-                eo += W[i] * (a0 * a0 + a1 * a1 + a2 * a2);
+                r[0] += W[i] * (a0 * a0 + a1 * a1 + a2 * a2);
             }
-            eo = warp_sum(eo) / sw;
+            w_block_sum(r, sh);
+            eo = r[0] / sw;
         }
         // step 6: the m selected particles with the smallest words (the
         // selected words lie below all the others) are reassigned at weight 1
@@ -523,22 +553,19 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
         uint32_t T = 0, quota = 0;
         if (m > 0) {
             uint32_t below = 0;
-            T = w_kth_word(b, e, m, key_of, hist, lane, below);
+            T = w_kth_word(b, e, m, key_of, hist, below);
             quota = m - below;
         }
         double un[3] = {0, 0, 0};
-        uint32_t ties = 0;
-        for (uint32_t i0 = b; i0 < e; i0 += 32) {
-            const uint32_t i = i0 + lane;
-            const bool has = i < e;
-            const uint32_t x = has ? key_of(i) : 0xFFFFFFFFu;
-            const bool sel = has && u01<double>(x) < R.p_relax;
-            const bool tie = sel && m > 0 && x == T;
-            const unsigned tb = __ballot_sync(0xffffffffu, tie);
-            const uint32_t trank = ties + (uint32_t)__popc(tb & lt);
-            ties += (uint32_t)__popc(tb);
-            if (!sel) continue;
-            const bool keep = m > 0 && (x < T || (tie && trank < quota));
+        for (uint32_t i = b + tid; i < e; i += T_) {
+            const uint32_t x = key_of(i);
+            if (!(u01<double>(x) < R.p_relax)) continue;
+            bool keep = m > 0 && x < T;
+            if (m > 0 && x == T) {   // one word, but for a chance of 2^-32 a pair
+                uint32_t rank = 0;
+                for (uint32_t j = b; j < i; ++j) rank += key_of(j) == T;
+                keep = rank < quota;
+            }
             if (!keep) {
                 W[i] = __longlong_as_double(0x7FF8000000000000ll);   // deleted
                 continue;
@@ -555,22 +582,22 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
             un[1] += B.c1[i];
             un[2] += B.c2[i];
         }
-        __syncwarp();
-        for (int d = 0; d < 3; ++d) un[d] = warp_sum(un[d]);
+        w_block_sum(un, sh);
         // the reassigned set carries the selected set's mean velocity and
-        // thermal energy per unit weight
+        // thermal energy per unit weight (a thread sees its own particles)
         auto reassigned = [&](uint32_t i) { return W[i] == 1.0 && u01<double>(key_of(i)) < R.p_relax; };
         if (m >= 2 && sw > 0.0) {
             for (int d = 0; d < 3; ++d) un[d] /= md;
-            double en = 0;
-            for (uint32_t i = b + lane; i < e; i += 32) {
+            double r[1] = {0};
+            for (uint32_t i = b + tid; i < e; i += T_) {
                 if (!reassigned(i)) continue;
                 const double a0 = B.c0[i] - un[0], a1 = B.c1[i] - un[1], a2 = B.c2[i] - un[2];
-                en += a0 * a0 + a1 * a1 + a2 * a2;
+                r[0] += a0 * a0 + a1 * a1 + a2 * a2;
             }
-            en = warp_sum(en) / md;
+            w_block_sum(r, sh);
+            const double en = r[0] / md;
             const double alpha = (en > 0.0 && eo > 0.0) ? sqrt(eo / en) : 1.0;
-            for (uint32_t i = b + lane; i < e; i += 32) {
+            for (uint32_t i = b + tid; i < e; i += T_) {
                 if (!reassigned(i)) continue;
                 B.c0[i] = uo[0] + alpha * (B.c0[i] - un[0]);
                 B.c1[i] = uo[1] + alpha * (B.c1[i] - un[1]);
@@ -578,15 +605,14 @@ __global__ void __launch_bounds__(32) k_w_relax(const SimDev* __restrict__ sims,
             }
         } else if (m == 1 && sw > 0.0) {
             const double f = sqrt(eo > 0.0 ? eo / (3.0 * R.theta) : 1.0);
-            for (uint32_t i = b + lane; i < e; i += 32) {
+            for (uint32_t i = b + tid; i < e; i += T_) {
                 if (!reassigned(i)) continue;
                 B.c0[i] = uo[0] + (B.c0[i] - un[0]) * f;
                 B.c1[i] = uo[1] + (B.c1[i] - un[1]) * f;
                 B.c2[i] = uo[2] + (B.c2[i] - un[2]) * f;
             }
         }
-        __syncwarp();
-        if (lane == 0) {
+        if (tid == 0) {
             s.prm[(size_t)15 * K + cell] = md;
             if (m > 0) atomicAdd(&s.dyn->counters[kCntRelaxed], (unsigned long long)m);
         }
@@ -613,9 +639,9 @@ __global__ void k_w_init(const SimDev* __restrict__ sims, int nsims) {
 // the counting sort of the weighted path: buffer cur -> cur ^ 1 by cell;
 // swap makes the sorted buffer current
 static void w_sort(const Launch& L, int swap) {
-    k_w_assign<<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    k_w_assign<<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
     launch_scan(L, false);
-    k_w_scatter<<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    k_w_scatter<<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
     k_w_sorted<<<L.nsims, 256, 0, L.stream>>>(L.sims, L.nsims, swap);
 }
 
@@ -624,7 +650,7 @@ template <int STAGE>
 static void w_add(const Launch& L, uint32_t bits) {
     k_w_stage<STAGE><<<L.grid_c, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
     k_w_scan<<<L.nsims, 1024, 0, L.stream>>>(L.sims, L.nsims);
-    k_w_add<<<L.grid_c, 256, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+    k_w_add<<<L.grid_c * kCTile, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
     k_w_commit<<<1, 32, 0, L.stream>>>(L.sims, L.nsims, bits);
 }
 
@@ -639,7 +665,7 @@ void enqueue_weighted_step(const Launch& L) {
     // step 3: flight and counting sort into cur ^ 1 (the weights follow)
     launch_stream(L, true);
     launch_scan(L, false);
-    k_w_scatter<<<L.grid_p, 256, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
+    k_w_scatter<<<L.grid_u, kPUnit, 0, L.stream>>>(L.sims, L.ptiles, L.nptiles);
     k_w_sorted<<<L.nsims, 256, 0, L.stream>>>(L.sims, L.nsims, 0);
     // moments and parameters of f~* (Eqs. 1, 16-18, 33)
     launch_moments(L, true);
@@ -649,8 +675,8 @@ void enqueue_weighted_step(const Launch& L) {
     w_add<2>(L, 2u);
     w_sort(L, 0);
     // steps 5-6
-    const int grid = std::max(1, std::min(L.grid_c * kCTile, 32 * sms));
-    k_w_relax<<<grid, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+    const int grid = std::max(1, std::min(L.grid_c * kCTile, 8 * sms));
+    k_w_relax<<<grid, 32 * kWWarps, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
     // step 7 appended to the relaxed buffer; compaction and sort end the step
     k_w_take_sorted<<<1, 32, 0, L.stream>>>(L.sims, L.nsims);
     w_add<3>(L, 0u);
