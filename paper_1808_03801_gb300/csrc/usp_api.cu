@@ -272,9 +272,11 @@ static int choose_R(int64_t cells, int ppc_ref, int dim) {
     return cells <= 2 * (int64_t)sms && ppc_ref > 128 ? 12 : 8;
 }
 
-// a load goes back to the default variant
+// a load goes back to the default variant (graphs captured with another go)
 static void set_default_R(usp_handle* h) {
-    h->fused_R = choose_R(h->host.K, h->ppc_ref, h->host.dim);
+    const int R = choose_R(h->host.K, h->ppc_ref, h->host.dim);
+    if (R != h->fused_R) destroy_graphs(h->graphs);
+    h->fused_R = R;
     h->tuned = false;
 }
 
@@ -605,10 +607,11 @@ static int alloc_particles(usp_handle* h, int64_t n) {
     }
     cap = (cap + 3) & ~(int64_t)3;   // whole 16-byte groups of FP32 slots (bulk copies of the fused pipeline)
     if (cap > (int64_t)0x7FFFFFFFll) return fail(h, USP_ERR_CAPACITY, "particle capacity exceeds 2^31 - 1");
-    destroy_graphs(h->graphs);
     // storage of a similar size is kept (a re-load of the same problem
-    // allocates nothing); the tile tables depend only on the capacity
+    // allocates nothing); the tile tables and the captured graphs depend only
+    // on the capacity
     if (!h->part_allocs.empty() && cap <= s.cap && 2 * cap > s.cap) return USP_OK;
+    destroy_graphs(h->graphs);
     free_particles(h);
     const size_t es = h->precision == USP_FP64 ? 8 : 4;
     auto grab = [&](size_t bytes) -> void* {
