@@ -491,16 +491,37 @@ __device__ __forceinline__ T sample_time(T U, T nu_es, T dt) {
     return dt + log(U + ((T)1 - U) * exp(-a)) / nu_es;
 }
 
+// the same in FP64, with its exponential and reciprocal once per cell
+struct TimeLaw64 {
+    double ea = 0.0, inv = 0.0, dt = 0.0;
+    bool small = false;
+    __device__ __forceinline__ void set(double nu_es, double dt_) {
+        dt = dt_;
+        const double a = nu_es * dt;
+        small = a < 1.0;
+        ea = small ? expm1(a) : exp(-a);
+        inv = 1.0 / nu_es;
+    }
+    __device__ __forceinline__ double instant(double U) const {
+        return small ? log1p64(U * ea) * inv : dt + log64(U + (1.0 - U) * ea) * inv;
+    }
+};
+
+// u01<double>(x) < p, in integers: the word has to lie below this (x + 1/2 <
+// 2^32 p; exact, since 2^32 p - 1/2 is a double where it is positive)
+__device__ __forceinline__ uint64_t word_limit(double p) {
+    return p > 0.0 ? (uint64_t)ceil(fmin(p, 1.0) * 4294967296.0 - 0.5) : 0u;
+}
+
 struct CellRelax {
     double u[3], theta, L[6], p_relax, nu, nu_es, pne;
 };
 
-// new peculiar velocity of a relaxed particle: ES Gaussian with covariance
+// new peculiar velocity of a particle relaxed at the instant t: ES Gaussian with covariance
 // theta I + s (1 - 1/Pr) sigma*/rho = s L L^T + (1 - s) theta I, s from Eq. 32
 template <class T>
 __device__ __forceinline__ void es_draw(const SimDev& s, const CellRelax& R, uint32_t pid, uint32_t step,
-                                        const uint4& w, T* C) {
-    const T t = sample_time<T>(u01<T>(w.y), (T)R.nu_es, (T)s.dt);
+                                        const uint4& w, T t, T* C) {
     // Eq. 32; the SP-ESBGK step holds the target for the whole step (Eq. 8b)
     const T sf = s.mode == kModeSPESBGK ? (T)1 : (T)R.pne + (T)(1.0 - R.pne) * exp(-(T)R.nu * t);
     const uint4 v = draw(s, pid, step, kRelax, 1);

@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "usp_math64.cuh"
+
 namespace usp {
 
 constexpr int kMaxSeg = 4;
@@ -182,11 +184,7 @@ template <> __device__ __forceinline__ float u01<float>(uint32_t x) {
 // Box-Muller pair from two words.
 template <class T> __device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, T& z0, T& z1);
 template <> __device__ __forceinline__ void box_muller<double>(uint32_t a, uint32_t b, double& z0, double& z1) {
-    double r = sqrt(-2.0 * log(u01<double>(a)));
-    double sn, cs;
-    sincospi(2.0 * u01<double>(b), &sn, &cs);
-    z0 = r * cs;
-    z1 = r * sn;
+    normal_pair64(a, b, z0, z1);
 }
 template <> __device__ __forceinline__ void box_muller<float>(uint32_t a, uint32_t b, float& z0, float& z1) {
     // -2 ln u = -2 ln2 * log2(u); the angle is shifted by pi, which flips the
@@ -199,10 +197,10 @@ template <> __device__ __forceinline__ void box_muller<float>(uint32_t a, uint32
 }
 
 template <class T> __device__ __forceinline__ T dev_sqrt(T x);
-template <> __device__ __forceinline__ double dev_sqrt<double>(double x) { return sqrt(x); }
+template <> __device__ __forceinline__ double dev_sqrt<double>(double x) { return sqrt64(x); }
 template <> __device__ __forceinline__ float dev_sqrt<float>(float x) { return sqrtf(x); }
 template <class T> __device__ __forceinline__ T dev_log(T x);
-template <> __device__ __forceinline__ double dev_log<double>(double x) { return log(x); }
+template <> __device__ __forceinline__ double dev_log<double>(double x) { return log64(x); }
 template <> __device__ __forceinline__ float dev_log<float>(float x) { return 0.6931471805599453f * __log2f(x); }
 template <class T> __device__ __forceinline__ T dev_floor(T x);
 template <> __device__ __forceinline__ double dev_floor<double>(double x) { return floor(x); }

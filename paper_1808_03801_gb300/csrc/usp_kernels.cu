@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
 // K7: relaxation of each cell with conservation of momentum and energy
 // ---------------------------------------------------------------------------
 // is the particle at slot i of the cell [b, e) relaxed?  Bernoulli: its
-// selection word against the probability; fixed count (Eq. 9): its rank
+// selection word against the probability (in FP64 as its limit in integers); fixed count (Eq. 9): its rank
 // among the cell's selection words below ns.  `words` holds the cell's
 // selection words (staged once per cell) when the cell fits, else null and
 // the words are drawn again.
@@ -519,8 +519,8 @@ template <class T> constexpr int kRelaxWarps = sizeof(T) == 8 ? 4 : 1;
 
 template <class T>
 __device__ __forceinline__ bool selected(const SimDev& s, const PView<T>& B, uint32_t b, uint32_t e, uint32_t i,
-                                         uint32_t wx, T pth, uint32_t ns, uint32_t step, const uint32_t* words) {
-    if (!s.selection) return u01<T>(wx) < pth;
+                                         uint32_t wx, T pth, uint64_t limit, uint32_t ns, uint32_t step, const uint32_t* words) {
+    if (!s.selection) return sizeof(T) == 8 ? wx < limit : u01<T>(wx) < pth;
     if (ns == 0) return false;
     uint32_t rank = 0;
     for (uint32_t j = b; j < e && rank < ns; ++j) {
@@ -539,9 +539,13 @@ __device__ __forceinline__ bool selected(const SimDev& s, const PView<T>& B, uin
 //  * the draw of a particle is split over the four warps (the time instant, and
 //    one Box-Muller pair each), which keep the FP64 pipe busy together where a
 //    domain has about one cell per SM.
+//  * the draws' functions are those of usp_math64.cuh, and the selection
+//    compares integers.
 // Measured per launch, one warp per cell on all particles before: 100 cells of
 // 100 particles, a quarter selected, 60 -> 20 us; 1000 cells of 360 / 45, all
-// selected, 208 -> 175 us (FP64 issue); FP32, 4e4 cells of 100, 719 -> 432 us.
+// selected, 208 -> 175 us, with these functions 130 us (FP64 issue: about 230
+// instructions a particle, 74 us at two lanes a clock); FP32, 4e4 cells of
+// 100, 719 -> 432 us.
 template <class T>
 __global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __restrict__ sims,
                                                                const int2* __restrict__ tiles,
@@ -589,6 +593,7 @@ __global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __r
         const uint32_t cap = (uint32_t)s.cap;
         const uint32_t b = min(s.start[cell], cap), e = min(s.start[cell + 1], cap);
         const T pth = (T)R.p_relax;
+        const uint64_t limit = sizeof(T) == 8 ? word_limit(R.p_relax) : 0u;
         // Eq. 9 fixed count: the ns particles with the smallest selection
         // words (ties: lower position first)
         const uint32_t ns = s.selection ? (uint32_t)floor((double)(e - b) * R.p_relax + 0.5) : 0u;
@@ -608,7 +613,7 @@ __global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __r
                 const uint32_t k = warp * Q_ + j + lane, i = c0 + k;
                 if (c0 + warp * Q_ + j >= e) break;
                 bool sel = false;
-                if (i < e) sel = selected<T>(s, V, b, e, i, draw(s, V.pid[i], step, kRelax, 0).x, pth, ns, step, words);
+                if (i < e) sel = selected<T>(s, V, b, e, i, draw(s, V.pid[i], step, kRelax, 0).x, pth, limit, ns, step, words);
                 const unsigned m = __ballot_sync(0xffffffffu, sel);
                 if (sel) part[warp * Q_ + mine + __popc(m & lt)] = (unsigned short)k;
                 mine += __popc(m);
@@ -618,7 +623,8 @@ __global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __r
                 for (uint32_t k = lane; k < mine; k += 32) {
                     const uint32_t id = V.pid[c0 + part[k]];
                     T C[3];
-                    es_draw<T>(s, R, id, step, draw(s, id, step, kRelax, 0), C);
+                    const uint4 w = draw(s, id, step, kRelax, 0);
+                    es_draw<T>(s, R, id, step, w, sample_time<T>(u01<T>(w.y), (T)R.nu_es, (T)s.dt), C);
                     zc[0][k] = C[0];   // (read again by this thread alone)
                     zc[1][k] = C[1];
                     zc[2][k] = C[2];
@@ -634,19 +640,13 @@ __global__ void __launch_bounds__(32 * kRelaxWarps<T>) k_relax(const SimDev* __r
             }
             for (uint32_t k = lane; k < mine; k += 32) list[first + k] = part[warp * Q_ + k];
             __syncthreads();
-            // time instant (Eqs. 29-30): its cell constants once, by this warp alone
-            const T dt = (T)s.dt, nues = (T)R.nu_es, a = nues * dt;
-            const bool small = a < (T)1;
-            T ea = (T)0, inv = (T)0;
-            if (warp == 0) {
-                ea = small ? expm1(a) : exp(-a);
-                inv = (T)1 / nues;
-            }
+            TimeLaw64 law;   // time instant (Eqs. 29-30): of this warp alone
+            if (warp == 0) law.set(R.nu_es, s.dt);
             for (uint32_t k = lane; k < all; k += 32) {
                 const uint32_t id = V.pid[c0 + list[k]];
                 if (warp == 0) {
                     const T U = u01<T>(draw(s, id, step, kRelax, 0).y);
-                    const T t = small ? log1p(U * ea) * inv : dt + log(U + ((T)1 - U) * ea) * inv;
+                    const T t = law.instant(U);
                     // Eq. 32; the SP-ESBGK step holds the target for the whole step (Eq. 8b)
                     const T sf = s.mode == kModeSPESBGK ? (T)1 : (T)R.pne + (T)(1.0 - R.pne) * exp(-(T)R.nu * t);
                     ab[0][k] = s.es_sampler ? sf : dev_sqrt<T>(sf);

@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
         const uint32_t cap = (uint32_t)s.cap;
         const uint32_t b = min(s.start[cell], cap), e = min(s.start[cell + 1], cap);
         const bool cached = e - b <= (uint32_t)kWKeys;
+        const uint64_t limit = word_limit(R.p_relax);
         auto key_of = [&](uint32_t i) -> uint32_t {
             return cached ? keys[i - b] : draw(s, B.pid[i], step, kRelax, 0).x;
         };
@@ -515,7 +516,7 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
         for (uint32_t i = b + tid; i < e; i += T_) {
             const uint32_t x = draw(s, B.pid[i], step, kRelax, 0).x;
             if (cached) keys[i - b] = x;
-            if (!(u01<double>(x) < R.p_relax)) continue;
+            if (!(x < limit)) continue;
             const double w = W[i];
             q[0] += 1.0;
             q[1] += w;
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
             for (int d = 0; d < 3; ++d) uo[d] = q[2 + d] / sw;
             double r[1] = {0};
             for (uint32_t i = b + tid; i < e; i += T_) {
-                if (!(u01<double>(key_of(i)) < R.p_relax)) continue;
+                if (!(key_of(i) < limit)) continue;
                 const double a0 = B.c0[i] - uo[0], a1 = B.c1[i] - uo[1], a2 = B.c2[i] - uo[2];
                 r[0] += W[i] * (a0 * a0 + a1 * a1 + a2 * a2);
             }
@@ -556,10 +557,12 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
             T = w_kth_word(b, e, m, key_of, hist, below);
             quota = m - below;
         }
+        TimeLaw64 law;
+        law.set(R.nu_es, s.dt);
         double un[3] = {0, 0, 0};
         for (uint32_t i = b + tid; i < e; i += T_) {
             const uint32_t x = key_of(i);
-            if (!(u01<double>(x) < R.p_relax)) continue;
+            if (!(x < limit)) continue;
             bool keep = m > 0 && x < T;
             if (m > 0 && x == T) {   // one word, but for a chance of 2^-32 a pair
                 uint32_t rank = 0;
@@ -573,7 +576,7 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
             const uint32_t pid = B.pid[i];
             const uint4 w = draw(s, pid, step, kRelax, 0);
             double C[3];
-            es_draw<double>(s, R, pid, step, w, C);
+            es_draw<double>(s, R, pid, step, w, law.instant(u01<double>(w.y)), C);
             B.c0[i] = R.u[0] + C[0];
             B.c1[i] = R.u[1] + C[1];
             B.c2[i] = R.u[2] + C[2];
@@ -585,7 +588,7 @@ __global__ void __launch_bounds__(32 * kWWarps) k_w_relax(const SimDev* __restri
         w_block_sum(un, sh);
         // the reassigned set carries the selected set's mean velocity and
         // thermal energy per unit weight (a thread sees its own particles)
-        auto reassigned = [&](uint32_t i) { return W[i] == 1.0 && u01<double>(key_of(i)) < R.p_relax; };
+        auto reassigned = [&](uint32_t i) { return W[i] == 1.0 && key_of(i) < limit; };
         if (m >= 2 && sw > 0.0) {
             for (int d = 0; d < 3; ++d) un[d] /= md;
             double r[1] = {0};
