@@ -566,7 +566,7 @@ def run_gpu(args):
             "frac": achieved / hbm, "traffic": traffic, "peak_source": f"{src} hbm_gbs (copy, burst)",
             "stage_ms": {names[k]: 1e3 * v for k, v in st.items()},
             "step_frac": alg / (el / args.steps) / 1e9 / hbm}
-    launches = U.launches_per_step(pipeline, reservoir=False) * args.steps
+    launches = U.launches_per_step(pipeline, reservoir=False, cells=1000) * args.steps
 
     result = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": world, "steps": args.steps,
               "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",

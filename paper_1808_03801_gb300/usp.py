@@ -142,9 +142,10 @@ def lib(build_if_missing: bool = True):
 _STAGES = {
     "plain": [(0, "k_stream"), (2, "k_scan+k_scatter"), (3, "k_moments"), (4, "k_params"), (5, "k_relax"),
               (6, "k_finish")],
-    "fused": [(10, "k_g2"), (12, "k_g1"), (13, "k_params_f"), (14, "k_lay_sum+scan+put+k_step_end")],
+    "fused": [(10, "k_g2"), (12, "k_g1"), (13, "k_params_f"), (14, "layout+k_step_end")],
 }
 _LAUNCHES = {"plain": 7, "fused": 7}
+_LAYOUT_ONE_KERNEL = 8192   # cells per simulation up to which one kernel lays out the buckets (else three)
 
 
 def fused_available() -> bool:
@@ -156,8 +157,10 @@ def stage_list(pipeline: str):
     return list(_STAGES[pipeline])
 
 
-def launches_per_step(pipeline: str, reservoir: bool = False) -> int:
-    return _LAUNCHES[pipeline] + (1 if reservoir else 0)
+def launches_per_step(pipeline: str, reservoir: bool = False, cells: int | None = None) -> int:
+    """Kernels of one step; `cells`: of the largest simulation (None: a domain above the one-kernel layout)."""
+    one = pipeline == "fused" and cells is not None and cells <= _LAYOUT_ONE_KERNEL
+    return _LAUNCHES[pipeline] + (1 if reservoir else 0) - (2 if one else 0)
 
 
 def exported_symbols():
