@@ -1796,9 +1796,17 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// k_params_f: per-cell parameters; FP64 for the stress tensor, Eq. 33 and the
-// Cholesky factor, FP32 for viscosity, mean free path, Kn_GLL and P_ne
+// k_params_f: per-cell parameters in FP32; the number density and the Eq. 34
+// averages in FP64
 // ---------------------------------------------------------------------------
+// A warp per tile of 32 cells, which takes as long as one cell's chain of
+// loads and arithmetic (10 us): all tiles in one wave where they fit.  16 blocks
+// of one warp per SM are what 128 registers a thread allow (18 and 24 with fewer
+// registers: small domains 1 us slower).  Against 8 per SM: 4e4 cells 19.5 ->
+// 14.2 us, 8e4 28.5 -> 26 us, 64 x 1000 cells 20.4 -> 17.7 us; a second warp for
+// the fields and averages gave no more.
+constexpr int kParamsBlocks = 16;
+
 struct LocalF {
     int valid, N;
     float n, T, umag;
@@ -1877,8 +1885,9 @@ __device__ __forceinline__ bool nb_state(const SimDev* __restrict__ sims, const 
     return L.valid != 0;
 }
 
-__global__ void __launch_bounds__(128) k_params_f(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
-                                                  const int* __restrict__ ntiles) {
+__global__ void __launch_bounds__(32, kParamsBlocks) k_params_f(const SimDev* __restrict__ sims,
+                                                                const int2* __restrict__ tiles,
+                                                                const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
     const int nt = *ntiles;
     for (int t = blockIdx.x; t < nt; t += gridDim.x) {
@@ -2620,7 +2629,16 @@ void launch_fused_moments(const Launch& L, int R) {
     k_g1<<<L.grid_f, 32 * kG1Warps, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 
-void launch_fused_params(const Launch& L) { k_params_f<<<L.grid_c, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles); }
+void launch_fused_params(const Launch& L) {
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0, n = 152;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms = n;
+    }
+    const int grid = std::max(1, std::min((L.cells - 1) / kCTile + 1, kParamsBlocks * sms));
+    k_params_f<<<grid, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
+}
 
 // the bucket layout of the next step's destination buffer (reads only the
 // arrivals of this step, so it may run beside k_g1 and k_params_f)
