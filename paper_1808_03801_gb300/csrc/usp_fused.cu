@@ -875,11 +875,11 @@ __device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, in
 // per SM with 128 registers and no spills measured best (12 and 14 warps with
 // more staging, 18 and 20 with less and some spills: 3-50 % slower), and so did
 // bulk copies (per-lane 16-byte copies took three times as long to issue).
-// What bounds it: the warps' dependent instructions (352 per 32 particles in
-// 1-D, 49 % issue) and, for dense cells, the copy that cannot start before the
+// What bounds it: the warps' dependent instructions (370 per 32 particles in
+// 1-D, 48 % issue) and, for dense cells, the copy that cannot start before the
 // cell ahead is written.  Against the form before it (a producer warp feeding
-// seven consumer warps): 64 shock tubes 301 -> 250 us, cavity 200 x 200 168 ->
-// 117 us, slit 522 -> 366 us per launch.
+// seven consumer warps): 64 shock tubes 301 -> 255 us, cavity 200 x 200 168 ->
+// 119 us, slit 522 -> 388 us per launch.
 // Cells above the staging area, and cells with spill-list entries, take the
 // general form of the same code: loaded by the lanes, in chunks, the draws of
 // all but one chunk made twice.
