@@ -334,8 +334,12 @@ struct Local {
 // local state of one cell from its shifted sums (means, Eq. 1; Eqs. 35-36)
 __device__ __forceinline__ void local_state(const SimDev& s, int cell, Local& L, double* P6, double* Q3) {
     const int K = s.K;
-    const double* M = s.mom;
-    const int N = (int)M[cell];
+    double M[13], us[3];   // every load first: one round of latency
+#pragma unroll
+    for (int k = 0; k < 13; ++k) M[k] = s.mom[(size_t)k * K + cell];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) us[d] = s.ushift[(size_t)d * K + cell];
+    const int N = (int)M[0];
     // with weighted particles the sums are W-weighted and N_eff = sum W
     // stands for N in the means and the density
     const double we = s.weighted ? s.wneff[cell] : (double)N;
@@ -346,12 +350,12 @@ __device__ __forceinline__ void local_state(const SimDev& s, int cell, Local& L,
     L.theta = 0.0;
     if (N < 1 || !(we > 0.0)) return;
     const double inv = 1.0 / we;
-    const double d0 = M[K + cell] * inv, d1 = M[2 * K + cell] * inv, d2 = M[3 * K + cell] * inv;
-    L.u[0] = s.ushift[cell] + d0;
-    L.u[1] = s.ushift[K + cell] + d1;
-    L.u[2] = s.ushift[2 * K + cell] + d2;
-    const double m00 = M[4 * K + cell] * inv, m11 = M[5 * K + cell] * inv, m22 = M[6 * K + cell] * inv;
-    const double m01 = M[7 * K + cell] * inv, m02 = M[8 * K + cell] * inv, m12 = M[9 * K + cell] * inv;
+    const double d0 = M[1] * inv, d1 = M[2] * inv, d2 = M[3] * inv;
+    L.u[0] = us[0] + d0;
+    L.u[1] = us[1] + d1;
+    L.u[2] = us[2] + d2;
+    const double m00 = M[4] * inv, m11 = M[5] * inv, m22 = M[6] * inv;
+    const double m01 = M[7] * inv, m02 = M[8] * inv, m12 = M[9] * inv;
     double P[6] = {m00 - d0 * d0, m11 - d1 * d1, m22 - d2 * d2, m01 - d0 * d1, m02 - d0 * d2, m12 - d1 * d2};
     L.theta = (P[0] + P[1] + P[2]) * (1.0 / 3.0);
     if (P6)
@@ -359,7 +363,7 @@ __device__ __forceinline__ void local_state(const SimDev& s, int cell, Local& L,
     if (Q3) {
         // central third moment from shifted raw moments: with d the mean of the
         // shifted velocities, E[|C|^2 C_i] = T3_i - d_i tr M2 - 2 (M2 d)_i + 2 d_i |d|^2
-        const double t0 = M[10 * K + cell] * inv, t1 = M[11 * K + cell] * inv, t2 = M[12 * K + cell] * inv;
+        const double t0 = M[10] * inv, t1 = M[11] * inv, t2 = M[12] * inv;
         const double tr = m00 + m11 + m22, dd = d0 * d0 + d1 * d1 + d2 * d2;
         const double md0 = m00 * d0 + m01 * d1 + m02 * d2;
         const double md1 = m01 * d0 + m11 * d1 + m12 * d2;

@@ -350,9 +350,14 @@ __global__ void __launch_bounds__(32) k_moments(const SimDev* __restrict__ sims,
 
 // ---------------------------------------------------------------------------
 // K6: per-cell USP parameters, fields and the Eq. 34 average
+//
+// A lane per cell, a warp per block: as long as one cell's chain of FP64
+// instructions, about 20 us, on domains of a few thousand cells (100 cells: 30 us
+// with plain divisions and the stencil's states formed again, 22 with loads
+// where they were needed, 20 with all of them first; 4e4 cells 67 -> 56).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
-                                                const int* __restrict__ ntiles) {
+__global__ void __launch_bounds__(32) k_params(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
+                                               const int* __restrict__ ntiles) {
     __shared__ SimDev sim_sh;
     const int nt = *ntiles;
     for (int t = blockIdx.x; t < nt; t += gridDim.x) {
@@ -365,6 +370,30 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
         for (int cc = threadIdx.x; cc < kCTile; cc += blockDim.x) {
             const int cell = tile.y + cc;
             if (cell >= K) break;
+            // every load of the cell first, as one round of latency (stores
+            // to the fields would hold the averages' loads back one by one):
+            // the running averages, the neighbours' stencil states, the sums
+            const bool first = s.dyn->nsamples == 0;
+            double av[kNFields];
+#pragma unroll
+            for (int k = 0; k < kNFields; ++k) av[k] = first ? 0.0 : s.avg[(size_t)k * K + cell];
+            const bool avg = gll_averaged(s);
+            GradState Nb[2][2];   // by axis and side
+            bool has[2][2] = {{false, false}, {false, false}};
+            if (s.mode == kModeUSP) {
+#pragma unroll
+                for (int axis = 0; axis < 2; ++axis) {
+                    if (axis == 0 && s.dim == 1) continue;
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) {
+                        const int c = neighbor(s, cell, axis, side ? +1 : -1);
+                        if (c < 0) continue;
+                        if (avg) grad_from_avg(s, c, Nb[axis][side], false);
+                        else load_grad_state(s, c, Nb[axis][side]);
+                        has[axis][side] = Nb[axis][side].valid != 0;
+                    }
+                }
+            }
             Local L;
             double P[6], Q[3];
             local_state(s, cell, L, P, Q);
@@ -392,7 +421,6 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                 else {
                     // gradient-length local Knudsen number (Eqs. 17-18): central
                     // differences, one-sided next to a missing or invalid neighbour
-                    const bool avg = gll_averaged(s);
                     GradState G;
                     if (avg) grad_from_avg(s, cell, G, true);
                     else grad_from_local(L, G);
@@ -400,20 +428,12 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                     if (G.valid) {
                         const double Qc[3] = {G.n, G.T, G.umag};
                         double g2[3] = {0.0, 0.0, 0.0};
-                        for (int axis = s.dim == 1 ? 1 : 0; axis < 2; ++axis) {
+#pragma unroll
+                        for (int axis = 0; axis < 2; ++axis) {
+                            if (axis == 0 && s.dim == 1) continue;
                             const double ih = s.inv_d[axis];
-                            int m = neighbor(s, cell, axis, -1), p = neighbor(s, cell, axis, +1);
-                            GradState Gm, Gp;
-                            if (m >= 0) {
-                                if (avg) grad_from_avg(s, m, Gm, false);
-                                else load_grad_state(s, m, Gm);
-                                if (!Gm.valid) m = -1;
-                            }
-                            if (p >= 0) {
-                                if (avg) grad_from_avg(s, p, Gp, false);
-                                else load_grad_state(s, p, Gp);
-                                if (!Gp.valid) p = -1;
-                            }
+                            const GradState &Gm = Nb[axis][0], &Gp = Nb[axis][1];
+                            const int m = has[axis][0] ? 1 : -1, p = has[axis][1] ? 1 : -1;
                             double Qm[3], Qp[3];
                             if (m >= 0) { Qm[0] = Gm.n; Qm[1] = Gm.T; Qm[2] = Gm.umag; }
                             if (p >= 0) { Qp[0] = Gp.n; Qp[1] = Gp.T; Qp[2] = Gp.umag; }
@@ -490,11 +510,10 @@ __global__ void __launch_bounds__(128) k_params(const SimDev* __restrict__ sims,
                 f[14] = pne;
             }
             for (int k = 0; k < kNPrm; ++k) prm[(size_t)k * K + cell] = pr[k];
-            const bool first = s.dyn->nsamples == 0;
+#pragma unroll
             for (int k = 0; k < kNFields; ++k) {
                 s.inst[(size_t)k * K + cell] = f[k];
-                double* a = &s.avg[(size_t)k * K + cell];
-                *a = first ? f[k] : s.avg_keep * *a + f[k] * s.avg_new;   // Eq. 34
+                s.avg[(size_t)k * K + cell] = first ? f[k] : s.avg_keep * av[k] + f[k] * s.avg_new;   // Eq. 34
             }
         }
     }

@@ -59,16 +59,23 @@ __device__ __forceinline__ double pne_of(const SimDev& s, int cell) {
 __device__ __forceinline__ double nu_of_state(const SimDev& s, double neff, double theta) {
     const double n = neff * s.w, T = theta / s.R;
     const double rho = n * s.mass, p = rho * theta;
-    const double mu = s.mu_ref * pow(T / s.T_ref, s.omega);
+    const double r = T / s.T_ref;
+    const double mu = s.mu_ref * (s.omega == 0.5 ? sqrt(r) : pow(r, s.omega));
     return p / mu;
 }
 
 // Eq. 34 average of a weight-field record, started at zero stress and heat
-// flux and at the first u, theta, nu
-__device__ __forceinline__ void average_record(const SimDev& s, double* a, const double* f, bool first) {
+// flux and at the first u, theta, nu; the record becomes the average.  (All
+// loads before the first store, which would hold them back one by one.)
+__device__ __forceinline__ void average_record(const SimDev& s, double* a, double* f, bool first) {
+    double o[kWFPref];
+#pragma unroll
+    for (int k = 0; k < kWFPref; ++k) o[k] = a[k];
+#pragma unroll
     for (int k = 0; k < kWFPref; ++k) {
-        if (first) a[k] = (k >= kWFSig && k < kWFNu) ? 0.0 : f[k];
-        else a[k] = s.avg_keep * a[k] + s.avg_new * f[k];
+        if (first) f[k] = (k >= kWFSig && k < kWFNu) ? 0.0 : f[k];
+        else f[k] = s.avg_keep * o[k] + s.avg_new * f[k];
+        a[k] = f[k];
     }
 }
 
@@ -115,7 +122,6 @@ __global__ void __launch_bounds__(128) k_w_stage(const SimDev* __restrict__ sims
                 if (s.weight_average) {
                     double* a = s.wan + (size_t)kNWF * cell;
                     average_record(s, a, rec, !(s.dyn->w_started & 1u));
-                    for (int k = 0; k < kWFPref; ++k) rec[k] = a[k];
                 }
                 pne = pne_of(s, cell);
                 live = pne != 0.0 && neff > 1.0;
@@ -131,7 +137,6 @@ __global__ void __launch_bounds__(128) k_w_stage(const SimDev* __restrict__ sims
                 if (s.weight_average) {
                     double* a = s.was + (size_t)kNWF * cell;
                     average_record(s, a, rec, !(s.dyn->w_started & 2u));
-                    for (int k = 0; k < kWFPref; ++k) rec[k] = a[k];
                 }
                 pne = pne_of(s, cell);
                 live = valid && pne != 0.0;
