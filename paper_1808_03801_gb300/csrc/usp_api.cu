@@ -1351,6 +1351,8 @@ static uint64_t batch_key(const usp_batch* b) {
         if (s.flux_axis) k |= 8u;
         if (s.selection || s.es_sampler) k |= 16u;
         if (s.has_reservoir) k |= 32u;
+        if (h->precision == USP_FP64) k |= 64u;             // an emptied batch may take another
+        if (h->pipeline == USP_PIPE_FUSED) k |= 128u;       // precision or pipeline
         per_sm = std::max(per_sm, h->grid_per_sm);
     }
     return k | (uint64_t)batch_R(b) << 8 | (uint64_t)per_sm << 16 | (uint64_t)b->members.size() << 32;
