@@ -1405,6 +1405,7 @@ __device__ __noinline__ G2Acc g2w_cell_general(Sh& sh, G2Sim S, G2Job J, int lan
     G2Acc acc = {0u, 0u};
     uint32_t nsp = 0;
     if (J.arrived > J.nb) nsp = collect_spill(sh.sim, S.p, J.cell, sh.spl, kG2wSpill, lane);
+    if (J.nb + nsp == 0) return acc;   // no bucket, and the spill list was full when its particles arrived
     g2w_cell_impl<DIM, MODE, true>(sh, S, J, 0u, nsp, lane, acc);
     return acc;
 }
