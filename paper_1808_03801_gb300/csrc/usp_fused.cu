@@ -2159,7 +2159,7 @@ __device__ __forceinline__ uint32_t bucket_size(const SimDev& s, const uint32_t*
     uint32_t m = 0;
     for (int dy = -1; dy <= 1; ++dy) {
         const int jy = iy + dy;
-        if (jy < 0 || jy >= s.ny) continue;
+        if (jy < 0 || jy >= s.rows) continue;   // (the counts of a slab are those of its own rows)
         for (int dx = (s.dim == 2 ? -1 : 0); dx <= (s.dim == 2 ? 1 : 0); ++dx) {
             const int jx = ix + dx;
             if (jx < 0 || jx >= s.nx) continue;

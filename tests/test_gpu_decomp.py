@@ -116,3 +116,41 @@ def test_slab_errors(env):
     bad["grid"] = dict(bad["grid"], ny=202)          # not a multiple of 4
     with pytest.raises(U.UspError):
         U.Simulation(bad)
+
+
+@pytest.mark.parametrize("name,nslabs", [("sod", 4), ("cavity", 3)])
+def test_slab_buckets_follow_from_the_slabs_own_counts(env, monkeypatch, name, nslabs):
+    """Memory that the library has not written holds 0xCCCCCCCC, behind the
+    counts of a slab too.  Taken for a count, that word makes a bucket of 16
+    slots (0xCC..C and a quarter of it wrap), and cells of 30 or 80 particles
+    spill; from the slab's own counts a bucket has a quarter and 16 slots to
+    spare, above the four standard deviations of any arrival count here."""
+    import ctypes
+    import torch
+    U, D = env
+    held = {}
+
+    def filled(nbytes, ctx):
+        t = torch.full(((int(nbytes) + 4096) // 4,), 0xCCCCCCCC - (1 << 32), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    def allocator():
+        a = U.Allocator()
+        a.alloc = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p)(filled)
+        a.free = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p)(lambda p, ctx: held.__delitem__(p))
+        a.ctx = None
+        return a, (a.alloc, a.free)
+
+    monkeypatch.setattr(U, "_torch_allocator", allocator)
+    real = U.Simulation
+    w = _case(name)
+    P = real(w).init_particles().particles()
+    monkeypatch.setattr(U, "Simulation", lambda ws: real(ws, allocator="torch"))
+    dec = D.DecomposedSim(w, nslabs).load(P)
+    assert len(held) > 0
+    dec.step(3)
+    c = dec.counters()
+    assert c[5] == 0 and c[6] == 0, c
+    dec.close()
