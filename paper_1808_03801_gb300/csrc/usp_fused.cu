@@ -1518,7 +1518,8 @@ __global__ void __launch_bounds__(32 * kG2wWarps, kG2wBlocks) k_g2(const SimDev*
                 }
             }
             if (bulk) {
-                ok = mbar_wait(&sh.full[par], phase >> par & 1u);
+                // one outcome for the warp: near the limit some lanes may see the copy land and others not
+                ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[par], phase >> par & 1u));
                 if (!ok) break;
                 phase ^= 1u << par;
             }
