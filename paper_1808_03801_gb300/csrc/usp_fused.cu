@@ -36,29 +36,25 @@ namespace {
 
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
 
-// the spill-list indices of `cell` (at most `most`; the others count as lost)
-// into spl (one warp); returns how many
-__device__ uint32_t collect_spill(const SimDev& s, int b, int cell, uint32_t* spl, uint32_t most, int lane) {
+// f(rank, i) for each entry i of buffer b's spill list that belongs to `cell`,
+// rank counting them (a warp; its lanes take entries side by side); returns
+// how many there are
+template <class F>
+__device__ __forceinline__ uint32_t each_spilled(const SimDev& s, int b, int cell, int lane, const F& f) {
     const uint32_t n = min(s.dyn->sp_n[b], (uint32_t)kSpillCap);
     uint32_t found = 0;
     for (uint32_t base = 0; base < n; base += 32) {
         const uint32_t i = base + lane;
         const bool hit = i < n && s.sp_cell[b][i] == (uint32_t)cell;
         const unsigned m = __ballot_sync(0xffffffffu, hit);
-        const uint32_t pos = found + __popc(m & lanemask_lt());
-        if (hit && pos < most) spl[pos] = i;
+        if (hit) f(found + __popc(m & lanemask_lt()), i);
         found += __popc(m);
-    }
-    __syncwarp();
-    if (found > most) {
-        if (lane == 0) atomicAdd(&s.dyn->counters[kCntOverflow], (unsigned long long)(found - most));
-        found = most;
     }
     return found;
 }
 
 template <int DIM>
-__device__ __forceinline__ void load_particle(const SimDev& s, int b, uint32_t base, uint32_t nb, const uint32_t* spl,
+__device__ __forceinline__ void load_particle(const SimDev& s, int b, uint32_t base, uint32_t nb, const uint16_t* spl,
                                               uint32_t j, float& x, float& y, float& v0, float& v1, float& v2,
                                               uint32_t& id) {
     if (j < nb) {
@@ -80,7 +76,7 @@ __device__ __forceinline__ void load_particle(const SimDev& s, int b, uint32_t b
     }
 }
 
-__device__ __forceinline__ void store_velocity(const SimDev& s, int b, uint32_t base, uint32_t nb, const uint32_t* spl,
+__device__ __forceinline__ void store_velocity(const SimDev& s, int b, uint32_t base, uint32_t nb, const uint16_t* spl,
                                                uint32_t j, float v0, float v1, float v2) {
     if (j < nb) {
         const uint32_t i = base + j;
@@ -267,7 +263,6 @@ enum { kFull = 0, kRelaxOnly = 1, kFullSlab = 2, kFullFlux = 3 };
 
 constexpr int kG2P = 4;         // particles per thread and chunk
 constexpr int kG2Warps = 16;    // resident warps per SM
-constexpr int kG2Spill = 512;   // spill-list entries one cell may add to its bucket
 
 // shared state of one block of k_g2b
 template <int G>
@@ -280,7 +275,7 @@ struct G2Shared {
     uint32_t part_n[G];         // per-warp relaxed particles
     uint32_t key[20];           // the ten round keys of the relaxation's Philox calls
     uint32_t hist[256];         // fixed-count selection: digits
-    uint32_t spl[kG2Spill];     // the cell's spill-list entries
+    uint16_t spl[kSpillCap];    // the cell's spill-list entries (all of them, if need be)
     uint32_t nsp;
     uint32_t next;              // next unit
     uint32_t sel[4];            // fixed-count selection: broadcast words
@@ -403,7 +398,7 @@ __device__ __forceinline__ void g2_flush(G2Acc& a, SimDyn* dyn, int tid) {
 }
 
 // the id of particle j of a cell (bucket, then its spill-list entries)
-__device__ __forceinline__ uint32_t g2_id(const SimDev& s, int p, uint32_t base, uint32_t nb, const uint32_t* spl,
+__device__ __forceinline__ uint32_t g2_id(const SimDev& s, int p, uint32_t base, uint32_t nb, const uint16_t* spl,
                                           uint32_t j) {
     return j < nb ? s.pid[p][base + j] : s.sp_pid[p][spl[j - nb]];
 }
@@ -531,15 +526,9 @@ __device__ __noinline__ uint32_t g2_collect(G2Shared<G>& sh, int p, int cell, in
     __syncthreads();
     const uint32_t n = min(s.dyn->sp_n[p], (uint32_t)kSpillCap);
     for (uint32_t i = tid; i < n; i += 32 * G)
-        if (s.sp_cell[p][i] == (uint32_t)cell) {
-            const uint32_t k = atomicAdd(&sh.nsp, 1u);
-            if (k < (uint32_t)kG2Spill) sh.spl[k] = i;
-        }
+        if (s.sp_cell[p][i] == (uint32_t)cell) sh.spl[atomicAdd(&sh.nsp, 1u)] = (uint16_t)i;
     __syncthreads();
-    const uint32_t found = sh.nsp;
-    if (found <= (uint32_t)kG2Spill) return found;
-    if (tid == 0) atomicAdd(&s.dyn->counters[kCntOverflow], (unsigned long long)(found - kG2Spill));
-    return kG2Spill;
+    return sh.nsp;
 }
 
 // one cell: bucket [base, base + nb) of buffer p, `arrived` arrivals
@@ -889,7 +878,6 @@ __device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, in
 // warp's work, so that a fault shows up as lost particles, not as a hang.
 // ---------------------------------------------------------------------------
 constexpr int kG2Stage1 = 448, kG2Stage2 = 384;   // staged particles per warp, 1-D and 2-D (multiples of 32)
-constexpr int kG2wSpill = 64;                     // spill-list entries one cell may add to its bucket
 
 constexpr int g2w_words(int dims) {   // 32-bit words of the staging area: (x,) y, v0, v1, v2, id and 16-bit slots
     return dims == 1 ? 5 * kG2Stage1 + kG2Stage1 / 2 : 6 * kG2Stage2 + kG2Stage2 / 2;
@@ -904,7 +892,6 @@ struct alignas(16) G2Warp {
     uint32_t wst[kWin];    // arrivals per window slot, then its first reserved index
     uint32_t wlo[kWin];    // start and end of the slot's bucket
     uint32_t wend[kWin];
-    uint32_t spl[kG2wSpill];
     int2 ptile[4];         // the cells on their way: tile,
     uint32_t pbound[4][4]; // bucket start, end and arrivals,
     uint32_t punit[4];     // unit number
@@ -1097,6 +1084,30 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
 #pragma unroll
     for (int k = 0; k < 8; ++k) R[k] = 0.0f;
     uint32_t nr = 0;
+    // GEN: particles [off, off + cnt) of the cell, the bucket's and then the spill list's
+    auto load_chunk = [&](uint32_t off, uint32_t cnt) {
+#pragma unroll 1
+        for (uint32_t j = lane; j < cnt && off + j < nb; j += 32) {
+            const uint32_t i = base + off + j;
+            if (DIM == 2) st_x[j] = ((const float*)s.pos[p][0])[i];
+            st_y[j] = ((const float*)s.pos[p][1])[i];
+            st_0[j] = ((const float*)s.vel[p][0])[i];
+            st_1[j] = ((const float*)s.vel[p][1])[i];
+            st_2[j] = ((const float*)s.vel[p][2])[i];
+            st_id[j] = s.pid[p][i];
+        }
+        if (off + cnt > nb) each_spilled(s, p, cell, lane, [&](uint32_t rank, uint32_t i) {
+            const uint32_t j = nb + rank - off;   // (far above cnt where it lies before off)
+            if (j >= cnt) return;
+            if (DIM == 2) st_x[j] = s.sp_pos[p][0][i];
+            st_y[j] = s.sp_pos[p][1][i];
+            st_0[j] = s.sp_vel[p][0][i];
+            st_1[j] = s.sp_vel[p][1][i];
+            st_2[j] = s.sp_vel[p][2][i];
+            st_id[j] = s.sp_pid[p][i];
+        });
+        __syncwarp();
+    };
     float al = 1.0f, uo0 = 0, uo1 = 0, uo2 = 0, mn0 = 0, mn1 = 0, mn2 = 0;
     bool apply = false;
 #pragma unroll 1
@@ -1105,18 +1116,7 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
         const uint32_t cnt = GEN ? min(CAP, n - off) : n;
         if (GEN) {
             __syncwarp();
-#pragma unroll 1
-            for (uint32_t j = lane; j < cnt; j += 32) {
-                float x = 0.0f, y, v0, v1, v2;
-                uint32_t id;
-                load_particle<DIM>(s, p, base, nb, sh.spl, off + j, x, y, v0, v1, v2, id);
-                if (DIM == 2) st_x[j] = x;
-                st_y[j] = y;
-                st_0[j] = v0;
-                st_1[j] = v1;
-                st_2[j] = v2;
-                st_id[j] = id;
-            }
+            load_chunk(off, cnt);
         }
         uint32_t selm = 0;   // bit i: the lane's particle of iteration i is relaxed
         // ---- sweep 1: each lane on its own particles, two at a time (lanes
@@ -1201,14 +1201,19 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                 }
             }
         }
-        if (!apply && selm) {   // fewer than two relaxed particles in the cell: reverted
+        if (GEN) {   // fewer than two relaxed particles in the cell: reverted
+            if (!apply && __any_sync(0xffffffffu, selm)) {
+                __syncwarp();
+                load_chunk(off, cnt);
+                selm = 0;
+            }
+        } else if (!apply && selm) {
 #pragma unroll 1
             for (uint32_t b = lane; b < cnt; b += 32, selm >>= 1)
                 if (selm & 1u) {
-                    float x, y;
-                    uint32_t id;
-                    load_particle<DIM>(s, p, base, nb, sh.spl, off + b, x, y, st_0[ro + b], st_1[ro + b],
-                                       st_2[ro + b], id);
+                    st_0[ro + b] = ((const float*)s.vel[p][0])[base + b];
+                    st_1[ro + b] = ((const float*)s.vel[p][1])[base + b];
+                    st_2[ro + b] = ((const float*)s.vel[p][2])[base + b];
                 }
             selm = 0;
         }
@@ -1404,7 +1409,7 @@ template <int DIM, int MODE, class Sh>
 __device__ __noinline__ G2Acc g2w_cell_general(Sh& sh, G2Sim S, G2Job J, int lane) {
     G2Acc acc = {0u, 0u};
     uint32_t nsp = 0;
-    if (J.arrived > J.nb) nsp = collect_spill(sh.sim, S.p, J.cell, sh.spl, kG2wSpill, lane);
+    if (J.arrived > J.nb) nsp = each_spilled(sh.sim, S.p, J.cell, lane, [](uint32_t, uint32_t) {});
     if (J.nb + nsp == 0) return acc;   // no bucket, and the spill list was full when its particles arrived
     g2w_cell_impl<DIM, MODE, true>(sh, S, J, 0u, nsp, lane, acc);
     return acc;
@@ -1604,7 +1609,6 @@ constexpr int kG1Units = 1;     // units per block wanted
 
 __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                      const int* __restrict__ ntiles) {
-    __shared__ uint32_t spl_all[kG1Warps][32];
     // the unit's per-cell headers, fetched in one round for all its cells:
     // bucket start, particles in the bucket, arrivals, and the shift u_s
     __shared__ uint32_t h_base[kCTile], h_nb[kCTile], h_arr[kCTile];
@@ -1700,9 +1704,7 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
             const uint32_t arrived = h_arr[cc];
             const float4 us = h_us[cc];
             const float u0 = us.x, u1 = us.y, u2 = us.z;
-            uint32_t nsp = 0;
-            if (arrived > nb) nsp = collect_spill(s, q, cell, spl_all[warp], 32u, lane);
-            const uint32_t n = nb + nsp;
+            uint32_t n = nb;
             float S[12];
 #pragma unroll
             for (int k = 0; k < 12; ++k) S[k] = 0.0f;
@@ -1733,10 +1735,10 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
                 __syncwarp();   // the stage is refilled by the copy issued two chunks on
                 ++done;
             }
-            for (uint32_t j = nb + lane; j < n; j += 32) {   // spill-list entries of the cell
-                const uint32_t i = spl_all[warp][j - nb];
-                add(s.sp_vel[q][0][i], s.sp_vel[q][1][i], s.sp_vel[q][2][i]);
-            }
+            if (arrived > nb)
+                n += each_spilled(s, q, cell, lane, [&](uint32_t, uint32_t i) {
+                    add(s.sp_vel[q][0][i], s.sp_vel[q][1][i], s.sp_vel[q][2][i]);
+                });
             // The cell's 64-byte record [N, 12 sums, shift u_s] as a warp
             // reduce-scatter: at each of four halving stages a lane keeps half
             // of its values and adds the partner's copy of that half (16

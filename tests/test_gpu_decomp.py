@@ -154,3 +154,23 @@ def test_slab_buckets_follow_from_the_slabs_own_counts(env, monkeypatch, name, n
     c = dec.counters()
     assert c[5] == 0 and c[6] == 0, c
     dec.close()
+
+
+def test_density_jump_at_a_slab_boundary(env):
+    """The bucket of the first cell behind the boundary does not know of the
+    dense cells before it: what enters there goes through the spill list, and
+    none of it is lost."""
+    U, D = env
+    w = _fused(W.sod(ny=1000, ppc_left=360, seed=2))
+    P = U.Simulation(w).init_particles().particles()
+    whole = U.Simulation(w).set_particles(P["pos"], P["vel"], P["pid"])
+    dec = D.DecomposedSim(w, 4).load(P)
+    whole.step(1)
+    dec.step(1)
+    assert dec.counters()[5] == 0 and dec.counters()[6] > 0
+    assert np.array_equal(dec.sample()[15], whole.sample()[15])
+    dec.step(20)
+    Q = dec.particles()
+    assert dec.counters()[5] == 0 and np.array_equal(np.sort(Q["pid"]), np.sort(P["pid"]))
+    assert np.array_equal(np.bincount(Q["cell"], minlength=1000), dec.sample()[15].astype(np.int64))
+    dec.close()

@@ -108,6 +108,21 @@ def test_fused_cell_sizes(usp, dim, R, reach):
     assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
 
 
+@pytest.mark.parametrize("R", [4, 12])
+def test_fused_cells_with_long_spill_lists(usp, R):
+    """Cells of 16 and 1500 particles side by side at reach 1: hundreds go to
+    the spill list for one cell.  All of them count in the cell's moments and go
+    on with it."""
+    counts = EDGES
+    w = _domain(1, len(counts), int(np.mean(counts)), 1.0)
+    g = usp.Simulation(dict(w, params=dict(w["params"], pipeline="fused"))).set_particles(*_state(w, counts, 5))
+    g.set_tuning(fused_R=R).step(1)
+    assert g.info()["counters"][5] == 0 and g.info()["counters"][6] > 128
+    g.close()
+    sets = [_differing_cells(usp, w, counts, R, 8, seed) for seed in (5, 6)]
+    assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
+
+
 @pytest.mark.parametrize("ncells", [1, 8191, 8192, 8193])
 def test_fused_layout_on_both_sides_of_the_one_kernel_limit(usp, ncells):
     w = _domain(1, ncells, 16, 0.02)
