@@ -9,22 +9,37 @@ on the simulation's stream, after warm-up) and keeps the fastest:
 * grid_per_sm: persistent blocks per SM of the tiled kernels.
 
 Results are cached in a JSON file keyed by the workload shape (dimension,
-cells, particles per cell, precision, pipeline, GPU name).
+cells, particles per cell, precision, pipeline, GPU name) and the kernels'
+source: what a value of fused_R selects, and which is the fastest, changes with
+them, and a record of other kernels could pick one that takes twice as long.
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import os
+
+from . import build
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), ".tune_cache.json")
 CANDIDATES_R = (4, 8, 12)
 CANDIDATES_GRID = (4, 8, 16)
 
 
+def _source_hash():
+    h = hashlib.sha1()
+    for name in sorted(os.listdir(build.CSRC)):
+        if name.endswith((".cu", ".cuh")):
+            with open(os.path.join(build.CSRC, name), "rb") as f:
+                h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:16]
+
+
 def _key(w, device_name):
     g, p = w["grid"], w["params"]
     cells = (g["nx"] if g["dim"] == 2 else 1) * g["ny"]
-    return f'{device_name}|{g["dim"]}|{cells}|{p["ppc_ref"]}|{p["precision"]}|{p.get("pipeline", "plain")}'
+    return (f'{device_name}|{g["dim"]}|{cells}|{p["ppc_ref"]}|{p["precision"]}|{p.get("pipeline", "plain")}'
+            f'|{_source_hash()}')
 
 
 def _load():
