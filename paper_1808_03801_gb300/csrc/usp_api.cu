@@ -189,6 +189,47 @@ static int upload_sim(usp_handle* h) {
     return USP_OK;
 }
 
+// k_g2 variant for `cells` cells in all of `ppc` particles.  R: one warp per
+// cell (4) is the cheapest per particle but takes the latency of a whole cell
+// (a dense one of a shock tube: 25 us); with few cells a block per cell spreads
+// each one over several warps (8: four, 12: eight).  blocks: of the warp form
+// per SM; three of them stage more particles per warp than four.
+//
+// Few cells: up to ten per SM.  Measured per k_g2 launch, R = 4 / 8 / 12: 100
+// cells of 200 particles 21 / 15 / 13 us; 1000 cells of 360 / 45 particles 30 /
+// 18 / 23 us; 5929 cells of 37 particles 28 / 44 / - us.  Eight warps pay where
+// every block has an SM to itself, and for cells above the 512 particles that
+// four warps hold (per step, 8 / 12: 1000 cells of 400 particles 31 / 35 us, of
+// 600 40.5 / 39).
+//
+// Many cells: a cell above the warp's staging area costs two to three times as
+// much, and three blocks per SM are slower than four by a tenth, so the line lies
+// where a cell two standard deviations above ppc still fits.  Per step, four
+// blocks / three / R = 8 / R = 12: 20 000 1-D cells of 400 particles 162 / 177 /
+// 257 / 332 us, of 450 277 / 193 / 276 / 340, of 600 324 / 234 / 407 / 408; 64
+// tubes of 420 / 52 particles 416 / 399 / 592 / 839 us; 10^4 2-D cells of 340 125 /
+// 123 / 146 / 195 us, of 400 204 / 133 / 160 / 204.  Three blocks pay up to one
+// deviation below their own area (1-D cells of 700: 352 / 277 / 444 / 422; 2-D of
+// 600: 243 / 201 / 252 / 256).  Above it four in 1-D (of 800: 383 us, R = 12 475),
+// blocks of eight warps in 2-D (of 800: 320 us, R = 12 294) and where the many
+// cells are few, up to twenty per SM (2000 1-D cells of 700: 63 us with three
+// blocks, R = 12 59; 2025 2-D cells of 600: 81, 69).
+struct G2Form {
+    int R, blocks;
+};
+
+static G2Form choose_form(int64_t cells, int ppc, int dim) {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const double dense = ppc, sd = std::sqrt(dense);
+    const int blocks = dense + 2 * sd > kG2Stage[1][dim - 1] && dense + sd <= kG2Stage[0][dim - 1] ? 3 : 4;
+    int R;
+    if (cells <= 10 * (int64_t)sms) R = (cells <= 2 * (int64_t)sms && ppc > 128) || dense + 2 * sd > 512 ? 12 : 8;
+    else if (cells <= 20 * (int64_t)sms && dense + 2 * sd > kG2Stage[0][dim - 1]) R = 12;
+    else R = dim == 2 && ppc > 700 ? 12 : 4;
+    return {R, blocks};
+}
+
 static Launch make_launch(usp_handle* h) {
     Launch L;
     L.sims = h->d_sim;
@@ -207,6 +248,7 @@ static Launch make_launch(usp_handle* h) {
     L.grid_u = persistent_grid(h->nptiles * (kPTile / kPUnit), 2 * h->grid_per_sm);
     L.grid_c = persistent_grid(h->nctiles, h->grid_per_sm);
     L.grid_f = persistent_grid(8 * h->nctiles, h->grid_per_sm);
+    L.g2_blocks = choose_form(h->host.K, h->ppc_ref, h->host.dim).blocks;
     L.lay_tiles = (h->host.K + kLayTile - 1) / kLayTile;
     L.stream = h->stream;
     return L;
@@ -254,27 +296,9 @@ static void enqueue_any(usp_handle* h, const Launch& L) {
     else enqueue_step(L, h->precision == USP_FP64, h->host.has_reservoir != 0);
 }
 
-// k_g2 variant for `cells` cells in all.  One warp per cell (4) is the
-// cheapest per particle but takes the latency of a whole cell (a dense one
-// of a shock tube: 25 us); with few cells a block per cell spreads each one
-// over several warps (8: four warps, 12: eight).  Measured per k_g2 launch:
-// 100 cells of 200 particles 21 us (4), 15 us (8), 13 us (12); 1000 cells of
-// 360 / 45 particles 30, 18, 23 us; 5929 cells of 37 particles 28, 44 us; so
-// the line lies at ten cells per SM, and eight warps pay where every block
-// has an SM to itself.  Cells above a warp's staging area (kG2Stage1 / 2, with
-// a margin for the scatter about the mean) go to the eight-warp blocks, which
-// hold 1024 particles in registers.
-static int choose_R(int64_t cells, int ppc_ref, int dim) {
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (ppc_ref > (dim == 1 ? 370 : 320)) return 12;
-    if (cells > 10 * (int64_t)sms) return 4;
-    return cells <= 2 * (int64_t)sms && ppc_ref > 128 ? 12 : 8;
-}
-
 // a load goes back to the default variant (graphs captured with another go)
 static void set_default_R(usp_handle* h) {
-    const int R = choose_R(h->host.K, h->ppc_ref, h->host.dim);
+    const int R = choose_form(h->host.K, h->ppc_ref, h->host.dim).R;
     if (R != h->fused_R) destroy_graphs(h->graphs);
     h->fused_R = R;
     h->tuned = false;
@@ -1325,19 +1349,27 @@ extern "C" int usp_batch_retire(usp_batch* b, usp_handle* h) {
     return bfail(b, USP_ERR_INVALID_ARG, "handle not in batch");
 }
 
-// k_g2 variant of a batch: the tuned one if a member was tuned, else by all
-// cells together and the particles per cell of the members that hold most
-static int batch_R(const usp_batch* b) {
+// k_g2 variant of a batch: by all cells together and the form that the members
+// holding most particles would take with that many cells; R is the tuned one if
+// a member was tuned
+static G2Form batch_form(const usp_batch* b) {
     int tuned = 0;
-    int64_t cells = 0, total = 0, dense = 0;
+    int64_t cells = 0, total = 0, dense = 0, three = 0;
     for (auto* h : b->members) {
         if (h->tuned) tuned = std::max(tuned, h->fused_R);
         cells += h->host.K;
-        total += h->host.cap;
-        if (choose_R(1 << 30, h->ppc_ref, h->host.dim) == 12) dense += h->host.cap;
     }
-    if (tuned) return tuned;
-    return choose_R(cells, 2 * dense > total ? 1 << 20 : 1, 1);
+    for (auto* h : b->members) {
+        const G2Form f = choose_form(cells, h->ppc_ref, h->host.dim);
+        total += h->host.cap;
+        if (f.R == 12) dense += h->host.cap;
+        if (f.blocks == 3) three += h->host.cap;
+    }
+    G2Form f = choose_form(cells, 1, 1);
+    if (2 * dense > total) f.R = 12;
+    if (2 * three > total) f.blocks = 3;
+    if (tuned) f.R = tuned;
+    return f;
 }
 
 // everything a captured graph depends on besides the device tables
@@ -1355,7 +1387,9 @@ static uint64_t batch_key(const usp_batch* b) {
         if (h->pipeline == USP_PIPE_FUSED) k |= 128u;       // precision or pipeline
         per_sm = std::max(per_sm, h->grid_per_sm);
     }
-    return k | (uint64_t)batch_R(b) << 8 | (uint64_t)per_sm << 16 | (uint64_t)b->members.size() << 32;
+    const G2Form f = batch_form(b);
+    if (f.blocks == 3) k |= 1ull << 12;
+    return k | (uint64_t)f.R << 8 | (uint64_t)per_sm << 16 | (uint64_t)b->members.size() << 32;
 }
 
 // rebuild the device tables of the batch (simulation list and tiles)
@@ -1462,6 +1496,7 @@ static Launch batch_launch(usp_batch* b) {
     L.grid_u = persistent_grid(1 << 30, 2 * per_sm);
     L.grid_c = persistent_grid(1 << 30, per_sm);
     L.grid_f = L.grid_c;
+    L.g2_blocks = batch_form(b).blocks;
     L.lay_tiles = b->lay_tiles;
     L.stream = b->stream;
     return L;
@@ -1472,7 +1507,7 @@ static int batch_capture(usp_batch* b, int nsteps, cudaGraphExec_t* exec) {
     const bool fp64 = b->precision == USP_FP64;
     bool res = false;
     for (auto* h : b->members) res |= h->host.has_reservoir != 0;
-    const int R = batch_R(b);
+    const int R = batch_form(b).R;
     if (b->pipeline == USP_PIPE_FUSED && b->fork.make()) b->fork.attach(L);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
@@ -1539,7 +1574,7 @@ extern "C" int usp_batch_run_stage(usp_batch* b, int stage) {
     const bool fp64 = b->precision == USP_FP64;
     bool res = false;
     for (auto* h : b->members) res |= h->host.has_reservoir != 0;
-    const int R = batch_R(b);
+    const int R = batch_form(b).R;
     if (stage_launch(L, b->pipeline, fp64, R, res, stage))
         return bfail(b, USP_ERR_INVALID_ARG, "stage must be 0..6 (plain) or 10..14 (fused)");
     cudaError_t e = cudaGetLastError();

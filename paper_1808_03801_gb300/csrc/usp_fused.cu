@@ -870,22 +870,21 @@ __device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, in
 // seven consumer warps): 64 shock tubes 301 -> 255 us, cavity 200 x 200 168 ->
 // 119 us, slit 522 -> 388 us per launch.
 // Cells above the staging area, and cells with spill-list entries, take the
-// general form of the same code: loaded by the lanes, in chunks, the draws of
-// all but one chunk made twice.
+// general form of the same code: loaded by the lanes (asynchronously, a chunk
+// at once: 20 000 cells of 600 particles 692 -> 324 us a step), in chunks, the
+// draws of all but one chunk made twice.  Domains whose cells are mostly above
+// the area of four blocks per SM run three with more staging (choose_form).
 //
 // The wait for a copy is bounded (kG2WaitNs of global time); one that runs out
 // adds kG2TimeoutMark to the overflow counter of simulation 0 and ends the
 // warp's work, so that a fault shows up as lost particles, not as a hang.
 // ---------------------------------------------------------------------------
-constexpr int kG2Stage1 = 448, kG2Stage2 = 384;   // staged particles per warp, 1-D and 2-D (multiples of 32)
+constexpr int kG2wWarps = 4;    // warps per block
 
-constexpr int g2w_words(int dims) {   // 32-bit words of the staging area: (x,) y, v0, v1, v2, id and 16-bit slots
-    return dims == 1 ? 5 * kG2Stage1 + kG2Stage1 / 2 : 6 * kG2Stage2 + kG2Stage2 / 2;
-}
-
-template <int DIMS>
+template <int DIMS, int BLOCKS>   // BLOCKS per SM
 struct alignas(16) G2Warp {
-    float stage[g2w_words(DIMS)];
+    static constexpr uint32_t CAP = kG2Stage[BLOCKS - 3][DIMS - 1];   // staged particles
+    float stage[(DIMS == 1 ? 5 : 6) * CAP + CAP / 2];                 // (x,) y, v0, v1, v2, id and 16-bit slots
     float prm[2][kNFPrm];  // parameter records of the cell and of the next one
     SimDev sim;
     uint32_t key[20];
@@ -1001,15 +1000,12 @@ struct G2Job {
     uint32_t ro;           // first staged particle
 };
 
-template <int DIM>
-__host__ __device__ constexpr uint32_t g2w_cap() { return DIM == 1 ? kG2Stage1 : kG2Stage2; }
-
 // start the bulk copies of a cell's bucket and parameter record (lane 0):
 // whole 16-byte groups, bucket starts and the capacity being multiples of
 // four slots
 template <int DIM, class Sh>
 __device__ __forceinline__ void g2w_copy(Sh& sh, const G2Job& J, int p, uint32_t parity) {
-    constexpr uint32_t CAP = g2w_cap<DIM>();
+    constexpr uint32_t CAP = Sh::CAP;
     const SimDev& s = sh.sim;
     float* const d = sh.stage + J.ro;
     const uint32_t bytes = 4u * ((J.nb + 3u) & ~3u);
@@ -1028,7 +1024,7 @@ __device__ __forceinline__ void g2w_copy(Sh& sh, const G2Job& J, int p, uint32_t
 // compact layout right after a set-up sort)
 template <int DIM, class Sh>
 __device__ __noinline__ void g2w_load(Sh& sh, G2Job J, int p, uint32_t parity, int lane) {
-    constexpr uint32_t CAP = g2w_cap<DIM>();
+    constexpr uint32_t CAP = Sh::CAP;
     const SimDev& s = sh.sim;
     float* const d = sh.stage + J.ro;
     if (lane < kNFPrm) sh.prm[parity][lane] = s.fprm[(size_t)J.cell * kNFPrm + lane];
@@ -1054,7 +1050,7 @@ struct Num {
 template <int DIM, int MODE, bool GEN, class Sh>
 __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Job& J, uint32_t parity, uint32_t nsp,
                                               int lane, G2Acc& acc) {
-    constexpr uint32_t CAP = g2w_cap<DIM>();
+    constexpr uint32_t CAP = Sh::CAP;
     const SimDev& s = sh.sim;
     const int p = S.p, q = p ^ 1, cell = J.cell;
     const uint32_t base = J.base, nb = J.nb, n = nb + nsp, ro = GEN ? 0u : J.ro;
@@ -1086,15 +1082,16 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
     uint32_t nr = 0;
     // GEN: particles [off, off + cnt) of the cell, the bucket's and then the spill list's
     auto load_chunk = [&](uint32_t off, uint32_t cnt) {
+        // (all of the chunk in flight at once)
 #pragma unroll 1
         for (uint32_t j = lane; j < cnt && off + j < nb; j += 32) {
             const uint32_t i = base + off + j;
-            if (DIM == 2) st_x[j] = ((const float*)s.pos[p][0])[i];
-            st_y[j] = ((const float*)s.pos[p][1])[i];
-            st_0[j] = ((const float*)s.vel[p][0])[i];
-            st_1[j] = ((const float*)s.vel[p][1])[i];
-            st_2[j] = ((const float*)s.vel[p][2])[i];
-            st_id[j] = s.pid[p][i];
+            if (DIM == 2) cp_async4(st_x + j, (const float*)s.pos[p][0] + i);
+            cp_async4(st_y + j, (const float*)s.pos[p][1] + i);
+            cp_async4(st_0 + j, (const float*)s.vel[p][0] + i);
+            cp_async4(st_1 + j, (const float*)s.vel[p][1] + i);
+            cp_async4(st_2 + j, (const float*)s.vel[p][2] + i);
+            cp_async4(st_id + j, s.pid[p] + i);
         }
         if (off + cnt > nb) each_spilled(s, p, cell, lane, [&](uint32_t rank, uint32_t i) {
             const uint32_t j = nb + rank - off;   // (far above cnt where it lies before off)
@@ -1106,6 +1103,7 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
             st_2[j] = s.sp_vel[p][2][i];
             st_id[j] = s.sp_pid[p][i];
         });
+        cp_async_wait_all();
         __syncwarp();
     };
     float al = 1.0f, uo0 = 0, uo1 = 0, uo2 = 0, mn0 = 0, mn1 = 0, mn2 = 0;
@@ -1415,20 +1413,17 @@ __device__ __noinline__ G2Acc g2w_cell_general(Sh& sh, G2Sim S, G2Job J, int lan
     return acc;
 }
 
-constexpr int kG2wWarps = 4;    // warps per block
-constexpr int kG2wBlocks = 4;   // blocks per SM
-
 // DIMS 1 or 2: the dimension of every cell of the tiles *first .. *first +
 // *ntiles (first null: 0)
-template <int DIMS, int MODE>
-__global__ void __launch_bounds__(32 * kG2wWarps, kG2wBlocks) k_g2(const SimDev* __restrict__ sims,
+template <int DIMS, int MODE, int BLOCKS>
+__global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __restrict__ sims,
                                                                    const int2* __restrict__ tiles,
                                                                    const int* __restrict__ ntiles,
                                                                    const int* __restrict__ first_tile,
                                                                    uint32_t* __restrict__ wq) {
     extern __shared__ __align__(16) unsigned char g2_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    G2Warp<DIMS>& sh = reinterpret_cast<G2Warp<DIMS>*>(g2_smem)[warp];
+    G2Warp<DIMS, BLOCKS>& sh = reinterpret_cast<G2Warp<DIMS, BLOCKS>*>(g2_smem)[warp];
     const SimDev& s = sh.sim;
     const uint32_t nunits = (uint32_t)*ntiles * kCTile;   // a unit is one cell slot of a tile
     if (first_tile) tiles += *first_tile;
@@ -1490,7 +1485,7 @@ __global__ void __launch_bounds__(32 * kG2wWarps, kG2wBlocks) k_g2(const SimDev*
             known = 0;
             staged = false;
         }
-        const uint32_t room = g2w_cap<DIMS>(), cap = (uint32_t)s.cap;
+        const uint32_t room = sh.CAP, cap = (uint32_t)s.cap;
         G2Job J;
         J.cell = tile.y + (int)(unit % kCTile);
         J.base = J.nb = J.arrived = 0;
@@ -2538,22 +2533,28 @@ void launch_g2b_one(const Launch& L) {
     k_g2b<DIMS, MODE, ABL, G><<<grid, 32 * G, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles, L.wq);
 }
 
-template <int DIMS, int MODE>
-void launch_g2_one(const Launch& L, cudaStream_t st, bool part) {
+template <int DIMS, int MODE, int BLOCKS>
+void launch_g2_blocks(const Launch& L, cudaStream_t st, bool part) {
     static int wave = 0;
-    constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS>));
+    constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS, BLOCKS>));
     if (!wave) {
         int dev = 0, sms = 152, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_g2<DIMS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE>, 32 * kG2wWarps, smem);
+        cudaFuncSetAttribute(k_g2<DIMS, MODE, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE, BLOCKS>, 32 * kG2wWarps, smem);
         wave = sms * std::max(per, 1);
     }
     const int grid = std::max(1, std::min(wave, (L.cells + kG2wWarps - 1) / kG2wWarps));
     const int* n = part ? (DIMS == 1 ? L.ndim : L.ndim + 1) : L.nctiles;
-    k_g2<DIMS, MODE><<<grid, 32 * kG2wWarps, smem, st>>>(L.sims, L.ctiles, n, part && DIMS == 2 ? L.ndim : nullptr,
+    k_g2<DIMS, MODE, BLOCKS><<<grid, 32 * kG2wWarps, smem, st>>>(L.sims, L.ctiles, n, part && DIMS == 2 ? L.ndim : nullptr,
                                                          DIMS == 1 ? L.wq : L.wq + 2);
+}
+
+template <int DIMS, int MODE>
+void launch_g2_one(const Launch& L, cudaStream_t st, bool part) {
+    if (L.g2_blocks == 3) launch_g2_blocks<DIMS, MODE, 3>(L, st, part);
+    else launch_g2_blocks<DIMS, MODE, 4>(L, st, part);
 }
 
 // A mixed batch runs the kernels of both dimensions side by side (one kernel

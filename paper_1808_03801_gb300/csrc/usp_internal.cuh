@@ -226,6 +226,7 @@ struct Launch {
     int grid_p, grid_c;   // persistent grid sizes
     int grid_u = 1;       // grid of the particle kernels (units of kPUnit)
     int grid_f = 1;       // grid of k_g1 (its units are parts of cell tiles)
+    int g2_blocks = 4;    // k_g2, a warp per cell: blocks per SM, 4 or (more staging per warp) 3
     int lay_tiles = 1;    // layout tiles (kLayTile cells) of the largest simulation
     cudaStream_t stream;
     // fused step: a second stream and two events let the layout kernels run
@@ -238,6 +239,7 @@ constexpr int kPTile = 512;   // particles per tile
 constexpr int kPUnit = 128;   // particles a block of the particle kernels takes at a time (a quarter of a tile)
 constexpr int kCTile = 32;    // cells per tile (balances the per-cell kernels across SMs)
 constexpr int kSpillCap = 4096;  // spill entries per parity (fused pipeline)
+constexpr uint32_t kG2Stage[2][2] = {{736, 640}, {448, 384}};   // k_g2: particles a warp stages with 3 and 4 blocks per SM, 1-D and 2-D (multiples of 32)
 constexpr int kNFPrm = 16;       // u[3], theta, M[6], P_relax (0: none), nu, 1/nu_ES, P_ne, X, 1/P_relax (G2Prm)
 constexpr int kLayTile = 1024;   // cells per block of the layout kernels (fused pipeline)
 

@@ -108,6 +108,22 @@ def test_fused_cell_sizes(usp, dim, R, reach):
     assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
 
 
+@pytest.mark.parametrize("ppc_ref", [100, 450])
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("reach", [0.02, 1.0])
+def test_fused_warp_per_cell_staging(usp, dim, ppc_ref, reach):
+    """The warp form with four blocks per SM (100 particles per cell meant) and
+    with three and more staging (450): cells at the edges of either area and in
+    several chunks, against blocks of four warps."""
+    counts = EDGES + [575, 577, 639, 640, 641, 704, 735, 736, 737, 800, 900]
+    if dim == 1:
+        counts = counts + counts[::-1]
+    w = _domain(dim, len(counts), int(np.mean(counts)), reach)
+    w["params"]["ppc_ref"] = ppc_ref
+    sets = [_differing_cells(usp, w, counts, 4, 8, seed) for seed in (14, 15)]
+    assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
+
+
 @pytest.mark.parametrize("R", [4, 12])
 def test_fused_cells_with_long_spill_lists(usp, R):
     """Cells of 16 and 1500 particles side by side at reach 1: hundreds go to
