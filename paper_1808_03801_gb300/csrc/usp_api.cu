@@ -65,6 +65,10 @@ struct Fork {
     }
 };
 
+// words of d_ntiles: two tile counts, two of k_g2's work queue for each group,
+// and (batches) the tiles of each group and their first one
+constexpr int kNTiles = 2 + 4 * kG2Groups;
+
 struct usp_handle {
     SimDev host{};            // host copy of the simulation description
     SimDev* d_sim = nullptr;  // device copy
@@ -85,7 +89,7 @@ struct usp_handle {
     size_t cell_bytes = 0, part_bytes = 0;
     int2* d_ptiles = nullptr;
     int2* d_ctiles = nullptr;
-    int* d_ntiles = nullptr;          // [0] particle tiles, [1] cell tiles, [2..5] k_g2 work queues
+    int* d_ntiles = nullptr;          // [0] particle tiles, [1] cell tiles, [2..9] k_g2 work queues
     int nptiles = 0, nctiles = 0;
     Graphs graphs;
     bool initialised = false;
@@ -113,7 +117,7 @@ struct usp_batch {
     SimDev* d_sims = nullptr;
     int2* d_ptiles = nullptr;
     int2* d_ctiles = nullptr;
-    int* d_ntiles = nullptr;          // as a handle's, then [6], [7] the cell tiles of each dimension
+    int* d_ntiles = nullptr;          // as a handle's, then [10..13] cell tiles of each group, [14..17] the first of them
     size_t ptile_cap = 0, ctile_cap = 0;
     int nptiles = 0, nctiles = 0;
     Graphs graphs;
@@ -230,6 +234,8 @@ static G2Form choose_form(int64_t cells, int ppc, int dim) {
     return {R, blocks};
 }
 
+static int group_of(const usp_handle* h) { return g2_group(h->host.dim, h->host.selection || h->host.es_sampler); }
+
 static Launch make_launch(usp_handle* h) {
     Launch L;
     L.sims = h->d_sim;
@@ -238,7 +244,8 @@ static Launch make_launch(usp_handle* h) {
     L.ctiles = h->d_ctiles;
     L.nctiles = h->d_ntiles + 1;
     L.wq = (uint32_t*)(h->d_ntiles + 2);
-    L.ndim = nullptr;   // one dimension
+    L.gtiles = nullptr;   // one group
+    L.groups = 1 << group_of(h);
     L.nsims = 1;
     L.dims = h->host.dim == 1 ? 1 : 2;
     L.flux = h->host.flux_axis != 0;
@@ -564,7 +571,7 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     if ((rc = cell_alloc(h, sizeof(SimDyn), &p)) != 0) { usp_destroy(h); return rc; }
     h->d_dyn = (SimDyn*)p;
     s.dyn = h->d_dyn;
-    if ((rc = cell_alloc(h, 8 * sizeof(int), &p)) != 0) { usp_destroy(h); return rc; }
+    if ((rc = cell_alloc(h, kNTiles * sizeof(int), &p)) != 0) { usp_destroy(h); return rc; }
     h->d_ntiles = (int*)p;
     h->nctiles = (K + kCTile - 1) / kCTile;
     if ((rc = cell_alloc(h, sizeof(int2) * (size_t)h->nctiles, &p)) != 0) { usp_destroy(h); return rc; }
@@ -589,7 +596,7 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     s.inj_total = total;
     std::vector<int2> ct(h->nctiles);
     for (int t = 0; t < h->nctiles; ++t) ct[t] = make_int2(0, t * kCTile);
-    int nt[8] = {0, h->nctiles, 0, 0, 0, 0, 0, 0};
+    int nt[kNTiles] = {0, h->nctiles};
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.inj_count, h->inj_count_host.data(), sizeof(uint32_t) * K, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.inj_pidoff, off.data(), sizeof(uint32_t) * K, cudaMemcpyHostToDevice, h->stream);
@@ -1285,8 +1292,8 @@ extern "C" int usp_batch_create(size_t hbm_budget, int max_sims, void* stream, u
         b->own_stream = true;
     }
     if (cudaMalloc(&b->d_sims, sizeof(SimDev) * max_sims) != cudaSuccess ||
-        cudaMalloc(&b->d_ntiles, 8 * sizeof(int)) != cudaSuccess ||
-        cudaMemsetAsync(b->d_ntiles, 0, 8 * sizeof(int), b->stream) != cudaSuccess) {
+        cudaMalloc(&b->d_ntiles, kNTiles * sizeof(int)) != cudaSuccess ||
+        cudaMemsetAsync(b->d_ntiles, 0, kNTiles * sizeof(int), b->stream) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(b->d_sims);
         cudaFree(b->d_ntiles);
@@ -1382,6 +1389,7 @@ static uint64_t batch_key(const usp_batch* b) {
         if (s.slab_count > 1) k |= 4u;
         if (s.flux_axis) k |= 8u;
         if (s.selection || s.es_sampler) k |= 16u;
+        k |= 1ull << (24 + group_of(h));
         if (s.has_reservoir) k |= 32u;
         if (h->precision == USP_FP64) k |= 64u;             // an emptied batch may take another
         if (h->pipeline == USP_PIPE_FUSED) k |= 128u;       // precision or pipeline
@@ -1401,13 +1409,15 @@ static int batch_rebuild(usp_batch* b) {
         sims.push_back(h->host);
         for (int t = 0; t < h->nptiles; ++t) pt.push_back(make_int2((int)i, t * kPTile));
     }
-    // the cells of the 1-D members first: k_g2 has a kernel for each dimension
-    int nd[2] = {0, 0};
-    for (int dim = 1; dim <= 2; ++dim)
+    // the cells by group: k_g2 has a kernel for each
+    int gt[2 * kG2Groups] = {};
+    for (int g = 0; g < kG2Groups; ++g) {
+        gt[kG2Groups + g] = (int)ct.size();
         for (size_t i = 0; i < b->members.size(); ++i)
-            if (b->members[i]->host.dim == dim)
-                for (int t = 0; t < b->members[i]->nctiles; ++t, ++nd[dim - 1])
-                    ct.push_back(make_int2((int)i, t * kCTile));
+            if (group_of(b->members[i]) == g)
+                for (int t = 0; t < b->members[i]->nctiles; ++t) ct.push_back(make_int2((int)i, t * kCTile));
+        gt[g] = (int)ct.size() - gt[kG2Groups + g];
+    }
     // the slabs of a decomposed domain must sit consecutively, in slab order,
     // each one pointing at slab 0 of its group
     for (size_t i = 0; i < sims.size(); ++i) {
@@ -1462,7 +1472,7 @@ static int batch_rebuild(usp_batch* b) {
     if (e == cudaSuccess && !pt.empty()) e = cudaMemcpyAsync(b->d_ptiles, pt.data(), sizeof(int2) * pt.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess && !ct.empty()) e = cudaMemcpyAsync(b->d_ctiles, ct.data(), sizeof(int2) * ct.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ntiles, nt, sizeof(nt), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ntiles + 6, nd, sizeof(nd), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_ntiles + 2 + 2 * kG2Groups, gt, sizeof(gt), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, USP_ERR_CUDA, cudaGetErrorString(e));
     if (regraph) destroy_graphs(b->graphs);
@@ -1478,7 +1488,8 @@ static Launch batch_launch(usp_batch* b) {
     L.ctiles = b->d_ctiles;
     L.nctiles = b->d_ntiles + 1;
     L.wq = (uint32_t*)(b->d_ntiles + 2);
-    L.ndim = b->d_ntiles + 6;
+    L.gtiles = b->d_ntiles + 2 + 2 * kG2Groups;
+    L.groups = 0;
     L.nsims = (int)b->members.size();
     L.dims = 0;
     for (auto* h : b->members) L.dims |= h->host.dim == 1 ? 1 : 2;
@@ -1486,6 +1497,7 @@ static Launch batch_launch(usp_batch* b) {
         L.slabs |= h->host.slab_count > 1;
         L.flux |= h->host.flux_axis != 0;
         L.ablation |= h->host.selection || h->host.es_sampler;
+        L.groups |= 1 << group_of(h);
     }
     L.cells = 1 << 30;   // members come and go under a captured graph
     // fixed persistent grids: the tile counts are read on the device, so the

@@ -414,6 +414,41 @@ struct G2Fixed {
     float inv_thr;
 };
 
+// the digit of the rem-th smallest word among the counted ones (one warp; lane l
+// looks at digits [8 l, 8 l + 8)); below: how many words have a smaller digit
+__device__ __forceinline__ uint32_t radix_digit(const uint32_t* hist, uint32_t rem, int lane, uint32_t& below) {
+    uint32_t h[8], tot = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        h[i] = hist[8 * lane + i];
+        tot += h[i];
+    }
+    uint32_t inc = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const uint32_t exc = inc - tot;
+    const unsigned own = __ballot_sync(0xffffffffu, exc < rem && rem <= inc);
+    const int L = __ffs(own) - 1;
+    uint32_t d = 0;
+    below = exc;
+    if (lane == L) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (below + h[i] >= rem) {
+                d = 8u * lane + i;
+                break;
+            }
+            below += h[i];
+        }
+    }
+    d = __shfl_sync(0xffffffffu, d, L);
+    below = __shfl_sync(0xffffffffu, below, L);
+    return d;
+}
+
 // radix select of the ns-th smallest word: four passes of 8-bit digits
 // counted in shared memory, then the ties and T2; every pass draws the words
 // again
@@ -439,35 +474,8 @@ __device__ __noinline__ G2Fixed g2_fixed(G2Shared<G>& sh, int p, uint32_t step, 
             if ((k & mask) == prefix) atomicAdd(&sh.hist[(k >> shift) & 255u], 1u);
         }
         __syncthreads();
-        // every warp: lane l holds digits [8l, 8l + 8); the digit where the running count reaches rem
-        uint32_t h[8], tot = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            h[i] = sh.hist[8 * lane + i];
-            tot += h[i];
-        }
-        uint32_t inc = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const uint32_t exc = inc - tot;
-        const unsigned own = __ballot_sync(0xffffffffu, exc < rem && rem <= inc);
-        const int L = __ffs(own) - 1;
-        uint32_t d = 0, below = exc;
-        if (lane == L) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (below + h[i] >= rem) {
-                    d = 8u * lane + i;
-                    break;
-                }
-                below += h[i];
-            }
-        }
-        d = __shfl_sync(0xffffffffu, d, L);
-        below = __shfl_sync(0xffffffffu, below, L);
+        uint32_t below;
+        const uint32_t d = radix_digit(sh.hist, rem, lane, below);   // (every warp for itself)
         rem -= below;
         prefix |= d << shift;
         mask |= 0xFFu << shift;
@@ -881,16 +889,17 @@ __device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, in
 // ---------------------------------------------------------------------------
 constexpr int kG2wWarps = 4;    // warps per block
 
-template <int DIMS, int BLOCKS>   // BLOCKS per SM
+template <int DIMS, bool ABL, int BLOCKS>   // BLOCKS per SM
 struct alignas(16) G2Warp {
-    static constexpr uint32_t CAP = kG2Stage[BLOCKS - 3][DIMS - 1];   // staged particles
+    // staged particles (an ablation's larger window takes some of three blocks' space)
+    static constexpr uint32_t CAP = kG2Stage[BLOCKS - 3][DIMS - 1] - (ABL && BLOCKS == 3 ? 32u : 0u);
     float stage[(DIMS == 1 ? 5 : 6) * CAP + CAP / 2];                 // (x,) y, v0, v1, v2, id and 16-bit slots
     float prm[2][kNFPrm];  // parameter records of the cell and of the next one
     SimDev sim;
     uint32_t key[20];
-    uint32_t wst[kWin];    // arrivals per window slot, then its first reserved index
-    uint32_t wlo[kWin];    // start and end of the slot's bucket
-    uint32_t wend[kWin];
+    // per window slot: its arrivals, then its first reserved index; start and end
+    // of its bucket (before that the digit counts of a fixed-count selection)
+    uint32_t win[ABL ? 256 : 3 * kWin];
     int2 ptile[4];         // the cells on their way: tile,
     uint32_t pbound[4][4]; // bucket start, end and arrivals,
     uint32_t punit[4];     // unit number
@@ -901,6 +910,7 @@ struct alignas(16) G2Warp {
 // cell share a slot)
 constexpr uint32_t kPackNone = 0xFFFFu;   // removed, nothing to write
 constexpr uint32_t kPackFar = 0xFFFEu;    // outside the window
+constexpr uint32_t kPackOther = 0xFFFDu;  // in another slab of a decomposed domain
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -1045,11 +1055,91 @@ struct Num {
     static constexpr int value = V;
 };
 
+// the fixed count of one cell by one warp, its ids staged at J.ro or (GEN) read
+// from the bucket and the spill list.  f(j, word) for every particle j
+template <bool GEN, class Sh, class F>
+__device__ __forceinline__ void g2w_words(const Sh& sh, const G2Sim& S, const G2Job& J, uint32_t nsp, int lane,
+                                          const F& f) {
+    const SimDev& s = sh.sim;
+    const uint32_t* const st_id = reinterpret_cast<const uint32_t*>(sh.stage + 4 * Sh::CAP) + J.ro;
+    for (uint32_t j = lane; j < J.nb; j += 32)
+        f(j, philox_keys(GEN ? s.pid[S.p][J.base + j] : st_id[j], S.step, sh.key).x);
+    if (GEN && nsp)
+        each_spilled(s, S.p, J.cell, lane, [&](uint32_t rank, uint32_t i) {
+            f(J.nb + rank, philox_keys(s.sp_pid[S.p][i], S.step, sh.key).x);
+        });
+}
+
+template <bool GEN, class Sh>
+__device__ __noinline__ G2Fixed g2w_fixed(Sh& sh, G2Sim S, G2Job J, uint32_t nsp, float pr, int lane) {
+    const uint32_t n = J.nb + nsp;
+    G2Fixed F;
+    F.ns = min((uint32_t)floorf((float)n * pr + 0.5f), n);
+    F.T = 0xFFFFFFFFu;
+    F.quota = F.eq = 0;
+    F.inv_thr = 1.0f;
+    if (F.ns == 0) return F;
+    uint32_t prefix = 0, mask = 0, rem = F.ns;
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        __syncwarp();
+        for (int b = lane; b < 256; b += 32) sh.win[b] = 0u;
+        __syncwarp();
+        g2w_words<GEN>(sh, S, J, nsp, lane, [&](uint32_t, uint32_t k) {
+            if ((k & mask) == prefix) atomicAdd(&sh.win[(k >> shift) & 255u], 1u);
+        });
+        __syncwarp();
+        uint32_t below;
+        const uint32_t d = radix_digit(sh.win, rem, lane, below);
+        rem -= below;
+        prefix |= d << shift;
+        mask |= 0xFFu << shift;
+    }
+    F.T = prefix;
+    F.quota = rem;
+    // words equal to T, and the smallest word above it
+    uint32_t eq = 0, above = 0xFFFFFFFFu;
+    bool any_above = false;
+    g2w_words<GEN>(sh, S, J, nsp, lane, [&](uint32_t, uint32_t k) {
+        eq += k == F.T;
+        if (k > F.T) {
+            any_above = true;
+            above = min(above, k);
+        }
+    });
+    __syncwarp();
+    F.eq = __reduce_add_sync(0xffffffffu, eq);
+    above = __reduce_min_sync(0xffffffffu, above);
+    if (F.eq > F.quota) F.inv_thr = 1.0f / u01<float>(F.T);
+    else if (__any_sync(0xffffffffu, any_above)) F.inv_thr = 1.0f / u01<float>(above);
+    return F;
+}
+
+// is particle j with word x among the fixed count?  (one lane; as g2_fixed_takes)
+template <bool GEN, class Sh>
+__device__ __noinline__ bool g2w_fixed_takes(const Sh& sh, G2Sim S, G2Job J, G2Fixed X, uint32_t j, uint32_t x) {
+    if (X.ns == 0 || x > X.T) return false;
+    if (x < X.T || X.eq <= X.quota) return true;
+    const SimDev& s = sh.sim;
+    const uint32_t* const st_id = reinterpret_cast<const uint32_t*>(sh.stage + 4 * Sh::CAP) + J.ro;
+    uint32_t rank = 0;
+    for (uint32_t i = 0; i < min(j, J.nb); ++i)
+        rank += philox_keys(GEN ? s.pid[S.p][J.base + i] : st_id[i], S.step, sh.key).x == X.T;
+    if (GEN && j > J.nb) {
+        const uint32_t m = min(s.dyn->sp_n[S.p], (uint32_t)kSpillCap);
+        for (uint32_t i = 0, k = J.nb; i < m && k < j; ++i)
+            if (s.sp_cell[S.p][i] == (uint32_t)J.cell) {
+                rank += philox_keys(s.sp_pid[S.p][i], S.step, sh.key).x == X.T;
+                ++k;
+            }
+    }
+    return rank < X.quota;
+}
+
 // one cell.  GEN: loaded here, in chunks, with spill-list entries; else it is
 // staged at J.ro
-template <int DIM, int MODE, bool GEN, class Sh>
-__device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Job& J, uint32_t parity, uint32_t nsp,
-                                              int lane, G2Acc& acc) {
+template <int DIM, int MODE, bool ABL, bool GEN, class Sh>
+__device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, Sh& sh, const G2Sim& S, const G2Job& J,
+                                              uint32_t parity, uint32_t nsp, int lane, G2Acc& acc) {
     constexpr uint32_t CAP = Sh::CAP;
     const SimDev& s = sh.sim;
     const int p = S.p, q = p ^ 1, cell = J.cell;
@@ -1061,20 +1151,30 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
     uint32_t* const st_id = reinterpret_cast<uint32_t*>(st_2 + CAP);
     float* const st_x = st_2 + 2 * CAP;   // 2-D only
     uint16_t* const st_r = reinterpret_cast<uint16_t*>(st_2 + (DIM == 2 ? 3 : 2) * CAP);
+    G2Prm f = GEN ? g2_prm(s.fprm, cell) : g2_prm(sh.prm[parity], 0);
+    const bool relax = S.pending && f.pr > 0.0f;
+    if (MODE == kRelaxOnly && !relax) return;
+    G2Fixed X = {0u, 0u, 0u, 0u, 1.0f};
+    if (ABL && relax && s.selection) {
+        X = g2w_fixed<GEN>(sh, S, J, nsp, f.pr, lane);
+        f.inv_pr = X.inv_thr;   // the instants scale with the threshold word instead of P_relax
+        __syncwarp();
+    }
     // the window: lane k looks after slots k and k + 32, their bucket bounds read ahead
     const int cy = DIM == 2 ? cell / s.nx : 0;
     const int cx = DIM == 2 ? cell - cy * s.nx : 0;
+    const int gcell = cell + (MODE == kFullSlab && DIM == 1 ? s.row0 : 0);   // 1-D: global cell of the slab's cell
+    const int row0 = MODE == kFullSlab && DIM == 2 ? s.row0 : 0;
+    const int cell0 = MODE == kFullSlab ? s.row0 * s.nx : 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; MODE != kRelaxOnly && h < 2; ++h) {
         const int k = lane + 32 * h, dest = win_cell<DIM>(k, cell, cx, cy, s.nx);
         if ((unsigned)dest < (unsigned)s.K) {
-            cp_async4(&sh.wlo[k], &s.lay[q][dest]);
-            cp_async4(&sh.wend[k], &s.lay[q][dest + 1]);
+            cp_async4(&sh.win[kWin + k], &s.lay[q][dest]);
+            cp_async4(&sh.win[2 * kWin + k], &s.lay[q][dest + 1]);
         }
-        sh.wst[k] = 0;
+        sh.win[k] = 0;
     }
-    const G2Prm f = GEN ? g2_prm(s.fprm, cell) : g2_prm(sh.prm[parity], 0);
-    const bool relax = S.pending && f.pr > 0.0f;
     const uint32_t nch = GEN ? (n + CAP - 1) / CAP : 1u;
     float R[8];
 #pragma unroll
@@ -1130,12 +1230,19 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
 #pragma unroll
                 for (int t = 0; t < N; ++t) {
                     u[t] = u01<float>(w[t].x);
-                    sel[t] = b + 32 * t + lane < cnt && u[t] < f.pr;
+                    sel[t] = b + 32 * t + lane < cnt;
+                    if (ABL && s.selection)
+                        sel[t] = sel[t] && g2w_fixed_takes<GEN>(sh, S, J, X, off + b + 32 * t + lane, w[t].x);
+                    else
+                        sel[t] = sel[t] && u[t] < f.pr;
                     any = any || sel[t];
                 }
                 if (!__any_sync(0xffffffffu, any)) return;
 #pragma unroll
-                for (int t = 0; t < N; ++t) es_draw1(s, f, u[t], w[t], C[t]);
+                for (int t = 0; t < N; ++t) {
+                    if (ABL && s.es_sampler) es_draw_gt(s, f, u[t], w[t], C[t]);
+                    else es_draw1(s, f, u[t], w[t], C[t]);
+                }
 #pragma unroll
                 for (int t = 0; t < N; ++t) {
                     const uint32_t j = ro + b + 32 * t + lane;
@@ -1199,6 +1306,31 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                 }
             }
         }
+        if (MODE == kRelaxOnly) {   // the new velocities back in place
+            if (!apply) return;
+#pragma unroll 1
+            for (uint32_t b = lane; b < cnt; b += 32, selm >>= 1) {
+                if (!(selm & 1u)) continue;
+                const uint32_t j = ro + b;
+                st_0[j] = uo0 + al * (st_0[j] - mn0);
+                st_1[j] = uo1 + al * (st_1[j] - mn1);
+                st_2[j] = uo2 + al * (st_2[j] - mn2);
+                if (off + b >= nb) continue;
+                ((float*)s.vel[p][0])[base + off + b] = st_0[j];
+                ((float*)s.vel[p][1])[base + off + b] = st_1[j];
+                ((float*)s.vel[p][2])[base + off + b] = st_2[j];
+            }
+            __syncwarp();
+            if (GEN && off + cnt > nb)   // (entries not relaxed get back what they hold)
+                each_spilled(s, p, cell, lane, [&](uint32_t rank, uint32_t i) {
+                    const uint32_t j = nb + rank - off;
+                    if (j >= cnt) return;
+                    s.sp_vel[p][0][i] = st_0[j];
+                    s.sp_vel[p][1][i] = st_1[j];
+                    s.sp_vel[p][2][i] = st_2[j];
+                });
+            continue;
+        }
         if (GEN) {   // fewer than two relaxed particles in the cell: reverted
             if (!apply && __any_sync(0xffffffffu, selm)) {
                 __syncwarp();
@@ -1232,9 +1364,13 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                 ++acc.removed;
                 alive = false;
             }
-            const int slot = win_slot_xy<DIM>(ix, iy, cell, cx, cy);
+            if (MODE == kFullSlab && alive) {
+                const int dc = (DIM == 2 ? iy * s.nx + ix : iy) - cell0;
+                if ((unsigned)dc >= (unsigned)s.K) return kPackOther;
+            }
+            const int slot = win_slot_xy<DIM>(ix, iy - row0, gcell, cx, cy);
             uint32_t sr = alive ? kPackFar : kPackNone;
-            if (alive && slot >= 0) sr = (uint32_t)slot | (atomicAdd(&sh.wst[slot], 1u) << 6);
+            if (alive && slot >= 0) sr = (uint32_t)slot | (atomicAdd(&sh.win[slot], 1u) << 6);
             return sr;
         };
         auto fly = [&](auto nt, uint32_t b) {
@@ -1273,7 +1409,7 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                     for (int t = 0; t < N; ++t)
                         if ((x[t] - ps) * (xn[t] - ps) <= 0.0f) inside[t] = false;
                 }
-            if (MODE == kFullFlux && s.flux_axis) {
+            if ((MODE == kFullFlux || MODE == kFullSlab) && s.flux_axis) {
 #pragma unroll
                 for (int t = 0; t < N; ++t)
                     if (has[t] && inside[t]) count_flux<float>(s, x[t], y[t], xn[t], yn[t]);
@@ -1304,7 +1440,7 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
             const uint32_t j = ro + 32u * (uint32_t)(__ffs(slow) - 1) + lane;
             const float x = DIM == 2 ? st_x[j] : 0.0f, y = st_y[j];
             const AdvOut o = advect_slow(s, S.step, st_id[j], x, y, st_0[j], st_1[j], st_2[j]);
-            if (MODE == kFullFlux && s.flux_axis) count_flux<float>(s, x, y, o.x, o.y);
+            if ((MODE == kFullFlux || MODE == kFullSlab) && s.flux_axis) count_flux<float>(s, x, y, o.x, o.y);
             st_r[j] = (uint16_t)place(o.alive != 0, o.x, o.y);
             if (DIM == 2) st_x[j] = o.x;
             st_y[j] = o.y;
@@ -1318,9 +1454,9 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = lane + 32 * h;
-            const uint32_t c = sh.wst[k];
-            if (c) sh.wst[k] = sh.wlo[k] + atom_add_global(&s.cnt[q][win_cell<DIM>(k, cell, cx, cy, s.nx)], c);
-            sh.wend[k] = min(sh.wend[k], (uint32_t)s.cap);
+            const uint32_t c = sh.win[k];
+            if (c) sh.win[k] = sh.win[kWin + k] + atom_add_global(&s.cnt[q][win_cell<DIM>(k, cell, cx, cy, s.nx)], c);
+            sh.win[2 * kWin + k] = min(sh.win[2 * kWin + k], (uint32_t)s.cap);
         }
         // ---- sweep 3 ----
         float* const dx = (float*)s.pos[q][0];
@@ -1347,8 +1483,8 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
             }
 #pragma unroll
             for (int t = 0; t < N; ++t) {
-                i[t] = sh.wst[sr[t] & 63u] + (sr[t] >> 6);
-                in[t] = sr[t] < kPackFar && i[t] < sh.wend[sr[t] & 63u];
+                i[t] = sh.win[sr[t] & 63u] + (sr[t] >> 6);
+                in[t] = sr[t] < kPackOther && i[t] < sh.win[2 * kWin + (sr[t] & 63u)];
                 odd = odd || (!in[t] && sr[t] != kPackNone);
             }
             if (__any_sync(0xffffffffu, odd)) {   // not in the window, or the bucket is full
@@ -1358,7 +1494,7 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                 for (int t = 0; t < N; ++t) {   // reservations of their own, all in flight together
                     int ix, iy;
                     cell_xy<DIM>(s, x[t], y[t], ix, iy);
-                    dc[t] = DIM == 2 ? iy * s.nx + ix : iy;
+                    dc[t] = (DIM == 2 ? iy * s.nx + ix : iy) - cell0;
                     r[t] = lo[t] = hi[t] = 0;
                     if (sr[t] == kPackFar) {
                         r[t] = atom_add_global(&s.cnt[q][dc[t]], 1u);
@@ -1372,7 +1508,9 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
                         i[t] = lo[t] + r[t];
                         in[t] = i[t] < min(hi[t], (uint32_t)s.cap);
                     }
-                    if (!in[t] && sr[t] != kPackNone)
+                    if (MODE == kFullSlab && sr[t] == kPackOther)   // into the buckets of another slab
+                        emit_other<DIM>(sims, s, q, x[t], y[t], v[t][0], v[t][1], v[t][2], id[t]);
+                    else if (!in[t] && sr[t] != kPackNone)
                         spill<DIM>(s, q, dc[t], x[t], y[t], v[t][0], v[t][1], v[t][2], id[t]);
                 }
             }
@@ -1396,26 +1534,31 @@ __device__ __forceinline__ void g2w_cell_impl(Sh& sh, const G2Sim& S, const G2Jo
         }
         if (GEN && it + 1 < 2 * nch - 1) {   // the window of the next chunk
             __syncwarp();
-            sh.wst[lane] = 0;
-            sh.wst[lane + 32] = 0;
+            sh.win[lane] = 0;
+            sh.win[lane + 32] = 0;
         }
     }
     __syncwarp();
 }
 
-template <int DIM, int MODE, class Sh>
-__device__ __noinline__ G2Acc g2w_cell_general(Sh& sh, G2Sim S, G2Job J, int lane) {
+// a cell out of line: the general form, and the ablations' (inline their state
+// spills: the 200 x 200 cavity with the fixed count 338 us a step, 330 like this)
+template <int DIM, int MODE, bool ABL, bool GEN, class Sh>
+__device__ __noinline__ G2Acc g2w_cell_call(const SimDev* __restrict__ sims, Sh& sh, G2Sim S, G2Job J, uint32_t parity,
+                                            int lane) {
     G2Acc acc = {0u, 0u};
     uint32_t nsp = 0;
-    if (J.arrived > J.nb) nsp = each_spilled(sh.sim, S.p, J.cell, lane, [](uint32_t, uint32_t) {});
-    if (J.nb + nsp == 0) return acc;   // no bucket, and the spill list was full when its particles arrived
-    g2w_cell_impl<DIM, MODE, true>(sh, S, J, 0u, nsp, lane, acc);
+    if (GEN) {
+        if (J.arrived > J.nb) nsp = each_spilled(sh.sim, S.p, J.cell, lane, [](uint32_t, uint32_t) {});
+        if (J.nb + nsp == 0) return acc;   // no bucket, and the spill list was full when its particles arrived
+    }
+    g2w_cell_impl<DIM, MODE, ABL, GEN>(sims, sh, S, J, parity, nsp, lane, acc);
     return acc;
 }
 
 // DIMS 1 or 2: the dimension of every cell of the tiles *first .. *first +
 // *ntiles (first null: 0)
-template <int DIMS, int MODE, int BLOCKS>
+template <int DIMS, int MODE, bool ABL, int BLOCKS>
 __global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __restrict__ sims,
                                                                    const int2* __restrict__ tiles,
                                                                    const int* __restrict__ ntiles,
@@ -1423,7 +1566,8 @@ __global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __r
                                                                    uint32_t* __restrict__ wq) {
     extern __shared__ __align__(16) unsigned char g2_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    G2Warp<DIMS, BLOCKS>& sh = reinterpret_cast<G2Warp<DIMS, BLOCKS>*>(g2_smem)[warp];
+    using Sh = G2Warp<DIMS, ABL, BLOCKS>;
+    Sh& sh = reinterpret_cast<Sh*>(g2_smem)[warp];
     const SimDev& s = sh.sim;
     const uint32_t nunits = (uint32_t)*ntiles * kCTile;   // a unit is one cell slot of a tile
     if (first_tile) tiles += *first_tile;
@@ -1566,13 +1710,12 @@ __global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __r
             }
         }
         if (J.arrived) {
-            if (general) {
-                const G2Acc a = g2w_cell_general<DIMS, MODE>(sh, S, J, lane);
-                acc.relaxed += a.relaxed;
-                acc.removed += a.removed;
-            } else {
-                g2w_cell_impl<DIMS, MODE, false>(sh, S, J, par, 0u, lane, acc);
-            }
+            G2Acc a = {0u, 0u};
+            if (general) a = g2w_cell_call<DIMS, MODE, ABL, true>(sims, sh, S, J, 0u, lane);
+            else if (ABL) a = g2w_cell_call<DIMS, MODE, ABL, false>(sims, sh, S, J, par, lane);
+            else g2w_cell_impl<DIMS, MODE, ABL, false>(sims, sh, S, J, par, 0u, lane, acc);
+            acc.relaxed += a.relaxed;
+            acc.removed += a.removed;
             fence_proxy_async_smem();   // later copies come after these accesses
             __syncwarp();
         }
@@ -2533,48 +2676,68 @@ void launch_g2b_one(const Launch& L) {
     k_g2b<DIMS, MODE, ABL, G><<<grid, 32 * G, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles, L.wq);
 }
 
-template <int DIMS, int MODE, int BLOCKS>
-void launch_g2_blocks(const Launch& L, cudaStream_t st, bool part) {
+template <int DIMS, int MODE, bool ABL, int BLOCKS>
+void launch_g2_blocks(const Launch& L, int group, cudaStream_t st) {
     static int wave = 0;
-    constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS, BLOCKS>));
+    constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS, ABL, BLOCKS>));
     if (!wave) {
         int dev = 0, sms = 152, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_g2<DIMS, MODE, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE, BLOCKS>, 32 * kG2wWarps, smem);
+        cudaFuncSetAttribute(k_g2<DIMS, MODE, ABL, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE, ABL, BLOCKS>, 32 * kG2wWarps, smem);
         wave = sms * std::max(per, 1);
     }
     const int grid = std::max(1, std::min(wave, (L.cells + kG2wWarps - 1) / kG2wWarps));
-    const int* n = part ? (DIMS == 1 ? L.ndim : L.ndim + 1) : L.nctiles;
-    k_g2<DIMS, MODE, BLOCKS><<<grid, 32 * kG2wWarps, smem, st>>>(L.sims, L.ctiles, n, part && DIMS == 2 ? L.ndim : nullptr,
-                                                         DIMS == 1 ? L.wq : L.wq + 2);
+    k_g2<DIMS, MODE, ABL, BLOCKS><<<grid, 32 * kG2wWarps, smem, st>>>(
+        L.sims, L.ctiles, L.gtiles ? L.gtiles + group : L.nctiles, L.gtiles ? L.gtiles + kG2Groups + group : nullptr,
+        L.wq + 2 * group);
 }
 
-template <int DIMS, int MODE>
-void launch_g2_one(const Launch& L, cudaStream_t st, bool part) {
-    if (L.g2_blocks == 3) launch_g2_blocks<DIMS, MODE, 3>(L, st, part);
-    else launch_g2_blocks<DIMS, MODE, 4>(L, st, part);
+template <int DIMS, int MODE, bool ABL>
+void launch_g2_one(const Launch& L, int group, cudaStream_t st) {
+    if constexpr (MODE != kRelaxOnly) {
+        if (L.g2_blocks == 3) return launch_g2_blocks<DIMS, MODE, ABL, 3>(L, group, st);
+    }
+    launch_g2_blocks<DIMS, MODE, ABL, 4>(L, group, st);
 }
 
-// A mixed batch runs the kernels of both dimensions side by side (one kernel
-// with both bodies overflows the instruction cache where a block's warps are
-// in different ones): the 2-D one on the second stream, its blocks following
-// as those of the 1-D one finish.
+// the cells of one group (g2_group).  The ablations' kernel counts the flux too,
+// and the one that relaxes in place holds the ablations' code.
+template <int MODE>
+void launch_g2_group(const Launch& L, int group, cudaStream_t st) {
+    constexpr int M = MODE == kFull ? kFullFlux : MODE;
+    const bool abl = MODE == kRelaxOnly || (group & 1);
+    if (group < 2) {
+        if (abl) return launch_g2_one<1, M, true>(L, group, st);
+        if constexpr (MODE != kRelaxOnly) launch_g2_one<1, MODE, false>(L, group, st);
+    } else {
+        if (abl) return launch_g2_one<2, M, true>(L, group, st);
+        if constexpr (MODE != kRelaxOnly) launch_g2_one<2, MODE, false>(L, group, st);
+    }
+}
+
+// A mixed batch runs the kernels of its groups side by side: one kernel with the
+// bodies of both dimensions overflows the instruction cache where a block's warps
+// are in different ones, and one that holds the ablations' code too costs the
+// other cells a sixth (64 shock tubes 325 -> 380 us a step).  One group of
+// ordinary cells takes the step's stream; the others follow on the second one,
+// an ablation's cells (few, and slow) before the rest, and their blocks run
+// where those of the first are done.
 template <int MODE>
 void launch_g2(const Launch& L) {
-    if (L.dims == 1) {
-        launch_g2_one<1, MODE>(L, L.stream, false);
-    } else if (L.dims == 2) {
-        launch_g2_one<2, MODE>(L, L.stream, false);
-    } else if (!L.side) {
-        launch_g2_one<1, MODE>(L, L.stream, true);
-        launch_g2_one<2, MODE>(L, L.stream, true);
-    } else {
+    constexpr int order[kG2Groups] = {1, 3, 0, 2};   // the ablations' first
+    int main = -1;
+    for (int g : {0, 2, 1, 3})
+        if (main < 0 && (L.groups >> g & 1)) main = g;
+    const bool fork = L.side && (L.groups & (L.groups - 1));
+    if (fork) {
         cudaEventRecord(L.ev_fork, L.stream);
         cudaStreamWaitEvent(L.side, L.ev_fork, 0);
-        launch_g2_one<1, MODE>(L, L.stream, true);
-        launch_g2_one<2, MODE>(L, L.side, true);
+    }
+    for (int g : order)
+        if (L.groups >> g & 1) launch_g2_group<MODE>(L, g, fork && g != main ? L.side : L.stream);
+    if (fork) {
         cudaEventRecord(L.ev_join, L.side);
         cudaStreamWaitEvent(L.stream, L.ev_join, 0);
     }
@@ -2594,18 +2757,16 @@ void launch_g2b(const Launch& L) {
 // R (tuning): 4 one warp per cell, 8 and 12 a block of 4 or 8 warps
 template <int MODE>
 void launch_g2_R(const Launch& L, int R) {
-    if (L.ablation) {
+    if (R <= 4) {
+        launch_g2<MODE>(L);
+    } else if (L.ablation) {
         launch_g2b<MODE, true, 4>(L);
     } else if constexpr (MODE == kRelaxOnly || MODE == kFullSlab) {
         launch_g2b<MODE, false, 4>(L);
+    } else if (R <= 8) {
+        launch_g2b<MODE, false, 4>(L);
     } else {
-        if (R <= 4) {
-            launch_g2<MODE>(L);
-        } else if (R <= 8) {
-            launch_g2b<MODE, false, 4>(L);
-        } else {
-            launch_g2b<MODE, false, 8>(L);
-        }
+        launch_g2b<MODE, false, 8>(L);
     }
 }
 

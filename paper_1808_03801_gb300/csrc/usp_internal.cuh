@@ -209,14 +209,20 @@ template <> __device__ __forceinline__ float dev_floor<float>(float x) { return 
 // -------------------------------------------------------------------------
 // launch helpers (defined in usp_kernels.cu)
 // -------------------------------------------------------------------------
+// k_g2 has kernels for each dimension, and for the ablations (fixed count,
+// Gallis-Torczynski): the group of a simulation's cells
+constexpr int kG2Groups = 4;
+constexpr int g2_group(int dim, bool ablation) { return 2 * (dim - 1) + (ablation ? 1 : 0); }
+
 struct Launch {
     const SimDev* sims;   // device array
     const int2* ptiles;   // (sim, first particle slot) tiles
     const int* nptiles;   // device scalar
     const int2* ctiles;   // (sim, first cell) tiles
     const int* nctiles;   // device scalar
-    uint32_t* wq;         // k_g2: units handed out and blocks done, for each dimension (zero between launches)
-    const int* ndim;      // device: 1-D and 2-D cell tiles of a batch (the 1-D ones come first)
+    uint32_t* wq;         // k_g2: units handed out and blocks done, for each group (zero between launches)
+    const int* gtiles;    // device: a batch's cell tiles by group (g2_group): how many, then the first of each
+    int groups;           // groups that have cells (bits)
     int nsims;
     int dims;             // bit 0: some simulation is 1-D, bit 1: some is 2-D
     int slabs = 0;        // some simulation is a slab of a decomposed domain

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 from paper_1808_03801_gb300 import workloads as W
-from tests._util import KB_M_AR, assert_particles_close
+from tests._util import KB_M_AR, assert_particles_close, by_pid
 
 pytestmark = pytest.mark.gpu
 
@@ -67,4 +67,41 @@ def test_batch_refilled_with_members_of_another_kind(usp, first, second):
         assert a["counters"][7] == b["counters"][7]
         assert_particles_close(s.particles(), alone.particles(), VSCALE, dy, rtol=rtol, check_cells=False)
         assert np.array_equal(s.sample()[15], alone.sample()[15])
+    B.close()
+
+
+def test_batch_of_every_kind_steps_as_each_alone(usp):
+    """1-D and 2-D members with and without ablations, more cells in all than
+    the block-per-cell form is used for: one kernel for each kind, side by side.
+    Three steps; a particle within rounding of a face or of a selection may change
+    its cells: three cells of a member at most."""
+    def workloads(seed):
+        out = [W.sod(ny=1000, ppc_left=80, seed=seed), W.couette(ny=700, ppc=60, seed=seed),
+               W.cavity(n=25, ppc=40, Kn=0.05, seed=seed), W.poiseuille(ny=60, ppc=90, seed=seed),
+               W.cavity(n=20, ppc=50, Kn=0.05, seed=seed), W.slit(nx=40, ny=20, ppc=30, seed=seed)]
+        out = [W.with_precision(w, "fp32") for w in out]
+        for w in out:
+            w["params"]["pipeline"] = "fused"
+        out[3]["params"]["selection"] = "fixed_count"
+        out[4]["params"].update(mode="spesbgk", es_sampler="gallis_torczynski")
+        return out
+
+    ws = workloads(31)
+    states = [usp.Simulation(w).init_particles().particles() for w in ws]
+    sims = [usp.Simulation(w).set_particles(P["pos"], P["vel"], P["pid"]) for w, P in zip(ws, states)]
+    alone = [usp.Simulation(w).set_particles(P["pos"], P["vel"], P["pid"]) for w, P in zip(ws, states)]
+    assert sum(s.K for s in sims) > 1520 and all(s.tuning()["fused_R"] > 4 for s in alone)
+    B = usp.Batch(hbm_budget=4 << 30, max_sims=len(ws))
+    for s in sims:
+        assert B.admit(s) == 0
+    B.step(3)
+    for s, a in zip(sims, alone):
+        B.retire(s)
+        a.step(3)
+        assert s.info()["counters"][5] == 0
+        assert abs(s.info()["counters"][4] - a.info()["counters"][4]) <= 3 * 100
+        P, Q = (by_pid(x.particles()) for x in (s, a))
+        assert np.array_equal(P["pid"], Q["pid"])
+        bad = np.abs(P["vel"] - Q["vel"]).max(1) > 1e-4 * VSCALE
+        assert len(set(Q["cell"][bad].tolist())) <= 3, (s.w["params"], bad.sum())
     B.close()

@@ -174,3 +174,32 @@ def test_density_jump_at_a_slab_boundary(env):
     assert dec.counters()[5] == 0 and np.array_equal(np.sort(Q["pid"]), np.sort(P["pid"]))
     assert np.array_equal(np.bincount(Q["cell"], minlength=1000), dec.sample()[15].astype(np.int64))
     dec.close()
+
+
+@pytest.mark.parametrize("name,nslabs", [("column", 4), ("cavity", 3)])
+def test_slabs_of_many_cells(env, name, nslabs):
+    """Domains above the cells that the block-per-cell form is used for: the
+    slabs step with a warp per cell.  One step as the whole domain's; particles
+    and cells consistent after more."""
+    U, D = env
+    if name == "column":
+        w = _fused(W.homogeneous_column(ny=2000, ppc=30, Kn=1.0, dt_over_tauc=1.0))
+    else:
+        w = _fused(W.cavity(n=42, ppc=30, Kn=0.05, seed=3))
+    P = U.Simulation(w).init_particles().particles()
+    whole = U.Simulation(w).set_particles(P["pos"], P["vel"], P["pid"])
+    assert whole.tuning()["fused_R"] == 4
+    dec = D.DecomposedSim(w, nslabs).load(P)
+    whole.step(1)
+    dec.step(1)
+    a, b = by_pid(whole.particles()), by_pid(dec.particles())
+    for k in ("pid", "pos", "cell"):
+        assert np.array_equal(a[k], b[k]), k
+    assert np.max(np.abs(a["vel"] - b["vel"])) < 1e-4 * np.sqrt(np.mean(a["vel"] ** 2))
+    dec.step(20)
+    N = dec.sample()[15].astype(np.int64)
+    Q = dec.particles()
+    assert dec.counters()[5] == 0 and dec.counters()[4] > 0
+    assert np.array_equal(np.sort(Q["pid"]), np.sort(P["pid"]))
+    assert np.array_equal(np.bincount(Q["cell"], minlength=len(N)), N)
+    dec.close()

@@ -124,6 +124,40 @@ def test_fused_warp_per_cell_staging(usp, dim, ppc_ref, reach):
     assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
 
 
+@pytest.mark.parametrize("ablation", [{"selection": "fixed_count"}, {"mode": "spesbgk", "es_sampler": "gallis_torczynski"},
+                                      {"selection": "fixed_count", "mode": "spesbgk", "es_sampler": "gallis_torczynski"}])
+@pytest.mark.parametrize("ppc_ref", [360, 500])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_fused_ablations_warp_per_cell(usp, dim, ppc_ref, ablation):
+    """The ablations with a warp per cell (four and three blocks per SM)
+    against blocks of four warps, at one collision time, so that the fixed count
+    takes a part of each cell; cells of several chunks and with spill-list
+    entries among them."""
+    counts = EDGES + EDGES[::-1] if dim == 1 else EDGES
+    n = len(counts)
+    for reach in (0.02, 1.0):
+        if dim == 1:
+            w = W.homogeneous_column(ny=n, ppc=360, Kn=reach, dt_over_tauc=1.0, precision="fp32")
+        else:
+            w = W.cavity(n=math.isqrt(n), ppc=360, Kn=reach / math.isqrt(n), dt_over_tauc=1.0)
+        w["params"].update(ablation, pipeline="fused", ppc_ref=ppc_ref)
+        bad = []
+        for seed in (16, 17):
+            st = _state(w, counts, seed)
+            P = []
+            for R in (4, 8):
+                g = usp.Simulation(w).set_particles(*st).set_tuning(fused_R=R).step(3)
+                assert g.info()["counters"][5] == 0 and 0 < g.info()["counters"][4] < 2 * len(st[2])
+                N = g.sample()[15]
+                P.append(by_pid(g.particles()))
+                assert np.array_equal(P[-1]["pid"], np.arange(len(st[2]), dtype=np.uint32))
+                assert np.array_equal(np.bincount(P[-1]["cell"], minlength=n), N.astype(np.int64))
+                g.close()
+            d = np.abs(P[0]["vel"] - P[1]["vel"]).max(1) > 1e-4 * VSCALE
+            bad.append(set(P[1]["cell"][d].tolist()))
+        assert max(map(len, bad)) <= 3 and not bad[0] & bad[1], (reach, bad)
+
+
 @pytest.mark.parametrize("R", [4, 12])
 def test_fused_cells_with_long_spill_lists(usp, R):
     """Cells of 16 and 1500 particles side by side at reach 1: hundreds go to
