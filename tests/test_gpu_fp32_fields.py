@@ -103,13 +103,15 @@ def oracle_means():
     return {c: np.array(v) for c, v in out.items()}
 
 
-def _gpu_means(usp, name):
+def _gpu_means(usp, name, R=0):
     out = []
     for seed in SEEDS_GPU:
         w, steps, t0 = _case(name, seed)
         w = W.with_precision(w, "fp32")
         w["params"]["pipeline"] = "fused"
         g = usp.Simulation(w).init_particles()
+        if R:
+            g.set_tuning(fused_R=R)
         g.step(t0)
         acc = None
         for _ in range(steps - t0):
@@ -136,6 +138,13 @@ def test_fp32_fields_within_three_standard_errors(usp, oracle_means, name):
         cur[name] = rows
         json.dump(cur, open(report, "w"), indent=1)
     assert_fields_agree(rows, name)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["sod", "couette"])
+def test_fp32_fields_with_a_warp_per_cell(usp, oracle_means, name):
+    """The 1-D cases in the form that larger domains and batches take."""
+    assert_fields_agree(compare(_gpu_means(usp, name, R=4), oracle_means[name]), name)
 
 
 def test_compare_detects_a_one_standard_error_bias():

@@ -173,6 +173,30 @@ def test_fused_cells_with_long_spill_lists(usp, R):
     assert max(map(len, sets)) <= 3 and not sets[0] & sets[1], sets
 
 
+@pytest.mark.parametrize("selection", ["bernoulli", "fixed_count"])
+@pytest.mark.parametrize("R", [4, 8, 12])
+@pytest.mark.parametrize("dim", [1, 2])
+def test_fused_counting_plane_in_every_form(usp, dim, R, selection):
+    """Net flow through a plane in closed walls: the particles at or above it
+    after each step less those before."""
+    w = W.couette(ny=30, ppc=80, dt_over_tauc=3.0) if dim == 1 else W.cavity(n=12, ppc=40, Kn=0.05)
+    w = W.with_precision(w, "fp32")
+    w["params"].update(pipeline="fused", selection=selection, flux_axis=2, flux_pos=0.37 * w["grid"]["hi"][1])
+    g = usp.Simulation(w).init_particles().set_tuning(fused_R=R)
+    plane = np.float32(w["params"]["flux_pos"])
+
+    def above():
+        return int(np.sum(g.particles()["pos"][:, 1].astype(np.float32) >= plane))
+
+    before, counted = above(), 0
+    for _ in range(4):
+        g.step(2)
+        now = above()
+        assert g.info()["counters"][7] - counted == now - before
+        counted, before = g.info()["counters"][7], now
+    assert g.info()["counters"][5] == 0
+
+
 @pytest.mark.parametrize("ncells", [1, 8191, 8192, 8193])
 def test_fused_layout_on_both_sides_of_the_one_kernel_limit(usp, ncells):
     w = _domain(1, ncells, 16, 0.02)
