@@ -286,13 +286,13 @@ static void enqueue_fused_step(const Launch& L, int R, bool reservoir) {
         Ls.stream = L.side;
         launch_fused_layout_parts(Ls);
         cudaEventRecord(L.ev_join, L.side);
-        launch_fused_moments(L, R);
+        launch_fused_moments(L);
         launch_fused_params(L);
         cudaStreamWaitEvent(L.stream, L.ev_join, 0);
         launch_fused_step_end(L);
         return;
     }
-    launch_fused_moments(L, R);
+    launch_fused_moments(L);
     launch_fused_params(L);
     launch_fused_layout(L);   // ends the step too
 }
@@ -541,7 +541,7 @@ extern "C" int usp_create(const usp_gas* gas, const usp_grid* grid, const usp_bc
     CALLOC(inj_pidoff, uint32_t, K);
     CALLOC(fprm, float, (size_t)kNFPrm * K);
     if (prm->gll_average && prm->pipeline == USP_PIPE_PLAIN) { CALLOC(gavg, double, 3 * (size_t)K); }
-    if (prm->pipeline == USP_PIPE_PLAIN) { CALLOC(gloc, double, 6 * (size_t)K); }
+    if (prm->pipeline == USP_PIPE_PLAIN) { CALLOC(gloc, double, 4 * (size_t)K); }
     if (prm->weighted) {
         CALLOC(wneff, double, K);
         CALLOC(wst, double, 9 * (size_t)K);
@@ -973,7 +973,7 @@ static int stage_launch(const Launch& L, int pipeline, bool fp64, int R, bool re
         switch (stage) {
         case 10: launch_fused_relax_stream(L, R, false); return 0;
         case 11: if (reservoir) launch_fused_inject(L); return 0;
-        case 12: launch_fused_moments(L, R); return 0;
+        case 12: launch_fused_moments(L); return 0;
         case 13: launch_fused_params(L); return 0;
         case 14: launch_fused_layout(L); return 0;   // layout + end of step
         default: return -1;

@@ -12,12 +12,13 @@
 //   k_g1      per cell (one warp): moments of Eq. 1 in one pass, as sums
 //             about the cell's mean velocity of the previous step, and the
 //             cell's n, T, |u| for its neighbours' Kn_GLL.
-//   k_params  per cell: Kn_GLL and P_ne (Eqs. 16-18), sigma* and q* (Eq. 33),
+//   k_params_f  per cell: Kn_GLL and P_ne (Eqs. 16-18), sigma* and q* (Eq. 33),
 //             the Cholesky factor of the ES covariance (Eq. 6c), the fields
 //             and the average of Eq. 34.
-//   k_layout  per simulation: histogram -> bucket sizes -> exclusive scan,
-//             the layout that the next step writes with; then the end of
-//             the step (swap buffers, advance the step).
+//   k_lay_small, or k_lay_sum, k_lay_scan and k_lay_put in larger domains:
+//             histogram -> bucket sizes -> exclusive scan, the layout that
+//             the next step writes with (beside k_g1 and k_params_f).
+//   k_step_end  per simulation: swap buffers, advance the step.
 // All arithmetic of a step is FP32 except the number density and the Eq. 34
 // running averages (FP64, in k_params_f).  FP64 issue rate is scarce on
 // GB300 (about two FP64 FMA per clock per SM).  The moments are sums about
@@ -644,8 +645,7 @@ __device__ __forceinline__ void g2_cell(const SimDev* __restrict__ sims, G2Share
             if ((lane & 3) == 0) sh.part[warp][lane >> 2] = R[0];
             if (lane == 0) sh.part_n[warp] = nr;
             __syncthreads();
-            float t = 0.0f;
-            if (G >= 4 || lane < 8 * G) t = sh.part[lane >> 3][lane & 7];
+            float t = sh.part[lane >> 3][lane & 7];
 #pragma unroll
             for (int g = 4; g < G; g += 4) t += sh.part[g + (lane >> 3)][lane & 7];
             t += __shfl_xor_sync(0xffffffffu, t, 8);
@@ -1738,12 +1738,11 @@ __global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __r
 // k_g1: per-cell moments (Eq. 1) in one pass, as sums of C = c - u_s about a
 // shift u_s: the cell's mean velocity of the previous step (the parameters
 // of that step, still in fprm).  The mean moves little in one step, so the
-// FP32 sums of the centred velocities do not cancel; k_params_f promotes
-// them to FP64 with the shift taken into account.
+// FP32 sums of the centred velocities do not cancel; k_params_f forms the
+// state from them in FP32 with the shift taken into account.
 // ---------------------------------------------------------------------------
 constexpr int kG1Warps = 4;     // warps per block; a block takes one 32-cell tile at a time
 constexpr int kG1Stage = 384;   // slots of one pipeline stage (a multiple of 4)
-constexpr int kG1Units = 1;     // units per block wanted
 
 __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__ sims, const int2* __restrict__ tiles,
                                                      const int* __restrict__ ntiles) {
@@ -1755,14 +1754,14 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
     __shared__ __align__(16) float stage[kG1Warps][2][3][kG1Stage];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ SimDev sim_sh;
-    // A unit is a whole tile or, until every block has kG1Units of them, a
+    // A unit is a whole tile or, until every block has one, a
     // half, quarter or eighth of one (down to one cell per warp), so that few
     // cells spread over all SMs: one shock tube of 1000 cells 16.6 -> 8.9 us.
     // More units than blocks cost what the next cell's copy ahead gains
-    // (cavity 200 x 200: 34 us with 1, 37 / 42 / 54 us with 2 / 4 / 8).
+    // (cavity 200 x 200: 34 us with one per block, 37 / 42 / 54 us with 2 / 4 / 8).
     const int nt = *ntiles;
     int parts = 1;
-    while (parts < kCTile / kG1Warps && nt * parts < kG1Units * (int)gridDim.x) parts *= 2;
+    while (parts < kCTile / kG1Warps && nt * parts < (int)gridDim.x) parts *= 2;
     const int ncell = kCTile / parts;   // cells of a unit
     int loaded = -1;
     for (int t = blockIdx.x; t < nt * parts; t += gridDim.x) {
@@ -1882,9 +1881,7 @@ __global__ void __launch_bounds__(32 * kG1Warps) k_g1(const SimDev* __restrict__
             // of its values and adds the partner's copy of that half (16
             // shuffles instead of 60 for twelve butterfly sums); lane 2v then
             // holds entry v of the record and writes it.  N and u_s come from
-            // lane 0 alone.  FP32 sums only: their promotion to FP64 happens in
-            // k_params_f, one cell per thread (an FP64 instruction costs the
-            // same for one lane).
+            // lane 0 alone.
             float v[16];
             v[0] = lane == 0 ? (float)n : 0.0f;
 #pragma unroll
@@ -2291,9 +2288,9 @@ __global__ void __launch_bounds__(256) k_inject_f(const SimDev* __restrict__ sim
 }
 
 // ---------------------------------------------------------------------------
-// k_layout: histogram -> bucket sizes (slack for arrivals) -> exclusive scan
-// setup == true builds the write layout of buffer cur ^ 1 right after the
-// initial fill (counts of buffer cur from the exact start offsets).
+// k_layout: histogram -> bucket sizes (slack for arrivals) -> exclusive scan, the
+// write layout of buffer cur ^ 1 right after the initial fill (counts of buffer
+// cur from the exact start offsets)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t bucket_size(const SimDev& s, const uint32_t* cnt, int c) {
     const int ix = c % s.nx, iy = c / s.nx;
@@ -2312,7 +2309,6 @@ __device__ __forceinline__ uint32_t bucket_size(const SimDev& s, const uint32_t*
     return (m + (m >> 2) + 16u + (s.has_reservoir ? s.inj_count[c] : 0u) + 3u) & ~3u;
 }
 
-template <bool SETUP>
 __global__ void __launch_bounds__(1024) k_layout(const SimDev* __restrict__ sims, int nsims) {
     __shared__ uint32_t warp_sums[32];
     __shared__ unsigned long long tot_full, tot_exact;
@@ -2322,16 +2318,13 @@ __global__ void __launch_bounds__(1024) k_layout(const SimDev* __restrict__ sims
         SimDyn* dyn = s.dyn;
         const int K = s.K;
         const int cur = dyn->cur;
-        const int src = SETUP ? cur : cur ^ 1;   // counts of the freshly written buffer
-        const int dst = SETUP ? cur ^ 1 : cur;   // layout for the next write
-        if (SETUP) {
-            for (int c = threadIdx.x; c <= K; c += blockDim.x) {
-                s.lay[cur][c] = s.start[c];
-                if (c < K) s.cnt[cur][c] = s.start[c + 1] - s.start[c];
-            }
-            __syncthreads();
+        const int dst = cur ^ 1;   // layout for the next write
+        for (int c = threadIdx.x; c <= K; c += blockDim.x) {
+            s.lay[cur][c] = s.start[c];
+            if (c < K) s.cnt[cur][c] = s.start[c + 1] - s.start[c];
         }
-        const uint32_t* C = s.cnt[src];
+        __syncthreads();
+        const uint32_t* C = s.cnt[cur];
         if (threadIdx.x == 0) {
             tot_full = 0;
             tot_exact = 0;
@@ -2394,25 +2387,12 @@ __global__ void __launch_bounds__(1024) k_layout(const SimDev* __restrict__ sims
         }
         if (threadIdx.x == 0) {
             s.lay[dst][K] = carry;
-            if (!SETUP) dyn->n = (uint32_t)min(tot_exact, (unsigned long long)0xFFFFFFFFu);
             dyn->sp_n[dst] = 0;
-            if (SETUP) {
-                dyn->sp_n[cur] = 0;
-                dyn->relax_pending = 0;
-            }
+            dyn->sp_n[cur] = 0;
+            dyn->relax_pending = 0;
         }
         for (int c = threadIdx.x; c < K; c += blockDim.x) s.cnt[dst][c] = 0;
         __syncthreads();
-        if (!SETUP && threadIdx.x == 0) {   // end of the step (every thread has read cur)
-            if (s.has_reservoir) {
-                dyn->next_pid += s.inj_total;
-                dyn->counters[kCntInjected] += s.inj_total;
-            }
-            dyn->cur ^= 1;
-            dyn->step += 1;
-            dyn->nsamples += 1;
-            dyn->relax_pending = 1;
-        }
     }
 }
 
@@ -2651,9 +2631,8 @@ __global__ void __launch_bounds__(kLayTile) k_lay_put(const SimDev* __restrict__
     }
 }
 
-// end of a fused step (mode 0) or after a flush of the pending relaxation (mode 1)
 // clears the pending relaxation once it has been applied in place before a
-// read-back (the end of a step is part of k_layout)
+// read-back
 __global__ void k_clear_pending(const SimDev* __restrict__ sims, int nsims) {
     for (int si = blockIdx.x * blockDim.x + threadIdx.x; si < nsims; si += gridDim.x * blockDim.x)
         sims[si].dyn->relax_pending = 0;
@@ -2772,7 +2751,7 @@ void launch_g2_R(const Launch& L, int R) {
 
 }  // namespace
 
-void launch_fused_setup(const Launch& L) { k_layout<true><<<L.nsims, 1024, 0, L.stream>>>(L.sims, L.nsims); }
+void launch_fused_setup(const Launch& L) { k_layout<<<L.nsims, 1024, 0, L.stream>>>(L.sims, L.nsims); }
 
 void launch_fused_relax_stream(const Launch& L, int R, bool flush_only) {
     if (flush_only) {
@@ -2790,8 +2769,7 @@ void launch_fused_inject(const Launch& L) {
     if (L.dims & 2) k_inject_f<2><<<L.grid_c, 256, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 
-void launch_fused_moments(const Launch& L, int R) {
-    (void)R;
+void launch_fused_moments(const Launch& L) {
     k_g1<<<L.grid_f, 32 * kG1Warps, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 

@@ -106,7 +106,7 @@ struct alignas(16) SimDev {
     double* avg;          // kNFields x K
     double* ushift;       // 3 x K, previous mean velocity (shift of the sums)
     double* gavg;         // 3 x K, averaged n, T, |u| at the start of the step (plain pipeline, gll_average)
-    double* gloc;         // 6 x K, each cell's stencil state (valid, n, T, |u|, a, lambda) of this step (plain)
+    double* gloc;         // 4 x K, each cell's stencil state (valid, n, T, |u|) of this step (plain)
     uint32_t* inj_count;  // K (buffer cells only)
     uint32_t* inj_pidoff; // K
     uint32_t inj_total;
@@ -275,7 +275,7 @@ void launch_zero(const ZeroList& z, cudaStream_t st);
 void launch_fused_setup(const Launch& L);
 void launch_fused_relax_stream(const Launch& L, int R, bool flush_only);
 void launch_fused_inject(const Launch& L);
-void launch_fused_moments(const Launch& L, int R);
+void launch_fused_moments(const Launch& L);
 void launch_fused_params(const Launch& L);
 void launch_fused_layout(const Launch& L);
 void launch_fused_layout_parts(const Launch& L);

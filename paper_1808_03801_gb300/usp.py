@@ -158,7 +158,9 @@ def stage_list(pipeline: str):
 
 
 def launches_per_step(pipeline: str, reservoir: bool = False, cells: int | None = None) -> int:
-    """Kernels of one step; `cells`: of the largest simulation (None: a domain above the one-kernel layout)."""
+    """Kernels of one step; `cells`: of the largest simulation (None: a domain above the one-kernel layout).  A
+    fused batch of many cells runs one more for each further kind of members (1-D and 2-D, with and without the
+    SP-ESBGK ablations)."""
     one = pipeline == "fused" and cells is not None and cells <= _LAYOUT_ONE_KERNEL
     return _LAUNCHES[pipeline] + (1 if reservoir else 0) - (2 if one else 0)
 
