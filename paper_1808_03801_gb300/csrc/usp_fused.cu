@@ -2641,32 +2641,37 @@ __global__ void k_clear_pending(const SimDev* __restrict__ sims, int nsims) {
 // ---------------------------------------------------------------------------
 // k_g2 launch configuration: one wave of resident blocks
 // ---------------------------------------------------------------------------
+static int sm_count() {
+    static const int sms = [] {
+        int dev = 0, n = 152;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return n;
+    }();
+    return sms;
+}
+
+// blocks of a kernel resident on the device (the same on every GB300), with its
+// shared memory allowed; each launcher asks once (the initialisation of its
+// static is the one that threads wait for)
+template <class K>
+int wave_of(K* kernel, int threads, int smem) {
+    int per = 0;
+    if (smem) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+    return sm_count() * std::max(per, 1);
+}
+
 template <int DIMS, int MODE, bool ABL, int G>
 void launch_g2b_one(const Launch& L) {
-    static int wave = 0;   // blocks resident on the device (the same on every GB300)
-    if (!wave) {
-        int dev = 0, sms = 152, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2b<DIMS, MODE, ABL, G>, 32 * G, 0);
-        wave = sms * std::max(per, 1);
-    }
+    static const int wave = wave_of(k_g2b<DIMS, MODE, ABL, G>, 32 * G, 0);
     const int grid = std::max(1, std::min(wave, L.cells));
     k_g2b<DIMS, MODE, ABL, G><<<grid, 32 * G, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles, L.wq);
 }
 
 template <int DIMS, int MODE, bool ABL, int BLOCKS>
 void launch_g2_blocks(const Launch& L, int group, cudaStream_t st) {
-    static int wave = 0;
     constexpr int smem = (int)(kG2wWarps * sizeof(G2Warp<DIMS, ABL, BLOCKS>));
-    if (!wave) {
-        int dev = 0, sms = 152, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_g2<DIMS, MODE, ABL, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2<DIMS, MODE, ABL, BLOCKS>, 32 * kG2wWarps, smem);
-        wave = sms * std::max(per, 1);
-    }
+    static const int wave = wave_of(k_g2<DIMS, MODE, ABL, BLOCKS>, 32 * kG2wWarps, smem);
     const int grid = std::max(1, std::min(wave, (L.cells + kG2wWarps - 1) / kG2wWarps));
     k_g2<DIMS, MODE, ABL, BLOCKS><<<grid, 32 * kG2wWarps, smem, st>>>(
         L.sims, L.ctiles, L.gtiles ? L.gtiles + group : L.nctiles, L.gtiles ? L.gtiles + kG2Groups + group : nullptr,
@@ -2774,13 +2779,7 @@ void launch_fused_moments(const Launch& L) {
 }
 
 void launch_fused_params(const Launch& L) {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0, n = 152;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        sms = n;
-    }
-    const int grid = std::max(1, std::min((L.cells - 1) / kCTile + 1, kParamsBlocks * sms));
+    const int grid = std::max(1, std::min((L.cells - 1) / kCTile + 1, kParamsBlocks * sm_count()));
     k_params_f<<<grid, 32, 0, L.stream>>>(L.sims, L.ctiles, L.nctiles);
 }
 

@@ -18,3 +18,11 @@ def test_a_bounded_wait_is_decided_by_the_whole_warp():
     body = code[code.index("k_g2(const SimDev"):]
     used = re.findall(r"=\s*(__all_sync\(0xffffffffu,\s*)?mbar_wait\(", body)
     assert used and all(used)
+
+
+def test_launchers_keep_no_state_that_threads_write():
+    """Handles are stepped from several threads: what a launcher finds out
+    once is initialised as a constant, which the language does under a lock."""
+    for name in os.listdir(build.CSRC):
+        code = _code(name)
+        assert not re.findall(r"\bstatic\s+(?:int|bool|unsigned|uint32_t|size_t|float|double)\s+\w+\s*(?:=|;|\[)", code), name
