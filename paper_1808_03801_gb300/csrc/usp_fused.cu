@@ -28,6 +28,7 @@
 // Each particle is read once and written once by k_g2 and its velocity is
 // read once more by k_g1.
 #include <algorithm>
+#include <cstddef>
 
 #include "usp_device.cuh"
 
@@ -897,9 +898,13 @@ struct alignas(16) G2Warp {
     float prm[2][kNFPrm];  // parameter records of the cell and of the next one
     SimDev sim;
     uint32_t key[20];
-    // per window slot: its arrivals, then its first reserved index; start and end
-    // of its bucket (before that the digit counts of a fixed-count selection)
-    uint32_t win[ABL ? 256 : 3 * kWin];
+    uint32_t wst[kWin];    // arrivals per window slot, then its first reserved index
+    uint32_t wlo[kWin];    // start and end of the slot's bucket
+    uint32_t wend[ABL ? 2 * kWin : kWin];
+    // the digit counts of a fixed-count selection, before the window is used
+    __device__ __forceinline__ uint32_t* hist() {
+        return reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(this) + offsetof(G2Warp, wst));
+    }
     int2 ptile[4];         // the cells on their way: tile,
     uint32_t pbound[4][4]; // bucket start, end and arrivals,
     uint32_t punit[4];     // unit number
@@ -1079,17 +1084,18 @@ __device__ __noinline__ G2Fixed g2w_fixed(Sh& sh, G2Sim S, G2Job J, uint32_t nsp
     F.quota = F.eq = 0;
     F.inv_thr = 1.0f;
     if (F.ns == 0) return F;
+    uint32_t* const hist = sh.hist();
     uint32_t prefix = 0, mask = 0, rem = F.ns;
     for (int shift = 24; shift >= 0; shift -= 8) {
         __syncwarp();
-        for (int b = lane; b < 256; b += 32) sh.win[b] = 0u;
+        for (int b = lane; b < 256; b += 32) hist[b] = 0u;
         __syncwarp();
         g2w_words<GEN>(sh, S, J, nsp, lane, [&](uint32_t, uint32_t k) {
-            if ((k & mask) == prefix) atomicAdd(&sh.win[(k >> shift) & 255u], 1u);
+            if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1u);
         });
         __syncwarp();
         uint32_t below;
-        const uint32_t d = radix_digit(sh.win, rem, lane, below);
+        const uint32_t d = radix_digit(hist, rem, lane, below);
         rem -= below;
         prefix |= d << shift;
         mask |= 0xFFu << shift;
@@ -1170,10 +1176,10 @@ __device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, S
     for (int h = 0; MODE != kRelaxOnly && h < 2; ++h) {
         const int k = lane + 32 * h, dest = win_cell<DIM>(k, cell, cx, cy, s.nx);
         if ((unsigned)dest < (unsigned)s.K) {
-            cp_async4(&sh.win[kWin + k], &s.lay[q][dest]);
-            cp_async4(&sh.win[2 * kWin + k], &s.lay[q][dest + 1]);
+            cp_async4(&sh.wlo[k], &s.lay[q][dest]);
+            cp_async4(&sh.wend[k], &s.lay[q][dest + 1]);
         }
-        sh.win[k] = 0;
+        sh.wst[k] = 0;
     }
     const uint32_t nch = GEN ? (n + CAP - 1) / CAP : 1u;
     float R[8];
@@ -1370,7 +1376,7 @@ __device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, S
             }
             const int slot = win_slot_xy<DIM>(ix, iy - row0, gcell, cx, cy);
             uint32_t sr = alive ? kPackFar : kPackNone;
-            if (alive && slot >= 0) sr = (uint32_t)slot | (atomicAdd(&sh.win[slot], 1u) << 6);
+            if (alive && slot >= 0) sr = (uint32_t)slot | (atomicAdd(&sh.wst[slot], 1u) << 6);
             return sr;
         };
         auto fly = [&](auto nt, uint32_t b) {
@@ -1454,9 +1460,9 @@ __device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, S
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int k = lane + 32 * h;
-            const uint32_t c = sh.win[k];
-            if (c) sh.win[k] = sh.win[kWin + k] + atom_add_global(&s.cnt[q][win_cell<DIM>(k, cell, cx, cy, s.nx)], c);
-            sh.win[2 * kWin + k] = min(sh.win[2 * kWin + k], (uint32_t)s.cap);
+            const uint32_t c = sh.wst[k];
+            if (c) sh.wst[k] = sh.wlo[k] + atom_add_global(&s.cnt[q][win_cell<DIM>(k, cell, cx, cy, s.nx)], c);
+            sh.wend[k] = min(sh.wend[k], (uint32_t)s.cap);
         }
         // ---- sweep 3 ----
         float* const dx = (float*)s.pos[q][0];
@@ -1483,8 +1489,8 @@ __device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, S
             }
 #pragma unroll
             for (int t = 0; t < N; ++t) {
-                i[t] = sh.win[sr[t] & 63u] + (sr[t] >> 6);
-                in[t] = sr[t] < kPackOther && i[t] < sh.win[2 * kWin + (sr[t] & 63u)];
+                i[t] = sh.wst[sr[t] & 63u] + (sr[t] >> 6);
+                in[t] = sr[t] < kPackOther && i[t] < sh.wend[sr[t] & 63u];
                 odd = odd || (!in[t] && sr[t] != kPackNone);
             }
             if (__any_sync(0xffffffffu, odd)) {   // not in the window, or the bucket is full
@@ -1534,8 +1540,8 @@ __device__ __forceinline__ void g2w_cell_impl(const SimDev* __restrict__ sims, S
         }
         if (GEN && it + 1 < 2 * nch - 1) {   // the window of the next chunk
             __syncwarp();
-            sh.win[lane] = 0;
-            sh.win[lane + 32] = 0;
+            sh.wst[lane] = 0;
+            sh.wst[lane + 32] = 0;
         }
     }
     __syncwarp();
@@ -1710,12 +1716,14 @@ __global__ void __launch_bounds__(32 * kG2wWarps, BLOCKS) k_g2(const SimDev* __r
             }
         }
         if (J.arrived) {
-            G2Acc a = {0u, 0u};
-            if (general) a = g2w_cell_call<DIMS, MODE, ABL, true>(sims, sh, S, J, 0u, lane);
-            else if (ABL) a = g2w_cell_call<DIMS, MODE, ABL, false>(sims, sh, S, J, par, lane);
-            else g2w_cell_impl<DIMS, MODE, ABL, false>(sims, sh, S, J, par, 0u, lane, acc);
-            acc.relaxed += a.relaxed;
-            acc.removed += a.removed;
+            if (ABL || general) {
+                const G2Acc a = !ABL || general ? g2w_cell_call<DIMS, MODE, ABL, true>(sims, sh, S, J, 0u, lane)
+                                                : g2w_cell_call<DIMS, MODE, ABL, false>(sims, sh, S, J, par, lane);
+                acc.relaxed += a.relaxed;
+                acc.removed += a.removed;
+            } else {
+                g2w_cell_impl<DIMS, MODE, ABL, false>(sims, sh, S, J, par, 0u, lane, acc);
+            }
             fence_proxy_async_smem();   // later copies come after these accesses
             __syncwarp();
         }
