@@ -33,7 +33,7 @@ FUSED_SRC = os.path.join(ROOT, "paper_1808_03801_gb300", "csrc", "usp_fused.cu")
 # dram__bytes_write.sum of the 32-tube Sod case divided by its particles),
 # valid only for the k_g2 source with this SHA-1; any other source reports
 # traffic as null until it is captured again
-KG2_TRAFFIC = {"sha1": "8c83d9cf92c90238f2b1b9e40bdefc4b699de37a", "bytes_per_particle": 38.81}
+KG2_TRAFFIC = {"sha1": "f57b01b769e92b80541702fdfa0cd5c3c6082d53", "bytes_per_particle": 38.75}
 
 
 def parse():
