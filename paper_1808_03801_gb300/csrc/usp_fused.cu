@@ -133,8 +133,7 @@ __device__ __forceinline__ void spill(const SimDev& s, int b, int cell, float x,
 // per thread (measured per launch, one warp per cell -> block per cell: 100
 // cells of 200 particles 21 -> 13 us, one shock tube of 1000 cells 30 -> 18 us;
 // with 4e4 cells of 100 particles the barriers and the per-warp share of the
-// cell's work cost more than they give, 117 -> 230 us).  It also carries the
-// forms that are seldom run: in-place relaxation, slabs, the ablations.
+// cell's work cost more than they give, 117 -> 230 us).
 // Cells above 32 G kG2P particles go through in chunks: a first sweep for the
 // conservation sums, a second one (in reverse, so that the last chunk is
 // still in registers) that draws the same counter-based random numbers again.
@@ -873,6 +872,9 @@ __device__ __forceinline__ void load_sim_warp(SimDev& dst, const SimDev& src, in
 // per SM with 128 registers and no spills measured best (12 and 14 warps with
 // more staging, 18 and 20 with less and some spills: 3-50 % slower), and so did
 // bulk copies (per-lane 16-byte copies took three times as long to issue).
+// Two codings of the same cell can differ by 1 % in 2-D, where the kernel is at
+// the edge of the instruction cache (the window as one array: 157.5 -> 158.3 us a
+// step of the cavity).
 // What bounds it: the warps' dependent instructions (370 per 32 particles in
 // 1-D, 48 % issue) and, for dense cells, the copy that cannot start before the
 // cell ahead is written.  Against the form before it (a producer warp feeding
