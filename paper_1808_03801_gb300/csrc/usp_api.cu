@@ -642,6 +642,7 @@ static int alloc_particles(usp_handle* h, int64_t n) {
     // allocates nothing); the tile tables and the captured graphs depend only
     // on the capacity
     if (!h->part_allocs.empty() && cap <= s.cap && 2 * cap > s.cap) return USP_OK;
+    h->initialised = false;   // should an allocation fail, there is nothing left to step
     destroy_graphs(h->graphs);
     free_particles(h);
     const size_t es = h->precision == USP_FP64 ? 8 : 4;
@@ -706,7 +707,10 @@ static int alloc_particles(usp_handle* h, int64_t n) {
     }
     void* p;
     int rc = cell_alloc(h, sizeof(int2) * (size_t)h->nptiles, &p);
-    if (rc) return rc;
+    if (rc) {
+        free_particles(h);   // (a retry must not take the storage for complete)
+        return rc;
+    }
     h->d_ptiles = (int2*)p;
     std::vector<int2> pt(h->nptiles);
     for (int t = 0; t < h->nptiles; ++t) pt[t] = make_int2(0, t * kPTile);
@@ -714,7 +718,10 @@ static int alloc_particles(usp_handle* h, int64_t n) {
     cudaError_t e = cudaMemcpyAsync(h->d_ptiles, pt.data(), sizeof(int2) * pt.size(), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d_ntiles, nt, sizeof(nt), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return fail(h, USP_ERR_CUDA, cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        free_particles(h);
+        return fail(h, USP_ERR_CUDA, cudaGetErrorString(e));
+    }
     return USP_OK;
 }
 
@@ -781,6 +788,7 @@ extern "C" int usp_init_particles(usp_handle* h, const usp_region* regions, int 
     start[K] = start[K + 1] = (uint32_t)total;
     int rc = alloc_particles(h, (int64_t)total);
     if (rc) return rc;
+    h->initialised = false;   // from here on the state is the load's
     s.key0 = (uint32_t)seed;
     s.key1 = (uint32_t)(seed >> 32);
     if ((rc = upload_sim(h)) != 0) return rc;
@@ -870,6 +878,7 @@ extern "C" int usp_set_particles(usp_handle* h, int64_t n, const double* pos, co
     if (n > (int64_t)0x7FFFFFF0) return fail(h, USP_ERR_CAPACITY, "too many particles");
     int rc = alloc_particles(h, n);
     if (rc) return rc;
+    h->initialised = false;   // from here on the state is the load's
     SimDev& s = h->host;
     s.key0 = (uint32_t)seed;
     s.key1 = (uint32_t)(seed >> 32);
