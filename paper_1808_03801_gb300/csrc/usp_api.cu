@@ -643,6 +643,8 @@ static int alloc_particles(usp_handle* h, int64_t n) {
     // on the capacity
     if (!h->part_allocs.empty() && cap <= s.cap && 2 * cap > s.cap) return USP_OK;
     h->initialised = false;   // should an allocation fail, there is nothing left to step
+    // a caller's allocator may hand memory out again at once: no step may still use it
+    if (!h->part_allocs.empty()) CK(cudaStreamSynchronize(h->stream));
     destroy_graphs(h->graphs);
     free_particles(h);
     const size_t es = h->precision == USP_FP64 ? 8 : 4;

@@ -1,6 +1,8 @@
-"""GPU tests of a load that runs out of memory on a handle that has stepped:
-whichever allocation fails, the handle has no state to step (STATE), is not
-left with part of its storage, and loads and steps again once there is memory."""
+"""GPU tests of loads that replace a stepped handle's storage.  One that runs
+out of memory: whichever allocation fails, the handle has no state to step
+(STATE), is not left with part of its storage, and loads and steps again once
+there is memory.  Storage goes back to the caller's allocator only when no step
+uses it any more."""
 import ctypes
 import math
 
@@ -100,3 +102,21 @@ def test_a_load_that_runs_out_of_memory(usp, memory, pipeline, how):
         if not failed:
             break
     assert 6 < k < 20 and not memory.held
+
+
+def test_storage_is_given_back_when_no_step_uses_it(usp, memory):
+    """Steps are still running when a larger state is loaded."""
+    w = W.cavity(n=100, ppc=100)
+    w["params"]["pipeline"] = "fused"
+    g = usp.Simulation(w, allocator="torch").init_particles().step(8)
+    g.synchronize()
+    idle = []
+    memory.on_free = lambda: idle.append(g.stream.query())
+    pos, vel, pid = W.bimaxwellian(3_000_000, seed=4, y_range=(0.0, 1.0e-4), x_range=(0.0, 1.0e-4))
+    g.step(2000)
+    assert not g.stream.query()
+    g.set_particles(pos, vel, pid)
+    memory.on_free = None
+    assert len(idle) >= 7 and all(idle)
+    assert g.step(1).info()["counters"][5] == 0
+    g.close()
