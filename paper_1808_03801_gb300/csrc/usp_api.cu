@@ -202,7 +202,9 @@ static int upload_sim(usp_handle* h) {
 // Few cells: up to ten per SM.  Measured per k_g2 launch, R = 4 / 8 / 12: 100
 // cells of 200 particles 21 / 15 / 13 us; 1000 cells of 360 / 45 particles 30 /
 // 18 / 23 us; 5929 cells of 37 particles 28 / 44 / - us.  Eight warps pay where
-// every block has an SM to itself, and for cells above the 512 particles that
+// there are no more than two cells per SM (300 cells of 200 particles 22.6 us a
+// step with four warps, 20.8 with eight; in a batch of three domains of 100, whose
+// slots are 384, 23.8 and 25.3), and for cells above the 512 particles that
 // four warps hold (per step, 8 / 12: 1000 cells of 400 particles 31 / 35 us, of
 // 600 40.5 / 39).
 //
@@ -222,13 +224,14 @@ struct G2Form {
     int R, blocks;
 };
 
-static G2Form choose_form(int64_t cells, int ppc, int dim) {
+// units: cell slots that the block form deals out (a batch's tiles are padded)
+static G2Form choose_form(int64_t cells, int ppc, int dim, int64_t units = 0) {
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const double dense = ppc, sd = std::sqrt(dense);
     const int blocks = dense + 2 * sd > kG2Stage[1][dim - 1] && dense + sd <= kG2Stage[0][dim - 1] ? 3 : 4;
     int R;
-    if (cells <= 10 * (int64_t)sms) R = (cells <= 2 * (int64_t)sms && ppc > 128) || dense + 2 * sd > 512 ? 12 : 8;
+    if (cells <= 10 * (int64_t)sms) R = (std::max(cells, units) <= 2 * (int64_t)sms && ppc > 128) || dense + 2 * sd > 512 ? 12 : 8;
     else if (cells <= 20 * (int64_t)sms && dense + 2 * sd > kG2Stage[0][dim - 1]) R = 12;
     else R = dim == 2 && ppc > 700 ? 12 : 4;
     return {R, blocks};
@@ -1372,13 +1375,14 @@ extern "C" int usp_batch_retire(usp_batch* b, usp_handle* h) {
 // a member was tuned
 static G2Form batch_form(const usp_batch* b) {
     int tuned = 0;
-    int64_t cells = 0, total = 0, dense = 0, three = 0;
+    int64_t cells = 0, units = 0, total = 0, dense = 0, three = 0;
     for (auto* h : b->members) {
         if (h->tuned) tuned = std::max(tuned, h->fused_R);
         cells += h->host.K;
+        units += (int64_t)h->nctiles * kCTile;
     }
     for (auto* h : b->members) {
-        const G2Form f = choose_form(cells, h->ppc_ref, h->host.dim);
+        const G2Form f = choose_form(cells, h->ppc_ref, h->host.dim, units);
         total += h->host.cap;
         if (f.R == 12) dense += h->host.cap;
         if (f.blocks == 3) three += h->host.cap;
